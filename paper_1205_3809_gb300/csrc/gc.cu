@@ -172,7 +172,7 @@ int ensure_device_limited(void** p, size_t* have, size_t need, int32_t limit_mb)
 
 struct Layout {
     size_t st, stats, rs, rv, rt, x0, x1, act0, act1, stat, hubs, defer;
-    size_t S[2], M[2], H[2], Hc[2], O[2];
+    size_t T[2], S[2], M[2], H[2], Hc[2], O[2];
     size_t total;
 };
 
@@ -197,7 +197,9 @@ Layout make_layout(int64_t n, int64_t nnz, size_t elem, const Stats& hs, int64_t
     L.hubs = take((size_t)hs.cap[gc::kBinH] * sizeof(gc::HubRecord));
     L.defer = take((size_t)hs.defer * sizeof(int32_t));
     for (int b = 0; b < 2; ++b) {
-        L.S[b] = take((size_t)hs.cap[gc::kBinS] * sizeof(int4));
+        // degree 1 .. s_max: T; longer rows whose active list has shrunk to s_max: S
+        L.T[b] = take((size_t)(hs.cap[gc::kBinS] - hs.cap[gc::kBinM]) * sizeof(int4));
+        L.S[b] = take((size_t)hs.cap[gc::kBinM] * sizeof(int4));
         L.M[b] = take((size_t)hs.cap[gc::kBinM] * sizeof(int4));
         L.H[b] = take((size_t)hs.cap[gc::kBinH] * sizeof(int4));
         L.Hc[b] = take((size_t)hs.cap[gc::kBinH] * sizeof(int32_t));
@@ -323,8 +325,8 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
     for (;; ++k) {
         GC_CUDA(cudaMemcpyAsync(h, &st->rc[k % 3], sizeof(gc::RoundCounts), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
-        const unsigned nS = h->s, nM = h->m, nH = gc::hub_count(h->hc), nHC = gc::hub_chunks(h->hc);
-        const unsigned size = nS + nM + nH;
+        const unsigned nT = h->t, nS = h->s, nM = h->m, nH = gc::hub_count(h->hc), nHC = gc::hub_chunks(h->hc);
+        const unsigned size = nT + nS + nM + nH;
         if (size == 0) break;
         if (k > p.max_rounds) {
             hs[1] = gc::kStatusMaxRounds;
@@ -337,11 +339,12 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
                                     cudaMemcpyHostToDevice, s));
         }
         GC_CUDA(cudaMemsetAsync(&st->rc[(k + 2) % 3], 0, sizeof(gc::RoundCounts), s));
-        const int64_t tasks = (int64_t)nHC + (nM + gc::kMedPerTask - 1) / gc::kMedPerTask + (nS + 31) / 32;
+        const int64_t tasks = (int64_t)nHC + (nM + gc::kMedPerTask - 1) / gc::kMedPerTask + (nS + 31) / 32 +
+                              (nT + 31) / 32;
         const int64_t warps_per_block = threads / 32;
         const int grid = (int)std::max<int64_t>(
             1, std::min<int64_t>((tasks + warps_per_block - 1) / warps_per_block, (int64_t)dc.sms * 8));
-        gc::round_kernel<T, P><<<grid, threads, 0, s>>>(p, k, nS, nM, nHC);
+        gc::round_kernel<T, P><<<grid, threads, 0, s>>>(p, k, nT, nS, nM, nHC);
         GC_CUDA(cudaGetLastError());
         *launches += 1;
     }
@@ -502,6 +505,7 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
             p.colidx = colidx;
             p.prio = priority;
             p.n = n;
+            p.nnz = hs.nnz;
             p.s_max = o.small_max_degree;
             p.m_max = o.medium_max_degree;
             p.max_rounds = max_rounds;
@@ -516,11 +520,13 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
             p.act0 = (int32_t*)(base + L.act0);
             p.act1 = (int32_t*)(base + L.act1);
             p.stat = (uint32_t*)(base + L.stat);
+            p.TA = (int4*)(base + L.T[0]);
             p.SA = (int4*)(base + L.S[0]);
             p.MA = (int4*)(base + L.M[0]);
             p.HA = (int4*)(base + L.H[0]);
             p.HcA = (int32_t*)(base + L.Hc[0]);
             p.OA = (int32_t*)(base + L.O[0]);
+            p.TB = (int4*)(base + L.T[1]);
             p.SB = (int4*)(base + L.S[1]);
             p.MB = (int4*)(base + L.M[1]);
             p.HB = (int4*)(base + L.H[1]);
@@ -698,6 +704,7 @@ int color_noalloc_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n
             p.colidx = colidx;
             p.prio = priority;
             p.n = n;
+            p.nnz = hs.nnz;
             p.s_max = o.small_max_degree;
             p.m_max = o.medium_max_degree;
             p.max_rounds = n;
@@ -711,11 +718,13 @@ int color_noalloc_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n
             p.act0 = (int32_t*)(base + L.act0);
             p.act1 = (int32_t*)(base + L.act1);
             p.stat = (uint32_t*)(base + L.stat);
+            p.TA = (int4*)(base + L.T[0]);
             p.SA = (int4*)(base + L.S[0]);
             p.MA = (int4*)(base + L.M[0]);
             p.HA = (int4*)(base + L.H[0]);
             p.HcA = (int32_t*)(base + L.Hc[0]);
             p.OA = (int32_t*)(base + L.O[0]);
+            p.TB = (int4*)(base + L.T[1]);
             p.SB = (int4*)(base + L.S[1]);
             p.MB = (int4*)(base + L.M[1]);
             p.HB = (int4*)(base + L.H[1]);
@@ -775,11 +784,13 @@ void fill_workspace(Params<T>& p, char* base, const Layout& L, RoundState* st, i
     p.act0 = (int32_t*)(base + L.act0);
     p.act1 = (int32_t*)(base + L.act1);
     p.stat = (uint32_t*)(base + L.stat);
+    p.TA = (int4*)(base + L.T[0]);
     p.SA = (int4*)(base + L.S[0]);
     p.MA = (int4*)(base + L.M[0]);
     p.HA = (int4*)(base + L.H[0]);
     p.HcA = (int32_t*)(base + L.Hc[0]);
     p.OA = (int32_t*)(base + L.O[0]);
+    p.TB = (int4*)(base + L.T[1]);
     p.SB = (int4*)(base + L.S[1]);
     p.MB = (int4*)(base + L.M[1]);
     p.HB = (int4*)(base + L.H[1]);
@@ -951,6 +962,7 @@ int batch_enqueue_typed(gc_batch& b, cudaStream_t s) {
     p.colidx = colidx_g;
     p.prio = b.prio;
     p.n = (int32_t)b.N;
+    p.nnz = (int32_t)b.NNZ;
     p.s_max = b.o.small_max_degree;
     p.m_max = b.o.medium_max_degree;
     p.max_rounds = b.o.max_rounds > 0 ? b.o.max_rounds : (int32_t)b.N;
@@ -1200,7 +1212,7 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     // the coloring layout's offsets are relative to its own base
     Layout& L = b->L;
     size_t* fields[] = {&L.st, &L.stats, &L.rs, &L.rv, &L.rt, &L.x0, &L.x1, &L.act0, &L.act1, &L.stat, &L.hubs,
-                        &L.defer, &L.S[0], &L.S[1], &L.M[0], &L.M[1], &L.H[0], &L.H[1], &L.Hc[0], &L.Hc[1],
+                        &L.defer, &L.T[0], &L.T[1], &L.S[0], &L.S[1], &L.M[0], &L.M[1], &L.H[0], &L.H[1], &L.Hc[0], &L.Hc[1],
                         &L.O[0], &L.O[1]};
     for (size_t* f : fields) *f += lay;
 

@@ -28,9 +28,14 @@
 // flag makes 16-bit state hold colors < 2^15: a larger color sets an
 // overflow status and the host reruns with 32-bit state.
 //
-// Work is split into warp-sized tasks, binned by the current active length:
-//   S bin (length <= s_max <= 32): 32 worklist entries per task (down to 4
-//     in the small rounds at the end), their lists walked as one flat range;
+// Work is split into warp-sized tasks, binned by the current active length
+// (T: by degree):
+//   T bin (degree <= s_max <= 32): the row is read from the graph itself in
+//     32-byte chunks, with one bit per entry for "not settled yet" in the
+//     worklist entry; no list is kept;
+//   S bin (longer rows whose list has shrunk to s_max): 32 worklist entries per
+//     task (down to 4 in the small rounds at the end), their lists walked as
+//     one flat range;
 //   M bin (s_max < length <= m_max <= 256): up to 16 worklist entries per
 //     task, each list read by the whole warp in turn (colors 1..64 in
 //     registers);
@@ -78,6 +83,11 @@ constexpr int kPass1LongBlocksPerSm = 8;      // pass 1, long rows: grid of 8 bl
 constexpr int kFlatBatches = GC_FLAT_BATCHES;  // flat tasks: batches in flight together
 constexpr int kMedPerTask = GC_MED_PER_TASK;   // M-bin vertices per task
 constexpr int kShortPerTaskMin = 4;            // S-bin vertices per task in a small round
+#ifndef GC_TINY_LANES
+#define GC_TINY_LANES 4
+#endif
+constexpr int kTinyLanes = GC_TINY_LANES;      // T bin: lanes per vertex
+constexpr int kTinyPerStep = 32 / kTinyLanes;  // T bin: vertices a warp reads side by side
 constexpr int kMinBlocks = GC_MIN_BLOCKS;      // round kernels: blocks per SM the registers allow
 constexpr int kWarpsPerBlockMax = 8;          // blocks of <= 256 threads
 
@@ -121,6 +131,7 @@ struct Stats {
 // than any other.  A hub's two counters (its worklist position and its first
 // chunk) share one 64-bit word, taken with one atomic.
 struct RoundCounts {
+    alignas(128) unsigned t;               // |U_k in T|
     alignas(128) unsigned s;               // |U_k in S|
     alignas(128) unsigned m;               // |U_k in M|
     alignas(128) unsigned long long hc;    // |U_k in H| (bits 0..31) | chunks of U_k in H (bits 32..63)
@@ -162,6 +173,7 @@ struct Params {
     const int32_t* __restrict__ colidx;
     const uint32_t* __restrict__ prio;  // NULL = index priority
     int32_t n;
+    int32_t nnz;                        // entries of colidx
     int32_t s_max, m_max;               // length bin limits
     int32_t max_rounds;
     int32_t tail_volume;                // rounds reading <= this many entries run in block 0 alone (< 0: never)
@@ -174,11 +186,11 @@ struct Params {
     int32_t* act0;                      // active lists (row starts as in colidx)
     int32_t* act1;
     uint32_t* stat;                     // static masks, 8 words per vertex
-    // worklists per parity (A: even k, B: odd k): S, M, H entries
-    // {vertex, row start, active length, degree}, first chunk of each H
-    // entry, owner position of each chunk
-    int4* SA; int4* MA; int4* HA; int32_t* HcA; int32_t* OA;
-    int4* SB; int4* MB; int4* HB; int32_t* HcB; int32_t* OB;
+    // worklists per parity (A: even k, B: odd k): T entries {vertex, row start,
+    // live entries, static mask}; S, M, H entries {vertex, row start, active
+    // length, degree}, first chunk of each H entry, owner position of each chunk
+    int4* TA; int4* SA; int4* MA; int4* HA; int32_t* HcA; int32_t* OA;
+    int4* TB; int4* SB; int4* MB; int4* HB; int32_t* HcB; int32_t* OB;
     int32_t* defer;                     // pass 1: rows longer than kPass1Flat
     HubRecord* hubs;
     RoundState* st;
@@ -298,7 +310,7 @@ __device__ __forceinline__ void warp_append_i32(bool flag, int32_t v, int32_t* l
 
 // Where the next round's worklists go.
 struct NextLists {
-    int4* S; int4* M; int4* H; int32_t* Hc; int32_t* O;
+    int4* T; int4* S; int4* M; int4* H; int32_t* Hc; int32_t* O;
     RoundCounts* cnt;  // the next round's counts
     int32_t s_max, m_max;
 };
@@ -350,6 +362,9 @@ __device__ __forceinline__ void warp_append_hubs(const NextLists& nl, bool flag,
     }
 }
 
+// The lowest d bits (0 <= d <= 32).
+__device__ __forceinline__ uint32_t low_bits(int32_t d) { return d >= 32 ? 0xffffffffu : (1u << d) - 1u; }
+
 // Append one entry held by lane 0 (any bin).  Called by all lanes of a warp.
 __device__ __forceinline__ void warp_append_one(const NextLists& nl, int4 e) {
     const int bin = bin_of(e.z, nl.s_max, nl.m_max);
@@ -359,6 +374,13 @@ __device__ __forceinline__ void warp_append_one(const NextLists& nl, int4 e) {
         int4* list = bin == kBinM ? nl.M : nl.S;
         list[atomicAdd(bin == kBinM ? &nl.cnt->m : &nl.cnt->s, 1u)] = e;
     }
+}
+
+// x << s with shifts of 32 and more (or "negative" ones) giving 0.
+__device__ __forceinline__ uint32_t shl_clamp(uint32_t x, uint32_t s) {
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));
+    return r;
 }
 
 // Bits of colors base+1 .. base+256 seen by one lane.
@@ -555,7 +577,7 @@ __device__ __forceinline__ void pass1_write(const Params<T>& p, int32_t v, bool 
 template <typename T>
 __device__ __forceinline__ NextLists pass1_next(const Params<T>& p) {
     NextLists nl;
-    nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
+    nl.T = p.TA; nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
     nl.cnt = &p.st->rc[2];
     nl.s_max = p.s_max;
     nl.m_max = p.m_max;
@@ -572,7 +594,7 @@ __device__ __forceinline__ NextLists pass1_next(const Params<T>& p) {
 // precedes it.  Longer rows go to pass1_long_kernel.
 template <typename T>
 __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_begin, int32_t v_end) {
-    // a warp takes two tasks (t, t + W) at a time and appends their S and M
+    // a warp takes two tasks (t, t + W) at a time and appends their T and M
     // entries with one atomic per bin: every task appends to both, and the
     // counters' lines were the busiest of the L2 in this kernel
     constexpr int NT = 2;
@@ -592,7 +614,7 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
     unsigned vol = 0;
     for (int64_t t0 = gw; t0 < ntasks; t0 += W * NT) {
         int4 ev[NT];
-        bool fS[NT], fM[NT];
+        bool fT[NT], fM[NT];
 #pragma unroll
         for (int jt = 0; jt < NT; ++jt) {
             const int64_t t = t0 + (int64_t)jt * W;
@@ -650,8 +672,9 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
             }
             const int bin = bin_of(d, p.s_max, p.m_max);
             const bool go = valid && !longrow && hit;
-            ev[jt] = make_int4(v, b, d, d);
-            fS[jt] = go && bin == kBinS;
+            // a row of at most s_max entries starts as a T entry: all of it live, no static mask
+            ev[jt] = bin == kBinS ? make_int4(v, b, (int32_t)low_bits(d), 0) : make_int4(v, b, d, d);
+            fT[jt] = go && bin == kBinS;
             fM[jt] = go && bin == kBinM;
             // hubs that stayed in the flat range (m_max < d <= kPass1Flat)
             unsigned hubs = __ballot_sync(kFull, go && bin == kBinH);
@@ -663,20 +686,20 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
             }
             warp_append_i32(valid && longrow, v, p.defer, &p.st->defer_cnt);
         }
-        // the S and M entries of these NT tasks, one atomic per bin
+        // the T and M entries of these NT tasks, one atomic per bin
 #pragma unroll
         for (int bin = 0; bin < 2; ++bin) {
             unsigned bal[NT], n = 0;
 #pragma unroll
             for (int jt = 0; jt < NT; ++jt) {
-                bal[jt] = __ballot_sync(kFull, bin == 0 ? fS[jt] : fM[jt]);
+                bal[jt] = __ballot_sync(kFull, bin == 0 ? fT[jt] : fM[jt]);
                 n += __popc(bal[jt]);
             }
             if (n == 0) continue;
             unsigned base = 0;
-            if (lane == 0) base = atomicAdd(bin == 0 ? &nl.cnt->s : &nl.cnt->m, n);
+            if (lane == 0) base = atomicAdd(bin == 0 ? &nl.cnt->t : &nl.cnt->m, n);
             base = __shfl_sync(kFull, base, 0);
-            int4* const list = bin == 0 ? nl.S : nl.M;
+            int4* const list = bin == 0 ? nl.T : nl.M;
 #pragma unroll
             for (int jt = 0; jt < NT; ++jt) {
                 if ((bal[jt] >> lane) & 1u) list[base + __popc(bal[jt] & ((1u << lane) - 1u))] = ev[jt];
@@ -751,7 +774,7 @@ struct PassIO {
     const int32_t* rin;     // active lists read this round (colidx in round 2)
     int32_t* rout;          // active lists written for the next round
     bool first;             // round 2: no static masks yet
-    const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
+    const int4* T_; const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
     NextLists next;
     uint64_t pol_row, pol_col;
 };
@@ -767,11 +790,13 @@ __device__ __forceinline__ PassIO<T> pass_io(const Params<T>& p, int k) {
     io.k = k;
     io.rin = k == 2 ? p.colidx : (odd ? p.act1 : p.act0);
     io.rout = odd ? p.act0 : p.act1;
+    io.T_ = odd ? p.TB : p.TA;
     io.S = odd ? p.SB : p.SA;
     io.M = odd ? p.MB : p.MA;
     io.H = odd ? p.HB : p.HA;
     io.Hc = odd ? p.HcB : p.HcA;
     io.O = odd ? p.OB : p.OA;
+    io.next.T = odd ? p.TA : p.TB;
     io.next.S = odd ? p.SA : p.SB;
     io.next.M = odd ? p.MA : p.MB;
     io.next.H = odd ? p.HA : p.HB;
@@ -804,29 +829,44 @@ __device__ __forceinline__ void recolor(const Params<T>& p, const PassIO<T>& io,
 
 // What a warp needs to start a task.  Loaded one task ahead.
 struct TaskHead {
-    int4 e;       // {vertex, row start, active length, degree}; x < 0 marks an empty slot
+    int4 e;       // worklist entry; x < 0 marks an empty slot
     int32_t pos;  // H chunk: worklist position of its vertex
     int32_t lo;   // H chunk: first entry of the chunk
 };
 
+// The tasks of one round, in the order they are dealt out: H chunks, M, S, T.
+struct TaskSplit {
+    unsigned nT, nS, nM, nHC;       // T, S, M entries; H chunks
+    unsigned mpt, spt, tsub;        // M and S entries per task; groups of kTinyPerStep T entries per task
+    unsigned tM, tS, total;         // tasks of M and S; of the round
+};
+
 template <typename T>
-__device__ __forceinline__ TaskHead load_head(const PassIO<T>& io, unsigned t, unsigned nS,
-                                              unsigned nM, unsigned nHC, unsigned tM, unsigned mpt,
-                                              unsigned spt) {
+__device__ __forceinline__ TaskHead load_head(const PassIO<T>& io, unsigned t, const TaskSplit& q) {
     TaskHead h;
     h.pos = 0;
     h.lo = 0;
-    if (t < nHC) {
+    if (t < q.nHC) {
         h.pos = __ldcg(io.O + t);
         h.e = __ldcg(io.H + h.pos);
         h.lo = h.e.y + ((int32_t)t - __ldcg(io.Hc + h.pos)) * kChunk;
-    } else if (t - nHC < tM) {
-        const unsigned i = (t - nHC) * mpt + lane_id();
-        h.e = (lane_id() < mpt && i < nM) ? __ldcg(io.M + i) : make_int4(-1, 0, 0, 0);
-    } else {
-        const unsigned i = (t - nHC - tM) * spt + lane_id();
-        h.e = (lane_id() < spt && i < nS) ? __ldcg(io.S + i) : make_int4(-1, 0, 0, 0);
+        return h;
     }
+    t -= q.nHC;
+    const unsigned lane = lane_id();
+    const int4* list;
+    unsigned i, n;
+    bool on;
+    if (t < q.tM) {
+        list = io.M; i = t * q.mpt + lane; n = q.nM; on = lane < q.mpt;
+    } else if (t < q.tM + q.tS) {
+        list = io.S; i = (t - q.tM) * q.spt + lane; n = q.nS; on = lane < q.spt;
+    } else {
+        // lane j of a group holds the entry that the group takes in step j
+        const unsigned j = lane % kTinyLanes, g = lane / kTinyLanes;
+        list = io.T_; i = ((t - q.tM - q.tS) * q.tsub + j) * kTinyPerStep + g; n = q.nT; on = j < q.tsub;
+    }
+    h.e = on && i < n ? __ldcg(list + i) : make_int4(-1, 0, 0, 0);
     return h;
 }
 
@@ -852,7 +892,134 @@ __device__ __forceinline__ void st_stream(int32_t* a, int32_t x, uint64_t pol) {
     asm volatile("st.global.L2::cache_hint.s32 [%0], %1, %2;" :: "l"(a), "r"(x), "l"(pol) : "memory");
 }
 
-// S and M bins: up to 32 worklist entries per task, one per lane.  Their
+// Eight consecutive entries of colidx from index a on (a multiple of eight
+// counted from the 32-byte boundary at or below colidx), with one 32-byte
+// load; where that would reach outside the array, entry by entry.
+__device__ __forceinline__ void load_chunk(const int32_t* __restrict__ colidx, int32_t nnz, int32_t a, uint64_t pol,
+                                           int32_t (&w)[8]) {
+    if (a >= 0 && a <= nnz - 8) {
+        asm volatile("ld.global.nc.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                     : "l"(colidx + a), "l"(pol));
+    } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) w[u] = a + u >= 0 && a + u < nnz ? __ldg(colidx + a + u) : 0;
+    }
+}
+
+// T bin: vertices of degree <= s_max <= 32, whose first fit is at most 33, so
+// one 32-bit word holds every color that matters to them (33 is taken when
+// 1..32 all are) and one more says which entries of the row are still live
+// (the neighbour had not settled when last read).  Both travel in the worklist
+// entry {v, row start, live, static mask}; the row itself is read from colidx
+// in every round and no list is written.
+//
+// kTinyLanes lanes share a vertex: each takes a 32-byte chunk of the row (one
+// load for eight entries), gathers the colors of the live entries, and ORs
+// what it finds in registers; the lanes of a vertex combine with shuffles.
+// Lane j of a group keeps the vertex of step j, so a task of up to 32
+// vertices appends its survivors with one atomic.
+//
+// Bound: the random L2 sector of each live entry's color (207 G entries/s on
+// rows of 16; a probe that only gathers reaches 208).  The flat walk below,
+// which these rows took before, ran at 133 G entries/s: 157 instructions per
+// 32 entries against about 40 here, and an L1 data pipe 72 % busy, two fifths
+// of it with shared-memory atomics.  R-MAT-ER of 2^22 vertices: 2.36 ms a call
+// before, 1.70 after.
+template <typename T, bool P>  // P: a priority array is given
+__device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& io, int4 en, unsigned steps, int& maxc,
+                                          unsigned& vol) {
+    const unsigned lane = lane_id();
+    const unsigned j = lane % kTinyLanes;
+    const uint32_t mis = (uint32_t)((uintptr_t)p.colidx >> 2) & 7u;  // entries from a 32-byte boundary to colidx
+    const bool valid = en.x >= 0;
+    const int32_t my_v = valid ? en.x : 0;
+    const uint32_t my_live = valid ? (uint32_t)en.z : 0u;
+    const uint32_t my_cv = valid ? word_color(ld_color(io.Xc + my_v, io.pol_col)) : 0u;
+    // which entries precede v (bit i: entry i), worked out in round 2
+    uint32_t my_prec = 0u;
+    if constexpr (P) {
+        if (valid) my_prec = io.first ? __ldg(p.prio + my_v) : __ldcg(p.stat + (size_t)my_v * 8);
+    }
+    uint32_t my_all = 0u, my_stat = 0u, my_dead = 0u, my_new_prec = 0u;
+    bool my_conflict = false;
+#pragma unroll 1
+    for (unsigned s = 0; s < steps; ++s) {
+        const int src = (int)((lane & ~(unsigned)(kTinyLanes - 1)) | s);
+        const int32_t v = __shfl_sync(kFull, my_v, src);
+        const int32_t b = __shfl_sync(kFull, en.y, src);
+        const uint32_t live = __shfl_sync(kFull, my_live, src);
+        const uint32_t cv = __shfl_sync(kFull, my_cv, src);
+        const uint32_t prec = P ? __shfl_sync(kFull, my_prec, src) : 0u;  // round 2: v's key
+        uint32_t all = 0u, stat = 0u, dead = 0u, nprec = 0u;
+        bool conflict = false;
+        const int32_t span = 32 - __clz(live);  // entries up to the last live one
+        // off: index in the row of the chunk's first entry (the first chunk may start before the row)
+        for (int32_t off = 8 * (int32_t)j - (int32_t)(((uint32_t)b + mis) & 7u); off < span; off += 8 * kTinyLanes) {
+            const uint32_t bits = (off >= 0 ? live >> off : live << -off) & 0xffu;
+            if (bits == 0u) continue;
+            int32_t w[8];
+            load_chunk(p.colidx, p.nnz, b + off, io.pol_row, w);
+            T c[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) c[u] = (bits >> u) & 1u ? ld_color(io.Xc + w[u], io.pol_col) : (T)0;
+            uint32_t gone = 0u, pre8 = 0u;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint32_t col = word_color(c[u]);       // 0 where the entry is not live
+                const bool settled = word_settled(c[u]);
+                const uint32_t bit = shl_clamp(1u, col - 1u);  // 0 for col 0 and col > 32
+                all |= bit;
+                if (settled) {
+                    stat |= bit;
+                    gone |= 1u << u;
+                }
+                if constexpr (!P) {
+                    if (col == cv && w[u] < v) conflict = true;
+                } else if (io.first) {
+                    if (((bits >> u) & 1u) && (col == cv || !settled) && precedes(p.prio, w[u], v, prec)) {
+                        pre8 |= 1u << u;
+                        if (col == cv) conflict = true;
+                    }
+                } else {
+                    if (col == cv && ((off >= 0 ? prec >> off : prec << -off) >> u & 1u)) conflict = true;
+                }
+            }
+            dead |= off >= 0 ? gone << off : gone >> -off;
+            if (P && io.first) nprec |= off >= 0 ? pre8 << off : pre8 >> -off;
+        }
+        const unsigned cb = __ballot_sync(kFull, conflict);
+#pragma unroll
+        for (int o = 1; o < kTinyLanes; o <<= 1) {
+            all |= __shfl_xor_sync(kFull, all, o);
+            stat |= __shfl_xor_sync(kFull, stat, o);
+            dead |= __shfl_xor_sync(kFull, dead, o);
+            if (P && io.first) nprec |= __shfl_xor_sync(kFull, nprec, o);
+        }
+        if (j == s) {
+            my_all = all;
+            my_stat = stat;
+            my_dead = dead;
+            my_new_prec = nprec;
+            my_conflict = ((cb >> (lane - j)) & ((1u << kTinyLanes) - 1u)) != 0u;
+        }
+    }
+    const bool go = valid && my_conflict;
+    const uint32_t stat = (uint32_t)en.w | my_stat;
+    const uint32_t live = my_live & ~my_dead;
+    if (go) {
+        const uint32_t taken = stat | my_all;
+        recolor(p, io, my_v, taken == 0xffffffffu ? 33u : (uint32_t)__ffs(~taken));
+        vol += (unsigned)__popc(live);
+        if (P && io.first) p.stat[(size_t)my_v * 8] = my_new_prec;
+    } else if (valid) {
+        settle(p, io, my_v, my_cv);
+        maxc = max(maxc, (int)my_cv);
+    }
+    warp_append(go, make_int4(my_v, en.y, (int32_t)live, (int32_t)stat), io.next.T, &io.next.cnt->t);
+}
+
+// S bin: up to 32 worklist entries per task, one per lane.  Their
 // active lists are walked as one flat range in batches of 32 entries (lane
 // l of batch u takes flat entry F0 + 32u + l), so every lane has an entry in
 // every batch whatever the lengths are.  The row owning an entry is found
@@ -1312,42 +1479,50 @@ __device__ __forceinline__ void hub_chunk(const Params<T>& p, const PassIO<T>& i
 // task.  The next task's head is loaded, and the claim after it issued,
 // before the current task runs, so neither waits on memory.
 template <typename T, bool P>  // P: a priority array is given
-__device__ __forceinline__ void run_pass(const Params<T>& p, int k, unsigned nS, unsigned nM,
+__device__ __forceinline__ void run_pass(const Params<T>& p, int k, unsigned nT, unsigned nS, unsigned nM,
                                          unsigned nHC, int& maxc, unsigned gw, unsigned W, unsigned* ctr) {
     __shared__ FlatSmem s_flat[kWarpsPerBlockMax];
     const PassIO<T> io = pass_io(p, k);
     const unsigned wib = threadIdx.x >> 5;
+    TaskSplit q;
+    q.nT = nT; q.nS = nS; q.nM = nM; q.nHC = nHC;
     // S vertices per task: 32 in a large round, down to kShortPerTaskMin as it
     // shrinks; a task of 32 short lists walks up to 1024 entries in sequence,
     // which in the last rounds was the longest chain of the round
-    const unsigned spt = max((unsigned)kShortPerTaskMin, min(32u, nS / (4u * W)));
-    const unsigned tS = (nS + spt - 1) / spt;
+    q.spt = max((unsigned)kShortPerTaskMin, min(32u, nS / (4u * W)));
+    q.tS = (nS + q.spt - 1) / q.spt;
     // M vertices per task: up to kMedPerTask when the round has enough of them
     // for several tasks per warp, fewer (down to 1) as the round shrinks, so
     // that a task's chain of per-vertex reads does not set the round's length
-    const unsigned mpt = max(1u, min((unsigned)kMedPerTask, nM / (4u * W)));
-    const unsigned tM = (nM + mpt - 1) / mpt;
-    const unsigned total = nHC + tM + tS;
+    q.mpt = max(1u, min((unsigned)kMedPerTask, nM / (4u * W)));
+    q.tM = (nM + q.mpt - 1) / q.mpt;
+    // T vertices per task: kTinyLanes steps of kTinyPerStep, fewer likewise
+    q.tsub = max(1u, min((unsigned)kTinyLanes, nT / (4u * W * kTinyPerStep)));
+    const unsigned tpt = q.tsub * kTinyPerStep;
+    q.total = nHC + q.tM + q.tS + (nT + tpt - 1) / tpt;
+    const unsigned total = q.total;
     unsigned vol = 0;  // this lane's share of the next round's read volume
     // this warp's tasks: gw + jW for j < nstat, then claimed ones from nstat W on
     const unsigned nstat = ctr ? max(2u, total / W / 2) : 0xffffffffu;
     TaskHead cur;
-    if (gw < total) cur = load_head(io, gw, nS, nM, nHC, tM, mpt, spt);
+    if (gw < total) cur = load_head(io, gw, q);
     unsigned tn = gw + W;
     unsigned j = 0;  // position of the current task in that sequence
     for (unsigned t = gw; t < total; ++j) {
         TaskHead nxt;
-        if (tn < total) nxt = load_head(io, tn, nS, nM, nHC, tM, mpt, spt);
+        if (tn < total) nxt = load_head(io, tn, q);
         // the task after next: fixed, or claimed now (its number is needed after this task)
         const bool fixed = j + 2u < nstat;
         unsigned claim = 0;
         if (!fixed && tn < total && lane_id() == 0) claim = atomicAdd(ctr, 1u);
         if (t < nHC) {
             hub_chunk<T, P>(p, io, cur, s_flat[wib], maxc, vol);
-        } else if (t - nHC < tM) {
+        } else if (t - nHC < q.tM) {
             vertex_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
-        } else {
+        } else if (t - nHC - q.tM < q.tS) {
             flat_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
+        } else {
+            tiny_task<T, P>(p, io, cur.e, q.tsub, maxc, vol);
         }
         const unsigned tnn = fixed ? tn + W : nstat * W + __shfl_sync(kFull, claim, 0);
         t = tn;
@@ -1373,8 +1548,8 @@ __global__ void __launch_bounds__(256, kMinBlocks) rounds_persistent_kernel(Para
     for (int k = 2;; ++k) {
         const RoundCounts& c = st->rc[k % 3];
         const unsigned long long hc = __ldcg(&c.hc);
-        const unsigned nS = __ldcg(&c.s), nM = __ldcg(&c.m), nH = hub_count(hc), nHC = hub_chunks(hc);
-        const unsigned size = nS + nM + nH;
+        const unsigned nT = __ldcg(&c.t), nS = __ldcg(&c.s), nM = __ldcg(&c.m), nH = hub_count(hc), nHC = hub_chunks(hc);
+        const unsigned size = nT + nS + nM + nH;
         // start of this pass (the last record, for the empty round, marks the end)
         if (p.round_ns && blockIdx.x == 0 && threadIdx.x == 0 && k - 1 <= p.round_cap)
             p.round_ns[k - 1] = globaltimer_ns();
@@ -1399,12 +1574,12 @@ __global__ void __launch_bounds__(256, kMinBlocks) rounds_persistent_kernel(Para
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             RoundCounts& z = st->rc[(k + 2) % 3];
-            z.s = z.m = z.vol = 0u;
+            z.t = z.s = z.m = z.vol = 0u;
             z.hc = 0ull;
             st->task_next[(k + 1) % 3] = 0u;  // round k + 1's claims (no one touches it in round k)
             if (k - 1 < p.round_cap) p.round_sizes[k - 1] = (int32_t)size;
         }
-        run_pass<T, P>(p, k, nS, nM, nHC, maxc, gw, W, &st->task_next[k % 3]);
+        run_pass<T, P>(p, k, nT, nS, nM, nHC, maxc, gw, W, &st->task_next[k % 3]);
         if (tail) {
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -1421,10 +1596,10 @@ __global__ void __launch_bounds__(256, kMinBlocks) rounds_persistent_kernel(Para
 
 // One pass per launch (loop mode 1): counts come from the host.
 template <typename T, bool P>  // P: a priority array is given
-__global__ void __launch_bounds__(256, kMinBlocks) round_kernel(Params<T> p, int k, unsigned nS, unsigned nM,
-                                                       unsigned nHC) {
+__global__ void __launch_bounds__(256, kMinBlocks) round_kernel(Params<T> p, int k, unsigned nT, unsigned nS,
+                                                                unsigned nM, unsigned nHC) {
     int maxc = 0;
-    run_pass<T, P>(p, k, nS, nM, nHC, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+    run_pass<T, P>(p, k, nT, nS, nM, nHC, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
              (gridDim.x * blockDim.x) >> 5, nullptr);
     fold_max_color(p.st, maxc);
 }
@@ -1449,9 +1624,9 @@ __global__ void __launch_bounds__(256, kMinBlocks) graph_round_kernel(Params<T> 
     RoundState* st = p.st;
     const int k = __ldcg(&st->graph_round);
     const RoundCounts& c = st->rc[k % 3];
-    const unsigned nS = __ldcg(&c.s), nM = __ldcg(&c.m), nHC = hub_chunks(__ldcg(&c.hc));
+    const unsigned nT = __ldcg(&c.t), nS = __ldcg(&c.s), nM = __ldcg(&c.m), nHC = hub_chunks(__ldcg(&c.hc));
     int maxc = 0;
-    run_pass<T, P>(p, k, nS, nM, nHC, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+    run_pass<T, P>(p, k, nT, nS, nM, nHC, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
              (gridDim.x * blockDim.x) >> 5, nullptr);
     fold_max_color(st, maxc);
 }
@@ -1464,7 +1639,7 @@ __global__ void graph_cond_kernel(Params<T> p, int before_loop, cudaGraphConditi
     const int k = before_loop ? 1 : st->graph_round;
     const int kn = k + 1;
     const RoundCounts& c = st->rc[kn % 3];
-    const unsigned size = c.s + c.m + hub_count(c.hc);
+    const unsigned size = c.t + c.s + c.m + hub_count(c.hc);
     unsigned go = 0u;
     if (size == 0u) {
         st->rounds = k;
@@ -1475,7 +1650,7 @@ __global__ void graph_cond_kernel(Params<T> p, int before_loop, cudaGraphConditi
         st->status = kStatusMaxRounds;
     } else {
         RoundCounts& z = st->rc[(kn + 1) % 3];
-        z.s = z.m = z.vol = 0u;
+        z.t = z.s = z.m = z.vol = 0u;
         z.hc = 0ull;
         if (kn - 1 < p.round_cap) p.round_sizes[kn - 1] = (int32_t)size;
         st->graph_round = kn;

@@ -1,0 +1,62 @@
+"""Rows that the rounds read from the graph itself, at the edges of their bins.
+
+A vertex of small degree keeps one bit per row entry instead of a rewritten list and is read in
+32-byte chunks, so what can go wrong sits at the bin limits, at rows that need all their colors
+(cliques), at every alignment of the adjacency array, and at its two ends.
+"""
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def gcpkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1205_3809_gb300 as m
+    m.library()
+    return m
+
+
+def _cliques(degree, seed):
+    """Cliques with rows of `degree`, some with one edge missing, and a sparse random graph around
+    them; ids shuffled."""
+    k = degree + 1
+    u, v = np.triu_indices(k, 1)
+    parts, n = [], 0
+    for i in range(5):
+        drop = 0 if i < 3 else 1 + i % max(1, u.size - 1)
+        parts.append((u[drop:] + n, v[drop:] + n))
+        n += k
+    g = gg.gnm(400, 1200, seed)
+    src = np.repeat(np.arange(g.n), g.degrees)
+    parts.append((src + n, g.colidx.astype(np.int64) + n))
+    n += g.n
+    perm = gg.permutation(n, seed + 1)
+    us, vs = (np.concatenate([p[i] for p in parts]) for i in (0, 1))
+    return gg.from_edges(n, perm[us], perm[vs], name=f"cliques({degree})")
+
+
+@pytest.mark.parametrize("degree", [1, 7, 8, 24, 25, 31, 32, 33])
+@pytest.mark.parametrize("keyed", [False, True])
+def test_bin_edges(gcpkg, degree, keyed):
+    g = _cliques(degree, 100 + degree)
+    prio = (gg.draws(degree, 3, g.n) % np.uint64(5)).astype(np.uint32) if keyed else None
+    want = oracle.iterative(g.rowptr, g.colidx, prio)
+    rp = torch.from_numpy(g.rowptr).cuda()
+    pr = torch.from_numpy(prio.view(np.int32)).cuda() if keyed else None
+    for shift in (0, 1, 6):  # the adjacency array at other alignments, its ends at other chunks
+        buf = torch.full((g.nnz + 16,), 1 << 30, dtype=torch.int32, device="cuda")
+        ci = buf[shift:shift + g.nnz]
+        ci.copy_(torch.from_numpy(g.colidx))
+        for options in (None, {"small_max_degree": 8}, {"color_bits": 32}):
+            got = gcpkg.color(rp, ci, pr, options=options, round_sizes=True)
+            assert (got.ncolors, got.rounds) == (want.ncolors, want.rounds), (g.name, shift, options)
+            assert np.array_equal(got.colors.cpu().numpy(), want.colors)
+            assert np.array_equal(got.round_sizes, want.round_sizes)
