@@ -171,8 +171,8 @@ int ensure_device_limited(void** p, size_t* have, size_t need, int32_t limit_mb)
 }
 
 struct Layout {
-    size_t st, stats, rs, rv, rt, x0, x1, act0, act1, stat, hubs, defer;
-    size_t T[2], S[2], M[2], H[2], Hc[2], O[2];
+    size_t st, rs, rv, rt, x0, x1, act0, act1, stat, hubs, defer;
+    size_t T[2], L8[2], L16[2], S[2], M[2], H[2], Hc[2], O[2];
     size_t total;
 };
 
@@ -185,10 +185,10 @@ Layout make_layout(int64_t n, int64_t nnz, size_t elem, const Stats& hs, int64_t
         return o;
     };
     L.st = take(sizeof(RoundState));
-    L.stats = take(sizeof(Stats));
-    L.rs = take((size_t)round_cap * sizeof(int32_t));
-    L.rv = take((size_t)round_cap * sizeof(unsigned long long));
-    L.rt = take((size_t)(round_cap + 1) * sizeof(unsigned long long));
+    // telemetry arrays, 8-byte words first, in one piece
+    L.rv = take((size_t)round_cap * 20 + 8);
+    L.rt = L.rv + (size_t)round_cap * sizeof(unsigned long long);
+    L.rs = L.rt + (size_t)(round_cap + 1) * sizeof(unsigned long long);
     L.x0 = take((size_t)n * elem);
     L.x1 = take((size_t)n * elem);
     L.act0 = take((size_t)nnz * sizeof(int32_t));
@@ -197,16 +197,56 @@ Layout make_layout(int64_t n, int64_t nnz, size_t elem, const Stats& hs, int64_t
     L.hubs = take((size_t)hs.cap[gc::kBinH] * sizeof(gc::HubRecord));
     L.defer = take((size_t)hs.defer * sizeof(int32_t));
     for (int b = 0; b < 2; ++b) {
-        // degree 1 .. s_max: T; longer rows whose active list has shrunk to s_max: S
-        L.T[b] = take((size_t)(hs.cap[gc::kBinS] - hs.cap[gc::kBinM]) * sizeof(int4));
-        L.S[b] = take((size_t)hs.cap[gc::kBinM] * sizeof(int4));
-        L.M[b] = take((size_t)hs.cap[gc::kBinM] * sizeof(int4));
+        // T: degree 1 .. s_max; L8 and L16: up to their limits; M: longer ones, and H
+        // lists that shrink to m_max; S: M and H lists that shrink to s_max
+        const size_t cT = hs.cap[gc::kBinS] - hs.cap[gc::kBinM], c8 = hs.cap[gc::kBinM] - hs.over8,
+                     c16 = hs.over8 - hs.over16, cM = hs.over16;
+        L.T[b] = take((cT + c8 + c16 + 2 * cM) * sizeof(int4));
+        L.L8[b] = L.T[b] + cT * sizeof(int4);
+        L.L16[b] = L.L8[b] + c8 * sizeof(int4);
+        L.M[b] = L.L16[b] + c16 * sizeof(int4);
+        L.S[b] = L.M[b] + cM * sizeof(int4);
         L.H[b] = take((size_t)hs.cap[gc::kBinH] * sizeof(int4));
         L.Hc[b] = take((size_t)hs.cap[gc::kBinH] * sizeof(int32_t));
         L.O[b] = take((size_t)hs.hub_chunks * sizeof(int32_t));
     }
     L.total = off;
     return L;
+}
+
+// A call's pointers into its workspace (p.s_max and p.m_max are set).
+template <typename T>
+void fill_workspace(Params<T>& p, char* base, const Layout& L, RoundState* st, int64_t round_cap) {
+    p.mid8 = gc::mid_limit(8, p.s_max, p.m_max);
+    p.mid16 = gc::mid_limit(16, p.s_max, p.m_max);
+    p.X0 = (T*)(base + L.x0);
+    p.X1 = (T*)(base + L.x1);
+    p.act0 = (int32_t*)(base + L.act0);
+    p.act1 = (int32_t*)(base + L.act1);
+    p.stat = (uint32_t*)(base + L.stat);
+    p.TA = (int4*)(base + L.T[0]);
+    p.L8A = (int4*)(base + L.L8[0]);
+    p.L16A = (int4*)(base + L.L16[0]);
+    p.SA = (int4*)(base + L.S[0]);
+    p.MA = (int4*)(base + L.M[0]);
+    p.HA = (int4*)(base + L.H[0]);
+    p.HcA = (int32_t*)(base + L.Hc[0]);
+    p.OA = (int32_t*)(base + L.O[0]);
+    p.TB = (int4*)(base + L.T[1]);
+    p.L8B = (int4*)(base + L.L8[1]);
+    p.L16B = (int4*)(base + L.L16[1]);
+    p.SB = (int4*)(base + L.S[1]);
+    p.MB = (int4*)(base + L.M[1]);
+    p.HB = (int4*)(base + L.H[1]);
+    p.HcB = (int32_t*)(base + L.Hc[1]);
+    p.OB = (int32_t*)(base + L.O[1]);
+    p.defer = (int32_t*)(base + L.defer);
+    p.hubs = (gc::HubRecord*)(base + L.hubs);
+    p.st = st;
+    p.round_sizes = (int32_t*)(base + L.rs);
+    p.round_vol = (unsigned long long*)(base + L.rv);
+    p.round_ns = nullptr;
+    p.round_cap = (int32_t)round_cap;
 }
 
 // Loop mode 2: rounds 2.. as one CUDA graph: a condition kernel, then a while
@@ -325,8 +365,9 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
     for (;; ++k) {
         GC_CUDA(cudaMemcpyAsync(h, &st->rc[k % 3], sizeof(gc::RoundCounts), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
-        const unsigned nT = h->t, nS = h->s, nM = h->m, nH = gc::hub_count(h->hc), nHC = gc::hub_chunks(h->hc);
-        const unsigned size = nT + nS + nM + nH;
+        const gc::RoundSizes r = {h->t, gc::low_count(h->mid), gc::high_count(h->mid), h->s, h->m,
+                                  gc::hub_chunks(h->hc)};
+        const unsigned size = r.nT + r.n8 + r.n16 + r.nS + r.nM + gc::hub_count(h->hc);
         if (size == 0) break;
         if (k > p.max_rounds) {
             hs[1] = gc::kStatusMaxRounds;
@@ -339,12 +380,12 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
                                     cudaMemcpyHostToDevice, s));
         }
         GC_CUDA(cudaMemsetAsync(&st->rc[(k + 2) % 3], 0, sizeof(gc::RoundCounts), s));
-        const int64_t tasks = (int64_t)nHC + (nM + gc::kMedPerTask - 1) / gc::kMedPerTask + (nS + 31) / 32 +
-                              (nT + 31) / 32;
+        const int64_t tasks = (int64_t)r.nHC + (r.nM + gc::kMedPerTask - 1) / gc::kMedPerTask + (r.nS + 31) / 32 +
+                              (r.nT + 31) / 32 + (r.n8 + 31) / 32 + (r.n16 + 15) / 16;
         const int64_t warps_per_block = threads / 32;
         const int grid = (int)std::max<int64_t>(
             1, std::min<int64_t>((tasks + warps_per_block - 1) / warps_per_block, (int64_t)dc.sms * 8));
-        gc::round_kernel<T, P><<<grid, threads, 0, s>>>(p, k, nT, nS, nM, nHC);
+        gc::round_kernel<T, P><<<grid, threads, 0, s>>>(p, k, r);
         GC_CUDA(cudaGetLastError());
         *launches += 1;
     }
@@ -513,32 +554,10 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
             p.barrier_polls = o.barrier_poll_limit > 0 ? (uint32_t)o.barrier_poll_limit : gc::kBarrierMaxPolls;
             p.color_limit = bits == 16 ? (o.narrow_color_limit > 0 ? (uint32_t)o.narrow_color_limit : 0x8000u)
                                        : 0x80000000u;
-            p.X0 = (T*)(base + L.x0);
-            p.X1 = (T*)(base + L.x1);
             p.colors_out = colors_out;
             p.settle_round = nullptr;
-            p.act0 = (int32_t*)(base + L.act0);
-            p.act1 = (int32_t*)(base + L.act1);
-            p.stat = (uint32_t*)(base + L.stat);
-            p.TA = (int4*)(base + L.T[0]);
-            p.SA = (int4*)(base + L.S[0]);
-            p.MA = (int4*)(base + L.M[0]);
-            p.HA = (int4*)(base + L.H[0]);
-            p.HcA = (int32_t*)(base + L.Hc[0]);
-            p.OA = (int32_t*)(base + L.O[0]);
-            p.TB = (int4*)(base + L.T[1]);
-            p.SB = (int4*)(base + L.S[1]);
-            p.MB = (int4*)(base + L.M[1]);
-            p.HB = (int4*)(base + L.H[1]);
-            p.HcB = (int32_t*)(base + L.Hc[1]);
-            p.OB = (int32_t*)(base + L.O[1]);
-            p.defer = (int32_t*)(base + L.defer);
-            p.hubs = (gc::HubRecord*)(base + L.hubs);
-            p.st = st;
-            p.round_sizes = (int32_t*)(base + L.rs);
-            p.round_vol = (unsigned long long*)(base + L.rv);
+            fill_workspace(p, base, L, st, round_cap);
             p.round_ns = o.telemetry && o.loop_mode == 0 ? (unsigned long long*)(base + L.rt) : nullptr;
-            p.round_cap = (int32_t)round_cap;
         };
         NvtxRange range(bits == 16 ? "gc rounds (16-bit colors)" : "gc rounds (32-bit colors)");
         if (bits == 16) {
@@ -711,32 +730,9 @@ int color_noalloc_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n
             p.tail_volume = o.tail_volume;
             p.barrier_polls = gc::kBarrierMaxPolls;
             p.color_limit = bits == 16 ? 0x8000u : 0x80000000u;
-            p.X0 = (T*)(base + L.x0);
-            p.X1 = (T*)(base + L.x1);
             p.colors_out = colors_out;
             p.settle_round = nullptr;
-            p.act0 = (int32_t*)(base + L.act0);
-            p.act1 = (int32_t*)(base + L.act1);
-            p.stat = (uint32_t*)(base + L.stat);
-            p.TA = (int4*)(base + L.T[0]);
-            p.SA = (int4*)(base + L.S[0]);
-            p.MA = (int4*)(base + L.M[0]);
-            p.HA = (int4*)(base + L.H[0]);
-            p.HcA = (int32_t*)(base + L.Hc[0]);
-            p.OA = (int32_t*)(base + L.O[0]);
-            p.TB = (int4*)(base + L.T[1]);
-            p.SB = (int4*)(base + L.S[1]);
-            p.MB = (int4*)(base + L.M[1]);
-            p.HB = (int4*)(base + L.H[1]);
-            p.HcB = (int32_t*)(base + L.Hc[1]);
-            p.OB = (int32_t*)(base + L.O[1]);
-            p.defer = (int32_t*)(base + L.defer);
-            p.hubs = (gc::HubRecord*)(base + L.hubs);
-            p.st = st;
-            p.round_sizes = (int32_t*)(base + L.rs);
-            p.round_vol = (unsigned long long*)(base + L.rv);
-            p.round_ns = nullptr;
-            p.round_cap = (int32_t)round_cap;
+            fill_workspace(p, base, L, st, round_cap);
         };
         if (bits == 16) {
             Params<uint16_t> p;
@@ -776,34 +772,6 @@ int color_noalloc_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n
 // kernels; no allocation, no host synchronisation), so a stream capture of
 // it is a CUDA graph of the whole batch, which gc_batch_launch_graph builds
 // once and replays.
-
-template <typename T>
-void fill_workspace(Params<T>& p, char* base, const Layout& L, RoundState* st, int64_t round_cap) {
-    p.X0 = (T*)(base + L.x0);
-    p.X1 = (T*)(base + L.x1);
-    p.act0 = (int32_t*)(base + L.act0);
-    p.act1 = (int32_t*)(base + L.act1);
-    p.stat = (uint32_t*)(base + L.stat);
-    p.TA = (int4*)(base + L.T[0]);
-    p.SA = (int4*)(base + L.S[0]);
-    p.MA = (int4*)(base + L.M[0]);
-    p.HA = (int4*)(base + L.H[0]);
-    p.HcA = (int32_t*)(base + L.Hc[0]);
-    p.OA = (int32_t*)(base + L.O[0]);
-    p.TB = (int4*)(base + L.T[1]);
-    p.SB = (int4*)(base + L.S[1]);
-    p.MB = (int4*)(base + L.M[1]);
-    p.HB = (int4*)(base + L.H[1]);
-    p.HcB = (int32_t*)(base + L.Hc[1]);
-    p.OB = (int32_t*)(base + L.O[1]);
-    p.defer = (int32_t*)(base + L.defer);
-    p.hubs = (gc::HubRecord*)(base + L.hubs);
-    p.st = st;
-    p.round_sizes = (int32_t*)(base + L.rs);
-    p.round_vol = (unsigned long long*)(base + L.rv);
-    p.round_ns = nullptr;
-    p.round_cap = (int32_t)round_cap;
-}
 
 }  // namespace
 
@@ -1211,8 +1179,8 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     fail(GC_OK);  // frees the head copy after the stream drains
     // the coloring layout's offsets are relative to its own base
     Layout& L = b->L;
-    size_t* fields[] = {&L.st, &L.stats, &L.rs, &L.rv, &L.rt, &L.x0, &L.x1, &L.act0, &L.act1, &L.stat, &L.hubs,
-                        &L.defer, &L.T[0], &L.T[1], &L.S[0], &L.S[1], &L.M[0], &L.M[1], &L.H[0], &L.H[1], &L.Hc[0], &L.Hc[1],
+    size_t* fields[] = {&L.st, &L.rs, &L.rv, &L.rt, &L.x0, &L.x1, &L.act0, &L.act1, &L.stat, &L.hubs,
+                        &L.defer, &L.T[0], &L.T[1], &L.L8[0], &L.L8[1], &L.L16[0], &L.L16[1], &L.S[0], &L.S[1], &L.M[0], &L.M[1], &L.H[0], &L.H[1], &L.Hc[0], &L.Hc[1],
                         &L.O[0], &L.O[1]};
     for (size_t* f : fields) *f += lay;
 

@@ -28,17 +28,19 @@
 // flag makes 16-bit state hold colors < 2^15: a larger color sets an
 // overflow status and the host reruns with 32-bit state.
 //
-// Work is split into warp-sized tasks, binned by the current active length
-// (T: by degree):
+// Work is split into warp-sized tasks, binned by degree (T, L8, L16) or by the
+// current active length (S, M, H):
 //   T bin (degree <= s_max <= 32): the row is read from the graph itself in
 //     32-byte chunks, with one bit per entry for "not settled yet" in the
 //     worklist entry; no list is kept;
+//   L8, L16 bins (longer rows of degree <= 57 and <= 121): likewise, by 8 or 16
+//     lanes, the bits beside the static mask;
 //   S bin (longer rows whose list has shrunk to s_max): 32 worklist entries per
 //     task (down to 4 in the small rounds at the end), their lists walked as
 //     one flat range;
-//   M bin (s_max < length <= m_max <= 256): up to 16 worklist entries per
-//     task, each list read by the whole warp in turn (colors 1..64 in
-//     registers);
+//   M bin (other lists of s_max < length <= m_max <= 256): up to 16 worklist
+//     entries per task, each list read by the whole warp in turn (colors 1..64
+//     in registers);
 //   H bin (length > m_max): one chunk of up to 1024 entries of one list per
 //     task; a list of one chunk is decided by its warp, and the chunks of a
 //     longer list OR their conflict flag and color windows into a per-vertex
@@ -88,6 +90,14 @@ constexpr int kShortPerTaskMin = 4;            // S-bin vertices per task in a s
 #endif
 constexpr int kTinyLanes = GC_TINY_LANES;      // T bin: lanes per vertex
 constexpr int kTinyPerStep = 32 / kTinyLanes;  // T bin: vertices a warp reads side by side
+constexpr int kMidSteps = 8;                   // L8, L16: steps of 32 / L vertices per task, at most
+
+// L8 and L16 bins: degrees above s_max (and up to m_max) whose row fits L
+// chunks of eight entries wherever it starts: 8 L - 7.
+__host__ __device__ __forceinline__ int32_t mid_limit(int L, int32_t s_max, int32_t m_max) {
+    const int32_t most = 8 * L - 7 < m_max ? 8 * L - 7 : m_max;
+    return most > s_max ? most : s_max;
+}
 constexpr int kMinBlocks = GC_MIN_BLOCKS;      // round kernels: blocks per SM the registers allow
 constexpr int kWarpsPerBlockMax = 8;          // blocks of <= 256 threads
 
@@ -121,7 +131,7 @@ struct Stats {
     int nnz;                      // rowptr[n]
     unsigned defer;               // vertices with degree > kPass1Flat
     unsigned cap[3];              // list capacities: degree >= 1, > s_max, > m_max
-    unsigned pad;
+    unsigned over8, over16;       // vertices with degree > mid_limit(8), > mid_limit(16)
     unsigned long long hub_chunks;  // sum over degree > m_max of ceil(degree / kChunk)
 };
 
@@ -132,12 +142,16 @@ struct Stats {
 // chunk) share one 64-bit word, taken with one atomic.
 struct RoundCounts {
     alignas(128) unsigned t;               // |U_k in T|
+    alignas(128) unsigned long long mid;   // |U_k in L8| (bits 0..31) | |U_k in L16| (bits 32..63)
     alignas(128) unsigned s;               // |U_k in S|
     alignas(128) unsigned m;               // |U_k in M|
     alignas(128) unsigned long long hc;    // |U_k in H| (bits 0..31) | chunks of U_k in H (bits 32..63)
     alignas(128) unsigned vol;             // active entries round k reads
 };
 
+// Two 32-bit counts in one 64-bit word.
+__host__ __device__ __forceinline__ unsigned low_count(unsigned long long x) { return (unsigned)x; }
+__host__ __device__ __forceinline__ unsigned high_count(unsigned long long x) { return (unsigned)(x >> 32); }
 __host__ __device__ __forceinline__ unsigned hub_count(unsigned long long hc) { return (unsigned)hc; }
 __host__ __device__ __forceinline__ unsigned hub_chunks(unsigned long long hc) { return (unsigned)(hc >> 32); }
 
@@ -175,6 +189,7 @@ struct Params {
     int32_t n;
     int32_t nnz;                        // entries of colidx
     int32_t s_max, m_max;               // length bin limits
+    int32_t mid8, mid16;                // degree limits of the L8 and L16 bins
     int32_t max_rounds;
     int32_t tail_volume;                // rounds reading <= this many entries run in block 0 alone (< 0: never)
     uint32_t barrier_polls;             // the grid barrier gives up after this many polls
@@ -187,10 +202,11 @@ struct Params {
     int32_t* act1;
     uint32_t* stat;                     // static masks, 8 words per vertex
     // worklists per parity (A: even k, B: odd k): T entries {vertex, row start,
-    // live entries, static mask}; S, M, H entries {vertex, row start, active
-    // length, degree}, first chunk of each H entry, owner position of each chunk
-    int4* TA; int4* SA; int4* MA; int4* HA; int32_t* HcA; int32_t* OA;
-    int4* TB; int4* SB; int4* MB; int4* HB; int32_t* HcB; int32_t* OB;
+    // live entries, static mask}; L8, L16, S, M, H entries {vertex, row start,
+    // active length (L8, L16: degree), degree}, first chunk of each H entry,
+    // owner position of each chunk
+    int4* TA; int4* L8A; int4* L16A; int4* SA; int4* MA; int4* HA; int32_t* HcA; int32_t* OA;
+    int4* TB; int4* L8B; int4* L16B; int4* SB; int4* MB; int4* HB; int32_t* HcB; int32_t* OB;
     int32_t* defer;                     // pass 1: rows longer than kPass1Flat
     HubRecord* hubs;
     RoundState* st;
@@ -310,7 +326,7 @@ __device__ __forceinline__ void warp_append_i32(bool flag, int32_t v, int32_t* l
 
 // Where the next round's worklists go.
 struct NextLists {
-    int4* T; int4* S; int4* M; int4* H; int32_t* Hc; int32_t* O;
+    int4* T; int4* L8; int4* L16; int4* S; int4* M; int4* H; int32_t* Hc; int32_t* O;
     RoundCounts* cnt;  // the next round's counts
     int32_t s_max, m_max;
 };
@@ -521,8 +537,9 @@ __device__ __forceinline__ void fold_volume(RoundState* st, unsigned long long* 
 __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int32_t s_max,
                              int32_t m_max, Stats* s) {
     int mx = 0, bad = 0;
-    unsigned c0 = 0, c1 = 0, c2 = 0, df = 0;
+    unsigned c0 = 0, c1 = 0, c2 = 0, df = 0, o8 = 0, o16 = 0;
     unsigned long long ch = 0;
+    const int32_t mid8 = mid_limit(8, s_max, m_max), mid16 = mid_limit(16, s_max, m_max);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int32_t d = __ldg(rowptr + v + 1) - __ldg(rowptr + v);
@@ -531,6 +548,8 @@ __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int3
         c0 += d >= 1;
         c1 += d > s_max;
         c2 += d > m_max;
+        o8 += d > mid8;
+        o16 += d > mid16;
         df += d > kPass1Flat;
         if (d > m_max) ch += (unsigned long long)((d + kChunk - 1) / kChunk);
     }
@@ -540,6 +559,8 @@ __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int3
     c1 = __reduce_add_sync(kFull, c1);
     c2 = __reduce_add_sync(kFull, c2);
     df = __reduce_add_sync(kFull, df);
+    o8 = __reduce_add_sync(kFull, o8);
+    o16 = __reduce_add_sync(kFull, o16);
     if (lane_id() == 0) {
         atomicMax(&s->max_degree, mx);
         if (bad) s->bad = 1;
@@ -547,6 +568,8 @@ __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int3
         if (c1) atomicAdd(&s->cap[1], c1);
         if (c2) atomicAdd(&s->cap[2], c2);
         if (df) atomicAdd(&s->defer, df);
+        if (o8) atomicAdd(&s->over8, o8);
+        if (o16) atomicAdd(&s->over16, o16);
     }
     for (int o = 16; o > 0; o >>= 1) ch += __shfl_xor_sync(kFull, ch, o);
     if (lane_id() == 0 && ch) atomicAdd(&s->hub_chunks, ch);
@@ -577,7 +600,7 @@ __device__ __forceinline__ void pass1_write(const Params<T>& p, int32_t v, bool 
 template <typename T>
 __device__ __forceinline__ NextLists pass1_next(const Params<T>& p) {
     NextLists nl;
-    nl.T = p.TA; nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
+    nl.T = p.TA; nl.L8 = p.L8A; nl.L16 = p.L16A; nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
     nl.cnt = &p.st->rc[2];
     nl.s_max = p.s_max;
     nl.m_max = p.m_max;
@@ -614,7 +637,7 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
     unsigned vol = 0;
     for (int64_t t0 = gw; t0 < ntasks; t0 += W * NT) {
         int4 ev[NT];
-        bool fT[NT], fM[NT];
+        int cls[NT];  // T, L8, L16, M (0..3), or -1
 #pragma unroll
         for (int jt = 0; jt < NT; ++jt) {
             const int64_t t = t0 + (int64_t)jt * W;
@@ -674,8 +697,7 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
             const bool go = valid && !longrow && hit;
             // a row of at most s_max entries starts as a T entry: all of it live, no static mask
             ev[jt] = bin == kBinS ? make_int4(v, b, (int32_t)low_bits(d), 0) : make_int4(v, b, d, d);
-            fT[jt] = go && bin == kBinS;
-            fM[jt] = go && bin == kBinM;
+            cls[jt] = !go || bin == kBinH ? -1 : (bin == kBinS ? 0 : (d <= p.mid8 ? 1 : (d <= p.mid16 ? 2 : 3)));
             // hubs that stayed in the flat range (m_max < d <= kPass1Flat)
             unsigned hubs = __ballot_sync(kFull, go && bin == kBinH);
             while (hubs) {
@@ -686,26 +708,34 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
             }
             warp_append_i32(valid && longrow, v, p.defer, &p.st->defer_cnt);
         }
-        // the T and M entries of these NT tasks, one atomic per bin
+        // the T, L8, L16 and M entries of these NT tasks, one atomic per counter
+        // (L8 and L16 share one)
+        unsigned bal[NT][4], n[4] = {0, 0, 0, 0};
 #pragma unroll
-        for (int bin = 0; bin < 2; ++bin) {
-            unsigned bal[NT], n = 0;
+        for (int jt = 0; jt < NT; ++jt)
 #pragma unroll
-            for (int jt = 0; jt < NT; ++jt) {
-                bal[jt] = __ballot_sync(kFull, bin == 0 ? fT[jt] : fM[jt]);
-                n += __popc(bal[jt]);
+            for (int c = 0; c < 4; ++c) {
+                bal[jt][c] = __ballot_sync(kFull, cls[jt] == c);
+                n[c] += __popc(bal[jt][c]);
             }
-            if (n == 0) continue;
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(bin == 0 ? &nl.cnt->t : &nl.cnt->m, n);
-            base = __shfl_sync(kFull, base, 0);
-            int4* const list = bin == 0 ? nl.T : nl.M;
+        unsigned long long base = 0;  // lane 0: T, lane 1: L8 and L16, lane 2: M
+        if (lane == 0 && n[0]) base = atomicAdd(&nl.cnt->t, n[0]);
+        if (lane == 1 && (n[1] | n[2]))
+            base = atomicAdd(&nl.cnt->mid, ((unsigned long long)n[2] << 32) | (unsigned long long)n[1]);
+        if (lane == 2 && n[3]) base = atomicAdd(&nl.cnt->m, n[3]);
+        unsigned at[4];
+        at[0] = __shfl_sync(kFull, (unsigned)base, 0);
+        at[1] = __shfl_sync(kFull, (unsigned)base, 1);
+        at[2] = __shfl_sync(kFull, (unsigned)(base >> 32), 1);
+        at[3] = __shfl_sync(kFull, (unsigned)base, 2);
 #pragma unroll
-            for (int jt = 0; jt < NT; ++jt) {
-                if ((bal[jt] >> lane) & 1u) list[base + __popc(bal[jt] & ((1u << lane) - 1u))] = ev[jt];
-                base += __popc(bal[jt]);
+        for (int jt = 0; jt < NT; ++jt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                int4* const list = c == 0 ? p.TA : (c == 1 ? p.L8A : (c == 2 ? p.L16A : p.MA));
+                if (cls[jt] == c) list[at[c] + __popc(bal[jt][c] & ((1u << lane) - 1u))] = ev[jt];
+                at[c] += __popc(bal[jt][c]);
             }
-        }
     }
     fold_max_color(p.st, maxc);
     fold_volume(p.st, p.round_vol, p.round_cap, 2, vol);
@@ -774,7 +804,7 @@ struct PassIO {
     const int32_t* rin;     // active lists read this round (colidx in round 2)
     int32_t* rout;          // active lists written for the next round
     bool first;             // round 2: no static masks yet
-    const int4* T_; const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
+    const int4* T_; const int4* L8; const int4* L16; const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
     NextLists next;
     uint64_t pol_row, pol_col;
 };
@@ -791,12 +821,16 @@ __device__ __forceinline__ PassIO<T> pass_io(const Params<T>& p, int k) {
     io.rin = k == 2 ? p.colidx : (odd ? p.act1 : p.act0);
     io.rout = odd ? p.act0 : p.act1;
     io.T_ = odd ? p.TB : p.TA;
+    io.L8 = odd ? p.L8B : p.L8A;
+    io.L16 = odd ? p.L16B : p.L16A;
     io.S = odd ? p.SB : p.SA;
     io.M = odd ? p.MB : p.MA;
     io.H = odd ? p.HB : p.HA;
     io.Hc = odd ? p.HcB : p.HcA;
     io.O = odd ? p.OB : p.OA;
     io.next.T = odd ? p.TA : p.TB;
+    io.next.L8 = odd ? p.L8A : p.L8B;
+    io.next.L16 = odd ? p.L16A : p.L16B;
     io.next.S = odd ? p.SA : p.SB;
     io.next.M = odd ? p.MA : p.MB;
     io.next.H = odd ? p.HA : p.HB;
@@ -834,39 +868,65 @@ struct TaskHead {
     int32_t lo;   // H chunk: first entry of the chunk
 };
 
-// The tasks of one round, in the order they are dealt out: H chunks, M, S, T.
+// The entries of one round.
+struct RoundSizes {
+    unsigned nT, n8, n16, nS, nM, nHC;  // T, L8, L16, S, M entries; H chunks
+};
+__device__ __forceinline__ RoundSizes round_sizes_of(const RoundCounts& c, unsigned* total) {
+    RoundSizes r;
+    const unsigned long long hc = __ldcg(&c.hc), mid = __ldcg(&c.mid);
+    r.nT = __ldcg(&c.t);
+    r.n8 = low_count(mid);
+    r.n16 = high_count(mid);
+    r.nS = __ldcg(&c.s);
+    r.nM = __ldcg(&c.m);
+    r.nHC = hub_chunks(hc);
+    *total = r.nT + r.n8 + r.n16 + r.nS + r.nM + hub_count(hc);
+    return r;
+}
+
+// Its tasks, in the order they are dealt out: H chunks, M, L16, L8, S, T.
 struct TaskSplit {
-    unsigned nT, nS, nM, nHC;       // T, S, M entries; H chunks
-    unsigned mpt, spt, tsub;        // M and S entries per task; groups of kTinyPerStep T entries per task
-    unsigned tM, tS, total;         // tasks of M and S; of the round
+    unsigned mpt, spt;              // M and S entries per task
+    unsigned s16, s8, sT;           // steps per task of L16, L8 and T
+    unsigned e0, e1, e2, e3, e4;    // ends of the H, M, L16, L8 and S tasks
+    unsigned total;
 };
 
+// Entry of step j < steps of a row task: lane j of every group of L lanes
+// holds the entry that the group takes in step j.
+template <int L>
+__device__ __forceinline__ unsigned step_entry(unsigned t, unsigned steps, unsigned* j) {
+    *j = lane_id() % L;
+    return (t * steps + *j) * (32 / L) + lane_id() / L;
+}
+
 template <typename T>
-__device__ __forceinline__ TaskHead load_head(const PassIO<T>& io, unsigned t, const TaskSplit& q) {
+__device__ __forceinline__ TaskHead load_head(const PassIO<T>& io, unsigned t, const RoundSizes& r,
+                                              const TaskSplit& q) {
     TaskHead h;
     h.pos = 0;
     h.lo = 0;
-    if (t < q.nHC) {
+    if (t < q.e0) {
         h.pos = __ldcg(io.O + t);
         h.e = __ldcg(io.H + h.pos);
         h.lo = h.e.y + ((int32_t)t - __ldcg(io.Hc + h.pos)) * kChunk;
         return h;
     }
-    t -= q.nHC;
-    const unsigned lane = lane_id();
     const int4* list;
-    unsigned i, n;
-    bool on;
-    if (t < q.tM) {
-        list = io.M; i = t * q.mpt + lane; n = q.nM; on = lane < q.mpt;
-    } else if (t < q.tM + q.tS) {
-        list = io.S; i = (t - q.tM) * q.spt + lane; n = q.nS; on = lane < q.spt;
+    unsigned i, n, j = lane_id(), most;
+    if (t < q.e1) {
+        list = io.M; n = r.nM; most = q.mpt; i = (t - q.e0) * q.mpt + j;
+    } else if (t < q.e2) {
+        list = io.L16; n = r.n16; most = q.s16; i = step_entry<16>(t - q.e1, q.s16, &j);
+    } else if (t < q.e3) {
+        list = io.L8; n = r.n8; most = q.s8; i = step_entry<8>(t - q.e2, q.s8, &j);
+    } else if (t < q.e4) {
+        list = io.S; n = r.nS; most = q.spt; i = (t - q.e3) * q.spt + j;
     } else {
-        // lane j of a group holds the entry that the group takes in step j
-        const unsigned j = lane % kTinyLanes, g = lane / kTinyLanes;
-        list = io.T_; i = ((t - q.tM - q.tS) * q.tsub + j) * kTinyPerStep + g; n = q.nT; on = j < q.tsub;
+        list = io.T_; n = r.nT; most = q.sT; i = step_entry<kTinyLanes>(t - q.e4, q.sT, &j);
     }
-    h.e = on && i < n ? __ldcg(list + i) : make_int4(-1, 0, 0, 0);
+    h.e = j < most && i < n ? __ldcg(list + i) : make_int4(-1, 0, 0, 0);
     return h;
 }
 
@@ -964,26 +1024,27 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
 #pragma unroll
             for (int u = 0; u < 8; ++u) c[u] = (bits >> u) & 1u ? ld_color(io.Xc + w[u], io.pol_col) : (T)0;
             uint32_t gone = 0u, pre8 = 0u;
+            if constexpr (P) {
+                if (!io.first) {
+                    pre8 = off >= 0 ? prec >> off : prec << -off;
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (((bits >> u) & 1u) && (word_color(c[u]) == cv || !word_settled(c[u])) &&
+                            precedes(p.prio, w[u], v, prec))
+                            pre8 |= 1u << u;
+                }
+            }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                const uint32_t col = word_color(c[u]);       // 0 where the entry is not live
-                const bool settled = word_settled(c[u]);
+                const uint32_t col = word_color(c[u]);         // 0 where the entry is not live
                 const uint32_t bit = shl_clamp(1u, col - 1u);  // 0 for col 0 and col > 32
                 all |= bit;
-                if (settled) {
+                if (word_settled(c[u])) {
                     stat |= bit;
                     gone |= 1u << u;
                 }
-                if constexpr (!P) {
-                    if (col == cv && w[u] < v) conflict = true;
-                } else if (io.first) {
-                    if (((bits >> u) & 1u) && (col == cv || !settled) && precedes(p.prio, w[u], v, prec)) {
-                        pre8 |= 1u << u;
-                        if (col == cv) conflict = true;
-                    }
-                } else {
-                    if (col == cv && ((off >= 0 ? prec >> off : prec << -off) >> u & 1u)) conflict = true;
-                }
+                if (col == cv && (P ? (pre8 >> u) & 1u : w[u] < v)) conflict = true;
             }
             dead |= off >= 0 ? gone << off : gone >> -off;
             if (P && io.first) nprec |= off >= 0 ? pre8 << off : pre8 >> -off;
@@ -1017,6 +1078,136 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
         maxc = max(maxc, (int)my_cv);
     }
     warp_append(go, make_int4(my_v, en.y, (int32_t)live, (int32_t)stat), io.next.T, &io.next.cnt->t);
+}
+
+// L8 and L16 bins (L = 8, 16): vertices of degree s_max < d <= 8 L - 7, read
+// like T rows: L lanes share a vertex, one 32-byte chunk of colidx each, 32 / L
+// vertices side by side, no list written.  Their first fit is at most
+// 8 L - 6, so W = L / 4 words hold the colors that matter.  The static mask
+// (words 0..W-1) and one byte of live entries per chunk (after it) share the
+// vertex's 32 bytes of p.stat; with a priority array, one byte per chunk of
+// p.act0's part of the row (which no list of this vertex uses) says which
+// entries precede v.
+//
+// Bound: as for T rows, one random L2 sector per live entry.  A warp per
+// vertex (the M bin, which these rows took before) leaves most of its lanes
+// without an entry on a list of 33..64 and repeats its per-vertex work 32
+// wide: 98 G entries/s on rows of 48 and 158 on rows of 96, against 214 and
+// 227 here; on rows of 192 the two are level (200), so longer rows stay there.
+// R-MAT-B of 2^24 vertices: 24.34 -> 22.40 ms a call, learned R-MAT-G of 2^23:
+// 17.15 -> 14.07 ms.
+template <typename T, bool P, int L>  // P: a priority array is given
+__device__ __forceinline__ void mid_task(const Params<T>& p, const PassIO<T>& io, int4 en, unsigned steps, int& maxc,
+                                         unsigned& vol) {
+    constexpr int W = L / 4;
+    const unsigned lane = lane_id();
+    const unsigned j = lane % L;
+    const uint32_t mis = (uint32_t)((uintptr_t)p.colidx >> 2) & 7u;
+    const bool first = io.first;
+    const bool valid = en.x >= 0;
+    const int32_t my_v = valid ? en.x : 0;
+    const int32_t my_d = valid ? en.z : 0;  // 0: nothing to read
+    const uint32_t my_cv = valid ? word_color(ld_color(io.Xc + my_v, io.pol_col)) : 0u;
+    const uint32_t my_key = P && first && valid ? __ldg(p.prio + my_v) : 0u;
+    bool my_conflict = false;
+    uint32_t my_color = 0u;
+#pragma unroll 1
+    for (unsigned s = 0; s < steps; ++s) {
+        const int src = (int)((lane & ~(unsigned)(L - 1)) | s);
+        const int32_t v = __shfl_sync(kFull, my_v, src);
+        const int32_t b = __shfl_sync(kFull, en.y, src);
+        const int32_t d = __shfl_sync(kFull, my_d, src);
+        const uint32_t cv = __shfl_sync(kFull, my_cv, src);
+        const uint32_t key = P ? __shfl_sync(kFull, my_key, src) : 0u;
+        // this lane's chunk: entries off .. off + 7 of the row
+        const int32_t off = 8 * (int32_t)j - (int32_t)(((uint32_t)b + mis) & 7u);
+        uint32_t* const st = p.stat + (size_t)v * 8;
+        uint8_t* const live_at = reinterpret_cast<uint8_t*>(st + W) + j;
+        uint8_t* const prec_at = reinterpret_cast<uint8_t*>(p.act0 + b) + j;
+        uint32_t live, old = 0u, prec = 0u;
+        if (first) {
+            live = low_bits(max(0, min(8, d - off))) & (off < 0 ? 0xffu << -off : 0xffu);
+        } else {
+            live = d ? (uint32_t)__ldcg(live_at) : 0u;
+            if (d && j < W) old = __ldcg(st + j);
+            if (P && d) prec = (uint32_t)__ldcg(prec_at);
+        }
+        uint32_t all[W], stat[W], gone = 0u;
+#pragma unroll
+        for (int q = 0; q < W; ++q) {
+            all[q] = 0u;
+            stat[q] = (int)j == q ? old : 0u;
+        }
+        bool conflict = false;
+        if (live) {
+            int32_t w[8];
+            load_chunk(p.colidx, p.nnz, b + off, io.pol_row, w);
+            T c[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) c[u] = (live >> u) & 1u ? ld_color(io.Xc + w[u], io.pol_col) : (T)0;
+            if (P && first) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (((live >> u) & 1u) && (word_color(c[u]) == cv || !word_settled(c[u])) &&
+                        precedes(p.prio, w[u], v, key))
+                        prec |= 1u << u;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint32_t col = word_color(c[u]);  // 0 where the entry is not live
+#pragma unroll
+                for (int q = 0; q < W; ++q) all[q] |= shl_clamp(1u, col - 1u - 32u * q);
+                if (word_settled(c[u])) {
+                    gone |= 1u << u;
+#pragma unroll
+                    for (int q = 0; q < W; ++q) stat[q] |= shl_clamp(1u, col - 1u - 32u * q);
+                }
+                if (col == cv && (P ? (prec >> u) & 1u : w[u] < v)) conflict = true;
+            }
+        }
+        const unsigned cb = __ballot_sync(kFull, conflict);
+        const bool conf = ((cb >> (lane - j)) & low_bits(L)) != 0u;
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1)
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+                all[q] |= __shfl_xor_sync(kFull, all[q], o);
+                stat[q] |= __shfl_xor_sync(kFull, stat[q], o);
+            }
+        uint32_t color = 0u, mine = 0u;  // v's next color; this lane's word of the static mask
+#pragma unroll
+        for (int q = W - 1; q >= 0; --q) {
+            const uint32_t taken = all[q] | stat[q];
+            if (taken != 0xffffffffu) color = 32u * q + (uint32_t)__ffs(~taken);
+            if ((int)j == q) mine = stat[q];
+        }
+        if (conf) {
+            const uint32_t now = live & ~gone;
+            if (j < W && (first || mine != old)) st[j] = mine;
+            if (first || gone) *live_at = (uint8_t)now;
+            if (P && first) *prec_at = (uint8_t)prec;
+            vol += (unsigned)__popc(now);
+        }
+        if (j == s) {
+            my_conflict = conf;
+            my_color = color;
+        }
+    }
+    const bool go = valid && my_conflict;
+    if (go) {
+        recolor(p, io, my_v, my_color);
+    } else if (valid) {
+        settle(p, io, my_v, my_cv);
+        maxc = max(maxc, (int)my_cv);
+    }
+    const unsigned bal = __ballot_sync(kFull, go);
+    if (bal) {
+        constexpr int kShift = L == 8 ? 0 : 32;
+        unsigned base = 0;
+        if (lane == 0) base = (unsigned)(atomicAdd(&io.next.cnt->mid, (unsigned long long)__popc(bal) << kShift) >> kShift);
+        base = __shfl_sync(kFull, base, 0);
+        if (go) (L == 8 ? io.next.L8 : io.next.L16)[base + __popc(bal & ((1u << lane) - 1u))] = en;
+    }
 }
 
 // S bin: up to 32 worklist entries per task, one per lane.  Their
@@ -1479,50 +1670,57 @@ __device__ __forceinline__ void hub_chunk(const Params<T>& p, const PassIO<T>& i
 // task.  The next task's head is loaded, and the claim after it issued,
 // before the current task runs, so neither waits on memory.
 template <typename T, bool P>  // P: a priority array is given
-__device__ __forceinline__ void run_pass(const Params<T>& p, int k, unsigned nT, unsigned nS, unsigned nM,
-                                         unsigned nHC, int& maxc, unsigned gw, unsigned W, unsigned* ctr) {
+__device__ __forceinline__ void run_pass(const Params<T>& p, int k, const RoundSizes& r, int& maxc, unsigned gw,
+                                         unsigned W, unsigned* ctr) {
     __shared__ FlatSmem s_flat[kWarpsPerBlockMax];
     const PassIO<T> io = pass_io(p, k);
     const unsigned wib = threadIdx.x >> 5;
     TaskSplit q;
-    q.nT = nT; q.nS = nS; q.nM = nM; q.nHC = nHC;
     // S vertices per task: 32 in a large round, down to kShortPerTaskMin as it
     // shrinks; a task of 32 short lists walks up to 1024 entries in sequence,
     // which in the last rounds was the longest chain of the round
-    q.spt = max((unsigned)kShortPerTaskMin, min(32u, nS / (4u * W)));
-    q.tS = (nS + q.spt - 1) / q.spt;
+    q.spt = max((unsigned)kShortPerTaskMin, min(32u, r.nS / (4u * W)));
     // M vertices per task: up to kMedPerTask when the round has enough of them
     // for several tasks per warp, fewer (down to 1) as the round shrinks, so
-    // that a task's chain of per-vertex reads does not set the round's length
-    q.mpt = max(1u, min((unsigned)kMedPerTask, nM / (4u * W)));
-    q.tM = (nM + q.mpt - 1) / q.mpt;
-    // T vertices per task: kTinyLanes steps of kTinyPerStep, fewer likewise
-    q.tsub = max(1u, min((unsigned)kTinyLanes, nT / (4u * W * kTinyPerStep)));
-    const unsigned tpt = q.tsub * kTinyPerStep;
-    q.total = nHC + q.tM + q.tS + (nT + tpt - 1) / tpt;
+    // that a task's chain of per-vertex reads does not set the round's length;
+    // likewise the steps of the T, L8 and L16 tasks
+    q.mpt = max(1u, min((unsigned)kMedPerTask, r.nM / (4u * W)));
+    q.sT = max(1u, min((unsigned)kTinyLanes, r.nT / (4u * W * kTinyPerStep)));
+    q.s8 = max(1u, min((unsigned)kMidSteps, r.n8 / (4u * W * 4u)));
+    q.s16 = max(1u, min((unsigned)kMidSteps, r.n16 / (4u * W * 2u)));
+    q.e0 = r.nHC;
+    q.e1 = q.e0 + (r.nM + q.mpt - 1) / q.mpt;
+    q.e2 = q.e1 + (r.n16 + 2u * q.s16 - 1) / (2u * q.s16);
+    q.e3 = q.e2 + (r.n8 + 4u * q.s8 - 1) / (4u * q.s8);
+    q.e4 = q.e3 + (r.nS + q.spt - 1) / q.spt;
+    q.total = q.e4 + (r.nT + q.sT * kTinyPerStep - 1) / (q.sT * kTinyPerStep);
     const unsigned total = q.total;
     unsigned vol = 0;  // this lane's share of the next round's read volume
     // this warp's tasks: gw + jW for j < nstat, then claimed ones from nstat W on
     const unsigned nstat = ctr ? max(2u, total / W / 2) : 0xffffffffu;
     TaskHead cur;
-    if (gw < total) cur = load_head(io, gw, q);
+    if (gw < total) cur = load_head(io, gw, r, q);
     unsigned tn = gw + W;
     unsigned j = 0;  // position of the current task in that sequence
     for (unsigned t = gw; t < total; ++j) {
         TaskHead nxt;
-        if (tn < total) nxt = load_head(io, tn, q);
+        if (tn < total) nxt = load_head(io, tn, r, q);
         // the task after next: fixed, or claimed now (its number is needed after this task)
         const bool fixed = j + 2u < nstat;
         unsigned claim = 0;
         if (!fixed && tn < total && lane_id() == 0) claim = atomicAdd(ctr, 1u);
-        if (t < nHC) {
+        if (t < q.e0) {
             hub_chunk<T, P>(p, io, cur, s_flat[wib], maxc, vol);
-        } else if (t - nHC < q.tM) {
+        } else if (t < q.e1) {
             vertex_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
-        } else if (t - nHC - q.tM < q.tS) {
+        } else if (t < q.e2) {
+            mid_task<T, P, 16>(p, io, cur.e, q.s16, maxc, vol);
+        } else if (t < q.e3) {
+            mid_task<T, P, 8>(p, io, cur.e, q.s8, maxc, vol);
+        } else if (t < q.e4) {
             flat_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
         } else {
-            tiny_task<T, P>(p, io, cur.e, q.tsub, maxc, vol);
+            tiny_task<T, P>(p, io, cur.e, q.sT, maxc, vol);
         }
         const unsigned tnn = fixed ? tn + W : nstat * W + __shfl_sync(kFull, claim, 0);
         t = tn;
@@ -1547,9 +1745,8 @@ __global__ void __launch_bounds__(256, kMinBlocks) rounds_persistent_kernel(Para
     bool tail = false;
     for (int k = 2;; ++k) {
         const RoundCounts& c = st->rc[k % 3];
-        const unsigned long long hc = __ldcg(&c.hc);
-        const unsigned nT = __ldcg(&c.t), nS = __ldcg(&c.s), nM = __ldcg(&c.m), nH = hub_count(hc), nHC = hub_chunks(hc);
-        const unsigned size = nT + nS + nM + nH;
+        unsigned size;
+        const RoundSizes r = round_sizes_of(c, &size);
         // start of this pass (the last record, for the empty round, marks the end)
         if (p.round_ns && blockIdx.x == 0 && threadIdx.x == 0 && k - 1 <= p.round_cap)
             p.round_ns[k - 1] = globaltimer_ns();
@@ -1575,11 +1772,11 @@ __global__ void __launch_bounds__(256, kMinBlocks) rounds_persistent_kernel(Para
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             RoundCounts& z = st->rc[(k + 2) % 3];
             z.t = z.s = z.m = z.vol = 0u;
-            z.hc = 0ull;
+            z.mid = z.hc = 0ull;
             st->task_next[(k + 1) % 3] = 0u;  // round k + 1's claims (no one touches it in round k)
             if (k - 1 < p.round_cap) p.round_sizes[k - 1] = (int32_t)size;
         }
-        run_pass<T, P>(p, k, nT, nS, nM, nHC, maxc, gw, W, &st->task_next[k % 3]);
+        run_pass<T, P>(p, k, r, maxc, gw, W, &st->task_next[k % 3]);
         if (tail) {
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -1596,10 +1793,9 @@ __global__ void __launch_bounds__(256, kMinBlocks) rounds_persistent_kernel(Para
 
 // One pass per launch (loop mode 1): counts come from the host.
 template <typename T, bool P>  // P: a priority array is given
-__global__ void __launch_bounds__(256, kMinBlocks) round_kernel(Params<T> p, int k, unsigned nT, unsigned nS,
-                                                                unsigned nM, unsigned nHC) {
+__global__ void __launch_bounds__(256, kMinBlocks) round_kernel(Params<T> p, int k, RoundSizes r) {
     int maxc = 0;
-    run_pass<T, P>(p, k, nT, nS, nM, nHC, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+    run_pass<T, P>(p, k, r, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
              (gridDim.x * blockDim.x) >> 5, nullptr);
     fold_max_color(p.st, maxc);
 }
@@ -1624,9 +1820,10 @@ __global__ void __launch_bounds__(256, kMinBlocks) graph_round_kernel(Params<T> 
     RoundState* st = p.st;
     const int k = __ldcg(&st->graph_round);
     const RoundCounts& c = st->rc[k % 3];
-    const unsigned nT = __ldcg(&c.t), nS = __ldcg(&c.s), nM = __ldcg(&c.m), nHC = hub_chunks(__ldcg(&c.hc));
+    unsigned size;
+    const RoundSizes r = round_sizes_of(c, &size);
     int maxc = 0;
-    run_pass<T, P>(p, k, nT, nS, nM, nHC, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+    run_pass<T, P>(p, k, r, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
              (gridDim.x * blockDim.x) >> 5, nullptr);
     fold_max_color(st, maxc);
 }
@@ -1639,7 +1836,7 @@ __global__ void graph_cond_kernel(Params<T> p, int before_loop, cudaGraphConditi
     const int k = before_loop ? 1 : st->graph_round;
     const int kn = k + 1;
     const RoundCounts& c = st->rc[kn % 3];
-    const unsigned size = c.t + c.s + c.m + hub_count(c.hc);
+    const unsigned size = c.t + low_count(c.mid) + high_count(c.mid) + c.s + c.m + hub_count(c.hc);
     unsigned go = 0u;
     if (size == 0u) {
         st->rounds = k;
@@ -1651,7 +1848,7 @@ __global__ void graph_cond_kernel(Params<T> p, int before_loop, cudaGraphConditi
     } else {
         RoundCounts& z = st->rc[(kn + 1) % 3];
         z.t = z.s = z.m = z.vol = 0u;
-        z.hc = 0ull;
+        z.mid = z.hc = 0ull;
         if (kn - 1 < p.round_cap) p.round_sizes[kn - 1] = (int32_t)size;
         st->graph_round = kn;
         go = 1u;

@@ -43,7 +43,7 @@ def _cliques(degree, seed):
     return gg.from_edges(n, perm[us], perm[vs], name=f"cliques({degree})")
 
 
-@pytest.mark.parametrize("degree", [1, 7, 8, 24, 25, 31, 32, 33])
+@pytest.mark.parametrize("degree", [1, 7, 8, 24, 25, 31, 32, 33, 56, 57, 58, 63, 120, 121, 122])
 @pytest.mark.parametrize("keyed", [False, True])
 def test_bin_edges(gcpkg, degree, keyed):
     g = _cliques(degree, 100 + degree)
@@ -55,7 +55,7 @@ def test_bin_edges(gcpkg, degree, keyed):
         buf = torch.full((g.nnz + 16,), 1 << 30, dtype=torch.int32, device="cuda")
         ci = buf[shift:shift + g.nnz]
         ci.copy_(torch.from_numpy(g.colidx))
-        for options in (None, {"small_max_degree": 8}, {"color_bits": 32}):
+        for options in (None, {"small_max_degree": 8}, {"medium_max_degree": 64}, {"color_bits": 32}):
             got = gcpkg.color(rp, ci, pr, options=options, round_sizes=True)
             assert (got.ncolors, got.rounds) == (want.ncolors, want.rounds), (g.name, shift, options)
             assert np.array_equal(got.colors.cpu().numpy(), want.colors)
