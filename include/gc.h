@@ -97,8 +97,12 @@ typedef struct gc_options {
                                   last rounds are bound by their longest
                                   task, not by the barrier) */
     int32_t batch_mode;        /* gc_batch_create only.  0: choose (default:
-                                  2 when no graph holds more than 2/SMs of
-                                  the batch's vertices + entries, else 1);
+                                  2 for all but the largest graphs, which are
+                                  colored first as one union as in 1, when
+                                  that is estimated to be faster than 1 for
+                                  all; a graph is split off when a block of
+                                  its own would outlast the others' even
+                                  share of the SMs);
                                   1: all graphs share one persistent grid and
                                   its rounds (the single-graph kernels on the
                                   union); 2: one thread block per graph, its
@@ -307,7 +311,8 @@ int gc_color_async(const int32_t* rowptr, const int32_t* colidx, int32_t n, cons
  * gc_batch_create plans the batch: it checks the offsets and every graph's
  * rowptr, builds the union rowptr, scans degrees, allocates the plan's
  * workspace (mode 1: roughly 80 bytes per vertex plus 12 per adjacency entry;
- * mode 2: roughly 45 bytes per vertex) and, with opt->validate, checks ids,
+ * mode 2: roughly 45 bytes per vertex, and mode 1's for the graphs it splits
+ * off) and, with opt->validate, checks ids,
  * self loops and symmetry.  It synchronises
  * `stream`.  The plan keeps the array pointers: later runs read the caller's
  * colidx_cat and priority and write the outputs, so their contents may change
@@ -383,8 +388,9 @@ size_t gc_batch_workspace_bytes(const gc_batch* plan);
 int64_t gc_batch_launch_count(const gc_batch* plan);
 
 /* gc_batch_mode - how the plan colors its graphs: 1 (one persistent grid over
- * the union) or 2 (one thread block per graph), as gc_options.batch_mode
- * describes; GC_ERR_INVALID for NULL. */
+ * the union) or 2 (one thread block per graph; with batch_mode 0 the largest may
+ * have been split off), as gc_options.batch_mode describes; GC_ERR_INVALID for
+ * NULL. */
 int gc_batch_mode(const gc_batch* plan);
 
 /*

@@ -802,6 +802,14 @@ struct gc_batch {
     size_t off_queue = 0, off_order = 0, off_lanes = 0, off_ovf = 0, off_wl0 = 0, off_wl1 = 0, off_gcol8 = 0,
            off_gcol32 = 0;
     int32_t* ucolidx = nullptr;  // mode 2: union colidx, allocated when validation or features need it
+    const int64_t* src_eoff = nullptr;  // mode 1 plan of some graphs of a batch: where their entries sit in colidx_cat
+    // mode 2: the graphs too large for one block, colored by a mode 1 plan of
+    // their own before the others (big_ws: its inputs and outputs)
+    gc_batch* big = nullptr;
+    int32_t nbig = 0;
+    void* big_ws = nullptr;
+    size_t big_ws_bytes = 0, off_big_voff = 0, off_big_src = 0, off_big_ids = 0, off_big_prio = 0, off_big_colors = 0,
+           off_big_nc = 0, off_big_rd = 0;
     cudaStream_t cap_stream = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -840,7 +848,7 @@ int batch_rebase(gc_batch& b, cudaStream_t s, int64_t* launches) {
     const int64_t spans = (b.NNZ + gc::kRebaseSpan - 1) / gc::kRebaseSpan;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((spans + 7) / 8, (int64_t)b.sms * 8));
     gc::batch_colidx_kernel<<<grid, 256, 0, s>>>(b.colidx_cat, (const int64_t*)(base + b.off_voff),
-                                                 (const int64_t*)(base + b.off_eoff), b.G, b.NNZ, colidx_g, fl);
+                                                 (const int64_t*)(base + b.off_eoff), b.src_eoff, b.G, b.NNZ, colidx_g, fl);
     GC_CUDA(cudaGetLastError());
     ++*launches;
     return GC_OK;
@@ -858,7 +866,7 @@ int batch_enqueue_local(gc_batch& b, cudaStream_t s) {
     lp.voff = (const int64_t*)(base + b.off_voff);
     lp.order = (const int32_t*)(base + b.off_order);
     lp.lanes_log2 = (const uint8_t*)(base + b.off_lanes);
-    lp.G = b.G;
+    lp.G = b.G - b.nbig;
     lp.max_rounds = b.o.max_rounds;
     lp.smem_bytes = b.local_smem;
     lp.wl0 = (int4*)(base + b.off_wl0);
@@ -884,7 +892,31 @@ int batch_enqueue_local(gc_batch& b, cudaStream_t s) {
     GC_CUDA(cudaGetLastError());
     gc::batch_local_kernel<uint32_t, P><<<b.sms, gc::kLocalThreads, b.local_smem, s>>>(lp, 1);
     GC_CUDA(cudaGetLastError());
-    b.launches_per_run = 2;
+    b.launches_per_run += 2;
+    return GC_OK;
+}
+
+// Mode 2: the graphs colored apart (b.big), as one union on the whole GPU.
+int batch_enqueue(gc_batch& b, cudaStream_t s);
+int batch_enqueue_big(gc_batch& b, cudaStream_t s) {
+    char* base = (char*)b.big_ws;
+    const int64_t* voff = (const int64_t*)(base + b.off_big_voff);
+    const int64_t* src = (const int64_t*)(base + b.off_big_src);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((b.big->N + 255) / 256, (int64_t)b.sms * 8));
+    if (b.prio) {
+        gc::subset_gather_kernel<<<grid, 256, 0, s>>>(b.prio, voff, src, b.nbig, b.big->N,
+                                                      (uint32_t*)(base + b.off_big_prio));
+        GC_CUDA(cudaGetLastError());
+        b.launches_per_run += 1;
+    }
+    const int rc = batch_enqueue(*b.big, s);
+    if (rc != GC_OK) return rc;
+    gc::subset_scatter_kernel<<<grid, 256, 0, s>>>(
+        (const int32_t*)(base + b.off_big_colors), (const int32_t*)(base + b.off_big_nc),
+        (const int32_t*)(base + b.off_big_rd), voff, src, (const int32_t*)(base + b.off_big_ids), b.nbig, b.big->N,
+        b.colors_out, b.ncolors_out, b.rounds_out);
+    GC_CUDA(cudaGetLastError());
+    b.launches_per_run += b.big->launches_per_run + 1;
     return GC_OK;
 }
 
@@ -986,7 +1018,14 @@ int batch_enqueue(gc_batch& b, cudaStream_t s) {
     GC_CUDA(cudaGetDevice(&dev));
     if (dev != b.device) return GC_ERR_INVALID;
     if (b.G == 0 || b.N == 0) return GC_OK;
-    if (b.mode == 2) return b.prio ? batch_enqueue_local<true>(b, s) : batch_enqueue_local<false>(b, s);
+    if (b.mode == 2) {
+        b.launches_per_run = 0;
+        if (b.big) {
+            const int rc = batch_enqueue_big(b, s);
+            if (rc != GC_OK) return rc;
+        }
+        return b.prio ? batch_enqueue_local<true>(b, s) : batch_enqueue_local<false>(b, s);
+    }
     return b.bits == 16 ? batch_enqueue_typed<uint16_t>(b, s) : batch_enqueue_typed<int32_t>(b, s);
 }
 
@@ -998,12 +1037,139 @@ void batch_free(gc_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-    if (b->ws || b->ucolidx) cudaDeviceSynchronize();
+    if (b->ws || b->ucolidx || b->big_ws) cudaDeviceSynchronize();
+    batch_free(b->big);
+    if (b->big_ws) cudaFree(b->big_ws);
     if (b->ws) cudaFree(b->ws);
     if (b->ucolidx) cudaFree(b->ucolidx);
     cudaSetDevice(cur);
     (void)cudaGetLastError();
     delete b;
+}
+
+constexpr int32_t kLocalSharedDefault = 164 * 1024;  // mode 2: bytes of shared memory per block for colors
+
+// How a batch with batch_mode 0 is split.  Costs are in vertices + entries of
+// a graph that one SM colors alone (about 2 ns each, over all its rounds).  The
+// `nbig` largest graphs go to the whole GPU as one union, which takes
+// kUnionFixed plus kUnionFactor times their even share of the SMs; the others
+// take a block each, as long as the largest of them or their even share,
+// whichever is longer; a graph whose colors do not fit shared memory counts
+// twice there.  All graphs in the union is mode 1.
+//
+// A block colors one graph's rounds in sequence, so one 262,144-vertex R-MAT
+// graph (14 ms alone) set the time of a 1,024-graph batch whose even share was
+// 5 ms: 15.13 ms with a block each, 10.69 with all in the union, 6.06 split; a
+// 2,500-graph batch 16.21 -> 14.34.  Factors from 2.5 to 4.5 pick splits within
+// 7 % of each other on eight batches of 96 to 2,500 graphs; 2 and less put so
+// many graphs in the union that the first takes 7.18 ms.
+constexpr double kUnionFixed = 1e5, kUnionFactor = 2.5;
+
+int32_t split_batch(const std::vector<int32_t>& order, const int64_t* voff, const int64_t* eoff, int sms,
+                    int64_t shared_vertices) {
+    const int32_t G = (int32_t)order.size();
+    auto work = [&](int32_t i) {
+        const int32_t g = order[(size_t)i];
+        return (double)((voff[g + 1] - voff[g]) + (eoff[g + 1] - eoff[g]));
+    };
+    auto alone = [&](int32_t i) {
+        const int32_t g = order[(size_t)i];
+        return work(i) * (voff[g + 1] - voff[g] > shared_vertices ? 2.0 : 1.0);
+    };
+    // largest single-block cost from i on
+    std::vector<double> most((size_t)G + 1, 0.0);
+    double rest = 0.0;
+    for (int32_t i = G - 1; i >= 0; --i) {
+        most[(size_t)i] = std::max(most[(size_t)i + 1], alone(i));
+        rest += alone(i);
+    }
+    int32_t best = 0;
+    double best_cost = std::max(rest / sms, most[0]), big = 0.0;
+    for (int32_t i = 0; i < G; ++i) {
+        big += work(i);
+        rest -= alone(i);
+        const double cost = kUnionFixed + kUnionFactor * big / sms + std::max(rest / sms, most[(size_t)i + 1]);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = i + 1;
+        }
+    }
+    if (most[(size_t)best] == 0.0) best = G;  // nothing but empty graphs left
+    return best;
+}
+
+int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, const int64_t* voff_h,
+                        const int64_t* eoff_h, int32_t G, const uint32_t* prio, int32_t* colors_out,
+                        int32_t* ncolors_out, int32_t* rounds_out, const gc_options* opt, cudaStream_t s,
+                        gc_batch* b);
+
+// Mode 2: plan the graphs order[0 .. nbig) as a union of their own.  Leaves
+// b->big empty (they then take a block each, like the others) when there is no
+// memory for it.
+int batch_plan_big(gc_batch* b, const std::vector<int32_t>& order, int32_t nbig, const int32_t* rowptr_cat,
+                   const int64_t* voff, const int64_t* eoff, cudaStream_t s) {
+    std::vector<int64_t> sv((size_t)nbig + 1, 0), se((size_t)nbig + 1, 0), src((size_t)nbig), esrc((size_t)nbig);
+    for (int32_t i = 0; i < nbig; ++i) {
+        const int32_t g = order[(size_t)i];
+        sv[(size_t)i + 1] = sv[(size_t)i] + voff[g + 1] - voff[g];
+        se[(size_t)i + 1] = se[(size_t)i] + eoff[g + 1] - eoff[g];
+        src[(size_t)i] = voff[g];
+        esrc[(size_t)i] = eoff[g];
+    }
+    const int64_t n = sv[(size_t)nbig];
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        size_t o = off;
+        off = align_up(off + std::max<size_t>(bytes, 16), 256);
+        return o;
+    };
+    b->off_big_voff = take(((size_t)nbig + 1) * 8);
+    b->off_big_src = take((size_t)nbig * 8);
+    const size_t off_esrc = take((size_t)nbig * 8), off_rowptr = take((size_t)(n + nbig) * 4);
+    b->off_big_ids = take((size_t)nbig * 4);
+    b->off_big_nc = take((size_t)nbig * 4);
+    b->off_big_rd = take((size_t)nbig * 4);
+    b->off_big_colors = take((size_t)n * 4);
+    b->off_big_prio = b->prio ? take((size_t)n * 4) : 0;
+    if (b->o.workspace_limit_mb > 0 && off > ((size_t)b->o.workspace_limit_mb << 20)) return GC_OK;
+    if (cudaMalloc(&b->big_ws, off) != cudaSuccess) {
+        (void)cudaGetLastError();
+        b->big_ws = nullptr;
+        return GC_OK;
+    }
+    b->big_ws_bytes = off;
+    char* base = (char*)b->big_ws;
+    GC_CUDA(cudaMemcpyAsync(base + b->off_big_voff, sv.data(), sv.size() * 8, cudaMemcpyHostToDevice, s));
+    GC_CUDA(cudaMemcpyAsync(base + b->off_big_src, src.data(), src.size() * 8, cudaMemcpyHostToDevice, s));
+    GC_CUDA(cudaMemcpyAsync(base + off_esrc, esrc.data(), esrc.size() * 8, cudaMemcpyHostToDevice, s));
+    GC_CUDA(cudaMemcpyAsync(base + b->off_big_ids, order.data(), (size_t)nbig * 4, cudaMemcpyHostToDevice, s));
+    int32_t* rp = (int32_t*)(base + off_rowptr);
+    for (int32_t i = 0; i < nbig; ++i) {
+        const int32_t g = order[(size_t)i];
+        GC_CUDA(cudaMemcpyAsync(rp + sv[(size_t)i] + i, rowptr_cat + voff[g] + g,
+                                (size_t)(voff[g + 1] - voff[g] + 1) * 4, cudaMemcpyDeviceToDevice, s));
+    }
+    gc_options o = b->o;
+    o.batch_mode = 1;
+    o.validate = 0;
+    gc_batch* big = new (std::nothrow) gc_batch();
+    if (!big) return GC_ERR_OOM;
+    const int rc = batch_create_locked(rp, b->colidx_cat, sv.data(), se.data(), nbig,
+                                       b->prio ? (const uint32_t*)(base + b->off_big_prio) : nullptr,
+                                       (int32_t*)(base + b->off_big_colors), (int32_t*)(base + b->off_big_nc),
+                                       (int32_t*)(base + b->off_big_rd), &o, s, big);
+    if (rc != GC_OK) {
+        batch_free(big);
+        if (rc != GC_ERR_OOM) return rc;
+        cudaFree(b->big_ws);
+        b->big_ws = nullptr;
+        b->big_ws_bytes = 0;
+        return GC_OK;
+    }
+    big->src_eoff = (const int64_t*)(base + off_esrc);
+    b->big = big;
+    b->nbig = nbig;
+    return GC_OK;
 }
 
 int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, const int64_t* voff_h,
@@ -1089,17 +1255,27 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     const int32_t max_rounds = b->o.max_rounds > 0 ? b->o.max_rounds : (int32_t)N;
     b->round_cap = std::max<int64_t>(1, std::min<int64_t>(max_rounds, 4096));
 
-    // Mode: one block per graph pays off when no graph is a large share of the
-    // batch's work (vertices + entries): then the graphs keep every SM busy.
-    int64_t max_work = 0;
-    for (int32_t g = 0; g < G; ++g)
-        max_work = std::max<int64_t>(max_work, (voff_h[g + 1] - voff_h[g]) + (eoff_h[g + 1] - eoff_h[g]));
-    b->mode = b->o.batch_mode != 0 ? b->o.batch_mode : (max_work * b->sms <= 2 * (N + NNZ) ? 2 : 1);
+    // graphs in the order the queue of mode 2 hands them out: most work first
+    std::vector<int32_t> order((size_t)G);
+    for (int32_t g = 0; g < G; ++g) order[(size_t)g] = g;
+    std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t c) {
+        return (voff_h[a + 1] - voff_h[a]) + (eoff_h[a + 1] - eoff_h[a]) >
+               (voff_h[c + 1] - voff_h[c]) + (eoff_h[c + 1] - eoff_h[c]);
+    });
+    // Mode: the caller's, or one block per graph for all but the largest graphs
+    // when that is cheaper than the union of all
+    int32_t nbig = 0;
+    b->mode = b->o.batch_mode;
+    if (b->mode == 0) {
+        nbig = split_batch(order, voff_h, eoff_h, b->sms,
+                           b->o.local_shared_bytes > 0 ? b->o.local_shared_bytes : kLocalSharedDefault);
+        b->mode = nbig < G ? 2 : 1;
+    }
     if (b->mode == 2) {
         rc = local_kernels_setup(b->device, &b->local_smem);
         if (rc != GC_OK) return fail(rc);
         b->local_smem = std::min<uint32_t>(
-            b->local_smem, b->o.local_shared_bytes > 0 ? (uint32_t)b->o.local_shared_bytes : 164u * 1024u);
+            b->local_smem, b->o.local_shared_bytes > 0 ? (uint32_t)b->o.local_shared_bytes : (uint32_t)kLocalSharedDefault);
         b->bits = 8;
         off = align_up(head, 256);
         b->L = Layout{};
@@ -1119,22 +1295,16 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
         b->off_eoff = h_eoff;
         b->off_rowptr = h_rowptr;
         b->off_flags = h_flags;
-        // queue order: most work first; lanes per vertex from the average degree
+        // lanes per vertex from the average degree
         const int64_t tpv = b->o.local_thread_degree == 0 ? 32 : b->o.local_thread_degree;
-        std::vector<int32_t> order((size_t)G);
         std::vector<uint8_t> lanes((size_t)G);
         for (int32_t g = 0; g < G; ++g) {
-            order[(size_t)g] = g;
             const int64_t ng = voff_h[g + 1] - voff_h[g], eg = eoff_h[g + 1] - eoff_h[g];
             const int64_t avg = ng > 0 ? (eg + ng - 1) / ng : 0;
             int lg = 2;
             while (lg < 5 && (int64_t(1) << lg) * 2 < avg) ++lg;  // about avg/2 lanes, 4..32
             lanes[(size_t)g] = (uint8_t)(avg <= tpv ? 0 : lg);
         }
-        std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t c) {
-            return (voff_h[a + 1] - voff_h[a]) + (eoff_h[a + 1] - eoff_h[a]) >
-                   (voff_h[c + 1] - voff_h[c]) + (eoff_h[c + 1] - eoff_h[c]);
-        });
         void* ws = nullptr;
         if (b->o.workspace_limit_mb > 0 && b->ws_bytes > ((size_t)b->o.workspace_limit_mb << 20))
             return fail(GC_ERR_OOM);
@@ -1144,10 +1314,14 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
             return fail(e == cudaErrorMemoryAllocation ? GC_ERR_OOM : GC_ERR_CUDA);
         }
         b->ws = ws;
+        if (nbig > 0) {
+            rc = batch_plan_big(b, order, nbig, rowptr_cat, voff_h, eoff_h, s);
+            if (rc != GC_OK) return fail(rc);
+        }
         char* base = (char*)b->ws;
         if (cudaMemcpyAsync(base, tmp, head, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
-            cudaMemcpyAsync(base + b->off_order, order.data(), (size_t)G * 4, cudaMemcpyHostToDevice, s) !=
-                cudaSuccess ||
+            cudaMemcpyAsync(base + b->off_order, order.data() + b->nbig, (size_t)(G - b->nbig) * 4,
+                            cudaMemcpyHostToDevice, s) != cudaSuccess ||
             cudaMemcpyAsync(base + b->off_lanes, lanes.data(), (size_t)G, cudaMemcpyHostToDevice, s) != cudaSuccess)
             return fail(GC_ERR_CUDA);
         fail(GC_OK);  // waits for the copies, frees the head copy
@@ -1207,8 +1381,8 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
         GC_CUDA(cudaMemsetAsync(fl, 0, sizeof(gc::BatchFlags), s));
         if (NNZ > 0) {
             gc::batch_colidx_kernel<<<grid, 256, 0, s>>>(colidx_cat, (const int64_t*)(base + b->off_voff),
-                                                         (const int64_t*)(base + b->off_eoff), G, NNZ, colidx_g,
-                                                         fl);
+                                                         (const int64_t*)(base + b->off_eoff), nullptr, G, NNZ,
+                                                         colidx_g, fl);
             GC_CUDA(cudaGetLastError());
         }
         GC_CUDA(cudaMemcpyAsync(&hf, fl, sizeof(hf), cudaMemcpyDeviceToHost, s));
@@ -1237,9 +1411,12 @@ int batch_status(gc_batch* b, cudaStream_t s, int32_t* max_rounds, int32_t* max_
     GC_CUDA(cudaMemcpyAsync(&hst, base + b->L.st, sizeof(hst), cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaMemcpyAsync(&hf, base + b->off_flags, sizeof(hf), cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaStreamSynchronize(s));
-    if (max_rounds) *max_rounds = hst.rounds;
-    if (max_colors) *max_colors = hst.max_color;
-    if (hf.bad_colidx) return GC_ERR_BAD_GRAPH;
+    int32_t big_rounds = 0, big_colors = 0;
+    const int big = b->big ? batch_status(b->big, s, &big_rounds, &big_colors) : GC_OK;
+    if (max_rounds) *max_rounds = std::max(hst.rounds, big_rounds);
+    if (max_colors) *max_colors = std::max(hst.max_color, big_colors);
+    if (hf.bad_colidx || big == GC_ERR_BAD_GRAPH) return GC_ERR_BAD_GRAPH;
+    if (big != GC_OK) return big;
     if (hst.status == gc::kStatusTimeout) return GC_ERR_TIMEOUT;
     if (hst.status == gc::kStatusMaxRounds) return GC_ERR_MAX_ROUNDS;
     if (hst.status != 0) return GC_ERR_CUDA;
@@ -1477,7 +1654,32 @@ int gc_batch_round_stats(gc_batch* plan, int32_t* sizes, int64_t* volumes, int32
     RoundState hst;
     GC_CUDA(cudaMemcpyAsync(&hst, base + b.L.st, sizeof(hst), cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaStreamSynchronize(s));
-    const int32_t m = (int32_t)std::min<int64_t>({(int64_t)hst.rounds, (int64_t)cap, b.round_cap});
+    // graphs colored apart: what they add comes from their settle rounds
+    int32_t rounds = hst.rounds;
+    std::vector<unsigned long long> big;  // per round: vertices that settle in it, then their entries
+    if (b.big) {
+        RoundState hb;
+        char* bb = (char*)b.big->ws;
+        GC_CUDA(cudaMemcpyAsync(&hb, bb + b.big->L.st, sizeof(hb), cudaMemcpyDeviceToHost, s));
+        GC_CUDA(cudaStreamSynchronize(s));
+        rounds = std::max(rounds, hb.rounds);
+        const int32_t bins = std::max(1, hb.rounds);
+        big.assign((size_t)bins * 2, 0ull);
+        unsigned long long* d = nullptr;
+        GC_CUDA(cudaMalloc(&d, big.size() * 8));
+        cudaError_t e = cudaMemsetAsync(d, 0, big.size() * 8, s);
+        if (e == cudaSuccess) {
+            gc::settle_histogram_kernel<<<b.sms * 2, 256, 0, s>>>((const int32_t*)(bb + b.big->off_rowptr),
+                                                                  (const int32_t*)(bb + b.big->off_settle),
+                                                                  (int32_t)b.big->N, bins, d, d + bins);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(big.data(), d, big.size() * 8, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        cudaFree(d);
+        GC_CUDA(e);
+    }
+    const int32_t m = (int32_t)std::min<int64_t>({(int64_t)rounds, (int64_t)cap, b.round_cap});
     if (m <= 0) return 0;
     if (sizes) {
         sizes[0] = (int32_t)b.N;
@@ -1492,6 +1694,13 @@ int gc_batch_round_stats(gc_batch* plan, int32_t* sizes, int64_t* volumes, int32
                                     cudaMemcpyDeviceToHost, s));
     }
     GC_CUDA(cudaStreamSynchronize(s));
+    unsigned long long left_n = 0, left_e = 0;
+    for (int32_t r = (int32_t)(big.size() / 2); r >= 2; --r) {
+        left_n += big[(size_t)r - 1];
+        left_e += big[big.size() / 2 + (size_t)r - 1];
+        if (r <= m && sizes) sizes[r - 1] += (int32_t)left_n;
+        if (r <= m && volumes) volumes[r - 1] += (int64_t)left_e;
+    }
     return m;
 }
 
@@ -1641,7 +1850,9 @@ int gc_batch_tune(const int32_t* rowptr_cat, const int32_t* colidx_cat, const in
     return rc;
 }
 
-size_t gc_batch_workspace_bytes(const gc_batch* plan) { return plan ? plan->ws_bytes : 0; }
+size_t gc_batch_workspace_bytes(const gc_batch* plan) {
+    return plan ? plan->ws_bytes + plan->big_ws_bytes + gc_batch_workspace_bytes(plan->big) : 0;
+}
 
 int64_t gc_batch_launch_count(const gc_batch* plan) { return plan ? plan->launches_per_run : 0; }
 

@@ -68,11 +68,14 @@ __global__ void batch_rowptr_kernel(const int32_t* __restrict__ rowptr_cat, cons
 // loads and stores, 16 in flight per lane); each lane walks its entries in
 // increasing order, so its graph only moves forward.  A local id outside
 // [0, n_g) is flagged and replaced by 0, so every id stays inside the union.
+// When the union is made of some graphs of a larger batch, src[g] is where
+// graph g's entries sit in colidx_cat (NULL: at eoff[g]).
 constexpr int kRebaseSpan = 512;
 
 __global__ void __launch_bounds__(256) batch_colidx_kernel(const int32_t* __restrict__ colidx_cat,
                                                            const int64_t* __restrict__ voff,
-                                                           const int64_t* __restrict__ eoff, int32_t G,
+                                                           const int64_t* __restrict__ eoff,
+                                                           const int64_t* __restrict__ src, int32_t G,
                                                            int64_t NNZ, int32_t* __restrict__ colidx_g,
                                                            BatchFlags* fl) {
     const unsigned lane = lane_id();
@@ -85,10 +88,23 @@ __global__ void __launch_bounds__(256) batch_colidx_kernel(const int32_t* __rest
         int32_t g = graph_of(eoff, G, s0);
         int64_t gend = __ldg(eoff + g + 1);
         int32_t x[kRebaseSpan / 32];
+        // entry e of the union is entry e + shift of colidx_cat; with src, the
+        // shift holds for the span when one graph owns all of it
+        const int64_t shift = src ? __ldg(src + g) - __ldg(eoff + g) : 0;
+        const bool whole = !src || gend >= min(NNZ, s0 + kRebaseSpan);
+        if (whole) {
 #pragma unroll
-        for (int i = 0; i < kRebaseSpan / 32; ++i) {
-            const int64_t e = s0 + i * 32 + lane;
-            x[i] = e < NNZ ? __ldg(colidx_cat + e) : 0;
+            for (int i = 0; i < kRebaseSpan / 32; ++i) {
+                const int64_t e = s0 + i * 32 + lane;
+                x[i] = e < NNZ ? __ldg(colidx_cat + e + shift) : 0;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kRebaseSpan / 32; ++i) {
+                const int64_t e = s0 + i * 32 + lane;
+                const int32_t h = e < NNZ ? graph_of(eoff, G, e) : 0;
+                x[i] = e < NNZ ? __ldg(colidx_cat + __ldg(src + h) + (e - __ldg(eoff + h))) : 0;
+            }
         }
 #pragma unroll
         for (int i = 0; i < kRebaseSpan / 32; ++i) {
@@ -165,6 +181,71 @@ __global__ void batch_reduce_kernel(const int32_t* __restrict__ colors, const in
             }
         }
     }
+}
+
+// Graphs of a batch colored apart as a union of their own: vertex i of its
+// graph g is vertex voff[g] + i of the union and src[g] + i of the batch.
+
+// to[union] = from[batch] (keys, before a run).
+__global__ void subset_gather_kernel(const uint32_t* __restrict__ from, const int64_t* __restrict__ voff,
+                                     const int64_t* __restrict__ src, int32_t G, int64_t N,
+                                     uint32_t* __restrict__ to) {
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < N; x += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t g = graph_of(voff, G, x);
+        to[x] = __ldg(from + __ldg(src + g) + (x - __ldg(voff + g)));
+    }
+}
+
+// Results of the union to the batch (after a run): colors by vertex, counts by graph.
+__global__ void subset_scatter_kernel(const int32_t* __restrict__ colors, const int32_t* __restrict__ ncolors,
+                                      const int32_t* __restrict__ rounds, const int64_t* __restrict__ voff,
+                                      const int64_t* __restrict__ src, const int32_t* __restrict__ ids, int32_t G,
+                                      int64_t N, int32_t* __restrict__ colors_out, int32_t* __restrict__ ncolors_out,
+                                      int32_t* __restrict__ rounds_out) {
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, T = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t x = tid; x < N; x += T) {
+        const int32_t g = graph_of(voff, G, x);
+        colors_out[__ldg(src + g) + (x - __ldg(voff + g))] = __ldg(colors + x);
+    }
+    for (int64_t g = tid; g < G; g += T) {
+        ncolors_out[__ldg(ids + g)] = __ldg(ncolors + g);
+        rounds_out[__ldg(ids + g)] = __ldg(rounds + g);
+    }
+}
+
+// Telemetry of a union run, from its settle rounds: cnt[r-1] vertices, with
+// deg[r-1] entries in their rows, settled in round r <= cap (the last bin
+// takes later ones too).
+constexpr int kSettleBins = 1024;
+
+__global__ void __launch_bounds__(256) settle_histogram_kernel(const int32_t* __restrict__ rowptr,
+                                                               const int32_t* __restrict__ settle, int32_t n,
+                                                               int32_t cap, unsigned long long* __restrict__ cnt,
+                                                               unsigned long long* __restrict__ deg) {
+    __shared__ unsigned s_cnt[kSettleBins];
+    __shared__ unsigned long long s_deg[kSettleBins];
+    for (int i = threadIdx.x; i < kSettleBins; i += blockDim.x) {
+        s_cnt[i] = 0u;
+        s_deg[i] = 0ull;
+    }
+    __syncthreads();
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t r = min(__ldg(settle + v), cap) - 1;
+        const unsigned long long d = (unsigned long long)(__ldg(rowptr + v + 1) - __ldg(rowptr + v));
+        if (r >= 0 && r < kSettleBins) {
+            atomicAdd(&s_cnt[r], 1u);
+            atomicAdd(&s_deg[r], d);
+        } else if (r >= 0) {
+            atomicAdd(cnt + r, 1ull);
+            atomicAdd(deg + r, d);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < min(cap, kSettleBins); i += blockDim.x)
+        if (s_cnt[i]) {
+            atomicAdd(cnt + i, (unsigned long long)s_cnt[i]);
+            atomicAdd(deg + i, s_deg[i]);
+        }
 }
 
 }  // namespace gc

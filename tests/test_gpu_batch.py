@@ -330,3 +330,46 @@ def test_color_batched_one_call(gcpkg, mode):
     with pytest.raises(gcpkg.GcError) as e:
         gcpkg.color_batched(_dev(rp), _dev(badc), voff, eoff, options={"batch_mode": mode})
     assert e.value.code == gcpkg.GC_ERR_BAD_GRAPH
+
+
+@pytest.mark.parametrize("keyed", [False, True])
+@pytest.mark.parametrize("large", [1, 3])
+def test_largest_graphs_split_off(gcpkg, keyed, large):
+    """With the default mode, graphs that would outlast the rest of the batch are colored
+    as a union of their own; every result is still each graph's own, wherever the large ones
+    sit, as launches and as graph replays, and the telemetry covers the whole batch."""
+    big = [gg.rmat(15, 16, gg.RMAT_G, 5), gg.rgg(30011, 6), gg.star(20000, 77)][:large]
+    gs = gg.batch_mix(3000, 8, n_min=1, n_max=250)
+    for i, g in enumerate(big):
+        gs.insert((0, 101, len(gs))[i], g)
+    keys = [(gg.draws(30 + i, 5, g.n) & np.uint64(0x7)).astype(np.uint32) for i, g in enumerate(gs)] if keyed else None
+    b, voff = _plan(gcpkg, gs, keys)
+    assert b.mode == 2
+    for graph in (False, True):
+        b.colors.fill_(-1)
+        b.run(graph=graph)
+        mr, mc = b.status()
+        _check(gs, b, voff, keys)
+    assert b.launch_count == 8 + keyed           # 2, and 5 of the union between gather and scatter
+    assert mr == int(b.rounds.max()) and mc == int(b.ncolors.max())
+    sizes, vols, _ = b.round_stats()
+    want, deg = np.zeros(mr, np.int64), np.zeros(mr, np.int64)
+    for i, g in enumerate(gs):
+        ref = oracle.iterative(g.rowptr, g.colidx, None if keys is None else keys[i])
+        want[:len(ref.round_sizes)] += ref.round_sizes
+        for k in range(1, mr + 1):
+            deg[k - 1] += int(g.degrees[ref.settle_round >= k].sum())
+    assert sizes.tolist() == want.tolist() and vols.tolist() == deg.tolist()
+    # an id outside a large graph is reported like any other
+    rp, ci, voff, eoff = gcpkg.pack_batch((g.rowptr, g.colidx) for g in gs)
+    ci[eoff[0] + 3] = gs[0].n
+    b = gcpkg.Batch(_dev(rp), _dev(ci), voff, eoff)
+    b.run()
+    with pytest.raises(gcpkg.GcError) as e:
+        b.status()
+    assert e.value.code == gcpkg.GC_ERR_BAD_GRAPH
+    # without room for the union the large graphs take a block each
+    room = gcpkg.Batch(_dev(rp), _dev(ci), voff, eoff, options={"batch_mode": 2}).workspace_bytes
+    lim = gcpkg.Batch(_dev(rp), _dev(ci), voff, eoff, options={"workspace_limit_mb": (room >> 20) + 1})
+    lim.run()
+    assert lim.mode == 2 and lim.launch_count == 2 and lim.workspace_bytes == room
