@@ -249,6 +249,14 @@ void fill_workspace(Params<T>& p, char* base, const Layout& L, RoundState* st, i
     p.round_cap = (int32_t)round_cap;
 }
 
+// Blocks of the cooperative rounds kernel: all that fit, or, for a small graph,
+// one warp per 8 vertices or 128 entries (what a warp reads side by side), so
+// that fewer blocks meet at the barriers.
+unsigned rounds_blocks(int64_t n, int64_t nnz, int threads, int64_t most) {
+    const int64_t warps = std::max(n / 8, nnz / 128) + 1, per_block = threads / 32;
+    return (unsigned)std::min(most, (warps + per_block - 1) / per_block);
+}
+
 // Loop mode 2: rounds 2.. as one CUDA graph: a condition kernel, then a while
 // node whose body is one round kernel and the condition kernel, so the loop
 // runs on the device without a cooperative launch or host round trips.  The
@@ -342,7 +350,7 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
         GC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
             &per_sm, gc::rounds_persistent_kernel<T, P>, threads, 0));
         if (per_sm < 1 || !dc.coop) return GC_ERR_CUDA;
-        dim3 grid(per_sm * dc.sms), block(threads);
+        dim3 grid(rounds_blocks(p.n, p.nnz, threads, (int64_t)per_sm * dc.sms)), block(threads);
         void* args[] = {&p};
         GC_CUDA(cudaLaunchCooperativeKernel((const void*)gc::rounds_persistent_kernel<T, P>, grid, block,
                                             args, 0, s));
@@ -366,7 +374,7 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
         GC_CUDA(cudaMemcpyAsync(h, &st->rc[k % 3], sizeof(gc::RoundCounts), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
         const gc::RoundSizes r = {h->t, gc::low_count(h->mid), gc::high_count(h->mid), h->s, h->m,
-                                  gc::hub_chunks(h->hc)};
+                                  gc::hub_chunks(h->hc), 0u};
         const unsigned size = r.nT + r.n8 + r.n16 + r.nS + r.nM + gc::hub_count(h->hc);
         if (size == 0) break;
         if (k > p.max_rounds) {
@@ -983,7 +991,7 @@ int batch_enqueue_typed(gc_batch& b, cudaStream_t s) {
     }
     {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(b.per_sm * b.sms));
+        cfg.gridDim = dim3(rounds_blocks(b.N, b.NNZ, b.o.block_threads, (int64_t)b.per_sm * b.sms));
         cfg.blockDim = dim3((unsigned)b.o.block_threads);
         cfg.dynamicSmemBytes = 0;
         cfg.stream = s;
