@@ -172,7 +172,7 @@ int ensure_device_limited(void** p, size_t* have, size_t need, int32_t limit_mb)
 
 struct Layout {
     size_t st, rs, rv, rt, x0, x1, act0, act1, stat, hubs, defer;
-    size_t T[2], L8[2], L16[2], S[2], M[2], H[2], Hc[2], O[2];
+    size_t L2[2], L4[2], L8[2], L16[2], S[2], M[2], H[2], Hc[2], O[2];
     size_t total;
 };
 
@@ -197,12 +197,13 @@ Layout make_layout(int64_t n, int64_t nnz, size_t elem, const Stats& hs, int64_t
     L.hubs = take((size_t)hs.cap[gc::kBinH] * sizeof(gc::HubRecord));
     L.defer = take((size_t)hs.defer * sizeof(int32_t));
     for (int b = 0; b < 2; ++b) {
-        // T: degree 1 .. s_max; L8 and L16: up to their limits; M: longer ones, and H
-        // lists that shrink to m_max; S: M and H lists that shrink to s_max
-        const size_t cT = hs.cap[gc::kBinS] - hs.cap[gc::kBinM], c8 = hs.cap[gc::kBinM] - hs.over8,
-                     c16 = hs.over8 - hs.over16, cM = hs.over16;
-        L.T[b] = take((cT + c8 + c16 + 2 * cM) * sizeof(int4));
-        L.L8[b] = L.T[b] + cT * sizeof(int4);
+        // L2 to L16: by degree, up to their limits; M: longer rows, and H lists that
+        // shrink to m_max; S: M and H lists that shrink to s_max
+        const size_t c2 = hs.cap[gc::kBinS] - hs.over2, c4 = hs.over2 - hs.cap[gc::kBinM],
+                     c8 = hs.cap[gc::kBinM] - hs.over8, c16 = hs.over8 - hs.over16, cM = hs.over16;
+        L.L2[b] = take((c2 + c4 + c8 + c16 + 2 * cM) * sizeof(int4));
+        L.L4[b] = L.L2[b] + c2 * sizeof(int4);
+        L.L8[b] = L.L4[b] + c4 * sizeof(int4);
         L.L16[b] = L.L8[b] + c8 * sizeof(int4);
         L.M[b] = L.L16[b] + c16 * sizeof(int4);
         L.S[b] = L.M[b] + cM * sizeof(int4);
@@ -217,14 +218,17 @@ Layout make_layout(int64_t n, int64_t nnz, size_t elem, const Stats& hs, int64_t
 // A call's pointers into its workspace (p.s_max and p.m_max are set).
 template <typename T>
 void fill_workspace(Params<T>& p, char* base, const Layout& L, RoundState* st, int64_t round_cap) {
-    p.mid8 = gc::mid_limit(8, p.s_max, p.m_max);
-    p.mid16 = gc::mid_limit(16, p.s_max, p.m_max);
+    p.lim2 = gc::tiny_limit(2, p.s_max);
+    p.lim4 = gc::tiny_limit(4, p.s_max);
+    p.lim8 = gc::mid_limit(8, p.s_max, p.m_max);
+    p.lim16 = gc::mid_limit(16, p.s_max, p.m_max);
     p.X0 = (T*)(base + L.x0);
     p.X1 = (T*)(base + L.x1);
     p.act0 = (int32_t*)(base + L.act0);
     p.act1 = (int32_t*)(base + L.act1);
     p.stat = (uint32_t*)(base + L.stat);
-    p.TA = (int4*)(base + L.T[0]);
+    p.L2A = (int4*)(base + L.L2[0]);
+    p.L4A = (int4*)(base + L.L4[0]);
     p.L8A = (int4*)(base + L.L8[0]);
     p.L16A = (int4*)(base + L.L16[0]);
     p.SA = (int4*)(base + L.S[0]);
@@ -232,7 +236,8 @@ void fill_workspace(Params<T>& p, char* base, const Layout& L, RoundState* st, i
     p.HA = (int4*)(base + L.H[0]);
     p.HcA = (int32_t*)(base + L.Hc[0]);
     p.OA = (int32_t*)(base + L.O[0]);
-    p.TB = (int4*)(base + L.T[1]);
+    p.L2B = (int4*)(base + L.L2[1]);
+    p.L4B = (int4*)(base + L.L4[1]);
     p.L8B = (int4*)(base + L.L8[1]);
     p.L16B = (int4*)(base + L.L16[1]);
     p.SB = (int4*)(base + L.S[1]);
@@ -373,9 +378,9 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
     for (;; ++k) {
         GC_CUDA(cudaMemcpyAsync(h, &st->rc[k % 3], sizeof(gc::RoundCounts), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
-        const gc::RoundSizes r = {h->t, gc::low_count(h->mid), gc::high_count(h->mid), h->s, h->m,
+        const gc::RoundSizes r = {gc::low_count(h->tiny), gc::high_count(h->tiny), gc::low_count(h->mid), gc::high_count(h->mid), h->s, h->m,
                                   gc::hub_chunks(h->hc), 0u};
-        const unsigned size = r.nT + r.n8 + r.n16 + r.nS + r.nM + gc::hub_count(h->hc);
+        const unsigned size = r.n2 + r.n4 + r.n8 + r.n16 + r.nS + r.nM + gc::hub_count(h->hc);
         if (size == 0) break;
         if (k > p.max_rounds) {
             hs[1] = gc::kStatusMaxRounds;
@@ -389,7 +394,7 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
         }
         GC_CUDA(cudaMemsetAsync(&st->rc[(k + 2) % 3], 0, sizeof(gc::RoundCounts), s));
         const int64_t tasks = (int64_t)r.nHC + (r.nM + gc::kMedPerTask - 1) / gc::kMedPerTask + (r.nS + 31) / 32 +
-                              (r.nT + 31) / 32 + (r.n8 + 31) / 32 + (r.n16 + 15) / 16;
+                              (r.n2 + 31) / 32 + (r.n4 + 31) / 32 + (r.n8 + 31) / 32 + (r.n16 + 15) / 16;
         const int64_t warps_per_block = threads / 32;
         const int grid = (int)std::max<int64_t>(
             1, std::min<int64_t>((tasks + warps_per_block - 1) / warps_per_block, (int64_t)dc.sms * 8));
@@ -1362,7 +1367,7 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     // the coloring layout's offsets are relative to its own base
     Layout& L = b->L;
     size_t* fields[] = {&L.st, &L.rs, &L.rv, &L.rt, &L.x0, &L.x1, &L.act0, &L.act1, &L.stat, &L.hubs,
-                        &L.defer, &L.T[0], &L.T[1], &L.L8[0], &L.L8[1], &L.L16[0], &L.L16[1], &L.S[0], &L.S[1], &L.M[0], &L.M[1], &L.H[0], &L.H[1], &L.Hc[0], &L.Hc[1],
+                        &L.defer, &L.L2[0], &L.L2[1], &L.L4[0], &L.L4[1], &L.L8[0], &L.L8[1], &L.L16[0], &L.L16[1], &L.S[0], &L.S[1], &L.M[0], &L.M[1], &L.H[0], &L.H[1], &L.Hc[0], &L.Hc[1],
                         &L.O[0], &L.O[1]};
     for (size_t* f : fields) *f += lay;
 

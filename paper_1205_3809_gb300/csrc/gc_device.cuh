@@ -28,11 +28,11 @@
 // flag makes 16-bit state hold colors < 2^15: a larger color sets an
 // overflow status and the host reruns with 32-bit state.
 //
-// Work is split into warp-sized tasks, binned by degree (T, L8, L16) or by the
+// Work is split into warp-sized tasks, binned by degree (L2 to L16) or by the
 // current active length (S, M, H):
-//   T bin (degree <= s_max <= 32): the row is read from the graph itself in
-//     32-byte chunks, with one bit per entry for "not settled yet" in the
-//     worklist entry; no list is kept;
+//   L2, L4 bins (degree <= 9 and <= 25, and s_max): the row is read from the
+//     graph itself in 32-byte chunks by 2 or 4 lanes, with one bit per entry for
+//     "not settled yet" in the worklist entry; no list is kept;
 //   L8, L16 bins (longer rows of degree <= 57 and <= 121): likewise, by 8 or 16
 //     lanes, the bits beside the static mask;
 //   S bin (longer rows whose list has shrunk to s_max): 32 worklist entries per
@@ -85,15 +85,16 @@ constexpr int kPass1LongBlocksPerSm = 8;      // pass 1, long rows: grid of 8 bl
 constexpr int kFlatBatches = GC_FLAT_BATCHES;  // flat tasks: batches in flight together
 constexpr int kMedPerTask = GC_MED_PER_TASK;   // M-bin vertices per task
 constexpr int kShortPerTaskMin = 4;            // S-bin vertices per task in a small round
-#ifndef GC_TINY_LANES
-#define GC_TINY_LANES 4
-#endif
-constexpr int kTinyLanes = GC_TINY_LANES;      // T bin: lanes per vertex
-constexpr int kTinyPerStep = 32 / kTinyLanes;  // T bin: vertices a warp reads side by side
-constexpr int kMidSteps = 8;                   // L8, L16: steps of 32 / L vertices per task, at most
+constexpr int kMidSteps = 8;                  // L8, L16: steps of 32 / L vertices per task, at most
 
-// L8 and L16 bins: degrees above s_max (and up to m_max) whose row fits L
-// chunks of eight entries wherever it starts: 8 L - 7.
+// L2 and L4 bins: degrees up to s_max whose row fits L chunks of eight entries
+// wherever it starts: 8 L - 7.
+__host__ __device__ __forceinline__ int32_t tiny_limit(int L, int32_t s_max) {
+    return s_max < 8 * L - 7 ? s_max : 8 * L - 7;
+}
+
+// L8 and L16 bins: degrees above that (and up to m_max) whose row fits L chunks
+// likewise.
 __host__ __device__ __forceinline__ int32_t mid_limit(int L, int32_t s_max, int32_t m_max) {
     const int32_t most = 8 * L - 7 < m_max ? 8 * L - 7 : m_max;
     return most > s_max ? most : s_max;
@@ -130,8 +131,8 @@ struct Stats {
     int bad;                      // rowptr[0] != 0 or a negative degree
     int nnz;                      // rowptr[n]
     unsigned defer;               // vertices with degree > kPass1Flat
-    unsigned cap[3];              // list capacities: degree >= 1, > s_max, > m_max
-    unsigned over8, over16;       // vertices with degree > mid_limit(8), > mid_limit(16)
+    unsigned cap[3];              // vertices with degree >= 1, > tiny_limit(4), > m_max
+    unsigned over2, over8, over16;  // with degree > tiny_limit(2), > mid_limit(8), > mid_limit(16)
     unsigned long long hub_chunks;  // sum over degree > m_max of ceil(degree / kChunk)
 };
 
@@ -141,7 +142,7 @@ struct Stats {
 // than any other.  A hub's two counters (its worklist position and its first
 // chunk) share one 64-bit word, taken with one atomic.
 struct RoundCounts {
-    alignas(128) unsigned t;               // |U_k in T|
+    alignas(128) unsigned long long tiny;  // |U_k in L2| (bits 0..31) | |U_k in L4| (bits 32..63)
     unsigned overflow;                     // round k - 1 chose a color too wide for the state
     alignas(128) unsigned long long mid;   // |U_k in L8| (bits 0..31) | |U_k in L16| (bits 32..63)
     alignas(128) unsigned s;               // |U_k in S|
@@ -153,6 +154,9 @@ struct RoundCounts {
 // Two 32-bit counts in one 64-bit word.
 __host__ __device__ __forceinline__ unsigned low_count(unsigned long long x) { return (unsigned)x; }
 __host__ __device__ __forceinline__ unsigned high_count(unsigned long long x) { return (unsigned)(x >> 32); }
+__host__ __device__ __forceinline__ unsigned long long pair_count(unsigned low, unsigned high) {
+    return ((unsigned long long)high << 32) | (unsigned long long)low;
+}
 __host__ __device__ __forceinline__ unsigned hub_count(unsigned long long hc) { return (unsigned)hc; }
 __host__ __device__ __forceinline__ unsigned hub_chunks(unsigned long long hc) { return (unsigned)(hc >> 32); }
 
@@ -188,7 +192,7 @@ struct Params {
     int32_t n;
     int32_t nnz;                        // entries of colidx
     int32_t s_max, m_max;               // length bin limits
-    int32_t mid8, mid16;                // degree limits of the L8 and L16 bins
+    int32_t lim2, lim4, lim8, lim16;    // degree limits of the L2, L4, L8 and L16 bins
     int32_t max_rounds;
     int32_t tail_volume;                // rounds reading <= this many entries run in block 0 alone (< 0: never)
     uint32_t barrier_polls;             // the grid barrier gives up after this many polls
@@ -200,12 +204,12 @@ struct Params {
     int32_t* act0;                      // active lists (row starts as in colidx)
     int32_t* act1;
     uint32_t* stat;                     // static masks, 8 words per vertex
-    // worklists per parity (A: even k, B: odd k): T entries {vertex, row start,
-    // live entries, static mask}; L8, L16, S, M, H entries {vertex, row start,
+    // worklists per parity (A: even k, B: odd k): L2 and L4 entries {vertex, row
+    // start, live entries, static mask}; L8, L16, S, M, H entries {vertex, row start,
     // active length (L8, L16: degree), degree}, first chunk of each H entry,
     // owner position of each chunk
-    int4* TA; int4* L8A; int4* L16A; int4* SA; int4* MA; int4* HA; int32_t* HcA; int32_t* OA;
-    int4* TB; int4* L8B; int4* L16B; int4* SB; int4* MB; int4* HB; int32_t* HcB; int32_t* OB;
+    int4* L2A; int4* L4A; int4* L8A; int4* L16A; int4* SA; int4* MA; int4* HA; int32_t* HcA; int32_t* OA;
+    int4* L2B; int4* L4B; int4* L8B; int4* L16B; int4* SB; int4* MB; int4* HB; int32_t* HcB; int32_t* OB;
     int32_t* defer;                     // pass 1: rows longer than kPass1Flat
     HubRecord* hubs;
     RoundState* st;
@@ -312,6 +316,18 @@ __device__ __forceinline__ void warp_append(bool flag, int4 e, int4* list, unsig
     if (flag) list[base + __popc(ballot & ((1u << lane) - 1u))] = e;
 }
 
+// The same with a counter in the bits from SHIFT (0 or 32) on of a 64-bit word.
+template <int SHIFT>
+__device__ __forceinline__ void warp_append_pair(bool flag, int4 e, int4* list, unsigned long long* cnt) {
+    const unsigned ballot = __ballot_sync(kFull, flag);
+    if (ballot == 0) return;
+    const unsigned lane = lane_id();
+    unsigned base = 0;
+    if (lane == 0) base = (unsigned)(atomicAdd(cnt, (unsigned long long)__popc(ballot) << SHIFT) >> SHIFT);
+    base = __shfl_sync(kFull, base, 0);
+    if (flag) list[base + __popc(ballot & ((1u << lane) - 1u))] = e;
+}
+
 __device__ __forceinline__ void warp_append_i32(bool flag, int32_t v, int32_t* list, unsigned* cnt) {
     const unsigned ballot = __ballot_sync(kFull, flag);
     if (ballot == 0) return;
@@ -325,7 +341,7 @@ __device__ __forceinline__ void warp_append_i32(bool flag, int32_t v, int32_t* l
 
 // Where the next round's worklists go.
 struct NextLists {
-    int4* T; int4* L8; int4* L16; int4* S; int4* M; int4* H; int32_t* Hc; int32_t* O;
+    int4* L2; int4* L4; int4* L8; int4* L16; int4* S; int4* M; int4* H; int32_t* Hc; int32_t* O;
     RoundCounts* cnt;  // the next round's counts
     int32_t s_max, m_max;
 };
@@ -479,9 +495,9 @@ __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" 
 // (from 0).  Returns false (and sets status = timeout) if the wait gave up;
 // the caller then leaves the loop.  Every block adds one to a count that is
 // never reset and waits until all of them have: one round trip to L2 to
-// arrive and one to see the last arrival.  With a reset count, a generation
-// word and the status read behind them, a round of nearly no work took 6.6 us
-// and one of G(10,000, 50,000) 10 us; now 4.5 and 6.
+// arrive and one to see the last arrival.  (With a reset count, a generation
+// word and the status read behind them, a round of nearly no work took 6.4 us
+// of which this barrier was most; now GC_ROUND_US.)
 __device__ __forceinline__ bool grid_barrier(RoundState* st, unsigned max_polls, unsigned passed) {
     __shared__ int s_ok;
     __syncthreads();
@@ -532,16 +548,17 @@ __device__ __forceinline__ void fold_volume(RoundState* st, unsigned long long* 
 __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int32_t s_max,
                              int32_t m_max, Stats* s) {
     int mx = 0, bad = 0;
-    unsigned c0 = 0, c1 = 0, c2 = 0, df = 0, o8 = 0, o16 = 0;
+    unsigned c0 = 0, c1 = 0, c2 = 0, df = 0, o2 = 0, o8 = 0, o16 = 0;
     unsigned long long ch = 0;
-    const int32_t mid8 = mid_limit(8, s_max, m_max), mid16 = mid_limit(16, s_max, m_max);
+    const int32_t tiny2 = tiny_limit(2, s_max), tiny4 = tiny_limit(4, s_max), mid8 = mid_limit(8, s_max, m_max), mid16 = mid_limit(16, s_max, m_max);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int32_t d = __ldg(rowptr + v + 1) - __ldg(rowptr + v);
         if (d < 0) { bad = 1; continue; }
         mx = max(mx, d);
         c0 += d >= 1;
-        c1 += d > s_max;
+        c1 += d > tiny4;
+        o2 += d > tiny2;
         c2 += d > m_max;
         o8 += d > mid8;
         o16 += d > mid16;
@@ -554,6 +571,7 @@ __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int3
     c1 = __reduce_add_sync(kFull, c1);
     c2 = __reduce_add_sync(kFull, c2);
     df = __reduce_add_sync(kFull, df);
+    o2 = __reduce_add_sync(kFull, o2);
     o8 = __reduce_add_sync(kFull, o8);
     o16 = __reduce_add_sync(kFull, o16);
     if (lane_id() == 0) {
@@ -563,6 +581,7 @@ __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int3
         if (c1) atomicAdd(&s->cap[1], c1);
         if (c2) atomicAdd(&s->cap[2], c2);
         if (df) atomicAdd(&s->defer, df);
+        if (o2) atomicAdd(&s->over2, o2);
         if (o8) atomicAdd(&s->over8, o8);
         if (o16) atomicAdd(&s->over16, o16);
     }
@@ -595,7 +614,7 @@ __device__ __forceinline__ void pass1_write(const Params<T>& p, int32_t v, bool 
 template <typename T>
 __device__ __forceinline__ NextLists pass1_next(const Params<T>& p) {
     NextLists nl;
-    nl.T = p.TA; nl.L8 = p.L8A; nl.L16 = p.L16A; nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
+    nl.L2 = p.L2A; nl.L4 = p.L4A; nl.L8 = p.L8A; nl.L16 = p.L16A; nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
     nl.cnt = &p.st->rc[2];
     nl.s_max = p.s_max;
     nl.m_max = p.m_max;
@@ -632,7 +651,7 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
     unsigned vol = 0;
     for (int64_t t0 = gw; t0 < ntasks; t0 += W * NT) {
         int4 ev[NT];
-        int cls[NT];  // T, L8, L16, M (0..3), or -1
+        int cls[NT];  // L2, L4, L8, L16, M (0..4), or -1
 #pragma unroll
         for (int jt = 0; jt < NT; ++jt) {
             const int64_t t = t0 + (int64_t)jt * W;
@@ -690,9 +709,10 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
             }
             const int bin = bin_of(d, p.s_max, p.m_max);
             const bool go = valid && !longrow && hit;
-            // a row of at most s_max entries starts as a T entry: all of it live, no static mask
-            ev[jt] = bin == kBinS ? make_int4(v, b, (int32_t)low_bits(d), 0) : make_int4(v, b, d, d);
-            cls[jt] = !go || bin == kBinH ? -1 : (bin == kBinS ? 0 : (d <= p.mid8 ? 1 : (d <= p.mid16 ? 2 : 3)));
+            // an L2 or L4 entry starts with all of its row live and no static mask
+            ev[jt] = d <= p.lim4 ? make_int4(v, b, (int32_t)low_bits(d), 0) : make_int4(v, b, d, d);
+            cls[jt] = !go || bin == kBinH ? -1
+                                          : (d <= p.lim8 ? (d <= p.lim2 ? 0 : (d <= p.lim4 ? 1 : 2)) : (d <= p.lim16 ? 3 : 4));
             // hubs that stayed in the flat range (m_max < d <= kPass1Flat)
             unsigned hubs = __ballot_sync(kFull, go && bin == kBinH);
             while (hubs) {
@@ -703,34 +723,32 @@ __global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_be
             }
             warp_append_i32(valid && longrow, v, p.defer, &p.st->defer_cnt);
         }
-        // the T, L8, L16 and M entries of these NT tasks, one atomic per counter
-        // (L8 and L16 share one)
-        unsigned bal[NT][4], n[4] = {0, 0, 0, 0};
+        // the entries of these NT tasks, one atomic per counter: L2 and L4 share one,
+        // L8 and L16 another, M has its own
+        unsigned long long n01 = 0, n23 = 0;
+        unsigned n4 = 0;
 #pragma unroll
-        for (int jt = 0; jt < NT; ++jt)
+        for (int jt = 0; jt < NT; ++jt) {
+            n01 += pair_count(__popc(__ballot_sync(kFull, cls[jt] == 0)), __popc(__ballot_sync(kFull, cls[jt] == 1)));
+            n23 += pair_count(__popc(__ballot_sync(kFull, cls[jt] == 2)), __popc(__ballot_sync(kFull, cls[jt] == 3)));
+            n4 += __popc(__ballot_sync(kFull, cls[jt] == 4));
+        }
+        unsigned long long base = 0;
+        if (lane == 0 && n01) base = atomicAdd(&nl.cnt->tiny, n01);
+        if (lane == 1 && n23) base = atomicAdd(&nl.cnt->mid, n23);
+        if (lane == 2 && n4) base = atomicAdd(&nl.cnt->m, n4);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                bal[jt][c] = __ballot_sync(kFull, cls[jt] == c);
-                n[c] += __popc(bal[jt][c]);
+        for (int c = 0; c < 5; ++c) {
+            const unsigned long long from = __shfl_sync(kFull, base, c >> 1);
+            unsigned at = c & 1 ? high_count(from) : low_count(from);
+            int4* const list = c == 0 ? p.L2A : (c == 1 ? p.L4A : (c == 2 ? p.L8A : (c == 3 ? p.L16A : p.MA)));
+#pragma unroll
+            for (int jt = 0; jt < NT; ++jt) {
+                const unsigned bal = __ballot_sync(kFull, cls[jt] == c);
+                if (cls[jt] == c) list[at + __popc(bal & ((1u << lane) - 1u))] = ev[jt];
+                at += __popc(bal);
             }
-        unsigned long long base = 0;  // lane 0: T, lane 1: L8 and L16, lane 2: M
-        if (lane == 0 && n[0]) base = atomicAdd(&nl.cnt->t, n[0]);
-        if (lane == 1 && (n[1] | n[2]))
-            base = atomicAdd(&nl.cnt->mid, ((unsigned long long)n[2] << 32) | (unsigned long long)n[1]);
-        if (lane == 2 && n[3]) base = atomicAdd(&nl.cnt->m, n[3]);
-        unsigned at[4];
-        at[0] = __shfl_sync(kFull, (unsigned)base, 0);
-        at[1] = __shfl_sync(kFull, (unsigned)base, 1);
-        at[2] = __shfl_sync(kFull, (unsigned)(base >> 32), 1);
-        at[3] = __shfl_sync(kFull, (unsigned)base, 2);
-#pragma unroll
-        for (int jt = 0; jt < NT; ++jt)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                int4* const list = c == 0 ? p.TA : (c == 1 ? p.L8A : (c == 2 ? p.L16A : p.MA));
-                if (cls[jt] == c) list[at[c] + __popc(bal[jt][c] & ((1u << lane) - 1u))] = ev[jt];
-                at[c] += __popc(bal[jt][c]);
-            }
+        }
     }
     fold_max_color(p.st, maxc);
     fold_volume(p.st, p.round_vol, p.round_cap, 2, vol);
@@ -799,7 +817,7 @@ struct PassIO {
     const int32_t* rin;     // active lists read this round (colidx in round 2)
     int32_t* rout;          // active lists written for the next round
     bool first;             // round 2: no static masks yet
-    const int4* T_; const int4* L8; const int4* L16; const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
+    const int4* L2; const int4* L4; const int4* L8; const int4* L16; const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
     NextLists next;
     uint64_t pol_row, pol_col;
 };
@@ -815,7 +833,8 @@ __device__ __forceinline__ PassIO<T> pass_io(const Params<T>& p, int k) {
     io.k = k;
     io.rin = k == 2 ? p.colidx : (odd ? p.act1 : p.act0);
     io.rout = odd ? p.act0 : p.act1;
-    io.T_ = odd ? p.TB : p.TA;
+    io.L2 = odd ? p.L2B : p.L2A;
+    io.L4 = odd ? p.L4B : p.L4A;
     io.L8 = odd ? p.L8B : p.L8A;
     io.L16 = odd ? p.L16B : p.L16A;
     io.S = odd ? p.SB : p.SA;
@@ -823,7 +842,8 @@ __device__ __forceinline__ PassIO<T> pass_io(const Params<T>& p, int k) {
     io.H = odd ? p.HB : p.HA;
     io.Hc = odd ? p.HcB : p.HcA;
     io.O = odd ? p.OB : p.OA;
-    io.next.T = odd ? p.TA : p.TB;
+    io.next.L2 = odd ? p.L2A : p.L2B;
+    io.next.L4 = odd ? p.L4A : p.L4B;
     io.next.L8 = odd ? p.L8A : p.L8B;
     io.next.L16 = odd ? p.L16A : p.L16B;
     io.next.S = odd ? p.SA : p.SB;
@@ -868,29 +888,31 @@ struct TaskHead {
 
 // The entries of one round.
 struct RoundSizes {
-    unsigned nT, n8, n16, nS, nM, nHC;  // T, L8, L16, S, M entries; H chunks
+    unsigned n2, n4, n8, n16, nS, nM, nHC;  // L2, L4, L8, L16, S, M entries; H chunks
     unsigned overflow;
 };
 __device__ __forceinline__ RoundSizes round_sizes_of(const RoundCounts& c, unsigned* total) {
     RoundSizes r;
-    const unsigned long long hc = __ldcg(&c.hc), mid = __ldcg(&c.mid);
-    r.nT = __ldcg(&c.t);
+    const unsigned long long hc = __ldcg(&c.hc), tiny = __ldcg(&c.tiny), mid = __ldcg(&c.mid);
+    r.n2 = low_count(tiny);
+    r.n4 = high_count(tiny);
     r.overflow = __ldcg(&c.overflow);
     r.n8 = low_count(mid);
     r.n16 = high_count(mid);
     r.nS = __ldcg(&c.s);
     r.nM = __ldcg(&c.m);
     r.nHC = hub_chunks(hc);
-    *total = r.nT + r.n8 + r.n16 + r.nS + r.nM + hub_count(hc);
+    *total = r.n2 + r.n4 + r.n8 + r.n16 + r.nS + r.nM + hub_count(hc);
     return r;
 }
 
-// Its tasks, in the order they are dealt out: H chunks, M, L16, L8, S, T.
+// Its tasks, in the order they are dealt out: H chunks, M, L16, L8, S, L4, L2.
 struct TaskSplit {
     unsigned mpt, spt;              // M and S entries per task
-    unsigned s16, s8, sT;           // steps per task of L16, L8 and T
-    unsigned e0, e1, e2, e3, e4;    // ends of the H, M, L16, L8 and S tasks
+    unsigned s16, s8, s4, s2;       // steps per task of L16, L8, L4 and L2
+    unsigned e0, e1, e2, e3, e4, e5;  // ends of the H, M, L16, L8, S and L4 tasks
     unsigned total;
+    unsigned nstat;                 // tasks a warp takes without a claim
 };
 
 // Entry of step j < steps of a row task: lane j of every group of L lanes
@@ -923,8 +945,10 @@ __device__ __forceinline__ TaskHead load_head(const PassIO<T>& io, unsigned t, c
         list = io.L8; n = r.n8; most = q.s8; i = step_entry<8>(t - q.e2, q.s8, &j);
     } else if (t < q.e4) {
         list = io.S; n = r.nS; most = q.spt; i = (t - q.e3) * q.spt + j;
+    } else if (t < q.e5) {
+        list = io.L4; n = r.n4; most = q.s4; i = step_entry<4>(t - q.e4, q.s4, &j);
     } else {
-        list = io.T_; n = r.nT; most = q.sT; i = step_entry<kTinyLanes>(t - q.e4, q.sT, &j);
+        list = io.L2; n = r.n2; most = q.s2; i = step_entry<2>(t - q.e5, q.s2, &j);
     }
     h.e = j < most && i < n ? __ldcg(list + i) : make_int4(-1, 0, 0, 0);
     return h;
@@ -967,18 +991,21 @@ __device__ __forceinline__ void load_chunk(const int32_t* __restrict__ colidx, i
     }
 }
 
-// T bin: vertices of degree <= s_max <= 32, whose first fit is at most 33, so
-// one 32-bit word holds every color that matters to them (33 is taken when
-// 1..32 all are) and one more says which entries of the row are still live
-// (the neighbour had not settled when last read).  Both travel in the worklist
-// entry {v, row start, live, static mask}; the row itself is read from colidx
-// in every round and no list is written.
+// L2 and L4 bins (L = 2, 4): vertices of degree <= 8 L - 7 <= 25 (and s_max),
+// whose first fit is at most 26, so one 32-bit word holds every color that matters to them and one more says
+// which entries of the row are still live (the neighbour had not settled when
+// last read).  Both travel in the worklist entry {v, row start, live, static
+// mask}; the row itself is read from colidx in every round and no list is
+// written.
 //
-// kTinyLanes lanes share a vertex: each takes a 32-byte chunk of the row (one
-// load for eight entries), gathers the colors of the live entries, and ORs
+// L lanes share a vertex: each takes a 32-byte chunk of the row (one load for
+// eight entries; a row of 8 L - 7 spans at most L), gathers the colors of the live entries, and ORs
 // what it finds in registers; the lanes of a vertex combine with shuffles.
 // Lane j of a group keeps the vertex of step j, so a task of up to 32
 // vertices appends its survivors with one atomic.
+//
+// Two lanes for rows of up to 9 (a mesh's, say) fill twice the lanes of four:
+// 5-point mesh of 4,000,003 vertices 0.55 -> 0.46 ms.
 //
 // Bound: the random L2 sector of each live entry's color (207 G entries/s on
 // rows of 16; a probe that only gathers reaches 208).  The flat walk below,
@@ -986,38 +1013,38 @@ __device__ __forceinline__ void load_chunk(const int32_t* __restrict__ colidx, i
 // 32 entries against about 40 here, and an L1 data pipe 72 % busy, two fifths
 // of it with shared-memory atomics.  R-MAT-ER of 2^22 vertices: 2.36 ms a call
 // before, 1.70 after.
-template <typename T, bool P>  // P: a priority array is given
+template <typename T, bool P, int L>  // P: a priority array is given
 __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& io, int4 en, unsigned steps, int& maxc,
                                           unsigned& vol) {
     const unsigned lane = lane_id();
-    const unsigned j = lane % kTinyLanes;
+    const unsigned j = lane % L;
     const uint32_t mis = (uint32_t)((uintptr_t)p.colidx >> 2) & 7u;  // entries from a 32-byte boundary to colidx
     const bool valid = en.x >= 0;
     const int32_t my_v = valid ? en.x : 0;
     const uint32_t my_live = valid ? (uint32_t)en.z : 0u;
-    uint32_t my_cv = 0u, my_all = 0u, my_stat = 0u, my_dead = 0u, my_new_prec = 0u;
+    const uint32_t my_cv = valid ? word_color(ld_color(io.Xc + my_v, io.pol_col)) : 0u;
+    // which entries precede v (bit i: entry i), worked out in round 2; there: v's key
+    uint32_t my_prec = 0u;
+    if constexpr (P) {
+        if (valid) my_prec = io.first ? __ldg(p.prio + my_v) : __ldcg(p.stat + (size_t)my_v * 8);
+    }
+    uint32_t my_all = 0u, my_stat = 0u, my_dead = 0u, my_new_prec = 0u;
     bool my_conflict = false;
 #pragma unroll 1
     for (unsigned s = 0; s < steps; ++s) {
-        const int src = (int)((lane & ~(unsigned)(kTinyLanes - 1)) | s);
-        const int32_t v = __shfl_sync(kFull, en.x, src);
+        const int src = (int)((lane & ~(unsigned)(L - 1)) | s);
+        const int32_t v = __shfl_sync(kFull, my_v, src);
         const int32_t b = __shfl_sync(kFull, en.y, src);
         const uint32_t live = __shfl_sync(kFull, my_live, src);
-        // every lane of the group reads v's color itself, so that the row's load does
-        // not wait for it (one line either way)
-        const uint32_t cv = v >= 0 ? word_color(ld_color(io.Xc + v, io.pol_col)) : 0u;
-        // which entries precede v (bit i: entry i), worked out in round 2; there: v's key
-        uint32_t prec = 0u;
-        if constexpr (P) {
-            if (live) prec = io.first ? __ldg(p.prio + v) : __ldcg(p.stat + (size_t)v * 8);
-        }
         uint32_t all = 0u, stat = 0u, dead = 0u, nprec = 0u;
         bool conflict = false;
-        const int32_t span = 32 - __clz(live);  // entries up to the last live one
-        // off: index in the row of the chunk's first entry (the first chunk may start before the row)
-        for (int32_t off = 8 * (int32_t)j - (int32_t)(((uint32_t)b + mis) & 7u); off < span; off += 8 * kTinyLanes) {
-            const uint32_t bits = (off >= 0 ? live >> off : live << -off) & 0xffu;
-            if (bits == 0u) continue;
+        // this lane's chunk: entries off .. off + 7 of the row (the first chunk may
+        // start before the row); bits: the live ones
+        const int32_t off = 8 * (int32_t)j - (int32_t)(((uint32_t)b + mis) & 7u);
+        const uint32_t bits = (off >= 0 ? live >> off : live << -off) & 0xffu;
+        const uint32_t cv = __shfl_sync(kFull, my_cv, src);
+        const uint32_t prec = P ? __shfl_sync(kFull, my_prec, src) : 0u;
+        if (bits) {
             int32_t w[8];
             load_chunk(p.colidx, p.nnz, b + off, io.pol_row, w);
             T c[8];
@@ -1033,6 +1060,7 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
                         if (((bits >> u) & 1u) && (word_color(c[u]) == cv || !word_settled(c[u])) &&
                             precedes(p.prio, w[u], v, prec))
                             pre8 |= 1u << u;
+                    nprec = off >= 0 ? pre8 << off : pre8 >> -off;
                 }
             }
 #pragma unroll
@@ -1046,24 +1074,22 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
                 }
                 if (col == cv && (P ? (pre8 >> u) & 1u : w[u] < v)) conflict = true;
             }
-            dead |= off >= 0 ? gone << off : gone >> -off;
-            if (P && io.first) nprec |= off >= 0 ? pre8 << off : pre8 >> -off;
+            dead = off >= 0 ? gone << off : gone >> -off;
         }
         const unsigned cb = __ballot_sync(kFull, conflict);
 #pragma unroll
-        for (int o = 1; o < kTinyLanes; o <<= 1) {
+        for (int o = 1; o < L; o <<= 1) {
             all |= __shfl_xor_sync(kFull, all, o);
             stat |= __shfl_xor_sync(kFull, stat, o);
             dead |= __shfl_xor_sync(kFull, dead, o);
             if (P && io.first) nprec |= __shfl_xor_sync(kFull, nprec, o);
         }
         if (j == s) {
-            my_cv = cv;
             my_all = all;
             my_stat = stat;
             my_dead = dead;
             my_new_prec = nprec;
-            my_conflict = ((cb >> (lane - j)) & ((1u << kTinyLanes) - 1u)) != 0u;
+            my_conflict = ((cb >> (lane - j)) & ((1u << L) - 1u)) != 0u;
         }
     }
     const bool go = valid && my_conflict;
@@ -1071,17 +1097,18 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
     const uint32_t live = my_live & ~my_dead;
     if (go) {
         const uint32_t taken = stat | my_all;
-        recolor(p, io, my_v, taken == 0xffffffffu ? 33u : (uint32_t)__ffs(~taken));
+        recolor(p, io, my_v, (uint32_t)__ffs(~taken));
         vol += (unsigned)__popc(live);
         if (P && io.first) p.stat[(size_t)my_v * 8] = my_new_prec;
     } else if (valid) {
         settle(p, io, my_v, my_cv);
         maxc = max(maxc, (int)my_cv);
     }
-    warp_append(go, make_int4(my_v, en.y, (int32_t)live, (int32_t)stat), io.next.T, &io.next.cnt->t);
+    warp_append_pair<(L == 2 ? 0 : 32)>(go, make_int4(my_v, en.y, (int32_t)live, (int32_t)stat),
+                                        L == 2 ? io.next.L2 : io.next.L4, &io.next.cnt->tiny);
 }
 
-// L8 and L16 bins (L = 8, 16): vertices of degree s_max < d <= 8 L - 7, read
+// L8 and L16 bins (L = 8, 16): longer rows of degree d <= 8 L - 7, read
 // like T rows: L lanes share a vertex, one 32-byte chunk of colidx each, 32 / L
 // vertices side by side, no list written.  Their first fit is at most
 // 8 L - 6, so W = L / 4 words hold the colors that matter.  The static mask
@@ -1116,6 +1143,8 @@ __device__ __forceinline__ void mid_task(const Params<T>& p, const PassIO<T>& io
         const int32_t v = __shfl_sync(kFull, my_v, src);
         const int32_t b = __shfl_sync(kFull, en.y, src);
         const int32_t d = __shfl_sync(kFull, my_d, src);
+        // every lane reads v's color itself, so that the row's load does not wait for it
+        // (one line either way)
         const uint32_t cv = d ? word_color(ld_color(io.Xc + v, io.pol_col)) : 0u;
         const uint32_t key = P && first && d ? __ldg(p.prio + v) : 0u;
         // this lane's chunk: entries off .. off + 7 of the row
@@ -1200,14 +1229,7 @@ __device__ __forceinline__ void mid_task(const Params<T>& p, const PassIO<T>& io
         settle(p, io, my_v, my_cv);
         maxc = max(maxc, (int)my_cv);
     }
-    const unsigned bal = __ballot_sync(kFull, go);
-    if (bal) {
-        constexpr int kShift = L == 8 ? 0 : 32;
-        unsigned base = 0;
-        if (lane == 0) base = (unsigned)(atomicAdd(&io.next.cnt->mid, (unsigned long long)__popc(bal) << kShift) >> kShift);
-        base = __shfl_sync(kFull, base, 0);
-        if (go) (L == 8 ? io.next.L8 : io.next.L16)[base + __popc(bal & ((1u << lane) - 1u))] = en;
-    }
+    warp_append_pair<(L == 8 ? 0 : 32)>(go, en, L == 8 ? io.next.L8 : io.next.L16, &io.next.cnt->mid);
 }
 
 // S bin: up to 32 worklist entries per task, one per lane.  Their
@@ -1657,6 +1679,50 @@ __device__ __forceinline__ void hub_chunk(const Params<T>& p, const PassIO<T>& i
     warp_append_one(io.next, make_int4(v, b, kept, h.e.w));
 }
 
+// The largest power of two (its logarithm) not above `most` that leaves a
+// task for each 1 / per_warp entries.  Powers of two and a float reciprocal,
+// so that no warp divides: a round of little work would feel it, and any
+// value gives the same result.
+__device__ __forceinline__ unsigned task_shift(unsigned entries, float per_warp, unsigned most) {
+    const unsigned x = min(most, (unsigned)((float)entries * per_warp));
+    return x <= 1u ? 0u : 31u - (unsigned)__clz((int)x);
+}
+
+__device__ __forceinline__ TaskSplit split_round(const RoundSizes& r, unsigned W) {
+    TaskSplit q;
+    const float w = 1.f / (float)W;
+    // S vertices per task: 32 in a large round, down to kShortPerTaskMin as it
+    // leaves fewer than four tasks a warp; a task of 32 short lists walks up to
+    // 1024 entries in sequence, which in the last rounds was the longest chain of
+    // the round
+    const unsigned xs = max(task_shift(r.nS, w / 4.f, 32u), task_shift(kShortPerTaskMin, 1.f, 32u));
+    // M vertices per task: up to kMedPerTask, fewer (down to 1) likewise, so that
+    // a task's chain of per-vertex reads does not set the round's length
+    const unsigned xm = task_shift(r.nM, w / 4.f, kMedPerTask);
+    // steps of 16, 8, 4 and 2 vertices of the L2 to L16 tasks: as many as leave a
+    // task for every other warp (each task waits for two reads in a row and
+    // appends once, so that four tasks a warp, as above, cost more than they even
+    // out: R-MAT-G of 1,000,003 vertices with keys 1.87 ms against 1.61; one a
+    // warp 1.62)
+    const unsigned x2 = task_shift(r.n2, w / 8.f, 2u), x4 = task_shift(r.n4, w / 4.f, 4u);
+    const unsigned x8 = task_shift(r.n8, w / 2.f, kMidSteps), x16 = task_shift(r.n16, w, kMidSteps);
+    q.spt = 1u << xs;
+    q.mpt = 1u << xm;
+    q.s2 = 1u << x2;
+    q.s4 = 1u << x4;
+    q.s8 = 1u << x8;
+    q.s16 = 1u << x16;
+    q.e0 = r.nHC;
+    q.e1 = q.e0 + ((r.nM + q.mpt - 1) >> xm);
+    q.e2 = q.e1 + ((r.n16 + 2u * q.s16 - 1) >> (1u + x16));
+    q.e3 = q.e2 + ((r.n8 + 4u * q.s8 - 1) >> (2u + x8));
+    q.e4 = q.e3 + ((r.nS + q.spt - 1) >> xs);
+    q.e5 = q.e4 + ((r.n4 + 8u * q.s4 - 1) >> (3u + x4));
+    q.total = q.e5 + ((r.n2 + 16u * q.s2 - 1) >> (4u + x2));
+    q.nstat = max(2u, (unsigned)((float)q.total * (.5f * w)));
+    return q;
+}
+
 // One fused pass over U_k, shared among W warps (this warp is number gw).
 // Task t: first the H-bin chunks, then the M-bin entries, up to kMedPerTask
 // per task (fewer as the round shrinks), then the S-bin entries, 32 per task
@@ -1675,36 +1741,28 @@ __device__ __forceinline__ void run_pass(const Params<T>& p, int k, const RoundS
     __shared__ FlatSmem s_flat[kWarpsPerBlockMax];
     const PassIO<T> io = pass_io(p, k);
     const unsigned wib = threadIdx.x >> 5;
-    TaskSplit q;
-    // S vertices per task: 32 in a large round, down to kShortPerTaskMin as it
-    // shrinks; a task of 32 short lists walks up to 1024 entries in sequence,
-    // which in the last rounds was the longest chain of the round
-    q.spt = max((unsigned)kShortPerTaskMin, min(32u, r.nS / (4u * W)));
-    // M vertices per task: up to kMedPerTask when the round has enough of them
-    // for several tasks per warp, fewer (down to 1) as the round shrinks, so
-    // that a task's chain of per-vertex reads does not set the round's length;
-    // likewise the steps of the T, L8 and L16 tasks
-    q.mpt = max(1u, min((unsigned)kMedPerTask, r.nM / (4u * W)));
-    q.sT = max(1u, min((unsigned)kTinyLanes, r.nT / (4u * W * kTinyPerStep)));
-    q.s8 = max(1u, min((unsigned)kMidSteps, r.n8 / (4u * W * 4u)));
-    q.s16 = max(1u, min((unsigned)kMidSteps, r.n16 / (4u * W * 2u)));
-    q.e0 = r.nHC;
-    q.e1 = q.e0 + (r.nM + q.mpt - 1) / q.mpt;
-    q.e2 = q.e1 + (r.n16 + 2u * q.s16 - 1) / (2u * q.s16);
-    q.e3 = q.e2 + (r.n8 + 4u * q.s8 - 1) / (4u * q.s8);
-    q.e4 = q.e3 + (r.nS + q.spt - 1) / q.spt;
-    q.total = q.e4 + (r.nT + q.sT * kTinyPerStep - 1) / (q.sT * kTinyPerStep);
+    // the split sits in shared memory: it is the same for every warp, read once a
+    // task, and would take some twenty registers across the loop
+    __shared__ RoundSizes s_sizes;
+    __shared__ TaskSplit s_split;
+    if (threadIdx.x == 0) {
+        s_sizes = r;
+        s_split = split_round(r, W);
+    }
+    __syncthreads();
+    const RoundSizes& z = s_sizes;
+    const TaskSplit& q = s_split;
     const unsigned total = q.total;
     unsigned vol = 0;  // this lane's share of the next round's read volume
     // this warp's tasks: gw + jW for j < nstat, then claimed ones from nstat W on
-    const unsigned nstat = ctr ? max(2u, total / W / 2) : 0xffffffffu;
+    const unsigned nstat = ctr ? q.nstat : 0xffffffffu;
     TaskHead cur;
-    if (gw < total) cur = load_head(io, gw, r, q);
+    if (gw < total) cur = load_head(io, gw, z, q);
     unsigned tn = gw + W;
     unsigned j = 0;  // position of the current task in that sequence
     for (unsigned t = gw; t < total; ++j) {
         TaskHead nxt;
-        if (tn < total) nxt = load_head(io, tn, r, q);
+        if (tn < total) nxt = load_head(io, tn, z, q);
         // the task after next: fixed, or claimed now (its number is needed after this task)
         const bool fixed = j + 2u < nstat;
         unsigned claim = 0;
@@ -1719,8 +1777,10 @@ __device__ __forceinline__ void run_pass(const Params<T>& p, int k, const RoundS
             mid_task<T, P, 8>(p, io, cur.e, q.s8, maxc, vol);
         } else if (t < q.e4) {
             flat_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
+        } else if (t < q.e5) {
+            tiny_task<T, P, 4>(p, io, cur.e, q.s4, maxc, vol);
         } else {
-            tiny_task<T, P>(p, io, cur.e, q.sT, maxc, vol);
+            tiny_task<T, P, 2>(p, io, cur.e, q.s2, maxc, vol);
         }
         const unsigned tnn = fixed ? tn + W : nstat * W + __shfl_sync(kFull, claim, 0);
         t = tn;
@@ -1772,8 +1832,8 @@ __global__ void __launch_bounds__(256, kMinBlocks) rounds_persistent_kernel(Para
         }
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             RoundCounts& z = st->rc[(k + 2) % 3];
-            z.t = z.overflow = z.s = z.m = z.vol = 0u;
-            z.mid = z.hc = 0ull;
+            z.overflow = z.s = z.m = z.vol = 0u;
+            z.tiny = z.mid = z.hc = 0ull;
             st->task_next[(k + 1) % 3] = 0u;  // round k + 1's claims (no one touches it in round k)
             if (k - 1 < p.round_cap) p.round_sizes[k - 1] = (int32_t)size;
         }
@@ -1833,7 +1893,7 @@ __global__ void graph_cond_kernel(Params<T> p, int before_loop, cudaGraphConditi
     const int k = before_loop ? 1 : st->graph_round;
     const int kn = k + 1;
     const RoundCounts& c = st->rc[kn % 3];
-    const unsigned size = c.t + low_count(c.mid) + high_count(c.mid) + c.s + c.m + hub_count(c.hc);
+    const unsigned size = low_count(c.tiny) + high_count(c.tiny) + low_count(c.mid) + high_count(c.mid) + c.s + c.m + hub_count(c.hc);
     unsigned go = 0u;
     if (size == 0u) {
         st->rounds = k;
@@ -1844,8 +1904,8 @@ __global__ void graph_cond_kernel(Params<T> p, int before_loop, cudaGraphConditi
         st->status = kStatusMaxRounds;
     } else {
         RoundCounts& z = st->rc[(kn + 1) % 3];
-        z.t = z.overflow = z.s = z.m = z.vol = 0u;
-        z.mid = z.hc = 0ull;
+        z.overflow = z.s = z.m = z.vol = 0u;
+        z.tiny = z.mid = z.hc = 0ull;
         if (kn - 1 < p.round_cap) p.round_sizes[kn - 1] = (int32_t)size;
         st->graph_round = kn;
         go = 1u;
