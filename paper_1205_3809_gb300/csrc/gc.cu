@@ -439,38 +439,48 @@ int normalise(const gc_options* opt, gc_options* o) {
     return GC_OK;
 }
 
+// The setup scan (Stats at the head of the workspace) and, when asked for, the
+// checks of every entry behind it, with one wait for both.
+int scan_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, int32_t s_max, int32_t m_max, bool validate,
+                const HostInput* hin, bool timed, cudaStream_t s, DeviceCache& dc, int64_t* launches, Stats* hs) {
+    constexpr size_t kOut = 1024, kHead = 2048;
+    static_assert(sizeof(Stats) <= kOut && sizeof(gc::ValidateOut) <= kHead - kOut, "workspace head");
+    Stats* stats = (Stats*)dc.ws;
+    gc::ValidateOut* out = (gc::ValidateOut*)((char*)dc.ws + kOut);
+    GC_CUDA(cudaMemsetAsync(dc.ws, 0, kHead, s));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)dc.sms * 8));
+    gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, s_max, m_max, stats);
+    GC_CUDA(cudaGetLastError());
+    *launches += 1;
+    if (validate) {
+        if (hin) GC_CUDA(cudaStreamWaitEvent(s, dc.chunk_ev[hin->nchunks - 1], 0));
+        gc::validate_kernel<<<grid, 256, 0, s>>>(rowptr, colidx, n, stats, out);
+        GC_CUDA(cudaGetLastError());
+        *launches += 1;
+    }
+    if (timed) GC_CUDA(cudaEventRecord(dc.ev[1], s));
+    GC_CUDA(cudaMemcpyAsync(dc.host, dc.ws, kHead, cudaMemcpyDeviceToHost, s));
+    GC_CUDA(cudaStreamSynchronize(s));
+    std::memcpy(hs, dc.host, sizeof(Stats));
+    if (hs->bad || hs->nnz < 0) return GC_ERR_BAD_GRAPH;
+    if (hs->nnz > 0 && !colidx) return GC_ERR_INVALID;
+    if (validate) {
+        gc::ValidateOut ho;
+        std::memcpy(&ho, (char*)dc.host + kOut, sizeof(ho));
+        if (ho.bad_index || ho.self_loop || ho.asym) return GC_ERR_BAD_GRAPH;
+    }
+    return GC_OK;
+}
+
 int validate_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, cudaStream_t s,
                     DeviceCache& dc, int64_t* launches) {
-    // workspace head is reused for the validation record
+    // workspace head is reused for the records
     int rc = ensure_device(&dc.ws, &dc.ws_bytes, std::max<size_t>(dc.ws_bytes, 4096));
     if (rc != GC_OK) return rc;
-    gc::ValidateOut* out = (gc::ValidateOut*)dc.ws;
-    Stats* stats = (Stats*)((char*)dc.ws + 1024);
-    GC_CUDA(cudaMemsetAsync(dc.ws, 0, 2048, s));
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)dc.sms * 8));
-    gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, gc::kSmallMaxLimit, gc::kMedMaxLimit, stats);
-    GC_CUDA(cudaGetLastError());
-    size_t hb = dc.host_bytes;
-    rc = ensure_host(&dc.host, &hb, 4096);
+    rc = ensure_host(&dc.host, &dc.host_bytes, 4096);
     if (rc != GC_OK) return rc;
-    dc.host_bytes = hb;
-    GC_CUDA(cudaMemcpyAsync(dc.host, stats, sizeof(Stats), cudaMemcpyDeviceToHost, s));
-    GC_CUDA(cudaStreamSynchronize(s));
     Stats hs;
-    std::memcpy(&hs, dc.host, sizeof(Stats));
-    *launches += 1;
-    if (hs.bad || hs.nnz < 0) return GC_ERR_BAD_GRAPH;
-    if (hs.nnz > 0 && !colidx) return GC_ERR_INVALID;
-    const int vgrid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n * 32 + 255) / 256, (int64_t)dc.sms * 16));
-    gc::validate_kernel<<<vgrid, 256, 0, s>>>(rowptr, colidx, n, out);
-    GC_CUDA(cudaGetLastError());
-    *launches += 1;
-    GC_CUDA(cudaMemcpyAsync(dc.host, out, sizeof(gc::ValidateOut), cudaMemcpyDeviceToHost, s));
-    GC_CUDA(cudaStreamSynchronize(s));
-    gc::ValidateOut ho;
-    std::memcpy(&ho, dc.host, sizeof(ho));
-    if (ho.bad_index || ho.self_loop || ho.sum_fwd != ho.sum_bwd) return GC_ERR_BAD_GRAPH;
-    return GC_OK;
+    return scan_locked(rowptr, colidx, n, gc::kSmallMaxLimit, gc::kMedMaxLimit, true, nullptr, false, s, dc, launches, &hs);
 }
 
 int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const uint32_t* priority,
@@ -498,11 +508,6 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
         rc = issue_host_chunks(dc, *hin, s);
         if (rc != GC_OK) return rc;
     }
-    if (o.validate) {
-        if (hin) GC_CUDA(cudaStreamWaitEvent(s, dc.chunk_ev[hin->nchunks - 1], 0));
-        rc = validate_locked(rowptr, colidx, n, s, dc, &launches);
-        if (rc != GC_OK) return rc;
-    }
     const int32_t max_rounds = o.max_rounds > 0 ? o.max_rounds : n;
     // telemetry covers the first min(rounds, max(4096, caller cap), 2^20) rounds
     const int64_t round_cap = std::max<int64_t>(1, std::min<int64_t>(
@@ -518,22 +523,13 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
     if (o.telemetry && !dc.ev[0])
         for (int i = 0; i < 4; ++i) GC_CUDA(cudaEventCreate(&dc.ev[i]));
     if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[0], s));
+    Stats hs;
     {
         NvtxRange range("gc setup scan");
-        Stats* stats = (Stats*)dc.ws;
-        GC_CUDA(cudaMemsetAsync(stats, 0, sizeof(Stats), s));
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)dc.sms * 8));
-        gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, o.small_max_degree, o.medium_max_degree, stats);
-        GC_CUDA(cudaGetLastError());
-        launches += 1;
-        if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[1], s));
-        GC_CUDA(cudaMemcpyAsync(dc.host, stats, sizeof(Stats), cudaMemcpyDeviceToHost, s));
-        GC_CUDA(cudaStreamSynchronize(s));
+        rc = scan_locked(rowptr, colidx, n, o.small_max_degree, o.medium_max_degree, o.validate != 0, hin,
+                         o.telemetry != 0, s, dc, &launches, &hs);
+        if (rc != GC_OK) return rc;
     }
-    Stats hs;
-    std::memcpy(&hs, dc.host, sizeof(Stats));
-    if (hs.bad || hs.nnz < 0) return GC_ERR_BAD_GRAPH;
-    if (hs.nnz > 0 && !colidx) return GC_ERR_INVALID;
     // 16-bit color words (flag + 15-bit color) unless asked for 32; a color
     // that does not fit makes the rounds stop with an overflow status, and the
     // call starts over with 32-bit words.
