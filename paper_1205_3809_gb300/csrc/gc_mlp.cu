@@ -27,39 +27,9 @@ constexpr int kIn = 6, kH = 32;
 constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kH * kIn, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH,
               kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH, kMlpParams = kOffB3 + 1;
 static_assert(kMlpParams == 1313, "parameter layout");
-constexpr int kTile = 64;   // samples per tile of the gradient kernel (static shared memory < 48 KB)
+constexpr int kTile = 128;  // samples per tile of the gradient kernel, one per thread
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-
-// Parameters with the matrix operands rounded to bf16 (biases stay fp32).
-__device__ __forceinline__ void load_params(const float* __restrict__ params, float* s) {
-    for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) {
-        const bool weight = i < kOffB1 || (i >= kOffW2 && i < kOffB2) || (i >= kOffW3 && i < kOffB3);
-        const float p = params[i];
-        s[i] = weight ? bf16r(p) : p;
-    }
-}
-
-// Layer 1 of one sample: a1 = bf16(relu(bf16(W1) a0 + b1)).
-__device__ __forceinline__ void layer1(const float* s, const float a0[kIn], float a1[kH]) {
-#pragma unroll
-    for (int j = 0; j < kH; ++j) {
-        float acc = 0.f;
-#pragma unroll
-        for (int i = 0; i < kIn; ++i) acc = fmaf(s[kOffW1 + j * kIn + i], a0[i], acc);
-        acc += s[kOffB1 + j];
-        a1[j] = bf16r(fmaxf(acc, 0.f));
-    }
-}
-
-// Unit j of layer 2: bf16(relu(bf16(W2[j]) . a1 + b2[j])).
-__device__ __forceinline__ float layer2_unit(const float* s, const float a1[kH], int j) {
-    float acc = 0.f;
-#pragma unroll
-    for (int i = 0; i < kH; ++i) acc = fmaf(s[kOffW2 + j * kH + i], a1[i], acc);
-    acc += s[kOffB2 + j];
-    return bf16r(fmaxf(acc, 0.f));
-}
 
 // Two fp32 values side by side, each lane of the arithmetic rounded as the
 // scalar instruction rounds it.
@@ -188,93 +158,169 @@ __global__ void __launch_bounds__(kForwardThreads, kForwardBlocks) mlp_forward_k
 // Gradient of scale * sum_b (y_b - t_b)^2 over n samples, added into grad;
 // the sum of squared errors is added into *sse.  Rounding to bf16 passes
 // gradients straight through, and the backward pass uses the same bf16
-// weights and activations as the forward.  One block handles kTile samples at
-// a time: forward and backward per sample (thread per sample) with
-// activations and deltas staged in shared memory, then each thread sums the
-// tile's contribution to the parameters it owns.
+// weights and activations as the forward.
+//
+// A block takes kTile samples at a time.  First a thread runs one sample
+// forward and backward (weights from shared memory, two units to an
+// instruction) and leaves its activations and deltas in shared memory; then
+// every warp takes 32 of the samples and adds their outer products to sums
+// that it keeps in registers over all tiles: lane l holds units 4 (l / 4) ..
+// + 3 by inputs 8 (l % 4) .. + 7 of W2's gradient (three reads of 16 bytes for
+// 32 multiply-adds), and unit l of the other gradients.  The warps' sums meet
+// once, at the end.
+//
+// Bound: reads of weights and activations from shared memory and the fp32
+// multiply-adds (3,552 a sample), about level.  With a thread per parameter
+// walking the tile (two reads a multiply-add) and 64 threads a block, 65,536
+// samples took 51 us, now 26 (262,144: 149 us, now 63).
+constexpr int kTileWarps = kTile / 32;
+struct __align__(16) GradShared {
+    ForwardParams p;
+    float w2r[kH][kRow];        // W2 by unit, for the way back
+    float a1[kTile][kRow], a2[kTile][kRow], d1[kTile][kRow], d2[kTile][kRow];
+    float a0[kTile][8];         // the inputs, then 1 and dy
+    float sum[kMlpParams];
+    float sse[kTileWarps];
+};
+
 __global__ void __launch_bounds__(kTile) mlp_grad_kernel(const float* __restrict__ params,
                                                          const float* __restrict__ x,
                                                          const float* __restrict__ t, int64_t n,
                                                          float scale, float* grad, float* sse) {
-    __shared__ float s[kMlpParams];
-    __shared__ float g[kMlpParams];
-    __shared__ float sa0[kTile][kIn + 1];
-    __shared__ float sa1[kTile][kH + 1];
-    __shared__ float sa2[kTile][kH + 1];
-    __shared__ float sd1[kTile][kH + 1];
-    __shared__ float sd2[kTile][kH + 1];
-    __shared__ float sdy[kTile];
-    __shared__ float s_sse;
-    load_params(params, s);
-    for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) g[i] = 0.f;
-    if (threadIdx.x == 0) s_sse = 0.f;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    GradShared& s = *reinterpret_cast<GradShared*>(s_raw);
+    load_forward_params(params, s.p);
+    for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) s.w2r[i / kH][i % kH] = bf16r(params[kOffW2 + i]);
+    for (int i = threadIdx.x; i < kMlpParams; i += blockDim.x) s.sum[i] = 0.f;
     __syncthreads();
-    float sse_local = 0.f;
-    const int q = threadIdx.x;
+    const int q = threadIdx.x, lane = q & 31, warp = q >> 5;
+    const int j0 = 4 * (lane >> 2), i0 = 8 * (lane & 3);
+    f32x2 gw2[4][4];             // W2: units j0 .. + 3, inputs i0 + 2 u, + 1
+    f32x2 gw1[4];                // W1 and b1 of unit `lane`: inputs 0 .. 5, then the bias and a term unused
+    float gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, sse_local = 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        gw1[u] = 0ull;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) gw2[u][v] = 0ull;
+    }
     for (int64_t base = (int64_t)blockIdx.x * kTile; base < n; base += (int64_t)gridDim.x * kTile) {
-        const int64_t r = base + q;
-        const bool valid = r < n;
-        float a0[kIn], a1[kH];
+        {
+            const int64_t r = base + q;
+            const bool valid = r < n;
+            float a0[1][kIn], a1[1][kH], a2[1][kH], d2[kH];
 #pragma unroll
-        for (int i = 0; i < kIn; ++i) {
-            a0[i] = valid ? bf16r(x[r * kIn + i]) : 0.f;
-            sa0[q][i] = a0[i];
-        }
-        layer1(s, a0, a1);
+            for (int i = 0; i < kIn; ++i) a0[0][i] = valid ? bf16r(x[r * kIn + i]) : 0.f;
+            layer_units<kIn, kH, 1>(s.p.w1, s.p.b1, 0, a0, a1);
+            layer_units<kH, kH, 1>(s.p.w2, s.p.b2, 0, a1, a2);
+            float out = 0.f;
 #pragma unroll
-        for (int i = 0; i < kH; ++i) sa1[q][i] = a1[i];
-        float out = 0.f;
-#pragma unroll 4
-        for (int j = 0; j < kH; ++j) {
-            const float a2 = layer2_unit(s, a1, j);
-            sa2[q][j] = a2;
-            out = fmaf(s[kOffW3 + j], a2, out);
-        }
-        out += s[kOffB3];
-        const float err = valid ? out - t[r] : 0.f;
-        sse_local += err * err;
-        const float dy = 2.f * scale * err;
-        sdy[q] = dy;
-        // relu masks: a > 0 exactly when z > 0 (rounding to bf16 keeps a positive value positive)
+            for (int j = 0; j < kH; ++j) out = fmaf(s.p.w3[j], a2[0][j], out);
+            out += s.p.b3;
+            const float err = valid ? out - t[r] : 0.f;
+            sse_local += err * err;
+            const float dy = 2.f * scale * err;
+            // relu masks: a > 0 exactly when z > 0 (rounding to bf16 keeps a positive value positive)
 #pragma unroll
-        for (int j = 0; j < kH; ++j) sd2[q][j] = sa2[q][j] > 0.f ? dy * s[kOffW3 + j] : 0.f;
-#pragma unroll 4
-        for (int i = 0; i < kH; ++i) {
-            float acc = 0.f;
+            for (int j = 0; j < kH; ++j) d2[j] = a2[0][j] > 0.f ? dy * s.p.w3[j] : 0.f;
 #pragma unroll
-            for (int j = 0; j < kH; ++j) acc = fmaf(s[kOffW2 + j * kH + i], sd2[q][j], acc);
-            sd1[q][i] = sa1[q][i] > 0.f ? acc : 0.f;
-        }
-        __syncthreads();
-        // parameter gradients of this tile: sums over its samples
-        for (int p = threadIdx.x; p < kMlpParams; p += blockDim.x) {
-            float acc = 0.f;
-            if (p < kOffB1) {
-                const int j = p / kIn, i = p % kIn;
-                for (int b = 0; b < kTile; ++b) acc = fmaf(sd1[b][j], sa0[b][i], acc);
-            } else if (p < kOffW2) {
-                const int j = p - kOffB1;
-                for (int b = 0; b < kTile; ++b) acc += sd1[b][j];
-            } else if (p < kOffB2) {
-                const int j = (p - kOffW2) / kH, i = (p - kOffW2) % kH;
-                for (int b = 0; b < kTile; ++b) acc = fmaf(sd2[b][j], sa1[b][i], acc);
-            } else if (p < kOffW3) {
-                const int j = p - kOffB2;
-                for (int b = 0; b < kTile; ++b) acc += sd2[b][j];
-            } else if (p < kOffB3) {
-                const int i = p - kOffW3;
-                for (int b = 0; b < kTile; ++b) acc = fmaf(sdy[b], sa2[b][i], acc);
-            } else {
-                for (int b = 0; b < kTile; ++b) acc += sdy[b];
+            for (int j = 0; j < kH; j += 4) {
+                *reinterpret_cast<float4*>(&s.a1[q][j]) = make_float4(a1[0][j], a1[0][j + 1], a1[0][j + 2], a1[0][j + 3]);
+                *reinterpret_cast<float4*>(&s.a2[q][j]) = make_float4(a2[0][j], a2[0][j + 1], a2[0][j + 2], a2[0][j + 3]);
+                *reinterpret_cast<float4*>(&s.d2[q][j]) = make_float4(d2[j], d2[j + 1], d2[j + 2], d2[j + 3]);
             }
-            g[p] += acc;
+            *reinterpret_cast<float4*>(&s.a0[q][0]) = make_float4(a0[0][0], a0[0][1], a0[0][2], a0[0][3]);
+            *reinterpret_cast<float4*>(&s.a0[q][4]) = make_float4(a0[0][4], a0[0][5], 1.f, dy);
+            f32x2 acc[kH / 2];
+#pragma unroll
+            for (int u = 0; u < kH / 2; ++u) acc[u] = 0ull;
+#pragma unroll
+            for (int j = 0; j < kH; ++j) {
+                const f32x2 dj = pack2(d2[j], d2[j]);
+#pragma unroll
+                for (int u = 0; u < kH / 2; u += 2) {
+                    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&s.w2r[j][2 * u]);
+                    acc[u] = fma2(w.x, dj, acc[u]);
+                    acc[u + 1] = fma2(w.y, dj, acc[u + 1]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kH / 2; u += 2) {
+                float4 d;
+                unpack2(acc[u], d.x, d.y);
+                unpack2(acc[u + 1], d.z, d.w);
+                d.x = a1[0][2 * u] > 0.f ? d.x : 0.f;
+                d.y = a1[0][2 * u + 1] > 0.f ? d.y : 0.f;
+                d.z = a1[0][2 * u + 2] > 0.f ? d.z : 0.f;
+                d.w = a1[0][2 * u + 3] > 0.f ? d.w : 0.f;
+                *reinterpret_cast<float4*>(&s.d1[q][2 * u]) = d;
+            }
+        }
+        __syncwarp();  // a warp adds up its own 32 samples: no other warp's are read
+#pragma unroll 2
+        for (int b = warp * 32; b < warp * 32 + 32; ++b) {
+            const float4 d = *reinterpret_cast<const float4*>(&s.d2[b][j0]);
+            const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(&s.a1[b][i0]);
+            const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(&s.a1[b][i0 + 4]);
+            const float dd[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const f32x2 e = pack2(dd[u], dd[u]);
+                gw2[u][0] = fma2(e, a.x, gw2[u][0]);
+                gw2[u][1] = fma2(e, a.y, gw2[u][1]);
+                gw2[u][2] = fma2(e, c.x, gw2[u][2]);
+                gw2[u][3] = fma2(e, c.y, gw2[u][3]);
+            }
+            const ulonglong2 f = *reinterpret_cast<const ulonglong2*>(&s.a0[b][0]);
+            const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(&s.a0[b][4]);
+            const f32x2 e = pack2(s.d1[b][lane], s.d1[b][lane]);
+            gw1[0] = fma2(e, f.x, gw1[0]);
+            gw1[1] = fma2(e, f.y, gw1[1]);
+            gw1[2] = fma2(e, g.x, gw1[2]);
+            gw1[3] = fma2(e, g.y, gw1[3]);
+            float one, dy;
+            unpack2(g.y, one, dy);
+            gb2 += s.d2[b][lane];
+            gw3 = fmaf(dy, s.a2[b][lane], gw3);
+            gb3 += dy;
+        }
+        __syncwarp();
+    }
+    for (int o = 16; o > 0; o >>= 1) sse_local += __shfl_xor_sync(0xffffffffu, sse_local, o);
+    if (lane == 0) s.sse[warp] = sse_local;
+    // the warps' sums, one warp after another
+    for (int w = 0; w < kTileWarps; ++w) {
+        if (w == warp) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    float lo, hi;
+                    unpack2(gw2[u][v], lo, hi);
+                    s.sum[kOffW2 + (j0 + u) * kH + i0 + 2 * v] += lo;
+                    s.sum[kOffW2 + (j0 + u) * kH + i0 + 2 * v + 1] += hi;
+                }
+                float lo, hi;
+                unpack2(gw1[u], lo, hi);
+                if (u < 3) {
+                    s.sum[kOffW1 + lane * kIn + 2 * u] += lo;
+                    s.sum[kOffW1 + lane * kIn + 2 * u + 1] += hi;
+                } else {
+                    s.sum[kOffB1 + lane] += lo;
+                }
+            }
+            s.sum[kOffB2 + lane] += gb2;
+            s.sum[kOffW3 + lane] += gw3;
+            if (lane == 0) s.sum[kOffB3] += gb3;
         }
         __syncthreads();
     }
-    atomicAdd(&s_sse, sse_local);
-    __syncthreads();
-    for (int p = threadIdx.x; p < kMlpParams; p += blockDim.x) atomicAdd(&grad[p], g[p]);
-    if (threadIdx.x == 0) atomicAdd(sse, s_sse);
+    for (int p = threadIdx.x; p < kMlpParams; p += blockDim.x) atomicAdd(&grad[p], s.sum[p]);
+    if (threadIdx.x == 0) {
+        float total = s.sse[0];
+        for (int w = 1; w < kTileWarps; ++w) total += s.sse[w];
+        atomicAdd(sse, total);
+    }
 }
 
 // Adam (Kingma & Ba): m <- b1 m + (1-b1) g; v <- b2 v + (1-b2) g^2;
@@ -433,7 +479,13 @@ int gc_mlp_grad(const float* params, const float* x, const float* t, int64_t n, 
                 float* sse, void* stream) {
     if (n < 0 || !params || !grad || !sse || (n > 0 && (!x || !t))) return GC_ERR_INVALID;
     if (n == 0) return GC_OK;
-    mlp_grad_kernel<<<grid_for(n, kTile, sm_count() * 4), kTile, 0, (cudaStream_t)stream>>>(
+    // (two blocks an SM: their shared memory)
+    if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradShared)) !=
+        cudaSuccess) {
+        (void)cudaGetLastError();
+        return GC_ERR_CUDA;
+    }
+    mlp_grad_kernel<<<grid_for(n, kTile, sm_count() * 2), kTile, sizeof(GradShared), (cudaStream_t)stream>>>(
         params, x, t, n, scale, grad, sse);
     return check_launch();
 }

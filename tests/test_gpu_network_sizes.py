@@ -1,0 +1,53 @@
+"""The network's kernels and the features at the edges of their tiles, grids and rows."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+from oracle import learned as L
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def gcpkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1205_3809_gb300 as m
+    m.library()
+    return m
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _uniform(seed, stream, count, lo, hi):
+    u = (gg.draws(seed, stream, count) >> np.uint64(11)).astype(np.float64) / float(1 << 53)
+    return (lo + (hi - lo) * u).astype(np.float32)
+
+
+# two samples a thread, 256 threads a block, two blocks an SM (152 of them): 155,648 a grid
+@pytest.mark.parametrize("n", [1, 2, 255, 257, 511, 512, 513, 155647, 155649])
+def test_forward_sizes(gcpkg, n):
+    p = _uniform(n, 7, L.N_PARAMS, -0.3, 0.3)
+    x = _uniform(n + 1, 9, n * L.N_IN, -2.0, 24.0).reshape(n, L.N_IN)
+    got = gcpkg.mlp_forward(_dev(p), _dev(x)).cpu().numpy()
+    assert np.array_equal(got.view(np.uint32), L.mlp_forward(p, x).view(np.uint32))
+
+
+# 128 samples a tile, two blocks an SM: 38,912 before a block takes a second tile
+@pytest.mark.parametrize("n", [2, 31, 33, 127, 128, 129, 38911, 38913, 80000])
+def test_gradient_sizes(gcpkg, n):
+    p = _uniform(n, 7, L.N_PARAMS, -0.3, 0.3)
+    x = _uniform(n + 1, 9, n * L.N_IN, 0.0, 16.0).reshape(n, L.N_IN)
+    t = np.linspace(-1.0, 1.0, n).astype(np.float32)
+    grad = torch.zeros(L.N_PARAMS, dtype=torch.float32, device="cuda")
+    sse = torch.zeros(1, dtype=torch.float32, device="cuda")
+    gcpkg.mlp_grad(_dev(p), _dev(x), _dev(t), 1.0 / n, grad, sse)
+    want, want_sse = L.mlp_grad(p, x, t, 1.0 / n, rounding=True)
+    got = grad.cpu().numpy().astype(np.float64)
+    # the bound of test_gpu_learned.test_grad_matches_oracle: fp32 sums of n terms in another order
+    assert np.all(np.abs(got - want) <= 1e-4 * np.abs(want).max() + 1e-5 * np.abs(want)), np.abs(got - want).max()
+    assert abs(float(sse.item()) - want_sse) <= 1e-4 * want_sse + 1e-6
