@@ -262,6 +262,15 @@ unsigned rounds_blocks(int64_t n, int64_t nnz, int threads, int64_t most) {
     return (unsigned)std::min(most, (warps + per_block - 1) / per_block);
 }
 
+// What a run needs cleared: the round state and the volume counters, which lie
+// side by side at the head of the layout, and the hub records, if any.
+int clear_workspace(char* base, const Layout& L, const Stats& hs, int64_t round_cap, cudaStream_t s) {
+    GC_CUDA(cudaMemsetAsync(base + L.st, 0, L.rv - L.st + (size_t)round_cap * sizeof(unsigned long long), s));
+    if (hs.cap[gc::kBinH])
+        GC_CUDA(cudaMemsetAsync(base + L.hubs, 0, (size_t)hs.cap[gc::kBinH] * sizeof(gc::HubRecord), s));
+    return GC_OK;
+}
+
 // Loop mode 2: rounds 2.. as one CUDA graph: a condition kernel, then a while
 // node whose body is one round kernel and the condition kernel, so the loop
 // runs on the device without a cooperative launch or host round trips.  The
@@ -328,8 +337,8 @@ int run_rounds_graph(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStr
 }
 
 template <typename T, bool P>
-int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_t s, int64_t* launches,
-                 const HostInput* hin) {
+int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, bool long_rows, cudaStream_t s,
+                 int64_t* launches, const HostInput* hin) {
     const int threads = o.block_threads;
     {
         // one warp task per 32 vertices, per input chunk when the input is still arriving
@@ -344,9 +353,11 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
             GC_CUDA(cudaGetLastError());
             *launches += 1;
         }
-        gc::pass1_long_kernel<T><<<dc.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
-        GC_CUDA(cudaGetLastError());
-        *launches += 1;
+        if (long_rows) {
+            gc::pass1_long_kernel<T><<<dc.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
+            GC_CUDA(cudaGetLastError());
+            *launches += 1;
+        }
         if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[2], s));
     }
     if (o.loop_mode == 2) return run_rounds_graph<T, P>(o, dc, p, s, launches);
@@ -411,10 +422,10 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_
 // The round kernels are compiled twice: with a priority array (its order
 // kept as a bit in the active lists) and without (index order).
 template <typename T>
-int run_rounds(const gc_options& o, DeviceCache& dc, Params<T>& p, cudaStream_t s, int64_t* launches,
+int run_rounds(const gc_options& o, DeviceCache& dc, Params<T>& p, bool long_rows, cudaStream_t s, int64_t* launches,
                const HostInput* hin = nullptr) {
-    return p.prio ? run_rounds_p<T, true>(o, dc, p, s, launches, hin)
-                  : run_rounds_p<T, false>(o, dc, p, s, launches, hin);
+    return p.prio ? run_rounds_p<T, true>(o, dc, p, long_rows, s, launches, hin)
+                  : run_rounds_p<T, false>(o, dc, p, long_rows, s, launches, hin);
 }
 
 int normalise(const gc_options* opt, gc_options* o) {
@@ -537,6 +548,7 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
     Layout L;
     char* base = nullptr;
     RoundState* st = nullptr;
+    RoundState hst;
     for (;;) {
         const size_t elem = bits == 16 ? 2 : 4;
         L = make_layout(n, hs.nnz, elem, hs, round_cap);
@@ -544,9 +556,8 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
         if (rc != GC_OK) return rc;
         base = (char*)dc.ws;
         st = (RoundState*)(base + L.st);
-        GC_CUDA(cudaMemsetAsync(st, 0, sizeof(RoundState), s));
-        GC_CUDA(cudaMemsetAsync(base + L.rv, 0, (size_t)round_cap * sizeof(unsigned long long), s));
-        GC_CUDA(cudaMemsetAsync(base + L.hubs, 0, (size_t)hs.cap[gc::kBinH] * sizeof(gc::HubRecord), s));
+        rc = clear_workspace(base, L, hs, round_cap, s);
+        if (rc != GC_OK) return rc;
 
         auto fill = [&](auto& p) {
             using PT = std::remove_reference_t<decltype(p)>;
@@ -572,28 +583,21 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
         if (bits == 16) {
             Params<uint16_t> p;
             fill(p);
-            rc = run_rounds(o, dc, p, s, &launches, hin);
+            rc = run_rounds(o, dc, p, hs.defer != 0, s, &launches, hin);
         } else {
             Params<int32_t> p;
             fill(p);
-            rc = run_rounds(o, dc, p, s, &launches, hin);
+            rc = run_rounds(o, dc, p, hs.defer != 0, s, &launches, hin);
         }
         if (rc != GC_OK) return rc;
-        if (bits == 32) break;
-        int status = 0;
-        GC_CUDA(cudaMemcpyAsync(dc.host, &st->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+        // results (and whether a color did not fit)
+        if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[3], s));
+        GC_CUDA(cudaMemcpyAsync(dc.host, st, sizeof(RoundState), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
-        std::memcpy(&status, dc.host, sizeof(int));
-        if (status != gc::kStatusColorOverflow) break;
+        std::memcpy(&hst, dc.host, sizeof(RoundState));
+        if (bits == 32 || hst.status != gc::kStatusColorOverflow) break;
         bits = 32;
     }
-
-    // 4. results
-    if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[3], s));
-    GC_CUDA(cudaMemcpyAsync(dc.host, st, sizeof(RoundState), cudaMemcpyDeviceToHost, s));
-    GC_CUDA(cudaStreamSynchronize(s));
-    RoundState hst;
-    std::memcpy(&hst, dc.host, sizeof(RoundState));
     if (hst.status == gc::kStatusTimeout) return GC_ERR_TIMEOUT;
     g_last.valid = 1;
     GC_CUDA(cudaGetDevice(&g_last.device));
@@ -722,9 +726,8 @@ int color_noalloc_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n
         const Layout L = make_layout(n, hs.nnz, elem, hs, round_cap);
         if (L.total > kNoAllocBytes) return GC_ERR_TOO_LARGE;
         st = (RoundState*)(base + L.st);
-        GC_CUDA(cudaMemsetAsync(st, 0, sizeof(RoundState), s));
-        GC_CUDA(cudaMemsetAsync(base + L.rv, 0, (size_t)round_cap * sizeof(unsigned long long), s));
-        GC_CUDA(cudaMemsetAsync(base + L.hubs, 0, (size_t)hs.cap[gc::kBinH] * sizeof(gc::HubRecord), s));
+        rc = clear_workspace(base, L, hs, round_cap, s);
+        if (rc != GC_OK) return rc;
         auto fill = [&](auto& p) {
             using PT = std::remove_reference_t<decltype(p)>;
             using T = std::remove_pointer_t<decltype(PT::X0)>;
@@ -746,11 +749,11 @@ int color_noalloc_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n
         if (bits == 16) {
             Params<uint16_t> p;
             fill(p);
-            rc = run_rounds(o, dc, p, s, &launches);
+            rc = run_rounds(o, dc, p, hs.defer != 0, s, &launches);
         } else {
             Params<int32_t> p;
             fill(p);
-            rc = run_rounds(o, dc, p, s, &launches);
+            rc = run_rounds(o, dc, p, hs.defer != 0, s, &launches);
         }
         if (rc != GC_OK) return rc;
         RoundState hst;
@@ -960,11 +963,10 @@ int batch_enqueue_typed(gc_batch& b, cudaStream_t s) {
     int32_t* colidx_g = (int32_t*)(base + b.off_colidx);
     int32_t* settle = (int32_t*)(base + b.off_settle);
     RoundState* st = (RoundState*)(base + b.L.st);
-    GC_CUDA(cudaMemsetAsync(st, 0, sizeof(RoundState), s));
-    GC_CUDA(cudaMemsetAsync(base + b.L.rv, 0, (size_t)b.round_cap * sizeof(unsigned long long), s));
-    GC_CUDA(cudaMemsetAsync(base + b.L.hubs, 0, (size_t)b.hs.cap[gc::kBinH] * sizeof(gc::HubRecord), s));
+    int rc = clear_workspace(base, b.L, b.hs, b.round_cap, s);
+    if (rc != GC_OK) return rc;
     int64_t launches = 0;
-    int rc = batch_rebase(b, s, &launches);
+    rc = batch_rebase(b, s, &launches);
     if (rc != GC_OK) return rc;
     Params<T> p;
     p.rowptr = rowptr_g;
@@ -986,9 +988,12 @@ int batch_enqueue_typed(gc_batch& b, cudaStream_t s) {
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)b.sms * 8));
         gc::pass1_kernel<T><<<grid, 256, 0, s>>>(p, 0, (int32_t)b.N);
         GC_CUDA(cudaGetLastError());
-        gc::pass1_long_kernel<T><<<b.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
-        GC_CUDA(cudaGetLastError());
-        launches += 2;
+        ++launches;
+        if (b.hs.defer) {
+            gc::pass1_long_kernel<T><<<b.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
+            GC_CUDA(cudaGetLastError());
+            ++launches;
+        }
     }
     {
         cudaLaunchConfig_t cfg = {};
