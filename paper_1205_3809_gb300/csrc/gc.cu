@@ -5,9 +5,9 @@
 //      checks; one device-to-host copy decides the color width (16-bit color
 //      state when every first-fit color fits, i.e. max degree + 1 <= 65535)
 //      and sizes the workspace;
-//   2. pass1_kernel (rows of up to 256 entries) + pass1_long_kernel (longer
-//      rows): round 1 (closed form, all colors 1), its conflict test, and
-//      round 2's colors (all 2);
+//   2. pass1_kernel (and pass1_long_kernel for long rows that a first look
+//      leaves open): round 1 (closed form, all colors 1), its conflict test,
+//      and round 2's colors (all 2);
 //   3. rounds_persistent_kernel: every later round in one cooperative launch
 //      (or, with loop_mode = 1, one round_kernel launch per round; with
 //      loop_mode = 2, graph_round_kernel in a CUDA graph's conditional loop);
@@ -271,6 +271,19 @@ int clear_workspace(char* base, const Layout& L, const Stats& hs, int64_t round_
     return GC_OK;
 }
 
+// Pass 1 over vertices [v0, v1).
+template <typename T>
+int launch_pass1(const Params<T>& p, int32_t v0, int32_t v1, int sms, cudaStream_t s) {
+    const int64_t count = (int64_t)v1 - v0;
+    if (count >= (int64_t)sms * 1024) {
+        gc::pass1_kernel<T, 4><<<(int)std::min<int64_t>((count + 1023) / 1024, (int64_t)sms * 4), 256, 0, s>>>(p, v0, v1);
+    } else {
+        gc::pass1_kernel<T, 1><<<(int)((count + 255) / 256), 256, 0, s>>>(p, v0, v1);
+    }
+    GC_CUDA(cudaGetLastError());
+    return GC_OK;
+}
+
 // Loop mode 2: rounds 2.. as one CUDA graph: a condition kernel, then a while
 // node whose body is one round kernel and the condition kernel, so the loop
 // runs on the device without a cooperative launch or host round trips.  The
@@ -341,16 +354,14 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, bool long_r
                  int64_t* launches, const HostInput* hin) {
     const int threads = o.block_threads;
     {
-        // one warp task per 32 vertices, per input chunk when the input is still arriving
+        // per input chunk when the input is still arriving
         const int nch = hin ? hin->nchunks : 1;
         for (int c = 0; c < nch; ++c) {
             const int32_t v0 = hin ? hin->vb[c] : 0, v1 = hin ? hin->vb[c + 1] : p.n;
             if (hin) GC_CUDA(cudaStreamWaitEvent(s, dc.chunk_ev[c], 0));
             if (v1 <= v0) continue;
-            const int64_t want = ((int64_t)v1 - v0 + 255) / 256;
-            const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)dc.sms * 8));
-            gc::pass1_kernel<T><<<grid, 256, 0, s>>>(p, v0, v1);
-            GC_CUDA(cudaGetLastError());
+            const int rc = launch_pass1(p, v0, v1, dc.sms, s);
+            if (rc != GC_OK) return rc;
             *launches += 1;
         }
         if (long_rows) {
@@ -984,10 +995,8 @@ int batch_enqueue_typed(gc_batch& b, cudaStream_t s) {
     p.settle_round = settle;
     fill_workspace(p, base, b.L, st, b.round_cap);
     {
-        const int64_t want = (b.N + 255) / 256;
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)b.sms * 8));
-        gc::pass1_kernel<T><<<grid, 256, 0, s>>>(p, 0, (int32_t)b.N);
-        GC_CUDA(cudaGetLastError());
+        rc = launch_pass1(p, 0, (int32_t)b.N, b.sms, s);
+        if (rc != GC_OK) return rc;
         ++launches;
         if (b.hs.defer) {
             gc::pass1_long_kernel<T><<<b.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);

@@ -70,7 +70,7 @@ constexpr int kSmallMaxLimit = 32;            // S bin: length <= 32
 constexpr int kMedMaxLimit = 32 * kPerLane;   // M bin: length <= 256
 constexpr int kHubSub = 32 * kPerLane;        // 256 entries: one sub-block of a hub chunk
 constexpr int kChunk = 4 * kHubSub;           // 1024 entries per H-bin task
-constexpr int kPass1Flat = 256;               // pass 1: longer rows go to pass1_long_kernel
+constexpr int kPass1Flat = 256;               // pass 1: longer open rows go to pass1_long_kernel
 constexpr int kPass1LongBlocksPerSm = 8;      // pass 1, long rows: grid of 8 blocks per SM
 #ifndef GC_FLAT_BATCHES
 #define GC_FLAT_BATCHES 4
@@ -165,7 +165,7 @@ __host__ __device__ __forceinline__ unsigned hub_chunks(unsigned long long hc) {
 // down the atomics of blocks still working.
 struct RoundState {
     RoundCounts rc[3];     // [k % 3]: the counts of U_k
-    alignas(128) unsigned defer_cnt;  // pass 1: vertices above kPass1Flat
+    alignas(128) unsigned defer_cnt;  // pass 1: rows left to pass1_long_kernel
     alignas(128) unsigned task_next[3];  // [k % 3]: tasks of round k claimed so far (beyond the first two per warp)
     alignas(128) unsigned bar_count;  // blocks that have reached a barrier, over all barriers
     alignas(128) int status;
@@ -210,7 +210,7 @@ struct Params {
     // owner position of each chunk
     int4* L2A; int4* L4A; int4* L8A; int4* L16A; int4* SA; int4* MA; int4* HA; int32_t* HcA; int32_t* OA;
     int4* L2B; int4* L4B; int4* L8B; int4* L16B; int4* SB; int4* MB; int4* HB; int32_t* HcB; int32_t* OB;
-    int32_t* defer;                     // pass 1: rows longer than kPass1Flat
+    int32_t* defer;                     // pass 1: long rows left open
     HubRecord* hubs;
     RoundState* st;
     int32_t* round_sizes;               // device telemetry, round_sizes[k-1] = |U_k|
@@ -621,141 +621,215 @@ __device__ __forceinline__ NextLists pass1_next(const Params<T>& p) {
     return nl;
 }
 
-// Round 1 on 32 consecutive vertices per task, over vertices [v_begin, v_end)
-// (v_begin a multiple of 32; the host may launch it per range as the input
-// arrives).  Their adjacency entries
-// (rows of degree <= kPass1Flat) are read as one flat, coalesced range;
-// lane l of batch u handles flat entry F0 + 32u + l, finds its row from the
-// batch's row starts (an OR-reduction over the warp and a table of the
-// non-empty rows' lanes), and marks the row in shared memory when the entry
-// precedes it.  Longer rows go to pass1_long_kernel.
-template <typename T>
-__global__ void __launch_bounds__(256, 5) pass1_kernel(Params<T> p, int32_t v_begin, int32_t v_end) {
-    // a warp takes two tasks (t, t + W) at a time and appends their T and M
-    // entries with one atomic per bin: every task appends to both, and the
-    // counters' lines were the busiest of the L2 in this kernel
-    constexpr int NT = 2;
-    struct P1Smem {
-        uint8_t lane_of[32];  // lane of the i-th non-empty row
-        unsigned hit[32];     // row r has a preceding neighbour
-    };
-    __shared__ P1Smem s_p1[8];
-    const unsigned wib = threadIdx.x >> 5;
-    const unsigned lane = lane_id();
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t ntasks = ((int64_t)v_end - v_begin + 31) / 32;
+// Eight consecutive entries of colidx from index a on (a multiple of eight
+// counted from the 32-byte boundary at or below colidx), with one 32-byte
+// load; where that would reach outside the array, entry by entry.
+__device__ __forceinline__ void load_chunk(const int32_t* __restrict__ colidx, int32_t nnz, int32_t a, uint64_t pol,
+                                           int32_t (&w)[8]) {
+    if (a >= 0 && a <= nnz - 8) {
+        asm volatile("ld.global.nc.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
+                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                     : "l"(colidx + a), "l"(pol));
+    } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) w[u] = a + u >= 0 && a + u < nnz ? __ldg(colidx + a + u) : 0;
+    }
+}
+
+// Whether one of the chunk's entries at positions [U0, U1) that `in` marks precedes v.
+template <int U0, int U1>
+__device__ __forceinline__ bool chunk_precedes(const uint32_t* __restrict__ prio, const int32_t (&w)[8], uint32_t in,
+                                               int32_t v, uint32_t pv) {
+    bool hit = false;
+    if (prio) {
+        uint32_t pw[U1 - U0];
+#pragma unroll
+        for (int u = U0; u < U1; ++u) pw[u - U0] = (in >> u) & 1u ? __ldg(prio + w[u]) : 0xffffffffu;
+#pragma unroll
+        for (int u = U0; u < U1; ++u)
+            hit |= ((in >> u) & 1u) && (pw[u - U0] < pv || (pw[u - U0] == pv && w[u] < v));
+    } else {
+#pragma unroll
+        for (int u = U0; u < U1; ++u) hit |= ((in >> u) & 1u) && w[u] < v;
+    }
+    return hit;
+}
+
+// The positions of a chunk at offset off of a row of d entries that lie in the row.
+__device__ __forceinline__ uint32_t chunk_in_row(int32_t off, int32_t d) {
+    return low_bits(max(0, min(8, d - off))) & (off < 0 ? 0xffu << -off : 0xffu);
+}
+
+// Round 1 over vertices [v_begin, v_end) (the host may launch it per range as
+// the input arrives): a vertex conflicts iff a neighbour precedes it, and one
+// such neighbour decides that, so a row is read only as far as needed.  A
+// block takes 256 PER vertices at a time.  Every thread reads the first
+// 32-byte chunk of its rows (all of it under index priority; half the chunk at a
+// time when a key has to be gathered for each entry).  Rows that this
+// leaves open, local minima for the most part, are read on by four lanes each
+// from a list in shared memory, or, when longer than kPass1Flat, go to
+// pass1_long_kernel.  The block appends its entries with one atomic per counter.
+//
+// Bound: one 32-byte sector of colidx per vertex, and its row start, buffers and
+// worklist entry.  Reading every row to its end as one flat range took 0.71 ms
+// for R-MAT-B of 2^24 vertices (now 0.38) and 0.24 for R-MAT-ER of 2^22 (now
+// 0.10).
+//
+// PER vertices a thread: 4, or 1 for a range too small to give every SM a block
+// of 1,024.
+template <typename T, int PER>
+__global__ void __launch_bounds__(256, 4) pass1_kernel(Params<T> p, int32_t v_begin, int32_t v_end) {
+    constexpr int kPass1Per = PER, kPass1Block = 256 * PER;
+    constexpr int kBins = 6;                // L2, L4, L8, L16, M entries; long rows left open
+    __shared__ int32_t s_b[kPass1Block], s_d[kPass1Block];
+    __shared__ uint16_t s_open[kPass1Block];  // vertices of this block whose first chunk left them open
+    __shared__ uint8_t s_hit[kPass1Block];
+    __shared__ unsigned s_nopen, s_cnt[kBins], s_base[kBins];
+    __shared__ unsigned long long s_hub, s_hub_base;
     const NextLists nl = pass1_next(p);
-    const uint64_t pol_adj = policy_evict_first();
+    const uint64_t pol = policy_evict_first();
+    const uint32_t mis = (uint32_t)((uintptr_t)p.colidx >> 2) & 7u;
+    const unsigned tid = threadIdx.x, lane = lane_id();
+    const unsigned below = (1u << lane) - 1u;
     int maxc = 0;
     unsigned vol = 0;
-    for (int64_t t0 = gw; t0 < ntasks; t0 += W * NT) {
-        int4 ev[NT];
-        int cls[NT];  // L2, L4, L8, L16, M (0..4), or -1
+    for (int64_t first = (int64_t)v_begin + (int64_t)blockIdx.x * kPass1Block; first < v_end;
+         first += (int64_t)gridDim.x * kPass1Block) {
+        if (tid < kBins) s_cnt[tid] = 0u;
+        if (tid == kBins) s_nopen = 0u;
+        if (tid == kBins + 1) s_hub = 0ull;
+        __syncthreads();
+        int32_t b[kPass1Per], d[kPass1Per];
+        unsigned hits = 0u, opens = 0u;  // bit i: this thread's vertex i
 #pragma unroll
-        for (int jt = 0; jt < NT; ++jt) {
-            const int64_t t = t0 + (int64_t)jt * W;
-            const int64_t vv = (int64_t)v_begin + t * 32 + lane;
-            const bool valid = t < ntasks && vv < v_end;
-            const int32_t v = valid ? (int32_t)vv : 0;
-            const int32_t b = valid ? __ldg(p.rowptr + v) : 0;
-            const int32_t d = valid ? __ldg(p.rowptr + v + 1) - b : 0;
-            const bool longrow = d > kPass1Flat;
-            const int32_t eff = longrow ? 0 : d;
-            const uint32_t pv = (p.prio && valid) ? __ldg(p.prio + v) : 0u;
-            int32_t incl = eff;
+        for (int i = 0; i < kPass1Per; ++i) {
+            const int64_t vv = first + i * 256 + tid;
+            b[i] = vv < v_end ? __ldg(p.rowptr + vv) : 0;
+            d[i] = vv < v_end ? __ldg(p.rowptr + vv + 1) - b[i] : 0;
+        }
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int32_t x = __shfl_up_sync(kFull, incl, o);
-                if ((int)lane >= o) incl += x;
+        for (int i = 0; i < kPass1Per; ++i) {
+            const int32_t v = (int32_t)(first + i * 256 + tid);
+            const int32_t off = -(int32_t)(((uint32_t)b[i] + mis) & 7u);
+            bool hit = false;
+            if (d[i] > 0) {
+                int32_t w[8];
+                load_chunk(p.colidx, p.nnz, b[i] + off, pol, w);
+                const uint32_t in = chunk_in_row(off, d[i]);
+                const uint32_t pv = p.prio ? __ldg(p.prio + v) : 0u;
+                hit = chunk_precedes<4, 8>(p.prio, w, in, v, pv);
+                if (!hit) hit = chunk_precedes<0, 4>(p.prio, w, in, v, pv);
             }
-            const int32_t off = incl - eff;
-            const int32_t D = __shfl_sync(kFull, incl, 31);
-            // entry f's row: the last non-empty row starting at or before f, found
-            // from the batch's row starts (one OR-reduction) and a lane table
-            const unsigned nz = __ballot_sync(kFull, eff > 0);
-            if (eff > 0) s_p1[wib].lane_of[__popc(nz & ((1u << lane) - 1u))] = (uint8_t)lane;
-            s_p1[wib].hit[lane] = 0u;
-            const int32_t b_off = b - off;  // entry f of this row sits at colidx[b_off + f]
-            __syncwarp();
-            for (int32_t F0 = 0; F0 < D; F0 += 32 * 4) {
-                int32_t w[4], own[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int32_t base = F0 + 32 * u;
-                    const int32_t f = base + (int32_t)lane;
-                    const int32_t rel = off - base;
-                    const unsigned before = __popc(__ballot_sync(kFull, eff > 0 && rel < 0));
-                    const unsigned starts = __reduce_or_sync(kFull, (eff > 0 && rel >= 0 && rel < 32) ? (1u << rel) : 0u);
-                    const unsigned rank = before + __popc(starts & (0xffffffffu >> (31 - lane)));
-                    const int o = (f < D && rank > 0) ? (int)s_p1[wib].lane_of[rank - 1] : 0;
-                    own[u] = o;
-                    const int32_t rb = __shfl_sync(kFull, b_off, o);
-                    w[u] = f < D ? ld_adj(p.colidx + rb + f, pol_adj) : 0;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int32_t f = F0 + 32 * u + (int32_t)lane;
-                    const uint32_t opv = __shfl_sync(kFull, pv, own[u]);
-                    if (f < D && precedes(p.prio, w[u], (int32_t)(v_begin + t * 32 + own[u]), opv))
-                        s_p1[wib].hit[own[u]] = 1u;
+            const bool open = !hit && off + 8 < d[i];
+            hits |= hit ? 1u << i : 0u;
+            opens |= open ? 1u << i : 0u;
+            const unsigned ball = __ballot_sync(kFull, open && d[i] <= kPass1Flat);
+            if (ball) {
+                unsigned at = 0;
+                if (lane == 0) at = atomicAdd(&s_nopen, (unsigned)__popc(ball));
+                at = __shfl_sync(kFull, at, 0) + __popc(ball & below);
+                if ((ball >> lane) & 1u) {
+                    const unsigned slot = i * 256 + tid;
+                    s_open[at] = (uint16_t)slot;
+                    s_b[slot] = b[i];
+                    s_d[slot] = d[i];
                 }
             }
-            __syncwarp();
-            const bool hit = s_p1[wib].hit[lane] != 0u;
-            if (valid && !longrow) {
-                pass1_write(p, v, hit, maxc);
-                if (hit) vol += (unsigned)d;
-            }
-            const int bin = bin_of(d, p.s_max, p.m_max);
-            const bool go = valid && !longrow && hit;
-            // an L2 or L4 entry starts with all of its row live and no static mask
-            ev[jt] = d <= p.lim4 ? make_int4(v, b, (int32_t)low_bits(d), 0) : make_int4(v, b, d, d);
-            cls[jt] = !go || bin == kBinH ? -1
-                                          : (d <= p.lim8 ? (d <= p.lim2 ? 0 : (d <= p.lim4 ? 1 : 2)) : (d <= p.lim16 ? 3 : 4));
-            // hubs that stayed in the flat range (m_max < d <= kPass1Flat)
-            unsigned hubs = __ballot_sync(kFull, go && bin == kBinH);
-            while (hubs) {
-                const int j = __ffs(hubs) - 1;
-                hubs &= hubs - 1;
-                const int32_t dj = __shfl_sync(kFull, d, j);
-                warp_append_hub(nl, make_int4(__shfl_sync(kFull, v, j), __shfl_sync(kFull, b, j), dj, dj));
-            }
-            warp_append_i32(valid && longrow, v, p.defer, &p.st->defer_cnt);
         }
-        // the entries of these NT tasks, one atomic per counter: L2 and L4 share one,
-        // L8 and L16 another, M has its own
-        unsigned long long n01 = 0, n23 = 0;
-        unsigned n4 = 0;
-#pragma unroll
-        for (int jt = 0; jt < NT; ++jt) {
-            n01 += pair_count(__popc(__ballot_sync(kFull, cls[jt] == 0)), __popc(__ballot_sync(kFull, cls[jt] == 1)));
-            n23 += pair_count(__popc(__ballot_sync(kFull, cls[jt] == 2)), __popc(__ballot_sync(kFull, cls[jt] == 3)));
-            n4 += __popc(__ballot_sync(kFull, cls[jt] == 4));
+        __syncthreads();
+        // open rows: four lanes each, 64 side by side
+        for (unsigned at = tid >> 2; at < ((s_nopen + 7u) & ~7u); at += 64u) {
+            const bool on = at < s_nopen;
+            const unsigned slot = on ? s_open[at] : 0u;
+            const int32_t v = (int32_t)(first + slot), ob = on ? s_b[slot] : 0, od = on ? s_d[slot] : 0;
+            const uint32_t pv = p.prio && on ? __ldg(p.prio + v) : 0u;
+            bool hit = false;
+            int32_t off = 8 + 8 * (int32_t)(lane & 3u) - (int32_t)(((uint32_t)ob + mis) & 7u);
+            for (; off < od && !hit; off += 32) {
+                int32_t w[8];
+                load_chunk(p.colidx, p.nnz, ob + off, pol, w);
+                hit = chunk_precedes<0, 8>(p.prio, w, chunk_in_row(off, od), v, pv);
+            }
+            const unsigned any = __ballot_sync(kFull, hit) >> (lane & ~3u) & 15u;
+            if (on && (lane & 3u) == 0u) s_hit[slot] = any != 0u;
         }
-        unsigned long long base = 0;
-        if (lane == 0 && n01) base = atomicAdd(&nl.cnt->tiny, n01);
-        if (lane == 1 && n23) base = atomicAdd(&nl.cnt->mid, n23);
-        if (lane == 2 && n4) base = atomicAdd(&nl.cnt->m, n4);
+        __syncthreads();
+        // outcome, and this block's share of every worklist
+        int cls[kPass1Per];
+        unsigned at[kPass1Per];
+        unsigned long long hub_at[kPass1Per];
 #pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            const unsigned long long from = __shfl_sync(kFull, base, c >> 1);
-            unsigned at = c & 1 ? high_count(from) : low_count(from);
-            int4* const list = c == 0 ? p.L2A : (c == 1 ? p.L4A : (c == 2 ? p.L8A : (c == 3 ? p.L16A : p.MA)));
+        for (int i = 0; i < kPass1Per; ++i) {
+            const int64_t vv = first + i * 256 + tid;
+            const bool later = (opens >> i & 1u) && d[i] > kPass1Flat;  // decided by pass1_long_kernel
+            const bool hit = (hits >> i & 1u) || ((opens >> i & 1u) && !later && s_hit[i * 256 + tid]);
+            cls[i] = -1;
+            if (vv < v_end) {
+                if (!later) {
+                    pass1_write(p, (int32_t)vv, hit, maxc);
+                    if (hit) vol += (unsigned)d[i];
+                }
+                if (later) cls[i] = 5;
+                else if (hit) cls[i] = d[i] <= p.lim8 ? (d[i] <= p.lim2 ? 0 : (d[i] <= p.lim4 ? 1 : 2))
+                                                      : (d[i] <= p.lim16 ? 3 : (d[i] <= p.m_max ? 4 : 6));
+            }
+            at[i] = 0u;
 #pragma unroll
-            for (int jt = 0; jt < NT; ++jt) {
-                const unsigned bal = __ballot_sync(kFull, cls[jt] == c);
-                if (cls[jt] == c) list[at + __popc(bal & ((1u << lane) - 1u))] = ev[jt];
-                at += __popc(bal);
+            for (int c = 0; c < kBins; ++c) {
+                const unsigned bal = __ballot_sync(kFull, cls[i] == c);
+                if (bal == 0u) continue;
+                unsigned base = 0;
+                if (lane == 0) base = atomicAdd(&s_cnt[c], (unsigned)__popc(bal));
+                base = __shfl_sync(kFull, base, 0);
+                if (cls[i] == c) at[i] = base + __popc(bal & below);
+            }
+            hub_at[i] = 0ull;
+            if (cls[i] == 6) hub_at[i] = atomicAdd(&s_hub, pair_count(1u, (unsigned)(d[i] + kChunk - 1) / kChunk));
+        }
+        __syncthreads();
+        if (tid == 0 && (s_cnt[0] | s_cnt[1])) {
+            const unsigned long long x = atomicAdd(&nl.cnt->tiny, pair_count(s_cnt[0], s_cnt[1]));
+            s_base[0] = low_count(x);
+            s_base[1] = high_count(x);
+        }
+        if (tid == 32 && (s_cnt[2] | s_cnt[3])) {
+            const unsigned long long x = atomicAdd(&nl.cnt->mid, pair_count(s_cnt[2], s_cnt[3]));
+            s_base[2] = low_count(x);
+            s_base[3] = high_count(x);
+        }
+        if (tid == 64 && s_cnt[4]) s_base[4] = atomicAdd(&nl.cnt->m, s_cnt[4]);
+        if (tid == 96 && s_cnt[5]) s_base[5] = atomicAdd(&p.st->defer_cnt, s_cnt[5]);
+        if (tid == 128 && s_hub) s_hub_base = atomicAdd(&nl.cnt->hc, s_hub);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kPass1Per; ++i) {
+            const int32_t v = (int32_t)(first + i * 256 + tid);
+            if (cls[i] == 6) {
+                // (both halves of the pair stay below 2^32: no carry)
+                const unsigned long long x = s_hub_base + hub_at[i];
+                const unsigned pos = hub_count(x), c0 = hub_chunks(x);
+                nl.H[pos] = make_int4(v, b[i], d[i], d[i]);
+                nl.Hc[pos] = (int32_t)c0;
+                for (unsigned j = 0; j < (unsigned)(d[i] + kChunk - 1) / kChunk; ++j) nl.O[c0 + j] = (int32_t)pos;
+            } else if (cls[i] == 5) {
+                p.defer[s_base[5] + at[i]] = v;
+            } else if (cls[i] >= 0) {
+                int4* const list = cls[i] == 0 ? p.L2A
+                                               : (cls[i] == 1 ? p.L4A : (cls[i] == 2 ? p.L8A : (cls[i] == 3 ? p.L16A : p.MA)));
+                // an L2 or L4 entry starts with all of its row live and no static mask
+                list[s_base[cls[i]] + at[i]] =
+                    cls[i] <= 1 ? make_int4(v, b[i], (int32_t)low_bits(d[i]), 0) : make_int4(v, b[i], d[i], d[i]);
             }
         }
+        __syncthreads();
     }
     fold_max_color(p.st, maxc);
     fold_volume(p.st, p.round_vol, p.round_cap, 2, vol);
 }
 
-// Round 1 for rows longer than kPass1Flat: a warp takes up to 32 of them (one
-// per lane; fewer when there are not many, so that every warp has some),
+// Round 1 for rows longer than kPass1Flat whose first chunk decided nothing: a
+// warp takes up to 32 of them (one per lane; fewer when there are not many, so
+// that every warp has some),
 // reads them one after another, 128 entries per step, stopping at the first
 // preceding neighbour, and appends the conflicting ones (all H bin: longer
 // than kPass1Flat >= m_max) with one atomic.
@@ -974,21 +1048,6 @@ __device__ __forceinline__ void prefetch_l1(const void* a) {
 // the next round, so evicted first.
 __device__ __forceinline__ void st_stream(int32_t* a, int32_t x, uint64_t pol) {
     asm volatile("st.global.L2::cache_hint.s32 [%0], %1, %2;" :: "l"(a), "r"(x), "l"(pol) : "memory");
-}
-
-// Eight consecutive entries of colidx from index a on (a multiple of eight
-// counted from the 32-byte boundary at or below colidx), with one 32-byte
-// load; where that would reach outside the array, entry by entry.
-__device__ __forceinline__ void load_chunk(const int32_t* __restrict__ colidx, int32_t nnz, int32_t a, uint64_t pol,
-                                           int32_t (&w)[8]) {
-    if (a >= 0 && a <= nnz - 8) {
-        asm volatile("ld.global.nc.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
-                     : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-                     : "l"(colidx + a), "l"(pol));
-    } else {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) w[u] = a + u >= 0 && a + u < nnz ? __ldg(colidx + a + u) : 0;
-    }
 }
 
 // L2 and L4 bins (L = 2, 4): vertices of degree <= 8 L - 7 <= 25 (and s_max),

@@ -60,3 +60,38 @@ def test_bin_edges(gcpkg, degree, keyed):
             assert (got.ncolors, got.rounds) == (want.ncolors, want.rounds), (g.name, shift, options)
             assert np.array_equal(got.colors.cpu().numpy(), want.colors)
             assert np.array_equal(got.round_sizes, want.round_sizes)
+
+
+def _reordered(g, order, seed):
+    """The same graph with the entries of every row shuffled or descending."""
+    ci = g.colidx.copy()
+    rng = np.random.default_rng(seed)
+    for v in range(g.n):
+        row = ci[g.rowptr[v]:g.rowptr[v + 1]]
+        row[:] = rng.permutation(row) if order == "shuffled" else row[::-1]
+    return ci
+
+
+@pytest.mark.parametrize("order", ["shuffled", "descending"])
+@pytest.mark.parametrize("make", [
+    lambda: _cliques(9, 3), lambda: gg.star(34, 0), lambda: gg.star(258, 257), lambda: gg.star(259, 0),
+    lambda: gg.complete(257), lambda: gg.star(5000, 0), lambda: gg.rmat(13, 8, gg.RMAT_B, 3), lambda: gg.gnm(3000, 40000, 5),
+])
+def test_rows_in_any_order(gcpkg, make, order):
+    """Round 1 looks at a row's first chunk first: rows whose only preceding neighbour comes late, at
+    every alignment, and rows longer than its limit, with index and key priority."""
+    g = make()
+    ci = _reordered(g, order, 11)
+    keys = (gg.draws(5, 3, g.n) % np.uint64(7)).astype(np.uint32)
+    rp = torch.from_numpy(g.rowptr).cuda()
+    for prio in (None, keys):
+        want = oracle.iterative(g.rowptr, ci, prio)
+        pr = None if prio is None else torch.from_numpy(prio.view(np.int32)).cuda()
+        for shift in (0, 3):
+            buf = torch.full((g.nnz + 16,), 1 << 30, dtype=torch.int32, device="cuda")
+            dev = buf[shift:shift + g.nnz]
+            dev.copy_(torch.from_numpy(ci))
+            got = gcpkg.color(rp, dev, pr, round_sizes=True)
+            assert (got.ncolors, got.rounds) == (want.ncolors, want.rounds), (g.name, order, shift)
+            assert np.array_equal(got.colors.cpu().numpy(), want.colors)
+            assert np.array_equal(got.round_sizes, want.round_sizes)
