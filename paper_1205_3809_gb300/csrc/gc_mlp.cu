@@ -358,68 +358,159 @@ __device__ __forceinline__ float mitchell_log2_1p(unsigned long long x) {
 
 __device__ __forceinline__ void write_features(float* f, int32_t d, unsigned long long sum, int32_t mx,
                                                int32_t mn) {
-    f[0] = mitchell_log2_1p((unsigned long long)d);
-    f[1] = (float)(31 - __clz(d + 1));
+    float2 x, y, z;
+    x.x = mitchell_log2_1p((unsigned long long)d);
+    x.y = (float)(31 - __clz(d + 1));
+    y = z = make_float2(0.f, 0.f);
     if (d > 0) {
-        f[2] = mitchell_log2_1p(sum / (unsigned long long)d);
-        f[3] = mitchell_log2_1p((unsigned long long)mx);
-        f[4] = mitchell_log2_1p(sum);
-        f[5] = mitchell_log2_1p((unsigned long long)mn);
+        y.x = mitchell_log2_1p(sum / (unsigned long long)d);
+        y.y = mitchell_log2_1p((unsigned long long)mx);
+        z.x = mitchell_log2_1p(sum);
+        z.y = mitchell_log2_1p((unsigned long long)mn);
+    }
+    if (((uintptr_t)f & 7u) == 0) {
+        float2* o = reinterpret_cast<float2*>(f);
+        o[0] = x;
+        o[1] = y;
+        o[2] = z;
     } else {
-        f[2] = f[3] = f[4] = f[5] = 0.f;
+        f[0] = x.x; f[1] = x.y; f[2] = y.x; f[3] = y.y; f[4] = z.x; f[5] = z.y;
     }
 }
 
-__global__ void features_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                                int32_t n, float* __restrict__ out) {
+// What the features need of a row's neighbours.
+struct RowDegrees {
+    unsigned long long sum = 0;
+    int32_t mx = 0, mn = 0x7fffffff;
+    __device__ __forceinline__ void add(int32_t d) {
+        sum += (unsigned long long)d;
+        mx = max(mx, d);
+        mn = min(mn, d);
+    }
+    // over the lanes of a group of L
+    template <int L>
+    __device__ __forceinline__ void combine() {
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        }
+    }
+};
+
+// A graph as the features read it.
+struct FeatureGraph {
+    const int32_t* __restrict__ rowptr;
+    const int32_t* __restrict__ colidx;
+    int32_t n, nnz;
+    uint32_t col_mis;  // entries from a 32-byte boundary to colidx
+
+    // (one line, most often one sector)
+    __device__ __forceinline__ int32_t degree(int32_t w) const { return __ldg(rowptr + w + 1) - __ldg(rowptr + w); }
+
+    // Lane j of a group of L: every L-th 32-byte chunk of the row [b, b + d).
+    template <int L>
+    __device__ __forceinline__ RowDegrees row(int32_t b, int32_t d, unsigned j) const {
+        RowDegrees r;
+        for (int64_t off = 8 * (int64_t)j - (int64_t)(((uint32_t)b + col_mis) & 7u); off < d; off += 8 * L) {
+            int32_t w[8];
+            const int64_t a = b + off;
+            if (a >= 0 && a + 8 <= nnz) {
+                asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                             : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
+                               "=r"(w[7])
+                             : "l"(colidx + a));
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) w[u] = a + u >= 0 && a + u < nnz ? __ldg(colidx + a + u) : 0;
+            }
+            int32_t dw[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) dw[u] = off + u >= 0 && off + u < d ? degree(w[u]) : -1;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (dw[u] >= 0) r.add(dw[u]);
+        }
+        return r;
+    }
+};
+
+// The rows of a warp's 32 vertices (one per lane), L lanes each, 32 / L side by side.
+template <int L>
+__device__ __forceinline__ void small_rows(const FeatureGraph& g, unsigned lane, int32_t b, int32_t d,
+                                           RowDegrees& mine) {
+#pragma unroll 1
+    for (unsigned s = 0; s < L; ++s) {
+        const int src = (int)((lane & ~(unsigned)(L - 1)) | s);
+        RowDegrees r = g.row<L>(__shfl_sync(0xffffffffu, b, src), __shfl_sync(0xffffffffu, d, src), lane % L);
+        r.combine<L>();
+        if (lane % L == s) mine = r;
+    }
+}
+
+// A warp takes 32 vertices.  Rows of up to 25 entries are read by 4 lanes, 8
+// rows side by side (by 2 lanes when none of the 32 is longer than 9), rows of
+// up to 121 by 16 lanes, longer ones by the whole warp, a 32-byte chunk a lane
+// at a time.
+//
+// Bound: one random L2 sector per entry (the neighbour's row starts; a probe
+// that only gathers reaches 208 G/s).  With a thread per short row and the
+// longest rows read 32 entries at a time with two waits each, R-MAT-B of 2^22
+// vertices took 446 us, now 394; R-MAT-ER 389 us, now 324 (207 G entries/s).
+// Six blocks an SM: with four (62 registers) 436 us for the first.
+__global__ void __launch_bounds__(256, 6) features_kernel(const int32_t* __restrict__ rowptr,
+                                                       const int32_t* __restrict__ colidx, int32_t n,
+                                                       float* __restrict__ out) {
+    constexpr int32_t kTiny = 8 * 2 - 7, kSmall = 8 * 4 - 7, kMid = 8 * 16 - 7;
+    FeatureGraph g;
+    g.rowptr = rowptr;
+    g.colidx = colidx;
+    g.n = n;
+    g.nnz = __ldg(rowptr + n);
+    g.col_mis = (uint32_t)((uintptr_t)colidx >> 2) & 7u;
     const unsigned lane = threadIdx.x & 31u;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t base = gw * 32; base < n; base += W * 32) {
         const int64_t v = base + lane;
         const bool valid = v < n;
-        const int32_t b = valid ? __ldg(rowptr + v) : 0, e = valid ? __ldg(rowptr + v + 1) : 0;
-        const int32_t d = e - b;
-        unsigned long long sum = 0;
-        int32_t mx = 0, mn = 0x7fffffff;
-        if (valid && d <= 32) {
-            // eight entries at a time: their ids first, then their degrees, so that a
-            // row costs two round trips per eight entries rather than per entry
-            for (int32_t i = b; i < e; i += 8) {
-                int32_t w[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) w[u] = i + u < e ? __ldg(colidx + i + u) : -1;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    if (w[u] >= 0) {
-                        const int32_t dw = __ldg(rowptr + w[u] + 1) - __ldg(rowptr + w[u]);
-                        sum += (unsigned long long)dw;
-                        mx = max(mx, dw);
-                        mn = min(mn, dw);
-                    }
-                }
-            }
-            write_features(out + v * 6, d, sum, mx, mn);
+        const int32_t b = valid ? __ldg(rowptr + v) : 0, d = valid ? __ldg(rowptr + v + 1) - b : 0;
+        RowDegrees mine;
+        if (__all_sync(0xffffffffu, d <= kTiny)) {
+            small_rows<2>(g, lane, b, d, mine);
+        } else {
+            small_rows<4>(g, lane, b, d <= kSmall ? d : 0, mine);
         }
-        unsigned big = __ballot_sync(0xffffffffu, valid && d > 32);
+        unsigned mid = __ballot_sync(0xffffffffu, d > kSmall && d <= kMid);
+        while (mid) {
+            // the lower half of the warp takes the first of them, the upper half the second
+            const unsigned rest = mid & (mid - 1);
+            const unsigned from = lane < 16u ? mid : rest;
+            const int o = __ffs(from) - 1;
+            const int32_t ob = __shfl_sync(0xffffffffu, b, o & 31), od = __shfl_sync(0xffffffffu, d, o & 31);
+            RowDegrees r = g.row<16>(ob, from ? od : 0, lane & 15u);
+            r.combine<16>();
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                RowDegrees x;
+                x.sum = __shfl_sync(0xffffffffu, r.sum, 16 * h);
+                x.mx = __shfl_sync(0xffffffffu, r.mx, 16 * h);
+                x.mn = __shfl_sync(0xffffffffu, r.mn, 16 * h);
+                const unsigned set = h == 0 ? mid : rest;
+                if (set && (int)lane == __ffs(set) - 1) mine = x;
+            }
+            mid = rest & (rest - 1);
+        }
+        unsigned big = __ballot_sync(0xffffffffu, d > kMid);
         while (big) {
-            const int j = __ffs(big) - 1;
+            const int o = __ffs(big) - 1;
             big &= big - 1;
-            const int32_t jb = __shfl_sync(0xffffffffu, b, j), je = __shfl_sync(0xffffffffu, e, j);
-            unsigned long long s2 = 0;
-            int32_t x2 = 0, n2 = 0x7fffffff;
-            for (int32_t i = jb + (int32_t)lane; i < je; i += 32) {
-                const int32_t w = __ldg(colidx + i);
-                const int32_t dw = __ldg(rowptr + w + 1) - __ldg(rowptr + w);
-                s2 += (unsigned long long)dw;
-                x2 = max(x2, dw);
-                n2 = min(n2, dw);
-            }
-            for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-            x2 = __reduce_max_sync(0xffffffffu, x2);
-            n2 = __reduce_min_sync(0xffffffffu, n2);
-            if ((int)lane == j) write_features(out + v * 6, d, s2, x2, n2);
+            RowDegrees r = g.row<32>(__shfl_sync(0xffffffffu, b, o), __shfl_sync(0xffffffffu, d, o), lane);
+            r.combine<32>();
+            if ((int)lane == o) mine = r;
         }
+        if (valid) write_features(out + v * 6, d, mine.sum, mine.mx, mine.mn);
     }
 }
 

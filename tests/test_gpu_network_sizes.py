@@ -51,3 +51,32 @@ def test_gradient_sizes(gcpkg, n):
     # the bound of test_gpu_learned.test_grad_matches_oracle: fp32 sums of n terms in another order
     assert np.all(np.abs(got - want) <= 1e-4 * np.abs(want).max() + 1e-5 * np.abs(want)), np.abs(got - want).max()
     assert abs(float(sse.item()) - want_sse) <= 1e-4 * want_sse + 1e-6
+
+
+def _rows_of(degree, seed):
+    """Vertices of exactly `degree` neighbours (stars), among a sparse random graph, ids shuffled."""
+    parts, n = [], 0
+    for _ in range(3):
+        parts.append((np.full(degree, n), n + 1 + np.arange(degree)))
+        n += degree + 1
+    g = gg.gnm(300, 700, seed)
+    parts.append((np.repeat(np.arange(g.n), g.degrees) + n, g.colidx.astype(np.int64) + n))
+    n += g.n
+    perm = gg.permutation(n, seed)
+    u, v = (np.concatenate([p[i] for p in parts]) for i in (0, 1))
+    return gg.from_edges(n, perm[u], perm[v])
+
+
+# rows read by 4 lanes (up to 25), 16 lanes (up to 121) or the warp, at every alignment of both arrays
+@pytest.mark.parametrize("degree", [1, 8, 25, 26, 57, 120, 121, 122, 255, 257, 1000])
+def test_feature_rows(gcpkg, degree):
+    g = _rows_of(degree, 40 + degree)
+    want = L.features(g.rowptr, g.colidx)
+    for shift in range(8):
+        rp = torch.full((g.n + 16,), -5, dtype=torch.int32, device="cuda")[shift % 4:][:g.n + 1]
+        ci = torch.full((g.nnz + 16,), 1 << 30, dtype=torch.int32, device="cuda")[shift:][:g.nnz]
+        rp.copy_(torch.from_numpy(g.rowptr))
+        ci.copy_(torch.from_numpy(g.colidx))
+        out = torch.empty(g.n * 6 + 1, dtype=torch.float32, device="cuda")[shift % 2:][:g.n * 6].view(g.n, 6)
+        got = gcpkg.features(rp, ci, out=out).cpu().numpy()
+        assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), (degree, shift)
