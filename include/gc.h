@@ -220,7 +220,8 @@ const char* gc_strerror(int code);
 /* The CUDA error code (cudaError_t) behind the last GC_ERR_CUDA, or 0. */
 int gc_last_cuda_error(void);
 
-/* Free the workspace of every device this process used.  Returns GC_OK. */
+/* Free the workspace of every device this process used, and the memory (at
+ * most 256 MiB per device) kept from destroyed batch plans.  Returns GC_OK. */
 int gc_release(void);
 
 /* Bytes of device workspace currently held on the current device. */

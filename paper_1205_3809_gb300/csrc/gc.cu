@@ -170,6 +170,71 @@ int ensure_device_limited(void** p, size_t* have, size_t need, int32_t limit_mb)
     return ensure_device(p, have, need);
 }
 
+// Device memory of batch plans.  A plan made, run and freed in one call (or one
+// per batch of work) would otherwise spend more time in cudaMalloc and cudaFree,
+// which also wait for the whole device, than in its kernels.  It comes from a
+// pool of its own per device that keeps at most kPlanPoolKeep bytes of freed
+// memory and gives them back in gc_release.  Both calls wait for the pool's
+// (otherwise idle) stream: memory handed out may be used on any stream, and
+// memory handed back must no longer be in use.
+constexpr size_t kPlanPoolKeep = 256ull << 20;
+struct PlanPool {
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t stream = nullptr;
+};
+std::mutex g_pool_mu;
+std::map<int, PlanPool> g_pools;
+
+cudaError_t plan_alloc(void** p, size_t bytes) {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    *p = nullptr;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    PlanPool& pp = g_pools[dev];
+    if (!pp.pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        e = cudaMemPoolCreate(&pool, &props);
+        if (e != cudaSuccess) return e;
+        uint64_t keep = kPlanPoolKeep;
+        e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&pp.stream, cudaStreamNonBlocking);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(pool);
+            return e;
+        }
+        pp.pool = pool;
+    }
+    e = cudaMallocFromPoolAsync(p, bytes, pp.pool, pp.stream);
+    if (e == cudaSuccess) {
+        e = cudaStreamSynchronize(pp.stream);
+        if (e != cudaSuccess) *p = nullptr;
+    }
+    return e;
+}
+
+void plan_free(void* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    PlanPool& pp = g_pools[dev];
+    cudaFreeAsync(p, pp.stream);
+    cudaStreamSynchronize(pp.stream);
+}
+
+void plan_pools_trim() {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    for (auto& kv : g_pools) {
+        cudaSetDevice(kv.first);
+        if (kv.second.pool) cudaMemPoolTrimTo(kv.second.pool, 0);
+    }
+}
+
 struct Layout {
     size_t st, rs, rv, rt, x0, x1, act0, act1, stat, hubs, defer;
     size_t L2[2], L4[2], L8[2], L16[2], S[2], M[2], H[2], Hc[2], O[2];
@@ -819,6 +884,7 @@ struct gc_batch {
     size_t ws_bytes = 0;
     size_t off_voff = 0, off_eoff = 0, off_rowptr = 0, off_colidx = 0, off_settle = 0, off_flags = 0;
     int64_t launches_per_run = 0;
+    bool idle = false;        // nothing of the plan can be running (no wait before it is freed)
     // 1: all graphs share the rounds kernel's grid; 2: one thread block per graph
     int mode = 1;
     uint32_t local_smem = 0;  // mode 2: dynamic shared memory per block
@@ -849,7 +915,7 @@ int union_colidx(gc_batch& b, int32_t** out) {
         return GC_OK;
     }
     if (!b.ucolidx) {
-        const cudaError_t e = cudaMalloc(&b.ucolidx, (size_t)std::max<int64_t>(b.NNZ, 1) * 4);
+        const cudaError_t e = plan_alloc((void**)&b.ucolidx, (size_t)std::max<int64_t>(b.NNZ, 1) * 4);
         if (e != cudaSuccess) {
             (void)cudaGetLastError();
             b.ucolidx = nullptr;
@@ -1060,11 +1126,12 @@ void batch_free(gc_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-    if (b->ws || b->ucolidx || b->big_ws) cudaDeviceSynchronize();
+    if ((b->ws || b->ucolidx || b->big_ws) && !b->idle) cudaDeviceSynchronize();
+    if (b->big) b->big->idle = true;
     batch_free(b->big);
-    if (b->big_ws) cudaFree(b->big_ws);
-    if (b->ws) cudaFree(b->ws);
-    if (b->ucolidx) cudaFree(b->ucolidx);
+    plan_free(b->big_ws);
+    plan_free(b->ws);
+    plan_free(b->ucolidx);
     cudaSetDevice(cur);
     (void)cudaGetLastError();
     delete b;
@@ -1155,7 +1222,7 @@ int batch_plan_big(gc_batch* b, const std::vector<int32_t>& order, int32_t nbig,
     b->off_big_colors = take((size_t)n * 4);
     b->off_big_prio = b->prio ? take((size_t)n * 4) : 0;
     if (b->o.workspace_limit_mb > 0 && off > ((size_t)b->o.workspace_limit_mb << 20)) return GC_OK;
-    if (cudaMalloc(&b->big_ws, off) != cudaSuccess) {
+    if (plan_alloc(&b->big_ws, off) != cudaSuccess) {
         (void)cudaGetLastError();
         b->big_ws = nullptr;
         return GC_OK;
@@ -1184,7 +1251,7 @@ int batch_plan_big(gc_batch* b, const std::vector<int32_t>& order, int32_t nbig,
     if (rc != GC_OK) {
         batch_free(big);
         if (rc != GC_ERR_OOM) return rc;
-        cudaFree(b->big_ws);
+        plan_free(b->big_ws);
         b->big_ws = nullptr;
         b->big_ws_bytes = 0;
         return GC_OK;
@@ -1246,10 +1313,10 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     const size_t h_stats = take(sizeof(Stats));
     const size_t head = off;
     void* tmp = nullptr;
-    GC_CUDA(cudaMalloc(&tmp, head));
+    GC_CUDA(plan_alloc(&tmp, head));
     auto fail = [&](int code) {
         cudaStreamSynchronize(s);
-        cudaFree(tmp);
+        plan_free(tmp);
         return code;
     };
     char* hb = (char*)tmp;
@@ -1331,7 +1398,7 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
         void* ws = nullptr;
         if (b->o.workspace_limit_mb > 0 && b->ws_bytes > ((size_t)b->o.workspace_limit_mb << 20))
             return fail(GC_ERR_OOM);
-        const cudaError_t e = cudaMalloc(&ws, b->ws_bytes);
+        const cudaError_t e = plan_alloc(&ws, b->ws_bytes);
         if (e != cudaSuccess) {
             (void)cudaGetLastError();
             return fail(e == cudaErrorMemoryAllocation ? GC_ERR_OOM : GC_ERR_CUDA);
@@ -1365,7 +1432,7 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
         void* ws = nullptr;
         if (b->o.workspace_limit_mb > 0 && b->ws_bytes > ((size_t)b->o.workspace_limit_mb << 20))
             return fail(GC_ERR_OOM);
-        const cudaError_t e = cudaMalloc(&ws, b->ws_bytes);
+        const cudaError_t e = plan_alloc(&ws, b->ws_bytes);
         if (e != cudaSuccess) {
             (void)cudaGetLastError();
             return fail(e == cudaErrorMemoryAllocation ? GC_ERR_OOM : GC_ERR_CUDA);
@@ -1613,6 +1680,7 @@ int gc_release(void) {
         if (kv.second.copy) cudaStreamDestroy(kv.second.copy);
     }
     g_cache.clear();
+    plan_pools_trim();
     g_last.valid = 0;
     cudaSetDevice(cur);
     (void)cudaGetLastError();
@@ -1689,7 +1757,7 @@ int gc_batch_round_stats(gc_batch* plan, int32_t* sizes, int64_t* volumes, int32
         const int32_t bins = std::max(1, hb.rounds);
         big.assign((size_t)bins * 2, 0ull);
         unsigned long long* d = nullptr;
-        GC_CUDA(cudaMalloc(&d, big.size() * 8));
+        GC_CUDA(plan_alloc((void**)&d, big.size() * 8));
         cudaError_t e = cudaMemsetAsync(d, 0, big.size() * 8, s);
         if (e == cudaSuccess) {
             gc::settle_histogram_kernel<<<b.sms * 2, 256, 0, s>>>((const int32_t*)(bb + b.big->off_rowptr),
@@ -1699,7 +1767,7 @@ int gc_batch_round_stats(gc_batch* plan, int32_t* sizes, int64_t* volumes, int32
         }
         if (e == cudaSuccess) e = cudaMemcpyAsync(big.data(), d, big.size() * 8, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        cudaFree(d);
+        plan_free(d);
         GC_CUDA(e);
     }
     const int32_t m = (int32_t)std::min<int64_t>({(int64_t)rounds, (int64_t)cap, b.round_cap});
@@ -1790,7 +1858,10 @@ int gc_color_batched(const int64_t* vertex_offsets, const int64_t* edge_offsets,
                              ncolors_out, rounds_out, opt, stream, &plan);
     if (rc != GC_OK) return rc;
     rc = gc_batch_run(plan, stream);
-    if (rc == GC_OK) rc = gc_batch_status(plan, stream, nullptr, nullptr);
+    if (rc == GC_OK) {
+        rc = gc_batch_status(plan, stream, nullptr, nullptr);
+        plan->idle = rc != GC_ERR_CUDA;  // the status waits for the run
+    }
     gc_batch_destroy(plan);
     return rc;
 }

@@ -373,3 +373,39 @@ def test_largest_graphs_split_off(gcpkg, keyed, large):
     lim = gcpkg.Batch(_dev(rp), _dev(ci), voff, eoff, options={"workspace_limit_mb": (room >> 20) + 1})
     lim.run()
     assert lim.mode == 2 and lim.launch_count == 2 and lim.workspace_bytes == room
+
+
+def test_plan_memory_is_shared_safely_and_given_back(gcpkg):
+    """Plans made, run and freed in one call by several threads, each on its own stream, share a
+    pool of device memory: every result is its own batch's, and the pool is empty after release()."""
+    import threading
+    gcpkg.release()
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    batches = [gg.batch_mix(12 + 5 * i, 50 + i, n_min=1, n_max=2000) for i in range(4)]
+    wrong = []
+
+    def work(i):
+        gs = batches[i]
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            rp, ci, voff, eoff = gcpkg.pack_batch((g.rowptr, g.colidx) for g in gs)
+            rp, ci = _dev(rp), _dev(ci)
+            for _ in range(6):
+                colors, nc, rd = gcpkg.color_batched(rp, ci, voff, eoff)
+                got = colors.cpu().numpy()
+                for k, g in enumerate(gs):
+                    if not np.array_equal(got[voff[k]:voff[k + 1]], want[i][k]):
+                        wrong.append((i, k))
+
+    want = [[oracle.iterative(g.rowptr, g.colidx).colors for g in gs] for gs in batches]
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+    gcpkg.release()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
