@@ -280,11 +280,11 @@ Layout make_layout(int64_t n, int64_t nnz, size_t elem, const Stats& hs, int64_t
     return L;
 }
 
-// A call's pointers into its workspace (p.s_max and p.m_max are set).
+// A call's pointers into its workspace (p.s_max, p.m_max and p.prio are set).
 template <typename T>
 void fill_workspace(Params<T>& p, char* base, const Layout& L, RoundState* st, int64_t round_cap) {
-    p.lim2 = gc::tiny_limit(2, p.s_max);
-    p.lim4 = gc::tiny_limit(4, p.s_max);
+    p.lim2 = gc::tiny_limit(2, p.s_max, p.prio != nullptr);
+    p.lim4 = gc::tiny_limit(4, p.s_max, p.prio != nullptr);
     p.lim8 = gc::mid_limit(8, p.s_max, p.m_max);
     p.lim16 = gc::mid_limit(16, p.s_max, p.m_max);
     p.X0 = (T*)(base + L.x0);
@@ -528,7 +528,7 @@ int normalise(const gc_options* opt, gc_options* o) {
 
 // The setup scan (Stats at the head of the workspace) and, when asked for, the
 // checks of every entry behind it, with one wait for both.
-int scan_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, int32_t s_max, int32_t m_max, bool validate,
+int scan_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, int32_t s_max, int32_t m_max, bool keyed, bool validate,
                 const HostInput* hin, bool timed, cudaStream_t s, DeviceCache& dc, int64_t* launches, Stats* hs) {
     constexpr size_t kOut = 1024, kHead = 2048;
     static_assert(sizeof(Stats) <= kOut && sizeof(gc::ValidateOut) <= kHead - kOut, "workspace head");
@@ -536,7 +536,7 @@ int scan_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, int32_t
     gc::ValidateOut* out = (gc::ValidateOut*)((char*)dc.ws + kOut);
     GC_CUDA(cudaMemsetAsync(dc.ws, 0, kHead, s));
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)dc.sms * 8));
-    gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, s_max, m_max, stats);
+    gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, s_max, m_max, keyed, stats);
     GC_CUDA(cudaGetLastError());
     *launches += 1;
     if (validate) {
@@ -567,7 +567,8 @@ int validate_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, cud
     rc = ensure_host(&dc.host, &dc.host_bytes, 4096);
     if (rc != GC_OK) return rc;
     Stats hs;
-    return scan_locked(rowptr, colidx, n, gc::kSmallMaxLimit, gc::kMedMaxLimit, true, nullptr, false, s, dc, launches, &hs);
+    return scan_locked(rowptr, colidx, n, gc::kSmallMaxLimit, gc::kMedMaxLimit, false, true, nullptr, false, s, dc,
+                       launches, &hs);
 }
 
 int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const uint32_t* priority,
@@ -613,7 +614,7 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
     Stats hs;
     {
         NvtxRange range("gc setup scan");
-        rc = scan_locked(rowptr, colidx, n, o.small_max_degree, o.medium_max_degree, o.validate != 0, hin,
+        rc = scan_locked(rowptr, colidx, n, o.small_max_degree, o.medium_max_degree, priority != nullptr, o.validate != 0, hin,
                          o.telemetry != 0, s, dc, &launches, &hs);
         if (rc != GC_OK) return rc;
     }
@@ -782,7 +783,8 @@ int color_noalloc_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n
         Stats* stats = (Stats*)base;
         GC_CUDA(cudaMemsetAsync(stats, 0, sizeof(Stats), s));
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)n + 255) / 256, (int64_t)nd->sms * 8));
-        gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, o.small_max_degree, o.medium_max_degree, stats);
+        gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, o.small_max_degree, o.medium_max_degree, priority != nullptr,
+                                              stats);
         GC_CUDA(cudaGetLastError());
         GC_CUDA(cudaMemcpyAsync(&hs, stats, sizeof(Stats), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
@@ -1331,7 +1333,7 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
                                                      (const int64_t*)(hb + h_eoff), G, N,
                                                      (int32_t*)(hb + h_rowptr), (gc::BatchFlags*)(hb + h_flags));
         gc::stats_kernel<<<grid, 256, 0, s>>>((const int32_t*)(hb + h_rowptr), (int32_t)N,
-                                              b->o.small_max_degree, b->o.medium_max_degree,
+                                              b->o.small_max_degree, b->o.medium_max_degree, prio != nullptr,
                                               (Stats*)(hb + h_stats));
         if (cudaGetLastError() != cudaSuccess) return fail(GC_ERR_CUDA);
     }

@@ -88,9 +88,12 @@ constexpr int kShortPerTaskMin = 4;            // S-bin vertices per task in a s
 constexpr int kMidSteps = 8;                  // L8, L16: steps of 32 / L vertices per task, at most
 
 // L2 and L4 bins: degrees up to s_max whose row fits L chunks of eight entries
-// wherever it starts: 8 L - 7.
-__host__ __device__ __forceinline__ int32_t tiny_limit(int L, int32_t s_max) {
-    return s_max < 8 * L - 7 ? s_max : 8 * L - 7;
+// wherever it starts (8 L - 7), and, with a priority array, whose state fits the
+// worklist entry: a live and a precedence bit per entry and the colors 1..22.
+constexpr int kKeyedBits = 21;
+__host__ __device__ __forceinline__ int32_t tiny_limit(int L, int32_t s_max, bool keyed) {
+    const int32_t fits = 8 * L - 7 < kKeyedBits || !keyed ? 8 * L - 7 : kKeyedBits;
+    return s_max < fits ? s_max : fits;
 }
 
 // L8 and L16 bins: degrees above that (and up to m_max) whose row fits L chunks
@@ -546,11 +549,11 @@ __device__ __forceinline__ void fold_volume(RoundState* st, unsigned long long* 
 
 // Degree statistics: max degree, list capacities, hub chunks, rowptr checks.
 __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int32_t s_max,
-                             int32_t m_max, Stats* s) {
+                             int32_t m_max, bool keyed, Stats* s) {
     int mx = 0, bad = 0;
     unsigned c0 = 0, c1 = 0, c2 = 0, df = 0, o2 = 0, o8 = 0, o16 = 0;
     unsigned long long ch = 0;
-    const int32_t tiny2 = tiny_limit(2, s_max), tiny4 = tiny_limit(4, s_max), mid8 = mid_limit(8, s_max, m_max), mid16 = mid_limit(16, s_max, m_max);
+    const int32_t tiny2 = tiny_limit(2, s_max, keyed), tiny4 = tiny_limit(4, s_max, keyed), mid8 = mid_limit(8, s_max, m_max), mid16 = mid_limit(16, s_max, m_max);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int32_t d = __ldg(rowptr + v + 1) - __ldg(rowptr + v);
@@ -1050,12 +1053,30 @@ __device__ __forceinline__ void st_stream(int32_t* a, int32_t x, uint64_t pol) {
     asm volatile("st.global.L2::cache_hint.s32 [%0], %1, %2;" :: "l"(a), "r"(x), "l"(pol) : "memory");
 }
 
+// The state of an L2 or L4 entry in its last two words.  With a priority array
+// the rows have at most kKeyedBits = 21 entries, so that the live bits, the
+// precedence bits and the mask of the colors 1..22 fill the 64 bits.
+template <bool P>
+struct TinyState {
+    uint32_t live, prec, stat;
+    __device__ __forceinline__ static TinyState of(int4 e) {
+        const uint32_t z = (uint32_t)e.z, w = (uint32_t)e.w;
+        if constexpr (!P) return {z, 0u, w};
+        return {z & ((1u << kKeyedBits) - 1u), (z >> kKeyedBits) | ((w & 0x3ffu) << 11), w >> 10};
+    }
+    __device__ __forceinline__ int4 entry(int32_t v, int32_t b) const {
+        if constexpr (!P) return make_int4(v, b, (int32_t)live, (int32_t)stat);
+        return make_int4(v, b, (int32_t)(live | prec << kKeyedBits), (int32_t)(prec >> 11 | stat << 10));
+    }
+};
+
 // L2 and L4 bins (L = 2, 4): vertices of degree <= 8 L - 7 <= 25 (and s_max),
 // whose first fit is at most 26, so one 32-bit word holds every color that matters to them and one more says
 // which entries of the row are still live (the neighbour had not settled when
 // last read).  Both travel in the worklist entry {v, row start, live, static
-// mask}; the row itself is read from colidx in every round and no list is
-// written.
+// mask}, with a priority array beside one bit per entry for "precedes v"
+// (TinyState); the row itself is read from colidx in every round and no list
+// is written.
 //
 // L lanes share a vertex: each takes a 32-byte chunk of the row (one load for
 // eight entries; a row of 8 L - 7 spans at most L), gathers the colors of the live entries, and ORs
@@ -1080,13 +1101,11 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
     const uint32_t mis = (uint32_t)((uintptr_t)p.colidx >> 2) & 7u;  // entries from a 32-byte boundary to colidx
     const bool valid = en.x >= 0;
     const int32_t my_v = valid ? en.x : 0;
-    const uint32_t my_live = valid ? (uint32_t)en.z : 0u;
+    const TinyState<P> my = TinyState<P>::of(valid ? en : make_int4(0, 0, 0, 0));
+    const uint32_t my_live = my.live;
     const uint32_t my_cv = valid ? word_color(ld_color(io.Xc + my_v, io.pol_col)) : 0u;
     // which entries precede v (bit i: entry i), worked out in round 2; there: v's key
-    uint32_t my_prec = 0u;
-    if constexpr (P) {
-        if (valid) my_prec = io.first ? __ldg(p.prio + my_v) : __ldcg(p.stat + (size_t)my_v * 8);
-    }
+    const uint32_t my_prec = P && io.first ? (valid ? __ldg(p.prio + my_v) : 0u) : my.prec;
     uint32_t my_all = 0u, my_stat = 0u, my_dead = 0u, my_new_prec = 0u;
     bool my_conflict = false;
 #pragma unroll 1
@@ -1152,18 +1171,18 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
         }
     }
     const bool go = valid && my_conflict;
-    const uint32_t stat = (uint32_t)en.w | my_stat;
-    const uint32_t live = my_live & ~my_dead;
+    TinyState<P> now;
+    now.live = my_live & ~my_dead;
+    now.prec = P && io.first ? my_new_prec : my.prec;
+    now.stat = my.stat | (P ? my_stat & ((1u << (kKeyedBits + 1)) - 1u) : my_stat);  // (first fit is at most 22)
     if (go) {
-        const uint32_t taken = stat | my_all;
-        recolor(p, io, my_v, (uint32_t)__ffs(~taken));
-        vol += (unsigned)__popc(live);
-        if (P && io.first) p.stat[(size_t)my_v * 8] = my_new_prec;
+        recolor(p, io, my_v, (uint32_t)__ffs(~(now.stat | my_all)));
+        vol += (unsigned)__popc(now.live);
     } else if (valid) {
         settle(p, io, my_v, my_cv);
         maxc = max(maxc, (int)my_cv);
     }
-    warp_append_pair<(L == 2 ? 0 : 32)>(go, make_int4(my_v, en.y, (int32_t)live, (int32_t)stat),
+    warp_append_pair<(L == 2 ? 0 : 32)>(go, now.entry(my_v, en.y),
                                         L == 2 ? io.next.L2 : io.next.L4, &io.next.cnt->tiny);
 }
 
@@ -1172,9 +1191,9 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
 // vertices side by side, no list written.  Their first fit is at most
 // 8 L - 6, so W = L / 4 words hold the colors that matter.  The static mask
 // (words 0..W-1) and one byte of live entries per chunk (after it) share the
-// vertex's 32 bytes of p.stat; with a priority array, one byte per chunk of
-// p.act0's part of the row (which no list of this vertex uses) says which
-// entries precede v.
+// vertex's 32 bytes of p.stat; with a priority array, one byte more per chunk
+// says which entries precede v (L8: after the live bytes; L16: in p.act0's part
+// of the row, which no list of this vertex uses).
 //
 // Bound: as for T rows, one random L2 sector per live entry.  A warp per
 // vertex (the M bin, which these rows took before) leaves most of its lanes
@@ -1210,7 +1229,7 @@ __device__ __forceinline__ void mid_task(const Params<T>& p, const PassIO<T>& io
         const int32_t off = 8 * (int32_t)j - (int32_t)(((uint32_t)b + mis) & 7u);
         uint32_t* const st = p.stat + (size_t)v * 8;
         uint8_t* const live_at = reinterpret_cast<uint8_t*>(st + W) + j;
-        uint8_t* const prec_at = reinterpret_cast<uint8_t*>(p.act0 + b) + j;
+        uint8_t* const prec_at = (L == 8 ? reinterpret_cast<uint8_t*>(st + 2 * W) : reinterpret_cast<uint8_t*>(p.act0 + b)) + j;
         uint32_t live, old = 0u, prec = 0u;
         if (first) {
             live = low_bits(max(0, min(8, d - off))) & (off < 0 ? 0xffu << -off : 0xffu);

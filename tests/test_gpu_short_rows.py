@@ -43,7 +43,7 @@ def _cliques(degree, seed):
     return gg.from_edges(n, perm[us], perm[vs], name=f"cliques({degree})")
 
 
-@pytest.mark.parametrize("degree", [1, 7, 8, 9, 10, 24, 25, 26, 31, 32, 33, 56, 57, 58, 63, 120, 121, 122])
+@pytest.mark.parametrize("degree", [1, 7, 8, 9, 10, 20, 21, 22, 24, 25, 26, 31, 32, 33, 56, 57, 58, 63, 120, 121, 122])
 @pytest.mark.parametrize("keyed", [False, True])
 def test_bin_edges(gcpkg, degree, keyed):
     g = _cliques(degree, 100 + degree)
