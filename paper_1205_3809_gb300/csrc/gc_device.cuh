@@ -16,16 +16,17 @@
 // start at 0), so pass 1 needs no color reads: v conflicts iff some
 // neighbour precedes it, and then its round-2 color is 2.
 //
-// Active lists.  A color word carries a flag bit once its vertex has settled
-// (its color is final).  A vertex v still in U reads each neighbour's word
-// anyway (the conflict test and first fit need this round's color), and a
-// flagged neighbour is then folded into v's static mask (the colors 1..256
-// held by settled neighbours, kept per vertex across rounds) and dropped
-// from v's active list, which pass k rewrites compacted into the other of
-// two buffers.  Later rounds read only the neighbours that had not settled,
-// plus v's static mask; first fit looks at static | this round's colors.  A
-// first fit beyond 256 rescans the original row (every neighbour).  The
-// flag makes 16-bit state hold colors < 2^15: a larger color sets an
+// Active neighbours.  A color word carries a flag bit once its vertex has
+// settled (its color is final).  A vertex v still in U reads each neighbour's
+// word anyway (the conflict test and first fit need this round's color), and
+// a flagged neighbour is then folded into v's static mask (the colors held by
+// settled neighbours, kept per vertex across rounds) and dropped: later rounds
+// read only the neighbours that had not settled, plus v's static mask; first
+// fit looks at static | this round's colors.  Rows of up to 121 entries drop a
+// neighbour by clearing its bit; longer rows keep an active list, which pass k
+// rewrites compacted into the other of two buffers, and a mask of the colors
+// 1..256 (a first fit beyond 256 rescans the original row, every neighbour).
+// The flag makes 16-bit state hold colors < 2^15: a larger color sets an
 // overflow status and the host reruns with 32-bit state.
 //
 // Work is split into warp-sized tasks, binned by degree (L2 to L16) or by the
@@ -51,8 +52,8 @@
 //
 // Priority: the round kernels are instantiated for index priority (the test
 // is one compare) and for a priority array, whose (key, index) order round 2
-// evaluates once per kept neighbour and stores in bit 31 of the active-list
-// entry.  Loops: all rounds in one cooperative launch with a bounded grid
+// evaluates once per kept neighbour and stores in a bit mask (rows read from
+// the graph) or in bit 31 of the active-list entry.  Loops: all rounds in one cooperative launch with a bounded grid
 // barrier (optionally handing the last rounds to block 0), one launch per
 // round, or a CUDA graph whose while node repeats a round kernel and a
 // one-thread condition kernel.
@@ -329,17 +330,6 @@ __device__ __forceinline__ void warp_append_pair(bool flag, int4 e, int4* list, 
     if (lane == 0) base = (unsigned)(atomicAdd(cnt, (unsigned long long)__popc(ballot) << SHIFT) >> SHIFT);
     base = __shfl_sync(kFull, base, 0);
     if (flag) list[base + __popc(ballot & ((1u << lane) - 1u))] = e;
-}
-
-__device__ __forceinline__ void warp_append_i32(bool flag, int32_t v, int32_t* list, unsigned* cnt) {
-    const unsigned ballot = __ballot_sync(kFull, flag);
-    if (ballot == 0) return;
-    const unsigned lane = lane_id();
-    const int leader = __ffs(ballot) - 1;
-    unsigned base = 0;
-    if ((int)lane == leader) base = atomicAdd(cnt, (unsigned)__popc(ballot));
-    base = __shfl_sync(kFull, base, leader);
-    if (flag) list[base + __popc(ballot & ((1u << lane) - 1u))] = v;
 }
 
 // Where the next round's worklists go.
@@ -1187,7 +1177,7 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
 }
 
 // L8 and L16 bins (L = 8, 16): longer rows of degree d <= 8 L - 7, read
-// like T rows: L lanes share a vertex, one 32-byte chunk of colidx each, 32 / L
+// like the short rows: L lanes share a vertex, one 32-byte chunk of colidx each, 32 / L
 // vertices side by side, no list written.  Their first fit is at most
 // 8 L - 6, so W = L / 4 words hold the colors that matter.  The static mask
 // (words 0..W-1) and one byte of live entries per chunk (after it) share the
@@ -1195,7 +1185,7 @@ __device__ __forceinline__ void tiny_task(const Params<T>& p, const PassIO<T>& i
 // says which entries precede v (L8: after the live bytes; L16: in p.act0's part
 // of the row, which no list of this vertex uses).
 //
-// Bound: as for T rows, one random L2 sector per live entry.  A warp per
+// Bound: as for the short rows, one random L2 sector per live entry.  A warp per
 // vertex (the M bin, which these rows took before) leaves most of its lanes
 // without an entry on a list of 33..64 and repeats its per-vertex work 32
 // wide: 98 G entries/s on rows of 48 and 158 on rows of 96, against 214 and
