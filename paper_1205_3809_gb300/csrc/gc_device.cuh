@@ -490,7 +490,7 @@ __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" 
 // never reset and waits until all of them have: one round trip to L2 to
 // arrive and one to see the last arrival.  (With a reset count, a generation
 // word and the status read behind them, a round of nearly no work took 6.4 us
-// of which this barrier was most; now GC_ROUND_US.)
+// of which this barrier was most; now 4.5 us.)
 __device__ __forceinline__ bool grid_barrier(RoundState* st, unsigned max_polls, unsigned passed) {
     __shared__ int s_ok;
     __syncthreads();
@@ -1311,8 +1311,13 @@ __device__ __forceinline__ void mid_task(const Params<T>& p, const PassIO<T>& io
 // its vertex's window in shared memory, flags a conflict, and, if the
 // neighbour has not settled, is copied to the next round's list at the
 // vertex's running write position.  Afterwards each lane decides its own
-// vertex.
-template <typename T, bool P>  // P: a priority array is given
+// vertex.  Round 2 with keys (F: keys are compared and kept as a bit of the
+// entry) is an instance of its own here and in the two functions that
+// follow; the later rounds then run without its branches, which matters
+// where most entries stand in lists: with keys by features and R-MAT-B at
+// 4M vertices 10.63 ms in one instance, 10.35 ms in two; short-row graphs
+// (G(1M, 8M), R-MAT-G at 8M) are unchanged.
+template <typename T, bool P, bool F>  // P: a priority array is given; F: and this is round 2
 __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& io, int4 en,
                                           FlatSmem& sm, int& maxc, unsigned& vol) {
     const unsigned lane = lane_id();
@@ -1393,8 +1398,8 @@ __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& i
             bool pre = false;
             if constexpr (!P) {
                 if (in && col == ocv) pre = wid < sm.vid[o];
-            } else if (in && (col == ocv || (io.first && !settled))) {
-                if (io.first) {
+            } else if (in && (col == ocv || (F && !settled))) {
+                if constexpr (F) {
                     const int32_t ov = sm.vid[o];
                     pre = precedes(p.prio, wid, ov, __ldg(p.prio + ov));
                 } else {
@@ -1414,7 +1419,7 @@ __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& i
             const unsigned below = kb & ((1u << lane) - 1u) & ~((1u << seglo[u]) - 1u);
             if (keep)
                 st_stream(io.rout + wbase + __popc(below),
-                          (P && io.first) ? (int32_t)((uint32_t)wid | (pre ? kPrecBit : 0u)) : w[u],
+                          F ? (int32_t)((uint32_t)wid | (pre ? kPrecBit : 0u)) : w[u],
                           io.pol_row);
             // my vertex's lanes in this batch: [lo, hi)
             const int32_t lo = max(0, min(32, off - base));
@@ -1478,7 +1483,7 @@ __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& i
 // long list.  The decisions stay in the lane of their entry, and the task
 // appends its conflicting vertices to the next round with one atomic per
 // bin.
-template <typename T, bool P>  // P: a priority array is given
+template <typename T, bool P, bool F>  // P: a priority array is given; F: and this is round 2
 __device__ __forceinline__ void vertex_task(const Params<T>& p, const PassIO<T>& io, int4 en,
                                             FlatSmem& sm, int& maxc, unsigned& vol) {
     constexpr int kB = 4;  // batches in flight
@@ -1502,7 +1507,7 @@ __device__ __forceinline__ void vertex_task(const Params<T>& p, const PassIO<T>&
             else if (lane == 8u) prefetch_l1(io.rin + bn + ln - 1);
         }
         const uint32_t cv = word_color(ld_color(io.Xc + v, io.pol_col));
-        const uint32_t pv = (P && first) ? __ldg(p.prio + v) : 0u;
+        const uint32_t pv = F ? __ldg(p.prio + v) : 0u;
         // v's static mask, word `lane` (read now, used after the list)
         const uint32_t old = (lane < 8u && !first) ? __ldcg(p.stat + (size_t)v * 8 + lane) : 0u;
         if (lane < 8u) { sm.dyn[lane] = 0u; sm.stat[lane] = 0u; }
@@ -1533,9 +1538,9 @@ __device__ __forceinline__ void vertex_task(const Params<T>& p, const PassIO<T>&
                 bool pre = false;
                 if constexpr (!P) {
                     pre = in && col == cv && wid < v;
-                } else if (in && (col == cv || (first && !settled))) {
-                    pre = first ? precedes(p.prio, wid, v, pv) : w[u] < 0;
-                    if (first) w[u] = (int32_t)((uint32_t)wid | (pre ? kPrecBit : 0u));  // the entry kept
+                } else if (in && (col == cv || (F && !settled))) {
+                    pre = F ? precedes(p.prio, wid, v, pv) : w[u] < 0;
+                    if (F) w[u] = (int32_t)((uint32_t)wid | (pre ? kPrecBit : 0u));  // the entry kept
                 }
                 if (in) {
                     if (col == cv && pre) conflict = true;
@@ -1602,7 +1607,7 @@ __device__ __forceinline__ void vertex_task(const Params<T>& p, const PassIO<T>&
 // vertex whose active list fits one chunk is decided by this warp at once;
 // otherwise the chunks OR their results into the vertex's record, and the
 // warp that completes the last chunk decides it and clears the record.
-template <typename T, bool P>  // P: a priority array is given
+template <typename T, bool P, bool F>  // P: a priority array is given; F: and this is round 2
 __device__ __forceinline__ void hub_chunk(const Params<T>& p, const PassIO<T>& io, TaskHead h,
                                           FlatSmem& sm, int& maxc, unsigned& vol) {
     constexpr int kHalf = kPerLane / 2;
@@ -1613,7 +1618,7 @@ __device__ __forceinline__ void hub_chunk(const Params<T>& p, const PassIO<T>& i
     const unsigned nch = (unsigned)(len + kChunk - 1) / kChunk;
     const bool single = nch == 1;
     const uint32_t cv = word_color(ld_color(io.Xc + v, io.pol_col));
-    const uint32_t pv = p.prio ? __ldg(p.prio + v) : 0u;
+    const uint32_t pv = F ? __ldg(p.prio + v) : 0u;
     // a vertex decided by this warp: its static mask word `lane`, read now
     const uint32_t old_single = (single && lane < 8u && !io.first) ? __ldcg(p.stat + (size_t)v * 8 + lane) : 0u;
     bool conflict = false;
@@ -1652,9 +1657,9 @@ __device__ __forceinline__ void hub_chunk(const Params<T>& p, const PassIO<T>& i
                 bool pre = false;
                 if constexpr (!P) {
                     pre = in && col == cv && wid < v;
-                } else if (in && (col == cv || (io.first && !settled))) {
-                    pre = io.first ? precedes(p.prio, wid, v, pv) : w[u] < 0;
-                    if (io.first) w[u] = (int32_t)((uint32_t)wid | (pre ? kPrecBit : 0u));  // the entry kept
+                } else if (in && (col == cv || (F && !settled))) {
+                    pre = F ? precedes(p.prio, wid, v, pv) : w[u] < 0;
+                    if (F) w[u] = (int32_t)((uint32_t)wid | (pre ? kPrecBit : 0u));  // the entry kept
                 }
                 if (in) {
                     if (col == cv && pre) conflict = true;
@@ -1836,15 +1841,18 @@ __device__ __forceinline__ void run_pass(const Params<T>& p, int k, const RoundS
         unsigned claim = 0;
         if (!fixed && tn < total && lane_id() == 0) claim = atomicAdd(ctr, 1u);
         if (t < q.e0) {
-            hub_chunk<T, P>(p, io, cur, s_flat[wib], maxc, vol);
+            if (P && io.first) hub_chunk<T, P, P>(p, io, cur, s_flat[wib], maxc, vol);
+            else hub_chunk<T, P, false>(p, io, cur, s_flat[wib], maxc, vol);
         } else if (t < q.e1) {
-            vertex_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
+            if (P && io.first) vertex_task<T, P, P>(p, io, cur.e, s_flat[wib], maxc, vol);
+            else vertex_task<T, P, false>(p, io, cur.e, s_flat[wib], maxc, vol);
         } else if (t < q.e2) {
             mid_task<T, P, 16>(p, io, cur.e, q.s16, maxc, vol);
         } else if (t < q.e3) {
             mid_task<T, P, 8>(p, io, cur.e, q.s8, maxc, vol);
         } else if (t < q.e4) {
-            flat_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
+            if (P && io.first) flat_task<T, P, P>(p, io, cur.e, s_flat[wib], maxc, vol);
+            else flat_task<T, P, false>(p, io, cur.e, s_flat[wib], maxc, vol);
         } else if (t < q.e5) {
             tiny_task<T, P, 4>(p, io, cur.e, q.s4, maxc, vol);
         } else {
