@@ -55,7 +55,7 @@ constexpr int kRow = kH + 4;
 struct __align__(16) ForwardParams {
     float w1[kIn][kRow];
     float w2[kH][kRow];
-    float w3[kH], b1[kH], b2[kH];
+    float w3[kH], b1[kH], b2[kH];  // (b1, b2: read two at a time)
     float b3;
 };
 __device__ __forceinline__ void load_forward_params(const float* __restrict__ params, ForwardParams& s) {
@@ -114,13 +114,75 @@ __device__ __forceinline__ void layer_units(const float (*w)[kRow], const float*
         }
 }
 
-// kForwardRows samples per thread, kForwardUnits units of layer 2 at a time.
-// Bound: the fp32 multiply-adds (1,248 a sample; 62 % of the fp32 rate).  With
-// one sample a thread, each read of four weights from shared memory served four
-// of them, and the kernel ran at 89 % of the L1 rate, 41 % of the fp32 rate:
-// 4,194,301 samples 319 us, now 221 (8 or 32 units at a time 231 and 242, three
-// samples 240, 128 threads a block 233).
-constexpr int kForwardRows = 2, kForwardUnits = 16, kForwardThreads = 256, kForwardBlocks = 2;
+// Two bf16 values in a word, the first in its low half: rounding to nearest
+// even (NaN stays NaN), max(., 0) of both (NaN gives 0, as fmaxf does; rounding
+// keeps the sign, so it commutes with the maximum), and a value back.
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+    uint32_t w;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(hi), "f"(lo));
+    return w;
+}
+__device__ __forceinline__ uint32_t relu_pair(uint32_t w) {
+    uint32_t m;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(w), "r"(0u));
+    return m;
+}
+__device__ __forceinline__ float bf16_of(uint32_t w, int half) {
+    return __uint_as_float(half ? w & 0xffff0000u : w << 16);
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// layer_units with the activations kept as pairs of bf16 (half the registers,
+// and bias, rounding and maximum take one instruction each for two units).
+template <int IN, int J, int R>
+__device__ __forceinline__ void layer_pairs(const float (*w)[kRow], const float* bias, int j0,
+                                            const uint32_t (&in)[R][IN / 2], uint32_t (&out)[R][J / 2]) {
+    f32x2 acc[R][J / 2];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int q = 0; q < J / 2; ++q) acc[r][q] = 0ull;
+#pragma unroll
+    for (int i = 0; i < IN; ++i) {
+        f32x2 a[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float v = bf16_of(in[r][i / 2], i & 1);
+            a[r] = pack2(v, v);
+        }
+#pragma unroll
+        for (int q = 0; q < J / 2; q += 2) {
+            const ulonglong2 wq = *reinterpret_cast<const ulonglong2*>(&w[i][j0 + 2 * q]);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                acc[r][q] = fma2(wq.x, a[r], acc[r][q]);
+                acc[r][q + 1] = fma2(wq.y, a[r], acc[r][q + 1]);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int q = 0; q < J / 2; ++q) {
+            float x, y;
+            unpack2(add2(acc[r][q], *reinterpret_cast<const f32x2*>(&bias[j0 + 2 * q])), x, y);
+            out[r][q] = relu_pair(bf16_pair(x, y));
+        }
+}
+
+// kForwardRows samples per thread, kForwardUnits units at a time.
+// Bound: the fp32 multiply-adds (1,248 a sample; 70 % of the fp32 rate) and the
+// 16-byte weight reads beside them, one for kForwardRows * 4 multiply-adds.
+// 4,194,301 samples take 197 us, 16,000,001 take 719 (one sample a thread,
+// scalar arithmetic: 319 for the first; two samples with activations as floats,
+// 128 registers: 223 and 818; two as pairs: 206 and 745; three 201 and 736;
+// four, 8 or 32 units at a time: 199 and 217).  Up to 155,648 samples (one
+// block per SM, once around) all of these take the same 16 us, launch included.
+constexpr int kForwardRows = 4, kForwardUnits = 16, kForwardThreads = 256, kForwardBlocks = 1;
 __global__ void __launch_bounds__(kForwardThreads, kForwardBlocks) mlp_forward_kernel(const float* __restrict__ params,
                                                           const float* __restrict__ x, int64_t n,
                                                           float* __restrict__ y) {
@@ -130,24 +192,34 @@ __global__ void __launch_bounds__(kForwardThreads, kForwardBlocks) mlp_forward_k
     __syncthreads();
     const int64_t T = (int64_t)gridDim.x * blockDim.x;
     for (int64_t r0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r0 < n; r0 += T * R) {
-        float a0[R][kIn], a1[R][kH], out[R];
+        uint32_t a0[R][kIn / 2], a1[R][kH / 2];
+        float out[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int64_t row = r0 + r * T < n ? r0 + r * T : r0;
 #pragma unroll
-            for (int i = 0; i < kIn; ++i) a0[r][i] = bf16r(__ldg(x + row * kIn + i));
+            for (int i = 0; i < kIn; i += 2)
+                a0[r][i / 2] = bf16_pair(__ldg(x + row * kIn + i), __ldg(x + row * kIn + i + 1));
             out[r] = 0.f;
         }
-        layer_units<kIn, kH, R>(s.w1, s.b1, 0, a0, a1);
+#pragma unroll
+        for (int j0 = 0; j0 < kH; j0 += J) {
+            uint32_t h[R][J / 2];
+            layer_pairs<kIn, J, R>(s.w1, s.b1, j0, a0, h);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int q = 0; q < J / 2; ++q) a1[r][j0 / 2 + q] = h[r][q];
+        }
         // output = bf16(W3) . a2 + b3, accumulated in unit order
 #pragma unroll 1
         for (int j0 = 0; j0 < kH; j0 += J) {
-            float a2[R][J];
-            layer_units<kH, J, R>(s.w2, s.b2, j0, a1, a2);
+            uint32_t a2[R][J / 2];
+            layer_pairs<kH, J, R>(s.w2, s.b2, j0, a1, a2);
 #pragma unroll
             for (int j = 0; j < J; ++j)
 #pragma unroll
-                for (int r = 0; r < R; ++r) out[r] = fmaf(s.w3[j0 + j], a2[r][j], out[r]);
+                for (int r = 0; r < R; ++r) out[r] = fmaf(s.w3[j0 + j], bf16_of(a2[r][j / 2], j & 1), out[r]);
         }
 #pragma unroll
         for (int r = 0; r < R; ++r)

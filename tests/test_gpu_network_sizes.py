@@ -28,13 +28,29 @@ def _uniform(seed, stream, count, lo, hi):
     return (lo + (hi - lo) * u).astype(np.float32)
 
 
-# two samples a thread, 256 threads a block, two blocks an SM (152 of them): 155,648 a grid
-@pytest.mark.parametrize("n", [1, 2, 255, 257, 511, 512, 513, 155647, 155649])
+# four samples a thread, 256 threads a block, a block an SM (152 of them): 155,648 a grid
+@pytest.mark.parametrize("n", [1, 2, 255, 257, 511, 512, 513, 1023, 1025, 155647, 155649])
 def test_forward_sizes(gcpkg, n):
     p = _uniform(n, 7, L.N_PARAMS, -0.3, 0.3)
     x = _uniform(n + 1, 9, n * L.N_IN, -2.0, 24.0).reshape(n, L.N_IN)
     got = gcpkg.mlp_forward(_dev(p), _dev(x)).cpu().numpy()
     assert np.array_equal(got.view(np.uint32), L.mlp_forward(p, x).view(np.uint32))
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf, -0.0, 3.4e38, -3.4e38, 1e-41, -1e-39])
+def test_forward_extreme_inputs(gcpkg, value):
+    """The maximum with 0 taken after the rounding, of two units at a time: not a number gives 0,
+    infinities and subnormal numbers pass through the rounding as they do one by one."""
+    n = 1300
+    p = _uniform(5, 7, L.N_PARAMS, -0.3, 0.3)
+    x = _uniform(6, 9, n * L.N_IN, -2.0, 24.0).reshape(n, L.N_IN)
+    x[np.arange(n), np.arange(n) % L.N_IN] = value
+    x[::7] = value
+    got = gcpkg.mlp_forward(_dev(p), _dev(x)).cpu().numpy()
+    want = L.mlp_forward(p, x)
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    ok = ~np.isnan(want)
+    assert np.array_equal(got[ok].view(np.uint32), want[ok].view(np.uint32))
 
 
 # 128 samples a tile, two blocks an SM: 38,912 before a block takes a second tile
