@@ -1253,6 +1253,7 @@ int batch_plan_big(gc_batch* b, const std::vector<int32_t>& order, int32_t nbig,
     if (rc != GC_OK) {
         batch_free(big);
         if (rc != GC_ERR_OOM) return rc;
+        cudaStreamSynchronize(s);  // the copies above; a refused first allocation returns without a wait
         plan_free(b->big_ws);
         b->big_ws = nullptr;
         b->big_ws_bytes = 0;

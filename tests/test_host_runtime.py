@@ -1,0 +1,95 @@
+"""Host code of the library against a fake CUDA runtime (no GPU).
+
+fake_cudart.cpp holds device memory in host memory, carries copies out only when
+their stream is waited for, and runs no kernel; it refuses chosen allocations and
+counts memory given back while work on it is still queued.  The library is
+compiled a second time, unoptimised, against it.
+"""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_1205_3809_gb300 as gc
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    out = str(tmp_path_factory.mktemp("fake") / "libgc_fake.so")
+    subprocess.run(["nvcc", "-gencode", "arch=compute_103a,code=compute_103a", "-O0", "-Xcicc", "-O0", "-std=c++17",
+                    "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-Xlinker", "-Bsymbolic", "--threads", "2", "-I", gc._INCLUDE,
+                    "-o", out, os.path.join(gc._CSRC, "gc.cu"), os.path.join(gc._CSRC, "gc_mlp.cu"), os.path.join(HERE, "fake_cudart.cpp")], check=True)
+    h = ctypes.CDLL(out)
+    vp, i32 = ctypes.c_void_p, ctypes.c_int32
+    h.gc_batch_create.argtypes = [vp, vp, vp, vp, i32, vp, vp, vp, vp, ctypes.POINTER(gc.Options), vp,
+                                  ctypes.POINTER(vp)]
+    h.gc_batch_destroy.argtypes = [vp]
+    h.gc_batch_workspace_bytes.argtypes = [vp]
+    h.gc_batch_workspace_bytes.restype = ctypes.c_size_t
+    h.fake_bytes_live.restype = ctypes.c_size_t
+    h.fake_bytes_taken.restype = ctypes.c_size_t
+    h.fake_capacity.argtypes = [ctypes.c_size_t]
+    h.fake_kernel_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]
+    yield h
+    h.gc_release()
+
+
+def _p(a):
+    return ctypes.c_void_p(a.ctypes.data)
+
+
+class EdgelessBatch:
+    """A plan of graphs without entries: sizes alone decide how a batch is split."""
+
+    def __init__(self, lib, sizes, keys=False, **options):
+        self.lib = lib
+        n, g = int(sum(sizes)), len(sizes)
+        self.voff = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        self.eoff = np.zeros(g + 1, np.int64)
+        self.rowptr = np.zeros(n + g, np.int32)
+        self.colors, self.nc, self.rd = (np.zeros(max(k, 1), np.int32) for k in (n, g, g))
+        self.prio = np.zeros(max(n, 1), np.uint32) if keys else None
+        self.plan = ctypes.c_void_p()
+        self.rc = lib.gc_batch_create(_p(self.rowptr), None, _p(self.voff), _p(self.eoff), g,
+                                      _p(self.prio) if keys else None, _p(self.colors), _p(self.nc), _p(self.rd),
+                                      ctypes.byref(gc._options(options)), None, ctypes.byref(self.plan))
+
+    def close(self):
+        self.lib.gc_batch_destroy(self.plan)
+
+
+SPLIT = [400000] + [500] * 199   # the first graph alone outlasts the others' share: colored apart
+
+
+def test_plan_of_a_split_batch_at_every_refused_allocation(lib):
+    """An allocation refused at any point gives a plan without the split or
+    GC_ERR_OOM, gives back no memory that queued work still uses, and leaves none
+    behind."""
+    b = EdgelessBatch(lib, SPLIT, keys=True)
+    assert b.rc == gc.GC_OK
+    whole = lib.gc_batch_workspace_bytes(b.plan)
+    b.close()
+    b = EdgelessBatch(lib, SPLIT, keys=True, batch_mode=2)
+    unsplit = lib.gc_batch_workspace_bytes(b.plan)
+    b.close()
+    assert whole > unsplit and lib.fake_misuse() == 0
+    start = lib.fake_bytes_live()
+    seen = []
+    for which in range(1, 20):
+        lib.fake_refuse_allocation(which)
+        b = EdgelessBatch(lib, SPLIT, keys=True)
+        lib.fake_refuse_allocation(0)
+        assert b.rc in (gc.GC_OK, gc.GC_ERR_OOM)
+        seen.append((b.rc, lib.gc_batch_workspace_bytes(b.plan) if b.rc == gc.GC_OK else 0))
+        if b.rc == gc.GC_OK:
+            b.close()
+        assert lib.fake_misuse() == 0, f"refused allocation {which}: memory given back in use"
+        assert lib.fake_bytes_live() == start
+        if seen[-1] == (gc.GC_OK, whole):
+            break
+    assert seen[-1] == (gc.GC_OK, whole)                 # past the last allocation
+    assert (gc.GC_ERR_OOM, 0) in seen and (gc.GC_OK, unsplit) in seen
