@@ -344,7 +344,7 @@ int gc_batch_launch_graph(gc_batch* plan, void* stream);
 /* gc_batch_status - wait for `stream`, then report the last run: the largest
  * round count and color count over the batch, and GC_OK, GC_ERR_BAD_GRAPH (a
  * neighbour id outside its graph; it was replaced by 0), GC_ERR_MAX_ROUNDS
- * or GC_ERR_TIMEOUT. */
+ * or GC_ERR_TIMEOUT.  Before a first run: GC_OK and zeros. */
 int gc_batch_status(gc_batch* plan, void* stream, int32_t* max_rounds, int32_t* max_colors);
 
 /* gc_batch_features - the six gc_features features of every vertex of the

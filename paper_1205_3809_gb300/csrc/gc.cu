@@ -1488,6 +1488,8 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
         rc = validate_locked((const int32_t*)(base + b->off_rowptr), colidx_g, (int32_t)N, s, *dcp, &launches);
         if (rc != GC_OK) return rc;
     }
+    // the status before a first run: memory from the pool may hold another plan's
+    GC_CUDA(cudaMemsetAsync((char*)b->ws + b->L.st, 0, sizeof(RoundState), s));
     GC_CUDA(cudaStreamSynchronize(s));
     return GC_OK;
 }

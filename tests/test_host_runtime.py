@@ -28,6 +28,8 @@ def lib(tmp_path_factory):
     h.gc_batch_create.argtypes = [vp, vp, vp, vp, i32, vp, vp, vp, vp, ctypes.POINTER(gc.Options), vp,
                                   ctypes.POINTER(vp)]
     h.gc_batch_destroy.argtypes = [vp]
+    h.gc_batch_status.argtypes = [vp, vp, vp, vp]
+    h.gc_batch_round_stats.argtypes = [vp, vp, vp, i32, vp, vp]
     h.gc_batch_workspace_bytes.argtypes = [vp]
     h.gc_batch_workspace_bytes.restype = ctypes.c_size_t
     h.fake_bytes_live.restype = ctypes.c_size_t
@@ -93,3 +95,17 @@ def test_plan_of_a_split_batch_at_every_refused_allocation(lib):
             break
     assert seen[-1] == (gc.GC_OK, whole)                 # past the last allocation
     assert (gc.GC_ERR_OOM, 0) in seen and (gc.GC_OK, unsplit) in seen
+
+
+@pytest.mark.parametrize("options", [{}, {"batch_mode": 1}, {"batch_mode": 2}], ids=["split", "shared-grid", "block-per-graph"])
+def test_status_of_a_plan_that_has_not_run(lib, options):
+    """The plan's memory may hold what an earlier plan left there: until a run
+    writes them, the status and the per-round record must not come from it."""
+    b = EdgelessBatch(lib, SPLIT, **options)
+    assert b.rc == gc.GC_OK
+    rounds, colors, bits = (ctypes.c_int32(-1) for _ in range(3))
+    assert lib.gc_batch_status(b.plan, None, ctypes.byref(rounds), ctypes.byref(colors)) == gc.GC_OK
+    assert (rounds.value, colors.value) == (0, 0)
+    sizes, volumes = np.full(8, -1, np.int32), np.full(8, -1, np.int64)
+    assert lib.gc_batch_round_stats(b.plan, _p(sizes), _p(volumes), 8, ctypes.byref(bits), None) == 0
+    b.close()
