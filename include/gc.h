@@ -193,9 +193,10 @@ int gc_last_round_stats(int32_t* sizes, int64_t* volumes, int32_t cap);
 /*
  * gc_last_phase_ms - phase timings, in milliseconds from CUDA events recorded
  * on the call's stream, of the last call made with opt->telemetry = 1:
- * ms[0] setup scan kernel, ms[1] round 1 (the two pass-1 kernels), ms[2]
- * every later round (the persistent kernel, or all per-round launches with
- * their host round trips in loop_mode 1), ms[3] the whole call.
+ * ms[0] setup scan kernel, ms[1] round 1 (pass 1, and the kernel for its long
+ * rows if there are any), ms[2] every later round (the persistent kernel, or
+ * all per-round launches with their host round trips in loop_mode 1), ms[3]
+ * the whole call, without the entry checks of opt->validate.
  * Returns the number of values written (<= cap, at most 4) or GC_ERR_INVALID.
  */
 int gc_last_phase_ms(float* ms, int32_t cap);

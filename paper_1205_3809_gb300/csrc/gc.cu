@@ -65,7 +65,7 @@ struct DeviceCache {
     size_t host_bytes = 0;
     int sms = 0;
     int coop = 0;
-    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t ev[5] = {};    // start, setup scan, round 1, end; entry checks
     cudaStream_t copy = nullptr;                 // host inputs: colidx copies in chunks
     cudaEvent_t chunk_ev[16] = {};               // one per chunk copied
     cudaEvent_t start_ev = nullptr;              // orders the copies after the caller's stream
@@ -539,13 +539,14 @@ int scan_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, int32_t
     gc::stats_kernel<<<grid, 256, 0, s>>>(rowptr, n, s_max, m_max, keyed, stats);
     GC_CUDA(cudaGetLastError());
     *launches += 1;
+    if (timed) GC_CUDA(cudaEventRecord(dc.ev[1], s));
     if (validate) {
         if (hin) GC_CUDA(cudaStreamWaitEvent(s, dc.chunk_ev[hin->nchunks - 1], 0));
         gc::validate_kernel<<<grid, 256, 0, s>>>(rowptr, colidx, n, stats, out);
         GC_CUDA(cudaGetLastError());
         *launches += 1;
+        if (timed) GC_CUDA(cudaEventRecord(dc.ev[4], s));
     }
-    if (timed) GC_CUDA(cudaEventRecord(dc.ev[1], s));
     GC_CUDA(cudaMemcpyAsync(dc.host, dc.ws, kHead, cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaStreamSynchronize(s));
     std::memcpy(hs, dc.host, sizeof(Stats));
@@ -609,7 +610,7 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
     if (rc != GC_OK) return rc;
     dc.host_bytes = hb;
     if (o.telemetry && !dc.ev[0])
-        for (int i = 0; i < 4; ++i) GC_CUDA(cudaEventCreate(&dc.ev[i]));
+        for (cudaEvent_t& e : dc.ev) GC_CUDA(cudaEventCreate(&e));
     if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[0], s));
     Stats hs;
     {
@@ -688,9 +689,14 @@ int color_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, const 
     g_last.timed = o.telemetry;
     if (o.telemetry) {
         GC_CUDA(cudaEventElapsedTime(&g_last.ms[0], dc.ev[0], dc.ev[1]));
-        GC_CUDA(cudaEventElapsedTime(&g_last.ms[1], dc.ev[1], dc.ev[2]));
+        GC_CUDA(cudaEventElapsedTime(&g_last.ms[1], dc.ev[o.validate ? 4 : 1], dc.ev[2]));
         GC_CUDA(cudaEventElapsedTime(&g_last.ms[2], dc.ev[2], dc.ev[3]));
         GC_CUDA(cudaEventElapsedTime(&g_last.ms[3], dc.ev[0], dc.ev[3]));
+        if (o.validate) {  // the entry checks are no phase of the coloring
+            float checks = 0.f;
+            GC_CUDA(cudaEventElapsedTime(&checks, dc.ev[1], dc.ev[4]));
+            g_last.ms[3] -= checks;
+        }
     }
     *rounds = hst.rounds;
     *ncolors = hst.max_color;
@@ -1677,8 +1683,8 @@ int gc_release(void) {
         if (kv.second.ws) cudaFree(kv.second.ws);
         if (kv.second.in) cudaFree(kv.second.in);
         if (kv.second.host) cudaFreeHost(kv.second.host);
-        for (int i = 0; i < 4; ++i)
-            if (kv.second.ev[i]) cudaEventDestroy(kv.second.ev[i]);
+        for (cudaEvent_t e : kv.second.ev)
+            if (e) cudaEventDestroy(e);
         for (int i = 0; i < kMaxChunks; ++i)
             if (kv.second.chunk_ev[i]) cudaEventDestroy(kv.second.chunk_ev[i]);
         if (kv.second.start_ev) cudaEventDestroy(kv.second.start_ev);

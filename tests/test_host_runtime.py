@@ -28,6 +28,8 @@ def lib(tmp_path_factory):
     h.gc_batch_create.argtypes = [vp, vp, vp, vp, i32, vp, vp, vp, vp, ctypes.POINTER(gc.Options), vp,
                                   ctypes.POINTER(vp)]
     h.gc_batch_destroy.argtypes = [vp]
+    h.gc_color_ex.argtypes = [vp, vp, i32, vp, vp, vp, vp, vp, ctypes.POINTER(gc.Options), vp, i32]
+    h.gc_last_phase_ms.argtypes = [vp, i32]
     h.gc_batch_status.argtypes = [vp, vp, vp, vp]
     h.gc_batch_round_stats.argtypes = [vp, vp, vp, i32, vp, vp]
     h.gc_batch_workspace_bytes.argtypes = [vp]
@@ -109,3 +111,26 @@ def test_status_of_a_plan_that_has_not_run(lib, options):
     sizes, volumes = np.full(8, -1, np.int32), np.full(8, -1, np.int64)
     assert lib.gc_batch_round_stats(b.plan, _p(sizes), _p(volumes), 8, ctypes.byref(bits), None) == 0
     b.close()
+
+
+def _phases(lib, **options):
+    n = 1000
+    rowptr, colors = np.zeros(n + 1, np.int32), np.zeros(n, np.int32)
+    nc, rd = ctypes.c_int32(), ctypes.c_int32()
+    rc = lib.gc_color_ex(_p(rowptr), None, n, None, _p(colors), ctypes.byref(nc), ctypes.byref(rd), None,
+                         ctypes.byref(gc._options(dict(options, telemetry=1))), None, 0)
+    assert rc == gc.GC_OK
+    ms = (ctypes.c_float * 4)()
+    assert lib.gc_last_phase_ms(ms, 4) == 4
+    return list(ms)
+
+
+def test_phase_times_leave_the_entry_checks_out(lib):
+    """One unit of time a kernel, a thousand for the entry checks: setup scan,
+    round 1, later rounds and their sum, with and without the checks."""
+    lib.fake_kernel_cost(b"validate_kernel", 1000.0)
+    try:
+        assert _phases(lib) == [1.0, 1.0, 1.0, 3.0]
+        assert _phases(lib, validate=1) == [1.0, 1.0, 1.0, 3.0]
+    finally:
+        lib.fake_kernel_cost(b"validate_kernel", 1.0)
