@@ -700,8 +700,10 @@ class Batch:
 
 TUNE_CANDIDATES = tuple({"small_max_degree": sm, "medium_max_degree": mm, "block_threads": bt}
                         for sm in (8, 16, 32) for mm in (64, 128, 256) for bt in (128, 256))
-# batches: one block per graph, or the grid above shared by all graphs
-BATCH_TUNE_CANDIDATES = (tuple({"batch_mode": 2, "local_shared_bytes": kb * 1024} for kb in (0, 132, 224))
+# batches: the library's own choice (one block per graph, the largest graphs on
+# the whole GPU if that is estimated to be faster), one block for every graph, or
+# the grid above shared by all graphs
+BATCH_TUNE_CANDIDATES = (tuple({"batch_mode": m, "local_shared_bytes": kb * 1024} for m in (0, 2) for kb in (0, 132, 224))
                          + tuple(dict(c, batch_mode=1) for c in TUNE_CANDIDATES))
 
 
@@ -800,7 +802,8 @@ def autotune_batch(rowptr_cat, colidx_cat, vertex_offsets, edge_offsets, priorit
     rp = rowptr_cat.cpu().numpy().astype(np.int64)
     keep = np.ones(max(rp.shape[0] - 1, 0), dtype=bool)
     keep[(voff[1:] + np.arange(G))[:-1]] = False   # the step from one graph's rowptr to the next
-    key = json.dumps(["batch", 2, _device_key(rowptr_cat.device), G, priority is not None,
+    # (the number goes up when winners stored before are out of date)
+    key = json.dumps(["batch", 3, _device_key(rowptr_cat.device), G, priority is not None,
                       _degree_signature(np.diff(rp)[keep] if rp.size > 1 else np.zeros(0))])
     if cache:
         hit = _cache_io(key)

@@ -42,3 +42,50 @@ def test_pack_batch_layout():
     assert rp.tolist() == [0, 1, 2, 0, 0, 0, 0, 0]
     assert ci.tolist() == [1, 0]
     assert voff.tolist() == [0, 2, 2, 5] and eoff.tolist() == [0, 2, 2, 2]
+
+
+def test_batch_candidates_hold_the_librarys_own_choice():
+    """What a call without options gets (batch_mode 0: the library decides, and may
+    split the batch) is among the candidates, with every size of shared memory, and
+    first, so that it wins a tie."""
+    own = [c for c in gc.BATCH_TUNE_CANDIDATES if c.get("batch_mode", 0) == 0]
+    assert own[0] is gc.BATCH_TUNE_CANDIDATES[0]
+    assert [c.get("local_shared_bytes", 0) for c in own] == [
+        c["local_shared_bytes"] for c in gc.BATCH_TUNE_CANDIDATES if c.get("batch_mode") == 2]
+    default, first = gc.Options(), gc._options_array(own)[0]
+    assert all(getattr(first, f) == getattr(default, f) for f, _ in gc.Options._fields_ if f != "reserved")
+
+
+def test_batch_winners_stored_before_the_split_are_not_served(tmp_path, monkeypatch):
+    """A winner chosen when no candidate could split a batch is tuned again."""
+    import contextlib
+
+    import torch
+
+    path = tmp_path / "tune.json"
+    monkeypatch.setenv("GC_TUNE_CACHE", str(path))
+    monkeypatch.setattr(gc, "_device_key", lambda device: "gpu")
+    monkeypatch.setattr(gc, "_dev_ptr", lambda *a: None)
+    monkeypatch.setattr(gc, "_stream_handle", lambda *a: None)
+    monkeypatch.setattr(torch.cuda, "device", lambda d: contextlib.nullcontext())
+    runs = []
+
+    class Native:
+        @staticmethod
+        def gc_batch_tune(*a):
+            arr, count, ms, best = a[9], a[10], a[13], a[14]
+            runs.append([arr[i].batch_mode for i in range(count)])
+            for i in range(count):
+                ms[i] = 1.0
+            best._obj.value = 0
+            return 0
+
+    monkeypatch.setattr(gc, "_load", lambda: Native)
+    rp, ci, voff, eoff = gc.pack_batch([(np.array([0, 1, 2], np.int32), np.array([1, 0], np.int32))] * 2)
+    sig = gc._degree_signature(np.ones(4))
+    old = json.dumps(["batch", 2, "gpu", 2, False, sig])
+    gc._cache_io(old, {"best": {"batch_mode": 2}, "table": []})
+    args = (torch.from_numpy(rp), torch.from_numpy(ci), voff, eoff)
+    best, table = gc.autotune_batch(*args)
+    assert len(runs) == 1 and 0 in runs[0] and best["batch_mode"] == 0
+    assert gc.autotune_batch(*args) == (best, table) and len(runs) == 1   # its own result is
