@@ -29,6 +29,7 @@
 #include "gc_batch.cuh"
 #include "gc_device.cuh"
 #include "gc_local.cuh"
+#include "gc_memory.cuh"
 
 namespace {
 
@@ -137,45 +138,12 @@ int device_cache(DeviceCache** out) {
     return GC_OK;
 }
 
-int ensure_device(void** p, size_t* have, size_t need) {
-    if (*have >= need && *p) return GC_OK;
-    if (*p) {
-        GC_CUDA(cudaDeviceSynchronize());
-        GC_CUDA(cudaFree(*p));
-        *p = nullptr;
-        *have = 0;
-    }
-    GC_CUDA(cudaMalloc(p, need));
-    *have = need;
-    return GC_OK;
-}
-
-int ensure_host(void** p, size_t* have, size_t need) {
-    if (*have >= need && *p) return GC_OK;
-    if (*p) {
-        GC_CUDA(cudaFreeHost(*p));
-        *p = nullptr;
-        *have = 0;
-    }
-    GC_CUDA(cudaMallocHost(p, need));
-    *have = need;
-    return GC_OK;
-}
-
-// A device workspace of `need` bytes, unless the caller's testing limit
-// (workspace_limit_mb) forbids growing the one held to that size: then
-// GC_ERR_OOM, as if cudaMalloc had refused, and the old workspace stays.
-int ensure_device_limited(void** p, size_t* have, size_t need, int32_t limit_mb) {
-    if (limit_mb > 0 && need > *have && need > ((size_t)limit_mb << 20)) return GC_ERR_OOM;
-    return ensure_device(p, have, need);
-}
-
 // Device memory of batch plans.  A plan made, run and freed in one call (or one
 // per batch of work) would otherwise spend more time in cudaMalloc and cudaFree,
 // which also wait for the whole device, than in its kernels.  It comes from a
 // pool of its own per device that keeps at most kPlanPoolKeep bytes of freed
-// memory and gives them back in gc_release.  Both calls wait for the pool's
-// (otherwise idle) stream: memory handed out may be used on any stream, and
+// memory and gives them back in gc_release, or when a workspace of another call
+// would be refused otherwise.  Both calls wait for the pool's (otherwise idle) stream: memory handed out may be used on any stream, and
 // memory handed back must no longer be in use.
 constexpr size_t kPlanPoolKeep = 256ull << 20;
 struct PlanPool {
@@ -233,6 +201,56 @@ void plan_pools_trim() {
         cudaSetDevice(kv.first);
         if (kv.second.pool) cudaMemPoolTrimTo(kv.second.pool, 0);
     }
+}
+
+}  // namespace
+
+namespace gc {
+cudaError_t malloc_device(void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    int dev = 0;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (cudaGetDevice(&dev) != cudaSuccess || !g_pools.count(dev) || !g_pools[dev].pool) return e;
+    (void)cudaGetLastError();
+    cudaMemPoolTrimTo(g_pools[dev].pool, 0);
+    return cudaMalloc(p, bytes);
+}
+}  // namespace gc
+
+namespace {
+
+int ensure_device(void** p, size_t* have, size_t need) {
+    if (*have >= need && *p) return GC_OK;
+    if (*p) {
+        GC_CUDA(cudaDeviceSynchronize());
+        GC_CUDA(cudaFree(*p));
+        *p = nullptr;
+        *have = 0;
+    }
+    GC_CUDA(gc::malloc_device(p, need));
+    *have = need;
+    return GC_OK;
+}
+
+int ensure_host(void** p, size_t* have, size_t need) {
+    if (*have >= need && *p) return GC_OK;
+    if (*p) {
+        GC_CUDA(cudaFreeHost(*p));
+        *p = nullptr;
+        *have = 0;
+    }
+    GC_CUDA(cudaMallocHost(p, need));
+    *have = need;
+    return GC_OK;
+}
+
+// A device workspace of `need` bytes, unless the caller's testing limit
+// (workspace_limit_mb) forbids growing the one held to that size: then
+// GC_ERR_OOM, as if cudaMalloc had refused, and the old workspace stays.
+int ensure_device_limited(void** p, size_t* have, size_t need, int32_t limit_mb) {
+    if (limit_mb > 0 && need > *have && need > ((size_t)limit_mb << 20)) return GC_ERR_OOM;
+    return ensure_device(p, have, need);
 }
 
 struct Layout {

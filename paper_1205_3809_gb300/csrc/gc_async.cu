@@ -18,6 +18,7 @@
 #include <mutex>
 
 #include "gc.h"
+#include "gc_memory.cuh"
 
 namespace {
 
@@ -144,7 +145,7 @@ extern "C" int gc_color_async(const int32_t* rowptr, const int32_t* colidx, int3
             ac.ws = nullptr;
             ac.bytes = 0;
         }
-        if (cudaMalloc(&ac.ws, need) != cudaSuccess) {
+        if (gc::malloc_device(&ac.ws, need) != cudaSuccess) {
             (void)cudaGetLastError();
             return GC_ERR_OOM;
         }

@@ -134,3 +134,24 @@ def test_phase_times_leave_the_entry_checks_out(lib):
         assert _phases(lib, validate=1) == [1.0, 1.0, 1.0, 3.0]
     finally:
         lib.fake_kernel_cost(b"validate_kernel", 1.0)
+
+
+def test_memory_kept_from_plans_does_not_refuse_a_later_call(lib):
+    """The pool keeps freed plan memory; a workspace that only fits without it is
+    still allocated."""
+    lib.gc_release()
+    b = EdgelessBatch(lib, [3000000])
+    assert b.rc == gc.GC_OK
+    b.close()
+    kept = lib.fake_bytes_taken() - lib.fake_bytes_live()
+    assert 100 << 20 < kept <= 256 << 20
+    n = 1000000                                          # about 36 bytes a vertex
+    rowptr, colors = np.zeros(n + 1, np.int32), np.zeros(n, np.int32)
+    nc, rd = ctypes.c_int32(), ctypes.c_int32()
+    lib.fake_capacity(lib.fake_bytes_taken() + (16 << 20))
+    try:
+        assert lib.gc_color_ex(_p(rowptr), None, n, None, _p(colors), ctypes.byref(nc), ctypes.byref(rd), None, None,
+                               None, 0) == gc.GC_OK
+    finally:
+        lib.fake_capacity(ctypes.c_size_t(-1).value)
+        lib.gc_release()
