@@ -155,6 +155,11 @@ size_t fake_bytes_live() {
     for (const auto& b : g_blocks) n += b.second.bytes;
     return n;
 }
+size_t fake_pool_bytes() {  // handed out from pools
+    size_t n = 0;
+    for (Pool* p : g_pools) n += p->used;
+    return n;
+}
 size_t fake_bytes_taken() { return taken(); }
 
 // ---- registration and launches

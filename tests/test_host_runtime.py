@@ -36,6 +36,7 @@ def lib(tmp_path_factory):
     h.gc_batch_workspace_bytes.restype = ctypes.c_size_t
     h.fake_bytes_live.restype = ctypes.c_size_t
     h.fake_bytes_taken.restype = ctypes.c_size_t
+    h.fake_pool_bytes.restype = ctypes.c_size_t
     h.fake_capacity.argtypes = [ctypes.c_size_t]
     h.fake_kernel_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]
     yield h
@@ -155,3 +156,17 @@ def test_memory_kept_from_plans_does_not_refuse_a_later_call(lib):
     finally:
         lib.fake_capacity(ctypes.c_size_t(-1).value)
         lib.gc_release()
+
+
+def test_large_plans_do_not_go_through_the_pool(lib):
+    """Memory that the pool would unmap when it is freed comes from cudaMalloc."""
+    lib.gc_release()
+    for n, pooled in ((3000000, True), (10000000, False)):
+        b = EdgelessBatch(lib, [n])
+        assert b.rc == gc.GC_OK
+        ws = lib.gc_batch_workspace_bytes(b.plan)
+        assert (ws <= 384 << 20) == pooled
+        assert (lib.fake_pool_bytes() >= ws) == pooled and lib.fake_bytes_live() >= ws
+        b.close()
+        assert lib.fake_pool_bytes() == 0 and lib.fake_misuse() == 0
+    lib.gc_release()
