@@ -1197,19 +1197,35 @@ constexpr int32_t kLocalSharedDefault = 164 * 1024;  // mode 2: bytes of shared 
 // 5 ms: 15.13 ms with a block each, 10.69 with all in the union, 6.06 split; a
 // 2,500-graph batch 16.21 -> 14.34.  Factors from 2.5 to 4.5 pick splits within
 // 7 % of each other on eight batches of 96 to 2,500 graphs; 2 and less put so
-// many graphs in the union that the first takes 7.18 ms.
-constexpr double kUnionFixed = 1e5, kUnionFactor = 2.5;
+// many graphs in the union that the first takes 7.18 ms.  That is how much the
+// factor matters, not how far a pick is from the best split: 300 graphs of the
+// mix take 3.98 ms as picked and 3.49 with all in the union.
+//
+// kUnionFixed: 1 to 64 graphs of 1,024 to 24,000 vertices (G(n, 4n), grids,
+// geometric graphs), either way.  With 1e5 one G(10000, 40000) took a block and
+// 146 us (130 when all such batches were a union, 96 with the union now); with
+// 7e4, 32 grids of 30,000 vertices go to the union, 208 us, where
+// blocks take 166.
+//
+// Skewed graphs cost a block more, for their many rounds and long rows: 4.4 to
+// 5.4 ns a vertex or entry on R-MAT-B of 4,096 to 131,072 vertices against 1.2
+// to 2.3 on the graphs above and 2.3 to 3.1 on R-MAT-G, and the union 1.9 times
+// as much.  A batch is taken as skewed when one row in 200 is longer than 121
+// (R-MAT-B 1.1 to 2.5 %, R-MAT-G and the mix at most 0.14): four R-MAT-B of 4,096
+// vertices 323 us in blocks, 238 in the union; sixteen of 8,192, 607 and 397.
+constexpr double kUnionFixed = 8.8e4, kUnionFactor = 2.5, kSkewedBlock = 2.5, kSkewedUnion = 1.9;
 
 int32_t split_batch(const std::vector<int32_t>& order, const int64_t* voff, const int64_t* eoff, int sms,
-                    int64_t shared_vertices) {
+                    int64_t shared_vertices, bool skewed) {
     const int32_t G = (int32_t)order.size();
+    const double block = skewed ? kSkewedBlock : 1.0, whole = kUnionFactor * (skewed ? kSkewedUnion : 1.0);
     auto work = [&](int32_t i) {
         const int32_t g = order[(size_t)i];
         return (double)((voff[g + 1] - voff[g]) + (eoff[g + 1] - eoff[g]));
     };
     auto alone = [&](int32_t i) {
         const int32_t g = order[(size_t)i];
-        return work(i) * (voff[g + 1] - voff[g] > shared_vertices ? 2.0 : 1.0);
+        return work(i) * block * (voff[g + 1] - voff[g] > shared_vertices ? 2.0 : 1.0);
     };
     // largest single-block cost from i on
     std::vector<double> most((size_t)G + 1, 0.0);
@@ -1223,7 +1239,7 @@ int32_t split_batch(const std::vector<int32_t>& order, const int64_t* voff, cons
     for (int32_t i = 0; i < G; ++i) {
         big += work(i);
         rest -= alone(i);
-        const double cost = kUnionFixed + kUnionFactor * big / sms + std::max(rest / sms, most[(size_t)i + 1]);
+        const double cost = kUnionFixed + whole * big / sms + std::max(rest / sms, most[(size_t)i + 1]);
         if (cost < best_cost) {
             best_cost = cost;
             best = i + 1;
@@ -1404,7 +1420,8 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     b->mode = b->o.batch_mode;
     if (b->mode == 0) {
         nbig = split_batch(order, voff_h, eoff_h, b->sms,
-                           b->o.local_shared_bytes > 0 ? b->o.local_shared_bytes : kLocalSharedDefault);
+                           b->o.local_shared_bytes > 0 ? b->o.local_shared_bytes : kLocalSharedDefault,
+                           (int64_t)b->hs.over16 * 200 >= N);
         b->mode = nbig < G ? 2 : 1;
     }
     if (b->mode == 2) {

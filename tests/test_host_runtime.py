@@ -29,7 +29,10 @@ def lib(tmp_path_factory):
                                   ctypes.POINTER(vp)]
     h.gc_batch_destroy.argtypes = [vp]
     h.gc_color_ex.argtypes = [vp, vp, i32, vp, vp, vp, vp, vp, ctypes.POINTER(gc.Options), vp, i32]
+    h.gc_validate_csr.argtypes = [vp, vp, i32, vp]
     h.gc_last_phase_ms.argtypes = [vp, i32]
+    h.gc_batch_mode.argtypes = [vp]
+    h.fake_result.argtypes = [ctypes.c_char_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_uint32]
     h.gc_batch_status.argtypes = [vp, vp, vp, vp]
     h.gc_batch_round_stats.argtypes = [vp, vp, vp, i32, vp, vp]
     h.gc_batch_workspace_bytes.argtypes = [vp]
@@ -38,6 +41,7 @@ def lib(tmp_path_factory):
     h.fake_bytes_taken.restype = ctypes.c_size_t
     h.fake_pool_bytes.restype = ctypes.c_size_t
     h.fake_capacity.argtypes = [ctypes.c_size_t]
+    h.fake_grid.argtypes = [ctypes.c_char_p]
     h.fake_kernel_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]
     yield h
     h.gc_release()
@@ -170,3 +174,31 @@ def test_large_plans_do_not_go_through_the_pool(lib):
         b.close()
         assert lib.fake_pool_bytes() == 0 and lib.fake_misuse() == 0
     lib.gc_release()
+
+
+STATS_ARG, STATS_CAP, STATS_OVER = 5, 16, 28   # stats_kernel's record: cap[0..1], over2, over8, over16 (bytes)
+
+
+@pytest.mark.parametrize("sizes, skewed, mode", [
+    ([85000], False, 2), ([90000], False, 1),            # one graph: a block up to about 89,500 vertices and entries
+    ([90000] * 32, False, 2), ([150000] * 32, False, 2),
+    ([150000] * 8, False, 1), ([150000] * 64, False, 2),
+    ([62500] * 4, False, 2), ([62500] * 4, True, 1), ([62500] * 64, True, 2),
+    ([30000], True, 2), ([128000] * 16, True, 1), ([128000] * 64, True, 2),
+])
+def test_split_of_a_batch_of_equal_graphs(lib, sizes, skewed, mode):
+    """Where the library's choice between a block a graph and one union changes, for even graphs and
+    for batches with one row in 200 longer than 121 (measured on both sides; the graphs here have no
+    entries, so their sizes stand for vertices and entries together)."""
+    lib.fake_no_results()
+    try:
+        if skewed:
+            for off in (STATS_CAP, STATS_CAP + 4, STATS_OVER, STATS_OVER + 4, STATS_OVER + 8):
+                lib.fake_result(b"stats_kernel", STATS_ARG, off, sum(sizes) // 200 + 1)
+        b = EdgelessBatch(lib, sizes)
+        assert b.rc == gc.GC_OK
+        assert lib.gc_batch_mode(b.plan) == mode
+        b.close()
+    finally:
+        lib.fake_no_results()
+        lib.gc_release()
