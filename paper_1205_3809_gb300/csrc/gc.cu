@@ -579,7 +579,8 @@ int scan_locked(const int32_t* rowptr, const int32_t* colidx, int32_t n, int32_t
     if (timed) GC_CUDA(cudaEventRecord(dc.ev[1], s));
     if (validate) {
         if (hin) GC_CUDA(cudaStreamWaitEvent(s, dc.chunk_ev[hin->nchunks - 1], 0));
-        gc::validate_kernel<<<grid, 256, 0, s>>>(rowptr, colidx, n, stats, out);
+        const int vgrid = (int)std::min<int64_t>(((int64_t)n + 7) / 8, (int64_t)dc.sms * 8);  // at most a warp per row
+        gc::validate_kernel<<<vgrid, 256, 0, s>>>(rowptr, colidx, n, stats, out);
         GC_CUDA(cudaGetLastError());
         *launches += 1;
         if (timed) GC_CUDA(cudaEventRecord(dc.ev[4], s));

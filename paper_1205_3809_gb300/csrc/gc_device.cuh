@@ -2005,15 +2005,19 @@ __device__ __forceinline__ uint64_t asymmetry(int32_t v, int32_t w) {
     return v < w ? h : 0ull - h;
 }
 
-// Range, self-loop and symmetry checks of every entry.  A warp takes 32 rows:
-// those of up to kPass1Flat entries are read as one flat, coalesced range (as
-// in pass 1), longer ones by the whole warp in turn.  Runs behind the setup
-// scan and does nothing when that found the row starts unusable.
+// Range, self-loop and symmetry checks of every entry.  A warp takes up to 32
+// rows: those of up to kPass1Flat entries are read as one flat, coalesced range,
+// longer ones by the whole warp in turn.  Fewer rows (a power of two) when that
+// would leave warps without any, as long as they hold 128 entries, so that a
+// graph of few long rows is spread over the GPU.  Runs behind the setup scan and
+// does nothing when that found the row starts unusable.
 //
 // Bound: the hash, some 25 instructions an entry; the entries are read once.  A
 // warp per row (4 of 32 lanes on a mesh), two hashes an entry and two global
 // atomics a thread, waited for on its own, cost 0.17 ms more on the 4.0 M
-// entries of a 997,399-vertex mesh (a checked call 0.42 ms, now 0.26).
+// entries of a 997,399-vertex mesh (a checked call 0.42 ms, now 0.26).  With 32
+// rows always, K(2000, 2000), 4,000 rows of 2,000 entries, took 217 us, now 20;
+// G(3000, 12000) 4.3, now 3.7; G(400000, 6000000) 38.9, now 37.0.
 __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ colidx, int32_t n,
                                                        const Stats* __restrict__ scan, ValidateOut* out) {
@@ -2022,11 +2026,15 @@ __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict
     };
     __shared__ Smem s_row[8];
     __shared__ unsigned long long s_sum[8];
-    if (__ldcg(&scan->bad) || __ldcg(&scan->nnz) < 0 || (__ldcg(&scan->nnz) > 0 && !colidx)) return;
+    // (read through L1: a word that every warp of the GPU takes from L2 costs 4 us)
+    const int bad_rows = __ldg(&scan->bad), nnz = __ldg(&scan->nnz);
+    if (bad_rows || nnz < 0 || (nnz > 0 && !colidx)) return;
     const unsigned lane = lane_id(), wib = threadIdx.x >> 5;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t ntasks = ((int64_t)n + 31) / 32;
+    const float most = fmaxf((float)n / (float)W, 128.f * (float)n / (float)max(nnz, 1));
+    const int shift = 31 - __clz((int)fminf(32.f, fmaxf(1.f, most))), rows = 1 << shift;
+    const int64_t ntasks = ((int64_t)n + rows - 1) >> shift;
     const uint64_t pol = policy_evict_first();
     uint64_t sum = 0;
     bool bad = false, loop = false;
@@ -2039,8 +2047,8 @@ __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict
         }
     };
     for (int64_t t = gw; t < ntasks; t += W) {
-        const int64_t vv = t * 32 + lane;
-        const bool valid = vv < n;
+        const int64_t vv = (t << shift) + lane;
+        const bool valid = (int)lane < rows && vv < n;
         const int32_t v = valid ? (int32_t)vv : 0;
         const int32_t b = valid ? __ldg(rowptr + v) : 0;
         const int32_t d = valid ? __ldg(rowptr + v + 1) - b : 0;
@@ -2073,13 +2081,13 @@ __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (F0 + 32 * u + (int32_t)lane < D) entry((int32_t)(t * 32 + own[u]), w[u]);
+                if (F0 + 32 * u + (int32_t)lane < D) entry((int32_t)(t << shift) + own[u], w[u]);
         }
         unsigned big = __ballot_sync(kFull, d > kPass1Flat);
         while (big) {
             const int j = __ffs(big) - 1;
             big &= big - 1;
-            const int32_t vj = (int32_t)(t * 32 + j);
+            const int32_t vj = (int32_t)(t << shift) + j;
             const int64_t bj = __shfl_sync(kFull, b, j), ej = bj + __shfl_sync(kFull, d, j);
             for (int64_t i = bj + lane; i < ej; i += 32 * 8) {
                 int32_t w[8];

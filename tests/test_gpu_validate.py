@@ -27,6 +27,8 @@ GRAPHS = [
     lambda: gg.path(2), lambda: gg.path(65), lambda: gg.grid2d(37, 53, 1), lambda: gg.gnm(5000, 40000, 2),
     lambda: gg.complete(256), lambda: gg.complete(257), lambda: gg.complete(258),  # rows of 255, 256, 257
     lambda: gg.star(3001, 17), lambda: gg.rmat(12, 16, gg.RMAT_B, 3),
+    # 16, 2 and 1 rows a warp (32, 8 and 4 above), the last with rows on both sides of 256
+    lambda: gg.gnm(999, 3900, 4), lambda: gg.gnm(1501, 37000, 5), lambda: gg.gnm(301, 38600, 6),
 ]
 
 

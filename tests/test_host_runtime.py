@@ -176,6 +176,14 @@ def test_large_plans_do_not_go_through_the_pool(lib):
     lib.gc_release()
 
 
+@pytest.mark.parametrize("n", [1, 9, 1500, 4000, 9728, 10000, 3000000])
+def test_entry_checks_have_a_warp_for_every_row_of_a_small_graph(lib, n):
+    """Blocks of eight warps, a warp a row as far as the GPU holds them (152 SMs, eight blocks each)."""
+    rowptr = np.zeros(n + 1, np.int32)
+    assert lib.gc_validate_csr(_p(rowptr), None, n, None) == gc.GC_OK
+    assert lib.fake_grid(b"validate_kernel") == min((n + 7) // 8, 152 * 8)
+
+
 STATS_ARG, STATS_CAP, STATS_OVER = 5, 16, 28   # stats_kernel's record: cap[0..1], over2, over8, over16 (bytes)
 
 
