@@ -174,19 +174,25 @@ __device__ __forceinline__ void layer_pairs(const float (*w)[kRow], const float*
         }
 }
 
-// kForwardRows samples per thread, kForwardUnits units at a time.
+// R samples per thread, kForwardUnits units at a time.
 // Bound: the fp32 multiply-adds (1,248 a sample; 70 % of the fp32 rate) and the
-// 16-byte weight reads beside them, one for kForwardRows * 4 multiply-adds.
-// 4,194,301 samples take 197 us, 16,000,001 take 719 (one sample a thread,
+// 16-byte weight reads beside them, one for R * 4 multiply-adds.  4,194,301
+// samples take 195 us, 16,000,001 take 719 with R = 4 (one sample a thread,
 // scalar arithmetic: 319 for the first; two samples with activations as floats,
 // 128 registers: 223 and 818; two as pairs: 206 and 745; three 201 and 736;
-// four, 8 or 32 units at a time: 199 and 217).  Up to 155,648 samples (one
-// block per SM, once around) all of these take the same 16 us, launch included.
-constexpr int kForwardRows = 4, kForwardUnits = 16, kForwardThreads = 256, kForwardBlocks = 1;
-__global__ void __launch_bounds__(kForwardThreads, kForwardBlocks) mlp_forward_kernel(const float* __restrict__ params,
+// four, 8 or 32 units at a time: 199 and 217).
+//
+// A thread takes its R samples whether they are there or not, so R is the
+// smallest of 1, 2 and 4 that covers n in one turn of the grid (one block per
+// SM).  On the device, 1,000 to 38,912 samples take 5.4 to 5.6 us
+// with R = 1 and 9.9 with 4 (5.2 to 5.5 before any of this, a sample a thread),
+// 39,000 to 77,824 take 6.9 with R = 2 and 9.9 with 4 (6.4 to 8.2 before).
+constexpr int kForwardUnits = 16, kForwardThreads = 256;
+template <int R>
+__global__ void __launch_bounds__(kForwardThreads, 1) mlp_forward_kernel(const float* __restrict__ params,
                                                           const float* __restrict__ x, int64_t n,
                                                           float* __restrict__ y) {
-    constexpr int R = kForwardRows, J = kForwardUnits;
+    constexpr int J = kForwardUnits;
     __shared__ ForwardParams s;
     load_forward_params(params, s);
     __syncthreads();
@@ -633,8 +639,16 @@ int gc_features(const int32_t* rowptr, const int32_t* colidx, int32_t n, float* 
 int gc_mlp_forward(const float* params, const float* x, int64_t n, float* y, void* stream) {
     if (n < 0 || !params || (n > 0 && (!x || !y))) return GC_ERR_INVALID;
     if (n == 0) return GC_OK;
-    mlp_forward_kernel<<<grid_for(n, kForwardThreads * kForwardRows, sm_count() * kForwardBlocks), kForwardThreads, 0,
-                         (cudaStream_t)stream>>>(params, x, n, y);
+    const cudaStream_t s = (cudaStream_t)stream;
+    const int most = sm_count();
+    const int64_t turn = (int64_t)most * kForwardThreads;
+    if (n <= turn) {
+        mlp_forward_kernel<1><<<grid_for(n, kForwardThreads, most), kForwardThreads, 0, s>>>(params, x, n, y);
+    } else if (n <= 2 * turn) {
+        mlp_forward_kernel<2><<<most, kForwardThreads, 0, s>>>(params, x, n, y);
+    } else {
+        mlp_forward_kernel<4><<<most, kForwardThreads, 0, s>>>(params, x, n, y);
+    }
     return check_launch();
 }
 

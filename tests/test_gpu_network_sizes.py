@@ -28,8 +28,9 @@ def _uniform(seed, stream, count, lo, hi):
     return (lo + (hi - lo) * u).astype(np.float32)
 
 
-# four samples a thread, 256 threads a block, a block an SM (152 of them): 155,648 a grid
-@pytest.mark.parametrize("n", [1, 2, 255, 257, 511, 512, 513, 1023, 1025, 155647, 155649])
+# 256 threads a block, a block an SM (152 of them): one sample a thread up to 38,912, two up to
+# 77,824, then four, and 155,648 in a turn of the grid
+@pytest.mark.parametrize("n", [1, 2, 255, 257, 511, 512, 513, 1023, 1025, 38912, 38913, 77824, 77825, 155647, 155649])
 def test_forward_sizes(gcpkg, n):
     p = _uniform(n, 7, L.N_PARAMS, -0.3, 0.3)
     x = _uniform(n + 1, 9, n * L.N_IN, -2.0, 24.0).reshape(n, L.N_IN)
