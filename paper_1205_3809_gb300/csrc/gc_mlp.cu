@@ -481,7 +481,7 @@ struct RowDegrees {
 struct FeatureGraph {
     const int32_t* __restrict__ rowptr;
     const int32_t* __restrict__ colidx;
-    int32_t n, nnz;
+    int32_t nnz;
     uint32_t col_mis;  // entries from a 32-byte boundary to colidx
 
     // (one line, most often one sector)
@@ -514,51 +514,81 @@ struct FeatureGraph {
     }
 };
 
-// The rows of a warp's 32 vertices (one per lane), L lanes each, 32 / L side by side.
-template <int L>
-__device__ __forceinline__ void small_rows(const FeatureGraph& g, unsigned lane, int32_t b, int32_t d,
-                                           RowDegrees& mine) {
-#pragma unroll 1
-    for (unsigned s = 0; s < L; ++s) {
-        const int src = (int)((lane & ~(unsigned)(L - 1)) | s);
-        RowDegrees r = g.row<L>(__shfl_sync(0xffffffffu, b, src), __shfl_sync(0xffffffffu, d, src), lane % L);
-        r.combine<L>();
-        if (lane % L == s) mine = r;
+// Its own row by each lane, four entries at a time.
+__device__ __forceinline__ RowDegrees lane_row(const FeatureGraph& g, int32_t b, int32_t d) {
+    RowDegrees r;
+    for (int32_t i = 0; i < d; i += 4) {
+        int32_t w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = i + u < d ? __ldg(g.colidx + b + i + u) : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = i + u < d ? g.degree(w[u]) : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (w[u] >= 0) r.add(w[u]);
     }
+    return r;
 }
 
-// A warp takes 32 vertices.  Rows of up to 25 entries are read by 4 lanes, 8
-// rows side by side (by 2 lanes when none of the 32 is longer than 9), rows of
-// up to 121 by 16 lanes, longer ones by the whole warp, a 32-byte chunk a lane
-// at a time.
+// The rows of a warp's vertices by four lanes each, eight side by side, in
+// `steps` steps: lane s of each group of four holds the row of step s.
+__device__ __forceinline__ RowDegrees small_rows(const FeatureGraph& g, unsigned lane, int32_t b, int32_t d, unsigned steps) {
+    RowDegrees mine;
+#pragma unroll 1
+    for (unsigned s = 0; s < steps; ++s) {
+        const int src = (int)((lane & ~3u) | s);
+        RowDegrees r = g.row<4>(__shfl_sync(0xffffffffu, b, src), __shfl_sync(0xffffffffu, d, src), lane & 3u);
+        r.combine<4>();
+        if ((lane & 3u) == s) mine = r;
+    }
+    return mine;
+}
+
+// A warp takes 32 vertices.  When none of their rows is longer than 12, each lane
+// reads its own; otherwise rows of up to 57 entries are read by 4 lanes, 8 rows
+// side by side, rows of up to 121 by 16 lanes and longer ones by the whole warp,
+// a 32-byte chunk a lane at a time.  A small graph (rows of 6 entries and more on
+// average) is dealt out 8 or 16 vertices a warp (STEPS = 1, 2: in as many steps of
+// 8 rows), so that all SMs have some.
 //
 // Bound: one random L2 sector per entry (the neighbour's row starts; a probe
 // that only gathers reaches 208 G/s).  With a thread per short row and the
 // longest rows read 32 entries at a time with two waits each, R-MAT-B of 2^22
-// vertices took 446 us, now 394; R-MAT-ER 389 us, now 324 (207 G entries/s).
+// vertices took 441 us, now 390; R-MAT-ER 386 us, now 320 (208 G entries/s).
 // Six blocks an SM: with four (62 registers) 436 us for the first.
-__global__ void __launch_bounds__(256, 6) features_kernel(const int32_t* __restrict__ rowptr,
+//
+// In the natural order of a mesh or band neighbouring lanes gather neighbouring
+// words when each has a row of its own: grid of 2,000 x 2,000 67.8 us (thread per
+// row, 8 entries at a time), 89.7 (two lanes in chunks), 56.3 now; 12 entries a
+// row 43.4, 79.3, 40; 26 entries 42.4, 168 (16 lanes), 48 (4 lanes, two chunks
+// each).  With own rows up to 16, R-MAT and G(n, m) are unchanged, but a geometric
+// graph of 1M vertices in random order (8 a row) takes 49.6 us, not 46.2.
+// Few vertices: G(3000, 12000) 3.3 us, 5.5 in warps of 32, 3.3; K(1500) 115, 132, 33.
+constexpr int kFeatureBlocks = 6;
+template <unsigned STEPS>
+__global__ void __launch_bounds__(256, kFeatureBlocks) features_kernel(const int32_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ colidx, int32_t n,
                                                        float* __restrict__ out) {
-    constexpr int32_t kTiny = 8 * 2 - 7, kSmall = 8 * 4 - 7, kMid = 8 * 16 - 7;
+    constexpr int32_t kOwn = 12, kSmall = 57, kMid = 8 * 16 - 7;
     FeatureGraph g;
     g.rowptr = rowptr;
     g.colidx = colidx;
-    g.n = n;
     g.nnz = __ldg(rowptr + n);
     g.col_mis = (uint32_t)((uintptr_t)colidx >> 2) & 7u;
     const unsigned lane = threadIdx.x & 31u;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t base = gw * 32; base < n; base += W * 32) {
-        const int64_t v = base + lane;
-        const bool valid = v < n;
+    const unsigned steps = STEPS == 4u || g.nnz / 6 >= n ? STEPS : 4u;
+    const unsigned rows = 8u * steps, own = (lane >> 2) * steps + (lane & 3u);
+    for (int64_t base = gw * rows; base < n; base += W * rows) {
+        const int64_t v = base + own;
+        const bool valid = (lane & 3u) < steps && v < n;
         const int32_t b = valid ? __ldg(rowptr + v) : 0, d = valid ? __ldg(rowptr + v + 1) - b : 0;
         RowDegrees mine;
-        if (__all_sync(0xffffffffu, d <= kTiny)) {
-            small_rows<2>(g, lane, b, d, mine);
+        if (steps == 4u && __all_sync(0xffffffffu, d <= kOwn)) {
+            mine = lane_row(g, b, d);
         } else {
-            small_rows<4>(g, lane, b, d <= kSmall ? d : 0, mine);
+            mine = small_rows(g, lane, b, d <= kSmall ? d : 0, steps);
         }
         unsigned mid = __ballot_sync(0xffffffffu, d > kSmall && d <= kMid);
         while (mid) {
@@ -631,8 +661,16 @@ extern "C" {
 int gc_features(const int32_t* rowptr, const int32_t* colidx, int32_t n, float* features, void* stream) {
     if (n < 0 || (n > 0 && (!rowptr || !features))) return GC_ERR_INVALID;
     if (n == 0) return GC_OK;
-    features_kernel<<<grid_for((int64_t)n, 256, sm_count() * 16), 256, 0, (cudaStream_t)stream>>>(
-        rowptr, colidx, n, features);
+    const int sms = sm_count();
+    const int64_t warps = (int64_t)sms * kFeatureBlocks * 8;
+    const cudaStream_t s = (cudaStream_t)stream;
+    if (n <= 8 * warps) {
+        features_kernel<1><<<grid_for((int64_t)n, 64, sms * 16), 256, 0, s>>>(rowptr, colidx, n, features);
+    } else if (n <= 16 * warps) {
+        features_kernel<2><<<grid_for((int64_t)n, 128, sms * 16), 256, 0, s>>>(rowptr, colidx, n, features);
+    } else {
+        features_kernel<4><<<grid_for((int64_t)n, 256, sms * 16), 256, 0, s>>>(rowptr, colidx, n, features);
+    }
     return check_launch();
 }
 

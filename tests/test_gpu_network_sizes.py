@@ -84,8 +84,9 @@ def _rows_of(degree, seed):
     return gg.from_edges(n, perm[u], perm[v])
 
 
-# rows read by 4 lanes (up to 25), 16 lanes (up to 121) or the warp, at every alignment of both arrays
-@pytest.mark.parametrize("degree", [1, 8, 25, 26, 57, 120, 121, 122, 255, 257, 1000])
+# rows read by their own lane (up to 12), 4 lanes (up to 57), 16 lanes (up to 121) or the warp, at every
+# alignment of both arrays
+@pytest.mark.parametrize("degree", [1, 8, 12, 13, 25, 26, 57, 58, 120, 121, 122, 255, 257, 1000])
 def test_feature_rows(gcpkg, degree):
     g = _rows_of(degree, 40 + degree)
     want = L.features(g.rowptr, g.colidx)
@@ -97,3 +98,22 @@ def test_feature_rows(gcpkg, degree):
         out = torch.empty(g.n * 6 + 1, dtype=torch.float32, device="cuda")[shift % 2:][:g.n * 6].view(g.n, 6)
         got = gcpkg.features(rp, ci, out=out).cpu().numpy()
         assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), (degree, shift)
+
+
+# vertices a warp takes: 8 up to 58,368 vertices, 16 up to 116,736, then 32; 32 below 6 entries a row
+@pytest.mark.parametrize("n", [1, 7, 9, 31, 33, 1000, 58367, 58368, 58369, 116736, 116737, 120001])
+def test_feature_vertices(gcpkg, n):
+    for edges in (2 * n, 3 * n, 5 * n):
+        g = gg.gnm(n, min(edges, n * (n - 1) // 2), n)
+        want = L.features(g.rowptr, g.colidx)
+        got = gcpkg.features(_dev(g.rowptr), _dev(g.colidx)).cpu().numpy()
+        assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), g.name
+
+
+def test_feature_rows_of_every_kind_together(gcpkg):
+    """Long, middle and short rows in one graph, in warps of 8, 16 and 32 vertices."""
+    for scale, ef in ((11, 16), (16, 8), (17, 8)):
+        g = gg.rmat(scale, ef, gg.RMAT_B, scale)
+        want = L.features(g.rowptr, g.colidx)
+        got = gcpkg.features(_dev(g.rowptr), _dev(g.colidx)).cpu().numpy()
+        assert np.array_equal(got.view(np.uint32), want.view(np.uint32)), g.name
