@@ -777,7 +777,19 @@ __global__ void __launch_bounds__(256, 4) pass1_kernel(Params<T> p, int32_t v_be
                 if (cls[i] == c) at[i] = base + __popc(bal & below);
             }
             hub_at[i] = 0ull;
-            if (cls[i] == 6) hub_at[i] = atomicAdd(&s_hub, pair_count(1u, (unsigned)(d[i] + kChunk - 1) / kChunk));
+            const unsigned hubs = __ballot_sync(kFull, cls[i] == 6);
+            if (hubs) {
+                const unsigned chunks = cls[i] == 6 ? (unsigned)(d[i] + kChunk - 1) / kChunk : 0u;
+                unsigned upto = chunks;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned x = __shfl_up_sync(kFull, upto, o);
+                    if ((int)lane >= o) upto += x;
+                }
+                unsigned long long base = 0ull;
+                if (lane == 31u) base = atomicAdd(&s_hub, pair_count(__popc(hubs), upto));
+                hub_at[i] = __shfl_sync(kFull, base, 31) + pair_count(__popc(hubs & below), upto - chunks);
+            }
         }
         __syncthreads();
         if (tid == 0 && (s_cnt[0] | s_cnt[1])) {

@@ -25,13 +25,14 @@ def gcpkg():
 
 
 def _cliques(degree, seed):
-    """Cliques with rows of `degree`, some with one edge missing, and a sparse random graph around
-    them; ids shuffled."""
+    """Cliques with rows of `degree`, two of them with edges missing, and a sparse random graph
+    around them; ids shuffled.  About 300 such rows at least, so that a task of one block's warps
+    takes all the steps it may."""
     k = degree + 1
     u, v = np.triu_indices(k, 1)
     parts, n = [], 0
-    for i in range(5):
-        drop = 0 if i < 3 else 1 + i % max(1, u.size - 1)
+    for i in range(max(5, 300 // k + 1)):
+        drop = 0 if i not in (3, 4) else 1 + i % max(1, u.size - 1)
         parts.append((u[drop:] + n, v[drop:] + n))
         n += k
     g = gg.gnm(400, 1200, seed)
@@ -51,11 +52,13 @@ def test_bin_edges(gcpkg, degree, keyed):
     want = oracle.iterative(g.rowptr, g.colidx, prio)
     rp = torch.from_numpy(g.rowptr).cuda()
     pr = torch.from_numpy(prio.view(np.int32)).cuda() if keyed else None
+    # one block for all rounds, and a launch per round: few warps, so several steps a task
+    few = ({"tail_volume": 1 << 30}, {"loop_mode": 1}, {"tail_volume": 1 << 30, "color_bits": 32})
     for shift in (0, 1, 6):  # the adjacency array at other alignments, its ends at other chunks
         buf = torch.full((g.nnz + 16,), 1 << 30, dtype=torch.int32, device="cuda")
         ci = buf[shift:shift + g.nnz]
         ci.copy_(torch.from_numpy(g.colidx))
-        for options in (None, {"small_max_degree": 8}, {"medium_max_degree": 64}, {"color_bits": 32}):
+        for options in (None, {"small_max_degree": 8}, {"medium_max_degree": 64}, {"color_bits": 32}) + few:
             got = gcpkg.color(rp, ci, pr, options=options, round_sizes=True)
             assert (got.ncolors, got.rounds) == (want.ncolors, want.rounds), (g.name, shift, options)
             assert np.array_equal(got.colors.cpu().numpy(), want.colors)
@@ -76,6 +79,8 @@ def _reordered(g, order, seed):
 @pytest.mark.parametrize("make", [
     lambda: _cliques(9, 3), lambda: gg.star(34, 0), lambda: gg.star(258, 257), lambda: gg.star(259, 0),
     lambda: gg.complete(257), lambda: gg.star(5000, 0), lambda: gg.rmat(13, 8, gg.RMAT_B, 3), lambda: gg.gnm(3000, 40000, 5),
+    # whole warps of rows of one and of two chunks to append
+    lambda: gg.complete(300), lambda: gg.complete_bipartite(1100, 270),
 ])
 def test_rows_in_any_order(gcpkg, make, order):
     """Round 1 looks at a row's first chunk first: rows whose only preceding neighbour comes late, at
@@ -93,5 +98,35 @@ def test_rows_in_any_order(gcpkg, make, order):
             dev.copy_(torch.from_numpy(ci))
             got = gcpkg.color(rp, dev, pr, round_sizes=True)
             assert (got.ncolors, got.rounds) == (want.ncolors, want.rounds), (g.name, order, shift)
+            assert np.array_equal(got.colors.cpu().numpy(), want.colors)
+            assert np.array_equal(got.round_sizes, want.round_sizes)
+
+
+def test_four_vertices_a_thread_in_round_1(gcpkg):
+    """A graph large enough for round 1's wide form (1,024 vertices for every SM), not a multiple of
+    its blocks: skewed, sparse and edgeless parts and long rows, entries shuffled in their rows, with
+    and without keys, at two alignments."""
+    parts = [gg.rmat(17, 8, gg.RMAT_B, 3), gg.gnm(70001, 250000, 4), gg.star(3000, 7), gg.star(300, 299), gg.edgeless(501)]
+    n, us, vs = 0, [], []
+    for g in parts:
+        us.append(np.repeat(np.arange(g.n, dtype=np.int64), g.degrees) + n)
+        vs.append(g.colidx.astype(np.int64) + n)
+        n += g.n
+    assert n >= 152 * 1024 and n % 1024
+    perm = gg.permutation(n, 9)
+    g = gg.from_edges(n, perm[np.concatenate(us)], perm[np.concatenate(vs)])
+    row = np.repeat(np.arange(n), g.degrees)
+    ci = g.colidx[np.lexsort((np.random.default_rng(5).random(g.nnz), row))]
+    keys = (gg.draws(6, 3, n) % np.uint64(9)).astype(np.uint32)
+    rp = torch.from_numpy(g.rowptr).cuda()
+    for prio in (None, keys):
+        want = oracle.iterative(g.rowptr, ci, prio)
+        pr = None if prio is None else torch.from_numpy(prio.view(np.int32)).cuda()
+        for shift in (0, 5):
+            buf = torch.full((g.nnz + 16,), 1 << 30, dtype=torch.int32, device="cuda")
+            dev = buf[shift:shift + g.nnz]
+            dev.copy_(torch.from_numpy(ci))
+            got = gcpkg.color(rp, dev, pr, round_sizes=True)
+            assert (got.ncolors, got.rounds) == (want.ncolors, want.rounds)
             assert np.array_equal(got.colors.cpu().numpy(), want.colors)
             assert np.array_equal(got.round_sizes, want.round_sizes)
