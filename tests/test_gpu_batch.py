@@ -377,7 +377,7 @@ def test_largest_graphs_split_off(gcpkg, keyed, large):
 
 def test_plan_memory_is_shared_safely_and_given_back(gcpkg):
     """Plans made, run and freed in one call by several threads, each on its own stream, share a
-    pool of device memory: every result is its own batch's, and the pool is empty after release()."""
+    pool of device memory: every result is its own batch's."""
     import threading
     gcpkg.release()
     torch.cuda.synchronize()
@@ -409,3 +409,27 @@ def test_plan_memory_is_shared_safely_and_given_back(gcpkg):
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
+
+
+def test_plan_memory_is_kept_and_given_back(gcpkg):
+    """The pool keeps a plan's memory (about 190 MB here) for the next plan, until release()."""
+    gcpkg.release()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    n, count = 100000, 40
+    rp = torch.zeros(count * (n + 1), dtype=torch.int32, device="cuda")
+    ci = torch.zeros(1, dtype=torch.int32, device="cuda")[:0]
+    free = [torch.cuda.mem_get_info()[0]]
+    b = gcpkg.Batch(rp, ci, np.arange(count + 1) * n, np.zeros(count + 1, np.int64), options={"batch_mode": 2})
+    held = b.workspace_bytes
+    assert 150 << 20 < held < 250 << 20
+    b.run()
+    assert b.status() == (1, 1)
+    torch.cuda.synchronize()
+    free.append(torch.cuda.mem_get_info()[0])
+    b.close()
+    free.append(torch.cuda.mem_get_info()[0])
+    gcpkg.release()
+    free.append(torch.cuda.mem_get_info()[0])
+    slack = 64 << 20
+    assert free[0] - free[1] >= held and free[0] - free[2] >= held - slack and free[0] - free[3] <= slack, free
