@@ -1323,13 +1323,10 @@ __device__ __forceinline__ void mid_task(const Params<T>& p, const PassIO<T>& io
 // its vertex's window in shared memory, flags a conflict, and, if the
 // neighbour has not settled, is copied to the next round's list at the
 // vertex's running write position.  Afterwards each lane decides its own
-// vertex.  Round 2 with keys (F: keys are compared and kept as a bit of the
-// entry) is an instance of its own here and in the two functions that
-// follow; the later rounds then run without its branches, which matters
-// where most entries stand in lists: with keys by features and R-MAT-B at
-// 4M vertices 10.63 ms in one instance, 10.35 ms in two; short-row graphs
-// (G(1M, 8M), R-MAT-G at 8M) are unchanged.
-template <typename T, bool P, bool F>  // P: a priority array is given; F: and this is round 2
+// vertex.  Round 2 has no S entries: pass 1 gives rows of up to s_max to the L2,
+// L4 and L8 bins, so every vertex here has a static mask, and with keys every
+// entry carries its precedence bit.
+template <typename T, bool P>  // P: a priority array is given
 __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& io, int4 en,
                                           FlatSmem& sm, int& maxc, unsigned& vol) {
     const unsigned lane = lane_id();
@@ -1338,8 +1335,8 @@ __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& i
     const int32_t b = en.y;
     const int32_t len = valid ? en.z : 0;
     const uint32_t cv = valid ? word_color(ld_color(io.Xc + v, io.pol_col)) : 0u;
-    // static mask of v (none yet in round 2)
-    if (valid && !io.first) {
+    // static mask of v
+    if (valid) {
         const uint4* src = reinterpret_cast<const uint4*>(p.stat + (size_t)v * 8);
         const uint4 a = __ldcg(src), c = __ldcg(src + 1);
         sm.stat[0 * 32 + lane] = a.x; sm.stat[1 * 32 + lane] = a.y;
@@ -1403,22 +1400,8 @@ __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& i
             const bool in = f < D;
             const uint32_t col = word_color(c[u]);
             const bool settled = in && word_settled(c[u]);
-            // does this neighbour precede its owner?  Round 2 works it out (for the
-            // conflict test and for the bit of every entry it keeps); later rounds read
-            // the bit.
-            const int32_t wid = P ? entry_id(w[u]) : w[u];
-            bool pre = false;
-            if constexpr (!P) {
-                if (in && col == ocv) pre = wid < sm.vid[o];
-            } else if (in && (col == ocv || (F && !settled))) {
-                if constexpr (F) {
-                    const int32_t ov = sm.vid[o];
-                    pre = precedes(p.prio, wid, ov, __ldg(p.prio + ov));
-                } else {
-                    pre = w[u] < 0;
-                }
-            }
-            if (in && col == ocv && pre) atomicOr(&sm.conf, 1u << o);
+            // (with keys, an entry's bit says that it precedes its owner)
+            if (in && col == ocv && (P ? w[u] < 0 : w[u] < sm.vid[o])) atomicOr(&sm.conf, 1u << o);
             {
                 const unsigned idx = col - 1u;
                 if (in && idx < 256u)
@@ -1430,9 +1413,7 @@ __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& i
             const unsigned kb = __ballot_sync(kFull, keep);
             const unsigned below = kb & ((1u << lane) - 1u) & ~((1u << seglo[u]) - 1u);
             if (keep)
-                st_stream(io.rout + wbase + __popc(below),
-                          F ? (int32_t)((uint32_t)wid | (pre ? kPrecBit : 0u)) : w[u],
-                          io.pol_row);
+                st_stream(io.rout + wbase + __popc(below), w[u], io.pol_row);
             // my vertex's lanes in this batch: [lo, hi)
             const int32_t lo = max(0, min(32, off - base));
             const int32_t hi = max(0, min(32, off + len - base));
@@ -1494,7 +1475,11 @@ __device__ __forceinline__ void flat_task(const Params<T>& p, const PassIO<T>& i
 // shared word, which the flat walk does when most of a batch belongs to one
 // long list.  The decisions stay in the lane of their entry, and the task
 // appends its conflicting vertices to the next round with one atomic per
-// bin.
+// bin.  Round 2 with keys (F: keys are compared and kept as a bit of the entry)
+// is an instance of its own here and in hub_chunk; the later rounds then run
+// without its branches, which matters where most entries stand in lists: with
+// keys by features and R-MAT-B at 4M vertices 10.63 ms in one instance, 10.35 ms
+// in two; short-row graphs (G(1M, 8M), R-MAT-G at 8M) are unchanged.
 template <typename T, bool P, bool F>  // P: a priority array is given; F: and this is round 2
 __device__ __forceinline__ void vertex_task(const Params<T>& p, const PassIO<T>& io, int4 en,
                                             FlatSmem& sm, int& maxc, unsigned& vol) {
@@ -1810,9 +1795,11 @@ __device__ __forceinline__ TaskSplit split_round(const RoundSizes& r, unsigned W
 
 // One fused pass over U_k, shared among W warps (this warp is number gw).
 // Task t: first the H-bin chunks, then the M-bin entries, up to kMedPerTask
-// per task (fewer as the round shrinks), then the S-bin entries, 32 per task
-// (down to kShortPerTaskMin as the round shrinks); an S or H task reads at
-// most 1024 entries.  Warp gw takes tasks gw, gw + W, ... for half of its even
+// per task (fewer as the round shrinks), L16 and L8 entries in steps of 2 and 4
+// (up to kMidSteps of them a task), the S-bin entries, 32 per task (down to
+// kShortPerTaskMin as the round shrinks), then L4 and L2 entries in steps of 8
+// and 16 (up to 4 and 2); an S or H task reads at most 1024 entries.  Warp gw
+// takes tasks gw, gw + W, ... for half of its even
 // share (at least two); then, with a counter (ctr), it claims one task at a
 // time (nstat W + the counter's old value), so that warps that drew cheap
 // tasks take more and the round ends when the work does, not when the
@@ -1863,8 +1850,7 @@ __device__ __forceinline__ void run_pass(const Params<T>& p, int k, const RoundS
         } else if (t < q.e3) {
             mid_task<T, P, 8>(p, io, cur.e, q.s8, maxc, vol);
         } else if (t < q.e4) {
-            if (P && io.first) flat_task<T, P, P>(p, io, cur.e, s_flat[wib], maxc, vol);
-            else flat_task<T, P, false>(p, io, cur.e, s_flat[wib], maxc, vol);
+            flat_task<T, P>(p, io, cur.e, s_flat[wib], maxc, vol);
         } else if (t < q.e5) {
             tiny_task<T, P, 4>(p, io, cur.e, q.s4, maxc, vol);
         } else {
