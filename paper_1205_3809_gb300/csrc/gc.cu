@@ -1214,12 +1214,20 @@ constexpr int32_t kLocalSharedDefault = 164 * 1024;  // mode 2: bytes of shared 
 // as much.  A batch is taken as skewed when one row in 200 is longer than 121
 // (R-MAT-B 1.1 to 2.5 %, R-MAT-G and the mix at most 0.14): four R-MAT-B of 4,096
 // vertices 323 us in blocks, 238 in the union; sixteen of 8,192, 607 and 397.
-constexpr double kUnionFixed = 8.8e4, kUnionFactor = 2.5, kSkewedBlock = 2.5, kSkewedUnion = 1.9;
+//
+// With keys a block costs 1.5 times as much (it gathers a key for every neighbour
+// of the same color, in every round) and the union 1.2 times: four R-MAT-G of
+// 4,096 vertices 296 us in blocks, 165 in the union, 64 of 65,536 vertices 4,529
+// and 2,949.  Of 236 keyed batches of 1 to 128 even graphs, 20 were slower than
+// as a union before without these factors, by up to 48 %, and none is with them.
+constexpr double kUnionFixed = 8.8e4, kUnionFactor = 2.5, kSkewedBlock = 2.5, kSkewedUnion = 1.9, kKeyedBlock = 1.5,
+                 kKeyedUnion = 1.2;
 
 int32_t split_batch(const std::vector<int32_t>& order, const int64_t* voff, const int64_t* eoff, int sms,
-                    int64_t shared_vertices, bool skewed) {
+                    int64_t shared_vertices, bool skewed, bool keyed) {
     const int32_t G = (int32_t)order.size();
-    const double block = skewed ? kSkewedBlock : 1.0, whole = kUnionFactor * (skewed ? kSkewedUnion : 1.0);
+    const double block = (skewed ? kSkewedBlock : 1.0) * (keyed ? kKeyedBlock : 1.0);
+    const double whole = kUnionFactor * (skewed ? kSkewedUnion : 1.0) * (keyed ? kKeyedUnion : 1.0);
     auto work = [&](int32_t i) {
         const int32_t g = order[(size_t)i];
         return (double)((voff[g + 1] - voff[g]) + (eoff[g + 1] - eoff[g]));
@@ -1422,7 +1430,7 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     if (b->mode == 0) {
         nbig = split_batch(order, voff_h, eoff_h, b->sms,
                            b->o.local_shared_bytes > 0 ? b->o.local_shared_bytes : kLocalSharedDefault,
-                           (int64_t)b->hs.over16 * 200 >= N);
+                           (int64_t)b->hs.over16 * 200 >= N, prio != nullptr);
         b->mode = nbig < G ? 2 : 1;
     }
     if (b->mode == 2) {

@@ -187,23 +187,26 @@ def test_entry_checks_have_a_warp_for_every_row_of_a_small_graph(lib, n):
 STATS_ARG, STATS_CAP, STATS_OVER = 5, 16, 28   # stats_kernel's record: cap[0..1], over2, over8, over16 (bytes)
 
 
-@pytest.mark.parametrize("sizes, skewed, mode", [
-    ([85000], False, 2), ([90000], False, 1),            # one graph: a block up to about 89,500 vertices and entries
-    ([90000] * 32, False, 2), ([150000] * 32, False, 2),
-    ([150000] * 8, False, 1), ([150000] * 64, False, 2),
-    ([62500] * 4, False, 2), ([62500] * 4, True, 1), ([62500] * 64, True, 2),
-    ([30000], True, 2), ([128000] * 16, True, 1), ([128000] * 64, True, 2),
+@pytest.mark.parametrize("sizes, skewed, keyed, mode", [
+    ([85000], False, False, 2), ([90000], False, False, 1),   # one graph: a block up to about 89,500
+    ([90000] * 32, False, False, 2), ([150000] * 32, False, False, 2),
+    ([150000] * 8, False, False, 1), ([150000] * 64, False, False, 2),
+    ([62500] * 4, False, False, 2), ([62500] * 4, True, False, 1), ([62500] * 64, True, False, 2),
+    ([30000], True, False, 2), ([128000] * 16, True, False, 1), ([128000] * 64, True, False, 2),
+    ([58000], False, True, 2), ([60000], False, True, 1),     # keys: up to about 59,500
+    ([67000] * 4, False, True, 1), ([67000] * 32, False, True, 2), ([147000] * 32, False, True, 1),
+    ([30000] * 4, True, True, 1), ([14700], True, True, 2),
 ])
-def test_split_of_a_batch_of_equal_graphs(lib, sizes, skewed, mode):
-    """Where the library's choice between a block a graph and one union changes, for even graphs and
-    for batches with one row in 200 longer than 121 (measured on both sides; the graphs here have no
-    entries, so their sizes stand for vertices and entries together)."""
+def test_split_of_a_batch_of_equal_graphs(lib, sizes, skewed, keyed, mode):
+    """Where the library's choice between a block a graph and one union changes, for even graphs, for
+    batches with one row in 200 longer than 121, and with keys (measured on both sides; the graphs
+    here have no entries, so their sizes stand for vertices and entries together)."""
     lib.fake_no_results()
     try:
         if skewed:
             for off in (STATS_CAP, STATS_CAP + 4, STATS_OVER, STATS_OVER + 4, STATS_OVER + 8):
                 lib.fake_result(b"stats_kernel", STATS_ARG, off, sum(sizes) // 200 + 1)
-        b = EdgelessBatch(lib, sizes)
+        b = EdgelessBatch(lib, sizes, keys=keyed)
         assert b.rc == gc.GC_OK
         assert lib.gc_batch_mode(b.plan) == mode
         b.close()
