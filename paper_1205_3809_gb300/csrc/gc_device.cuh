@@ -2005,7 +2005,8 @@ __device__ __forceinline__ uint64_t asymmetry(int32_t v, int32_t w) {
 
 // Range, self-loop and symmetry checks of every entry.  A warp takes up to 32
 // rows: those of up to kPass1Flat entries are read as one flat, coalesced range,
-// longer ones by the whole warp in turn.  Fewer rows (a power of two) when that
+// longer ones by the whole warp in turn, and those above kCheckFar by the whole
+// block when its warps are done with the others.  Fewer rows (a power of two) when that
 // would leave warps without any, as long as they hold 128 entries, so that a
 // graph of few long rows is spread over the GPU.  Runs behind the setup scan and
 // does nothing when that found the row starts unusable.
@@ -2015,7 +2016,10 @@ __device__ __forceinline__ uint64_t asymmetry(int32_t v, int32_t w) {
 // atomics a thread, waited for on its own, cost 0.17 ms more on the 4.0 M
 // entries of a 997,399-vertex mesh (a checked call 0.42 ms, now 0.26).  With 32
 // rows always, K(2000, 2000), 4,000 rows of 2,000 entries, took 217 us, now 20;
-// G(3000, 12000) 4.3, now 3.7; G(400000, 6000000) 38.9, now 37.0.
+// G(3000, 12000) 4.3, now 3.7; G(400000, 6000000) 38.9, now 37.0.  With the
+// longest rows left to a warp, K(2, 200000) took 1,179 us, now 151, and a star of
+// 1M vertices 2,964, now 380.
+constexpr int kCheckFar = 8192, kCheckFarRows = 64;
 __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ colidx, int32_t n,
                                                        const Stats* __restrict__ scan, ValidateOut* out) {
@@ -2024,9 +2028,13 @@ __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict
     };
     __shared__ Smem s_row[8];
     __shared__ unsigned long long s_sum[8];
+    __shared__ int32_t s_far[kCheckFarRows];  // rows for the whole block
+    __shared__ int s_nfar;
     // (read through L1: a word that every warp of the GPU takes from L2 costs 4 us)
     const int bad_rows = __ldg(&scan->bad), nnz = __ldg(&scan->nnz);
     if (bad_rows || nnz < 0 || (nnz > 0 && !colidx)) return;
+    if (threadIdx.x == 0) s_nfar = 0;
+    __syncthreads();
     const unsigned lane = lane_id(), wib = threadIdx.x >> 5;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -2042,6 +2050,17 @@ __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict
         } else {
             loop |= w == v;
             sum += asymmetry(v, w);
+        }
+    };
+    // entries [i, e) of row v, from i on every `step`-th group of 256
+    auto entries = [&](int32_t v, int64_t i, int64_t e, int step) {
+        for (i += lane; i < e; i += step) {
+            int32_t w[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) w[u] = i + 32 * u < e ? ld_adj(colidx + i + 32 * u, pol) : 0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (i + 32 * u < e) entry(v, w[u]);
         }
     };
     for (int64_t t = gw; t < ntasks; t += W) {
@@ -2081,22 +2100,25 @@ __global__ void __launch_bounds__(256) validate_kernel(const int32_t* __restrict
             for (int u = 0; u < 4; ++u)
                 if (F0 + 32 * u + (int32_t)lane < D) entry((int32_t)(t << shift) + own[u], w[u]);
         }
-        unsigned big = __ballot_sync(kFull, d > kPass1Flat);
+        bool later = false;
+        if (d > kCheckFar) {
+            const int at = atomicAdd(&s_nfar, 1);
+            later = at < kCheckFarRows;
+            if (later) s_far[at] = v;
+        }
+        unsigned big = __ballot_sync(kFull, d > kPass1Flat && !later);
         while (big) {
             const int j = __ffs(big) - 1;
             big &= big - 1;
-            const int32_t vj = (int32_t)(t << shift) + j;
-            const int64_t bj = __shfl_sync(kFull, b, j), ej = bj + __shfl_sync(kFull, d, j);
-            for (int64_t i = bj + lane; i < ej; i += 32 * 8) {
-                int32_t w[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) w[u] = i + 32 * u < ej ? ld_adj(colidx + i + 32 * u, pol) : 0;
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (i + 32 * u < ej) entry(vj, w[u]);
-            }
+            const int64_t bj = __shfl_sync(kFull, b, j);
+            entries((int32_t)(t << shift) + j, bj, bj + __shfl_sync(kFull, d, j), 256);
         }
         __syncwarp();
+    }
+    __syncthreads();
+    for (int j = 0; j < min(s_nfar, kCheckFarRows); ++j) {
+        const int32_t v = s_far[j];
+        entries(v, (int64_t)__ldg(rowptr + v) + 256 * wib, __ldg(rowptr + v + 1), 256 * (int)(blockDim.x / 32));
     }
     if (__any_sync(kFull, bad) && lane == 0) out->bad_index = 1;
     if (__any_sync(kFull, loop) && lane == 0) out->self_loop = 1;

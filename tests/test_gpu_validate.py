@@ -23,12 +23,20 @@ def _dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
+def _many_long_rows():
+    """70 rows of 8,200 in a row, among enough empty ones that a warp takes 32 and a block 256."""
+    g = gg.complete_bipartite(70, 8200)
+    return gg.from_edges(310000, np.repeat(np.arange(g.n), g.degrees), g.colidx, name="70 rows of 8,200")
+
+
 GRAPHS = [
     lambda: gg.path(2), lambda: gg.path(65), lambda: gg.grid2d(37, 53, 1), lambda: gg.gnm(5000, 40000, 2),
     lambda: gg.complete(256), lambda: gg.complete(257), lambda: gg.complete(258),  # rows of 255, 256, 257
     lambda: gg.star(3001, 17), lambda: gg.rmat(12, 16, gg.RMAT_B, 3),
     # 16, 2 and 1 rows a warp (32, 8 and 4 above), the last with rows on both sides of 256
     lambda: gg.gnm(999, 3900, 4), lambda: gg.gnm(1501, 37000, 5), lambda: gg.gnm(301, 38600, 6),
+    # rows for the whole block: one of 8,193, two of 9,000, and more than a block notes down (64)
+    lambda: gg.star(8194, 5), lambda: gg.complete_bipartite(2, 9000), lambda: _many_long_rows(),
 ]
 
 
