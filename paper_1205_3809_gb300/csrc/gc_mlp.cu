@@ -544,7 +544,7 @@ __device__ __forceinline__ RowDegrees small_rows(const FeatureGraph& g, unsigned
     return mine;
 }
 
-// A warp takes 32 vertices.  When none of their rows is longer than 12, each lane
+// A warp takes 32 vertices.  When none of their rows is longer than 16, each lane
 // reads its own; otherwise rows of up to 57 entries are read by 4 lanes, 8 rows
 // side by side, rows of up to 121 by 16 lanes and longer ones by the whole warp,
 // a 32-byte chunk a lane at a time.  A small graph (rows of 6 entries and more on
@@ -561,15 +561,16 @@ __device__ __forceinline__ RowDegrees small_rows(const FeatureGraph& g, unsigned
 // words when each has a row of its own: grid of 2,000 x 2,000 67.8 us (thread per
 // row, 8 entries at a time), 89.7 (two lanes in chunks), 56.3 now; 12 entries a
 // row 43.4, 79.3, 40; 26 entries 42.4, 168 (16 lanes), 48 (4 lanes, two chunks
-// each).  With own rows up to 16, R-MAT and G(n, m) are unchanged, but a geometric
-// graph of 1M vertices in random order (8 a row) takes 49.6 us, not 46.2.
+// each).  With own rows up to 12 only, a geometric graph of 1M vertices in random
+// order (8 a row) takes 46.2 us, not 49.6 (thread per row 53.4), but 200 graphs of
+// 4,096 vertices in a batch, 8 a row and near each other, 71, not 66 (65).
 // Few vertices: G(3000, 12000) 3.3 us, 5.5 in warps of 32, 3.3; K(1500) 115, 132, 33.
 constexpr int kFeatureBlocks = 6;
 template <unsigned STEPS>
 __global__ void __launch_bounds__(256, kFeatureBlocks) features_kernel(const int32_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ colidx, int32_t n,
                                                        float* __restrict__ out) {
-    constexpr int32_t kOwn = 12, kSmall = 57, kMid = 8 * 16 - 7;
+    constexpr int32_t kOwn = 16, kSmall = 57, kMid = 8 * 16 - 7;
     FeatureGraph g;
     g.rowptr = rowptr;
     g.colidx = colidx;
