@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -1206,7 +1207,10 @@ constexpr int32_t kLocalSharedDefault = 164 * 1024;  // mode 2: bytes of shared 
 // geometric graphs), either way.  With 1e5 one G(10000, 40000) took a block and
 // 146 us (130 when all such batches were a union, 96 with the union now); with
 // 7e4, 32 grids of 30,000 vertices go to the union, 208 us, where
-// blocks take 166.
+// blocks take 166.  A union of one, two or four graphs has fewer rounds and costs
+// 0.55, 0.7 or 0.85 of that: one graph breaks even at 40,000 to 60,000 vertices
+// and entries (one R-MAT-G of 4,096 vertices, 67,472 of them: 208 us in a block,
+// 126 in the union, 201 in the union before).
 //
 // Skewed graphs cost a block more, for their many rounds and long rows: 4.4 to
 // 5.4 ns a vertex or entry on R-MAT-B of 4,096 to 131,072 vertices against 1.2
@@ -1248,7 +1252,8 @@ int32_t split_batch(const std::vector<int32_t>& order, const int64_t* voff, cons
     for (int32_t i = 0; i < G; ++i) {
         big += work(i);
         rest -= alone(i);
-        const double cost = kUnionFixed + whole * big / sms + std::max(rest / sms, most[(size_t)i + 1]);
+        const double fixed = kUnionFixed * std::min(1.0, 0.55 + 0.15 * std::log2(i + 1.0));
+        const double cost = fixed + whole * big / sms + std::max(rest / sms, most[(size_t)i + 1]);
         if (cost < best_cost) {
             best_cost = cost;
             best = i + 1;

@@ -188,14 +188,15 @@ STATS_ARG, STATS_CAP, STATS_OVER = 5, 16, 28   # stats_kernel's record: cap[0..1
 
 
 @pytest.mark.parametrize("sizes, skewed, keyed, mode", [
-    ([85000], False, False, 2), ([90000], False, False, 1),   # one graph: a block up to about 89,500
+    ([48000], False, False, 2), ([50000], False, False, 1),   # one graph: a block up to about 49,200
+    ([60000] * 2, False, False, 2), ([65000] * 2, False, False, 1), ([85000] * 8, False, False, 2),
     ([90000] * 32, False, False, 2), ([150000] * 32, False, False, 2),
     ([150000] * 8, False, False, 1), ([150000] * 64, False, False, 2),
     ([62500] * 4, False, False, 2), ([62500] * 4, True, False, 1), ([62500] * 64, True, False, 2),
-    ([30000], True, False, 2), ([128000] * 16, True, False, 1), ([128000] * 64, True, False, 2),
-    ([58000], False, True, 2), ([60000], False, True, 1),     # keys: up to about 59,500
+    ([19000], True, False, 2), ([21000], True, False, 1), ([128000] * 16, True, False, 1), ([128000] * 64, True, False, 2),
+    ([32000], False, True, 2), ([34000], False, True, 1),     # keys: up to about 32,700
     ([67000] * 4, False, True, 1), ([67000] * 32, False, True, 2), ([147000] * 32, False, True, 1),
-    ([30000] * 4, True, True, 1), ([14700], True, True, 2),
+    ([30000] * 4, True, True, 1), ([12000], True, True, 2),
 ])
 def test_split_of_a_batch_of_equal_graphs(lib, sizes, skewed, keyed, mode):
     """Where the library's choice between a block a graph and one union changes, for even graphs, for
