@@ -1950,9 +1950,11 @@ template <typename T, bool P>  // P: a priority array is given
 __global__ void __launch_bounds__(256, kMinBlocks) graph_round_kernel(Params<T> p) {
     RoundState* st = p.st;
     const int k = __ldcg(&st->graph_round);
-    const RoundCounts& c = st->rc[k % 3];
+    // the counts by one thread, which alone splits them into tasks: six words that
+    // every warp of the GPU takes from one L2 line each are 2 us of a short round
+    RoundSizes r = {};
     unsigned size;
-    const RoundSizes r = round_sizes_of(c, &size);
+    if (threadIdx.x == 0) r = round_sizes_of(st->rc[k % 3], &size);
     int maxc = 0;
     run_pass<T, P>(p, k, r, maxc, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
              (gridDim.x * blockDim.x) >> 5, nullptr);
