@@ -251,6 +251,11 @@ __global__ void __launch_bounds__(kForwardThreads, 1) mlp_forward_kernel(const f
 // multiply-adds (3,552 a sample), about level.  With a thread per parameter
 // walking the tile (two reads a multiply-add) and 64 threads a block, 65,536
 // samples took 51 us, now 26 (262,144: 149 us, now 63).
+//
+// Error: a warp's sums run over all of its samples, n / 1,216 terms in a row, and
+// then over the blocks by atomics, which set the error: each part of the gradient
+// is off by 0.4 to 4e-7 of itself from 4,096 to 16.8 million samples (against 64
+// bits over the same activations), by 0.7 to 6e-7 with a sum a parameter and tile.
 constexpr int kTileWarps = kTile / 32;
 struct __align__(16) GradShared {
     ForwardParams p;

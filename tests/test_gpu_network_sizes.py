@@ -70,6 +70,54 @@ def test_gradient_sizes(gcpkg, n):
     assert abs(float(sse.item()) - want_sse) <= 1e-4 * want_sse + 1e-6
 
 
+def _gradient_64bit(p, x, t, scale):
+    """Gradient and squared error in 64 bits on the device, over the forward's own activations: its
+    products of bf16 values are exact in 32 bits, so a 32-bit sum in input order has its bits."""
+    W1, b1, W2, b2, W3, b3 = (p[a:b] for a, b in ((0, 192), (192, 224), (224, 1248), (1248, 1280), (1280, 1312), (1312, 1313)))
+    half = lambda z: z.to(torch.bfloat16).float()
+    W1, W2, W3 = half(W1).view(32, 6), half(W2).view(32, 32), half(W3)
+
+    def chain(a, w):
+        acc = torch.zeros(a.shape[0], w.shape[0], device=a.device)
+        for k in range(a.shape[1]):
+            acc = acc + a[:, k:k + 1] * w[:, k][None]
+        return acc
+
+    grad, sse = torch.zeros(L.N_PARAMS, dtype=torch.float64, device=p.device), 0.0
+    for a0, tt in zip(half(x).split(1 << 20), t.split(1 << 20)):
+        a1 = half(torch.relu(chain(a0, W1) + b1))
+        a2 = half(torch.relu(chain(a1, W2) + b2))
+        err = (chain(a2, W3[None])[:, 0] + b3) - tt
+        dy = (2 * scale * err).double()
+        d2 = dy[:, None] * W3.double()[None] * (a2 > 0)
+        d1 = (d2 @ W2.double()) * (a1 > 0)
+        grad += torch.cat([(d1.T @ a0.double()).reshape(-1), d1.sum(0), (d2.T @ a1.double()).reshape(-1), d2.sum(0),
+                           dy @ a2.double(), dy.sum()[None]])
+        sse += float((err.double() ** 2).sum())
+    return grad, sse
+
+
+# a warp's running sums are n / 1,216 terms long: 216, 3,449 and 13,798
+@pytest.mark.parametrize("n, shift", [(262145, 0.0), (4194301, 0.0), (4194301, 50.0), (16777213, 0.0)])
+def test_gradient_sums_of_many_samples(gcpkg, n, shift):
+    """Each part of the gradient and the squared error against 64 bits.  The sums end in one atomic a
+    block: 304 additions of 32 bits, each off by at most 2^-24 of the sum so far, which is half the
+    end's on average: 304 / 2 * 2^-24 = 9e-6 of it at worst.  A chain of k terms in a warp is off by
+    about sqrt(k / 3) * 2^-25 of its own sum, and 1,216 of them, independent, by 1/35 of that of the
+    whole: 6e-8 for the longest here.  Measured: 1 to 5e-7, and 2 to 6e-7 with short chains and one
+    sum a parameter."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    p = torch.randn(L.N_PARAMS, generator=g, device="cuda") * 0.25
+    x = torch.rand(n, L.N_IN, generator=g, device="cuda") * 12
+    t = torch.randn(n, generator=g, device="cuda") * 3 + shift
+    want, want_sse = _gradient_64bit(p, x, t, 1.0 / n)
+    grad, sse = torch.zeros(L.N_PARAMS, device="cuda"), torch.zeros(1, device="cuda")
+    gcpkg.mlp_grad(p, x, t, 1.0 / n, grad, sse)
+    for a, b in ((0, 192), (192, 224), (224, 1248), (1248, 1280), (1280, 1312), (1312, 1313)):
+        assert float((grad.double() - want)[a:b].norm()) <= 9e-6 * float(want[a:b].norm()), (a, b)
+    assert abs(float(sse) - want_sse) <= 9e-6 * want_sse
+
+
 def _rows_of(degree, seed):
     """Vertices of exactly `degree` neighbours (stars), among a sparse random graph, ids shuffled."""
     parts, n = [], 0
