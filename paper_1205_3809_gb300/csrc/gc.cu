@@ -1662,7 +1662,13 @@ int gc_color_host(const int32_t* rowptr, const int32_t* colidx, int32_t n, const
     hin.vb[hin.nchunks] = n;
     hin.eb[hin.nchunks] = nnz;
     rc = color_locked(d_rp, d_ci, n, d_pr, d_co, ncolors, rounds, s, opt, nullptr, 0, &hin);
-    if (rc != GC_OK) return rc;
+    if (rc != GC_OK) {
+        // the caller may free its arrays: no copy from them may be left in flight
+        cudaStreamSynchronize(s);
+        if (dc.copy) cudaStreamSynchronize(dc.copy);
+        (void)cudaGetLastError();
+        return rc;
+    }
     GC_CUDA(cudaMemcpyAsync(colors_out, d_co, (size_t)n * 4, cudaMemcpyDeviceToHost, s));
     GC_CUDA(cudaStreamSynchronize(s));
     return GC_OK;

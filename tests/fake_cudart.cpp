@@ -182,6 +182,11 @@ size_t fake_pool_bytes() {  // handed out from pools
     for (Pool* p : g_pools) n += p->used;
     return n;
 }
+int fake_pending() {  // copies, memsets and kernels not yet carried out
+    size_t n = 0;
+    for (Stream* s : g_streams) n += s->ops.size();
+    return (int)n;
+}
 size_t fake_bytes_taken() { return taken(); }
 
 // ---- registration and launches

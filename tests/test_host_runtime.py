@@ -32,6 +32,7 @@ def lib(tmp_path_factory):
     h.gc_validate_csr.argtypes = [vp, vp, i32, vp]
     h.gc_last_phase_ms.argtypes = [vp, i32]
     h.gc_batch_mode.argtypes = [vp]
+    h.gc_color_host.argtypes = [vp, vp, i32, vp, vp, vp, vp, vp, vp]
     h.fake_result.argtypes = [ctypes.c_char_p, ctypes.c_int, ctypes.c_size_t, ctypes.c_uint32]
     h.gc_batch_status.argtypes = [vp, vp, vp, vp]
     h.gc_batch_round_stats.argtypes = [vp, vp, vp, i32, vp, vp]
@@ -211,6 +212,23 @@ def test_split_of_a_batch_of_equal_graphs(lib, sizes, skewed, keyed, mode):
         assert b.rc == gc.GC_OK
         assert lib.gc_batch_mode(b.plan) == mode
         b.close()
+    finally:
+        lib.fake_no_results()
+        lib.gc_release()
+
+
+def test_rejected_host_graph_leaves_no_copy_of_it_queued(lib):
+    """After gc_color_host returns, with whatever status, the caller may free its arrays."""
+    n, nnz = 64, 3 << 20                                 # three chunks
+    rowptr = np.linspace(0, nnz, n + 1).astype(np.int32)
+    colidx, colors = np.zeros(nnz, np.int32), np.zeros(n, np.int32)
+    nc, rd = ctypes.c_int32(), ctypes.c_int32()
+    lib.fake_no_results()
+    try:
+        lib.fake_result(b"stats_kernel", STATS_ARG, 4, 1)   # the setup scan finds the row starts unusable
+        assert lib.gc_color_host(_p(rowptr), _p(colidx), n, None, _p(colors), ctypes.byref(nc), ctypes.byref(rd),
+                                 None, None) == gc.GC_ERR_BAD_GRAPH
+        assert lib.fake_pending() == 0
     finally:
         lib.fake_no_results()
         lib.gc_release()
