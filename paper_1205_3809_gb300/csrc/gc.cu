@@ -75,8 +75,8 @@ struct DeviceCache {
 };
 
 // Host inputs of gc_color_host: colidx goes to the device in chunks of whole
-// 32-vertex tasks on a copy stream, and round 1 runs on each chunk as soon as
-// it has arrived, so the copy overlaps the setup scan and round 1.
+// rows on a copy stream, and round 1 runs on each chunk as soon as it has
+// arrived, so the copy overlaps the setup scan and round 1.
 constexpr int kMaxChunks = 16;
 struct HostInput {
     const int32_t* h_colidx;
@@ -456,24 +456,22 @@ template <typename T, bool P>
 int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, bool long_rows, cudaStream_t s,
                  int64_t* launches, const HostInput* hin) {
     const int threads = o.block_threads;
-    {
-        // per input chunk when the input is still arriving
-        const int nch = hin ? hin->nchunks : 1;
-        for (int c = 0; c < nch; ++c) {
-            const int32_t v0 = hin ? hin->vb[c] : 0, v1 = hin ? hin->vb[c + 1] : p.n;
-            if (hin) GC_CUDA(cudaStreamWaitEvent(s, dc.chunk_ev[c], 0));
-            if (v1 <= v0) continue;
-            const int rc = launch_pass1(p, v0, v1, dc.sms, s);
-            if (rc != GC_OK) return rc;
-            *launches += 1;
-        }
-        if (long_rows) {
-            gc::pass1_long_kernel<T><<<dc.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
-            GC_CUDA(cudaGetLastError());
-            *launches += 1;
-        }
-        if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[2], s));
+    // round 1, per input chunk when the input is still arriving
+    const int nch = hin ? hin->nchunks : 1;
+    for (int c = 0; c < nch; ++c) {
+        const int32_t v0 = hin ? hin->vb[c] : 0, v1 = hin ? hin->vb[c + 1] : p.n;
+        if (hin) GC_CUDA(cudaStreamWaitEvent(s, dc.chunk_ev[c], 0));
+        if (v1 <= v0) continue;
+        const int rc = launch_pass1(p, v0, v1, dc.sms, s);
+        if (rc != GC_OK) return rc;
+        *launches += 1;
     }
+    if (long_rows) {
+        gc::pass1_long_kernel<T><<<dc.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
+        GC_CUDA(cudaGetLastError());
+        *launches += 1;
+    }
+    if (o.telemetry) GC_CUDA(cudaEventRecord(dc.ev[2], s));
     if (o.loop_mode == 2) return run_rounds_graph<T, P>(o, dc, p, s, launches);
     if (o.loop_mode == 0) {
         int per_sm = 0;
@@ -503,8 +501,8 @@ int run_rounds_p(const gc_options& o, DeviceCache& dc, Params<T>& p, bool long_r
     for (;; ++k) {
         GC_CUDA(cudaMemcpyAsync(h, &st->rc[k % 3], sizeof(gc::RoundCounts), cudaMemcpyDeviceToHost, s));
         GC_CUDA(cudaStreamSynchronize(s));
-        const gc::RoundSizes r = {gc::low_count(h->tiny), gc::high_count(h->tiny), gc::low_count(h->mid), gc::high_count(h->mid), h->s, h->m,
-                                  gc::hub_chunks(h->hc), 0u};
+        const gc::RoundSizes r = {gc::low_count(h->tiny), gc::high_count(h->tiny), gc::low_count(h->mid),
+                                  gc::high_count(h->mid), h->s, h->m, gc::hub_chunks(h->hc), 0u};
         const unsigned size = r.n2 + r.n4 + r.n8 + r.n16 + r.nS + r.nM + gc::hub_count(h->hc);
         if (size == 0) break;
         if (k > p.max_rounds) {
@@ -1107,15 +1105,13 @@ int batch_enqueue_typed(gc_batch& b, cudaStream_t s) {
     p.colors_out = b.colors_out;
     p.settle_round = settle;
     fill_workspace(p, base, b.L, st, b.round_cap);
-    {
-        rc = launch_pass1(p, 0, (int32_t)b.N, b.sms, s);
-        if (rc != GC_OK) return rc;
+    rc = launch_pass1(p, 0, (int32_t)b.N, b.sms, s);
+    if (rc != GC_OK) return rc;
+    ++launches;
+    if (b.hs.defer) {
+        gc::pass1_long_kernel<T><<<b.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
+        GC_CUDA(cudaGetLastError());
         ++launches;
-        if (b.hs.defer) {
-            gc::pass1_long_kernel<T><<<b.sms * gc::kPass1LongBlocksPerSm, 256, 0, s>>>(p);
-            GC_CUDA(cudaGetLastError());
-            ++launches;
-        }
     }
     {
         cudaLaunchConfig_t cfg = {};
@@ -1520,9 +1516,10 @@ int batch_create_locked(const int32_t* rowptr_cat, const int32_t* colidx_cat, co
     fail(GC_OK);  // frees the head copy after the stream drains
     // the coloring layout's offsets are relative to its own base
     Layout& L = b->L;
-    size_t* fields[] = {&L.st, &L.rs, &L.rv, &L.rt, &L.x0, &L.x1, &L.act0, &L.act1, &L.stat, &L.hubs,
-                        &L.defer, &L.L2[0], &L.L2[1], &L.L4[0], &L.L4[1], &L.L8[0], &L.L8[1], &L.L16[0], &L.L16[1], &L.S[0], &L.S[1], &L.M[0], &L.M[1], &L.H[0], &L.H[1], &L.Hc[0], &L.Hc[1],
-                        &L.O[0], &L.O[1]};
+    size_t* fields[] = {&L.st,    &L.rs,    &L.rv,    &L.rt,    &L.x0,     &L.x1,     &L.act0,  &L.act1, &L.stat,
+                        &L.hubs,  &L.defer, &L.L2[0], &L.L2[1], &L.L4[0],  &L.L4[1],  &L.L8[0], &L.L8[1],
+                        &L.L16[0], &L.L16[1], &L.S[0], &L.S[1], &L.M[0],   &L.M[1],   &L.H[0],  &L.H[1],
+                        &L.Hc[0], &L.Hc[1], &L.O[0],  &L.O[1]};
     for (size_t* f : fields) *f += lay;
 
     int per_sm = 0;

@@ -47,16 +47,16 @@
 //     longer list OR their conflict flag and color windows into a per-vertex
 //     record, write their survivors at offsets taken from an atomic counter,
 //     and the warp that finishes the last chunk decides.
-// Tasks are dealt to warps round-robin; no block-wide barrier is taken
-// inside a round.
+// Tasks are dealt to warps round-robin; after the round's split into tasks no
+// block-wide barrier is taken inside a round.
 //
 // Priority: the round kernels are instantiated for index priority (the test
 // is one compare) and for a priority array, whose (key, index) order round 2
 // evaluates once per kept neighbour and stores in a bit mask (rows read from
-// the graph) or in bit 31 of the active-list entry.  Loops: all rounds in one cooperative launch with a bounded grid
-// barrier (optionally handing the last rounds to block 0), one launch per
-// round, or a CUDA graph whose while node repeats a round kernel and a
-// one-thread condition kernel.
+// the graph) or in bit 31 of the active-list entry.  Loops: all rounds in one
+// cooperative launch with a bounded grid barrier (optionally handing the last
+// rounds to block 0), one launch per round, or a CUDA graph whose while node
+// repeats a round kernel and a one-thread condition kernel.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -543,7 +543,8 @@ __global__ void stats_kernel(const int32_t* __restrict__ rowptr, int32_t n, int3
     int mx = 0, bad = 0;
     unsigned c0 = 0, c1 = 0, c2 = 0, df = 0, o2 = 0, o8 = 0, o16 = 0;
     unsigned long long ch = 0;
-    const int32_t tiny2 = tiny_limit(2, s_max, keyed), tiny4 = tiny_limit(4, s_max, keyed), mid8 = mid_limit(8, s_max, m_max), mid16 = mid_limit(16, s_max, m_max);
+    const int32_t tiny2 = tiny_limit(2, s_max, keyed), tiny4 = tiny_limit(4, s_max, keyed);
+    const int32_t mid8 = mid_limit(8, s_max, m_max), mid16 = mid_limit(16, s_max, m_max);
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int32_t d = __ldg(rowptr + v + 1) - __ldg(rowptr + v);
@@ -607,7 +608,8 @@ __device__ __forceinline__ void pass1_write(const Params<T>& p, int32_t v, bool 
 template <typename T>
 __device__ __forceinline__ NextLists pass1_next(const Params<T>& p) {
     NextLists nl;
-    nl.L2 = p.L2A; nl.L4 = p.L4A; nl.L8 = p.L8A; nl.L16 = p.L16A; nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
+    nl.L2 = p.L2A; nl.L4 = p.L4A; nl.L8 = p.L8A; nl.L16 = p.L16A;
+    nl.S = p.SA; nl.M = p.MA; nl.H = p.HA; nl.Hc = p.HcA; nl.O = p.OA;
     nl.cnt = &p.st->rc[2];
     nl.s_max = p.s_max;
     nl.m_max = p.m_max;
@@ -665,8 +667,8 @@ __device__ __forceinline__ uint32_t chunk_in_row(int32_t off, int32_t d) {
 //
 // Bound: one 32-byte sector of colidx per vertex, and its row start, buffers and
 // worklist entry.  Reading every row to its end as one flat range took 0.71 ms
-// for R-MAT-B of 2^24 vertices (now 0.38) and 0.24 for R-MAT-ER of 2^22 (now
-// 0.10).
+// for R-MAT-B of 2^24 vertices (now 0.38; both with the setup scan, without it
+// now 0.29) and 0.24 for R-MAT-ER of 2^22 (now 0.10).
 //
 // PER vertices a thread: 4, or 1 for a range too small to give every SM a block
 // of 1,024.
@@ -896,7 +898,8 @@ struct PassIO {
     const int32_t* rin;     // active lists read this round (colidx in round 2)
     int32_t* rout;          // active lists written for the next round
     bool first;             // round 2: no static masks yet
-    const int4* L2; const int4* L4; const int4* L8; const int4* L16; const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
+    const int4* L2; const int4* L4; const int4* L8; const int4* L16;
+    const int4* S; const int4* M; const int4* H; const int32_t* Hc; const int32_t* O;
     NextLists next;
     uint64_t pol_row, pol_col;
 };
@@ -1969,7 +1972,8 @@ __global__ void graph_cond_kernel(Params<T> p, int before_loop, cudaGraphConditi
     const int k = before_loop ? 1 : st->graph_round;
     const int kn = k + 1;
     const RoundCounts& c = st->rc[kn % 3];
-    const unsigned size = low_count(c.tiny) + high_count(c.tiny) + low_count(c.mid) + high_count(c.mid) + c.s + c.m + hub_count(c.hc);
+    const unsigned size = low_count(c.tiny) + high_count(c.tiny) + low_count(c.mid) + high_count(c.mid) + c.s + c.m +
+                          hub_count(c.hc);
     unsigned go = 0u;
     if (size == 0u) {
         st->rounds = k;

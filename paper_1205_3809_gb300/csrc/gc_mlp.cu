@@ -77,41 +77,31 @@ __device__ __forceinline__ void load_forward_params(const float* __restrict__ pa
     }
 }
 
-// One layer of R samples for units j0 .. j0 + J - 1: every unit's sum runs over
-// the inputs in index order, two units to an instruction, and a weight read
-// from shared memory serves all R samples.
-template <int IN, int J, int R>
-__device__ __forceinline__ void layer_units(const float (*w)[kRow], const float* bias, int j0, const float (&in)[R][IN],
-                                            float (&out)[R][J]) {
-    f32x2 acc[R][J / 2];
+// One layer of one sample: every unit's sum runs over the inputs in index order,
+// two units to an instruction.
+template <int IN, int OUT>
+__device__ __forceinline__ void layer_units(const float (*w)[kRow], const float* bias, const float (&in)[IN],
+                                            float (&out)[OUT]) {
+    f32x2 acc[OUT / 2];
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int q = 0; q < J / 2; ++q) acc[r][q] = 0ull;
+    for (int q = 0; q < OUT / 2; ++q) acc[q] = 0ull;
 #pragma unroll
     for (int i = 0; i < IN; ++i) {
-        f32x2 a[R];
+        const f32x2 a = pack2(in[i], in[i]);
 #pragma unroll
-        for (int r = 0; r < R; ++r) a[r] = pack2(in[r][i], in[r][i]);
-#pragma unroll
-        for (int q = 0; q < J / 2; q += 2) {
-            const ulonglong2 wq = *reinterpret_cast<const ulonglong2*>(&w[i][j0 + 2 * q]);
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                acc[r][q] = fma2(wq.x, a[r], acc[r][q]);
-                acc[r][q + 1] = fma2(wq.y, a[r], acc[r][q + 1]);
-            }
+        for (int q = 0; q < OUT / 2; q += 2) {
+            const ulonglong2 wq = *reinterpret_cast<const ulonglong2*>(&w[i][2 * q]);
+            acc[q] = fma2(wq.x, a, acc[q]);
+            acc[q + 1] = fma2(wq.y, a, acc[q + 1]);
         }
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int q = 0; q < J / 2; ++q) {
-            float x, y;
-            unpack2(acc[r][q], x, y);
-            out[r][2 * q] = bf16r(fmaxf(x + bias[j0 + 2 * q], 0.f));
-            out[r][2 * q + 1] = bf16r(fmaxf(y + bias[j0 + 2 * q + 1], 0.f));
-        }
+    for (int q = 0; q < OUT / 2; ++q) {
+        float x, y;
+        unpack2(acc[q], x, y);
+        out[2 * q] = bf16r(fmaxf(x + bias[2 * q], 0.f));
+        out[2 * q + 1] = bf16r(fmaxf(y + bias[2 * q + 1], 0.f));
+    }
 }
 
 // Two bf16 values in a word, the first in its low half: rounding to nearest
@@ -136,8 +126,10 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
     return r;
 }
 
-// layer_units with the activations kept as pairs of bf16 (half the registers,
-// and bias, rounding and maximum take one instruction each for two units).
+// The same for R samples and units j0 .. j0 + J - 1, a weight read from shared
+// memory serving all samples, with the activations kept as pairs of bf16 (half the
+// registers, and bias, rounding and maximum take one instruction each for two
+// units).
 template <int IN, int J, int R>
 __device__ __forceinline__ void layer_pairs(const float (*w)[kRow], const float* bias, int j0,
                                             const uint32_t (&in)[R][IN / 2], uint32_t (&out)[R][J / 2]) {
@@ -253,9 +245,9 @@ __global__ void __launch_bounds__(kForwardThreads, 1) mlp_forward_kernel(const f
 // samples took 51 us, now 26 (262,144: 149 us, now 63).
 //
 // Error: a warp's sums run over all of its samples, n / 1,216 terms in a row, and
-// then over the blocks by atomics, which set the error: each part of the gradient
-// is off by 0.4 to 4e-7 of itself from 4,096 to 16.8 million samples (against 64
-// bits over the same activations), by 0.7 to 6e-7 with a sum a parameter and tile.
+// then over the blocks by atomics, which set the error: from 4,096 to 16.8 million
+// samples each part of the gradient is off by at most 5e-7 of itself (against 64
+// bits over the same activations; 9e-7 with a sum a parameter and tile).
 constexpr int kTileWarps = kTile / 32;
 struct __align__(16) GradShared {
     ForwardParams p;
@@ -291,29 +283,29 @@ __global__ void __launch_bounds__(kTile) mlp_grad_kernel(const float* __restrict
         {
             const int64_t r = base + q;
             const bool valid = r < n;
-            float a0[1][kIn], a1[1][kH], a2[1][kH], d2[kH];
+            float a0[kIn], a1[kH], a2[kH], d2[kH];
 #pragma unroll
-            for (int i = 0; i < kIn; ++i) a0[0][i] = valid ? bf16r(x[r * kIn + i]) : 0.f;
-            layer_units<kIn, kH, 1>(s.p.w1, s.p.b1, 0, a0, a1);
-            layer_units<kH, kH, 1>(s.p.w2, s.p.b2, 0, a1, a2);
+            for (int i = 0; i < kIn; ++i) a0[i] = valid ? bf16r(x[r * kIn + i]) : 0.f;
+            layer_units(s.p.w1, s.p.b1, a0, a1);
+            layer_units(s.p.w2, s.p.b2, a1, a2);
             float out = 0.f;
 #pragma unroll
-            for (int j = 0; j < kH; ++j) out = fmaf(s.p.w3[j], a2[0][j], out);
+            for (int j = 0; j < kH; ++j) out = fmaf(s.p.w3[j], a2[j], out);
             out += s.p.b3;
             const float err = valid ? out - t[r] : 0.f;
             sse_local += err * err;
             const float dy = 2.f * scale * err;
             // relu masks: a > 0 exactly when z > 0 (rounding to bf16 keeps a positive value positive)
 #pragma unroll
-            for (int j = 0; j < kH; ++j) d2[j] = a2[0][j] > 0.f ? dy * s.p.w3[j] : 0.f;
+            for (int j = 0; j < kH; ++j) d2[j] = a2[j] > 0.f ? dy * s.p.w3[j] : 0.f;
 #pragma unroll
             for (int j = 0; j < kH; j += 4) {
-                *reinterpret_cast<float4*>(&s.a1[q][j]) = make_float4(a1[0][j], a1[0][j + 1], a1[0][j + 2], a1[0][j + 3]);
-                *reinterpret_cast<float4*>(&s.a2[q][j]) = make_float4(a2[0][j], a2[0][j + 1], a2[0][j + 2], a2[0][j + 3]);
+                *reinterpret_cast<float4*>(&s.a1[q][j]) = make_float4(a1[j], a1[j + 1], a1[j + 2], a1[j + 3]);
+                *reinterpret_cast<float4*>(&s.a2[q][j]) = make_float4(a2[j], a2[j + 1], a2[j + 2], a2[j + 3]);
                 *reinterpret_cast<float4*>(&s.d2[q][j]) = make_float4(d2[j], d2[j + 1], d2[j + 2], d2[j + 3]);
             }
-            *reinterpret_cast<float4*>(&s.a0[q][0]) = make_float4(a0[0][0], a0[0][1], a0[0][2], a0[0][3]);
-            *reinterpret_cast<float4*>(&s.a0[q][4]) = make_float4(a0[0][4], a0[0][5], 1.f, dy);
+            *reinterpret_cast<float4*>(&s.a0[q][0]) = make_float4(a0[0], a0[1], a0[2], a0[3]);
+            *reinterpret_cast<float4*>(&s.a0[q][4]) = make_float4(a0[4], a0[5], 1.f, dy);
             f32x2 acc[kH / 2];
 #pragma unroll
             for (int u = 0; u < kH / 2; ++u) acc[u] = 0ull;
@@ -332,10 +324,10 @@ __global__ void __launch_bounds__(kTile) mlp_grad_kernel(const float* __restrict
                 float4 d;
                 unpack2(acc[u], d.x, d.y);
                 unpack2(acc[u + 1], d.z, d.w);
-                d.x = a1[0][2 * u] > 0.f ? d.x : 0.f;
-                d.y = a1[0][2 * u + 1] > 0.f ? d.y : 0.f;
-                d.z = a1[0][2 * u + 2] > 0.f ? d.z : 0.f;
-                d.w = a1[0][2 * u + 3] > 0.f ? d.w : 0.f;
+                d.x = a1[2 * u] > 0.f ? d.x : 0.f;
+                d.y = a1[2 * u + 1] > 0.f ? d.y : 0.f;
+                d.z = a1[2 * u + 2] > 0.f ? d.z : 0.f;
+                d.w = a1[2 * u + 3] > 0.f ? d.w : 0.f;
                 *reinterpret_cast<float4*>(&s.d1[q][2 * u]) = d;
             }
         }
