@@ -667,8 +667,8 @@ __device__ __forceinline__ uint32_t chunk_in_row(int32_t off, int32_t d) {
 //
 // Bound: one 32-byte sector of colidx per vertex, and its row start, buffers and
 // worklist entry.  Reading every row to its end as one flat range took 0.71 ms
-// for R-MAT-B of 2^24 vertices (now 0.38; both with the setup scan, without it
-// now 0.29) and 0.24 for R-MAT-ER of 2^22 (now 0.10).
+// for R-MAT-B of 2^24 vertices (now 0.38; both with the setup scan, 0.07 of it)
+// and 0.24 for R-MAT-ER of 2^22 (now 0.10).
 //
 // PER vertices a thread: 4, or 1 for a range too small to give every SM a block
 // of 1,024.
