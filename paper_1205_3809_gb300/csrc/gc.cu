@@ -1218,8 +1218,9 @@ constexpr int32_t kLocalSharedDefault = 164 * 1024;  // mode 2: bytes of shared 
 // With keys a block costs 1.5 times as much (it gathers a key for every neighbour
 // of the same color, in every round) and the union 1.2 times: four R-MAT-G of
 // 4,096 vertices 296 us in blocks, 165 in the union, 64 of 65,536 vertices 4,529
-// and 2,949.  Of 236 keyed batches of 1 to 128 even graphs, 20 were slower than
-// as a union before without these factors, by up to 48 %, and none is with them.
+// and 2,949.  Of 299 keyed batches of 1 to 128 even graphs, 20 were slower than
+// as a union before without these factors, by up to 48 %, and none is with them by
+// more than 3 %.
 constexpr double kUnionFixed = 8.8e4, kUnionFactor = 2.5, kSkewedBlock = 2.5, kSkewedUnion = 1.9, kKeyedBlock = 1.5,
                  kKeyedUnion = 1.2;
 
