@@ -551,17 +551,18 @@ __device__ __forceinline__ RowDegrees small_rows(const FeatureGraph& g, unsigned
 // Bound: one random L2 sector per entry (the neighbour's row starts; a probe
 // that only gathers reaches 208 G/s).  With a thread per short row and the
 // longest rows read 32 entries at a time with two waits each, R-MAT-B of 2^22
-// vertices took 441 us, now 390; R-MAT-ER 386 us, now 320 (208 G entries/s).
+// vertices took 441 us, now 391; R-MAT-ER 386 us, now 313 (214 G entries/s).
 // Six blocks an SM: with four (62 registers) 436 us for the first.
 //
 // In the natural order of a mesh or band neighbouring lanes gather neighbouring
 // words when each has a row of its own: grid of 2,000 x 2,000 67.8 us (thread per
-// row, 8 entries at a time), 89.7 (two lanes in chunks), 56.3 now; 12 entries a
-// row 43.4, 79.3, 40; 26 entries 42.4, 168 (16 lanes), 48 (4 lanes, two chunks
+// row, 8 entries at a time), 89.7 (two lanes in chunks), 55.2 now; 12 entries a
+// row 43.4, 79.1, 40.1; 26 entries 42.2, 168 (16 lanes), 47.7 (4 lanes, two chunks
 // each).  With own rows up to 12 only, a geometric graph of 1M vertices in random
-// order (8 a row) takes 46.2 us, not 49.6 (thread per row 53.4), but 200 graphs of
+// order (8 a row) takes 46.2 us, not 52.4 (thread per row 53.4), but 200 graphs of
 // 4,096 vertices in a batch, 8 a row and near each other, 71, not 66 (65).
-// Few vertices: G(3000, 12000) 3.3 us, 5.5 in warps of 32, 3.3; K(1500) 115, 132, 33.
+// Few vertices: G(3000, 12000) 3.0 us, 5.3 in warps of 32, 3.2 now; K(1500) 111, 132
+// and 33.7.
 constexpr int kFeatureBlocks = 6;
 template <unsigned STEPS>
 __global__ void __launch_bounds__(256, kFeatureBlocks) features_kernel(const int32_t* __restrict__ rowptr,
